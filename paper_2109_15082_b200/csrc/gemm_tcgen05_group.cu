@@ -123,48 +123,53 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer
-    if (lane == 0) {
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0;
-      const uint32_t stage_adv = (uint32_t)g.stage_bytes >> 4;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        int local;
-        const TcParams& p = g.p[find_problem(g, tile, local)];
-        // descriptor words of this problem's operand layouts (see tc_gemm_kernel)
-        const uint32_t adv_a = (p.a_mn ? 2048u : 32u) >> 4, adv_b = (p.b_mn ? 2048u : 32u) >> 4;
-        const uint64_t proto_a = smem_desc(tiles_base, p.a_mn ? 8192u : 16u, 1024u);
-        const uint64_t proto_b = smem_desc(tiles_base + A_STAGE_BYTES, p.b_mn ? 8192u : 16u, 1024u);
-        const uint32_t a_hi = (uint32_t)(proto_a >> 32), b_hi = (uint32_t)(proto_b >> 32);
-        const uint32_t a_lo0 = (uint32_t)proto_a, b_lo0 = (uint32_t)proto_b;
-        uint32_t a_lo = a_lo0 + (uint32_t)stage * stage_adv, b_lo = b_lo0 + (uint32_t)stage * stage_adv;
-        if (!mbar_wait_or_abort(smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, vabort, g.p[0].wait_ns)) {
-          if (!*vabort) fail(p, DEV_TIMEOUT_EPI, vabort);
+    // ---------------- MMA issuer: the whole warp walks the loop, one elected lane issues (see elect_one)
+    const bool leader = elect_one();
+    int stage = 0, acc = 0;
+    uint32_t phase = 0, acc_phase = 0;
+    const uint32_t stage_adv = (uint32_t)g.stage_bytes >> 4;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      int local;
+      const TcParams& p = g.p[find_problem(g, tile, local)];
+      // descriptor words of this problem's operand layouts (see tc_gemm_kernel)
+      const uint32_t adv_a = (p.a_mn ? 2048u : 32u) >> 4, adv_b = (p.b_mn ? 2048u : 32u) >> 4;
+      const uint64_t proto_a = smem_desc(tiles_base, p.a_mn ? 8192u : 16u, 1024u);
+      const uint64_t proto_b = smem_desc(tiles_base + A_STAGE_BYTES, p.b_mn ? 8192u : 16u, 1024u);
+      const uint32_t a_hi = (uint32_t)(proto_a >> 32), b_hi = (uint32_t)(proto_b >> 32);
+      const uint32_t a_lo0 = (uint32_t)proto_a, b_lo0 = (uint32_t)proto_b;
+      uint32_t a_lo = a_lo0 + (uint32_t)stage * stage_adv, b_lo = b_lo0 + (uint32_t)stage * stage_adv;
+      const uint32_t idesc = p.idesc;
+      const int k_blocks = p.k_blocks;
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, vabort, g.p[0].wait_ns)) {
+        if (leader && !*vabort) fail(p, DEV_TIMEOUT_EPI, vabort);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t tmem_d = tmem_base + (uint32_t)(acc * p.block_n);
+      for (int kb = 0; kb < k_blocks; ++kb) {
+        if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, vabort, g.p[0].wait_ns)) {
+          if (leader && !*vabort) fail(p, DEV_TIMEOUT_TMA, vabort);
+          ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * p.block_n);
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!mbar_wait_or_abort(smem_u32(&full_bar[stage]), phase, vabort, g.p[0].wait_ns)) {
-            if (!*vabort) fail(p, DEV_TIMEOUT_TMA, vabort);
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          tc_mma_lohi<0>(tmem_d, a_lo, a_hi, b_lo, b_hi, p.idesc, (uint32_t)(kb != 0));
-          tc_mma_lohi<0>(tmem_d, a_lo + adv_a, a_hi, b_lo + adv_b, b_hi, p.idesc, 1u);
-          tc_mma_lohi<0>(tmem_d, a_lo + 2 * adv_a, a_hi, b_lo + 2 * adv_b, b_hi, p.idesc, 1u);
-          tc_mma_lohi<0>(tmem_d, a_lo + 3 * adv_a, a_hi, b_lo + 3 * adv_b, b_hi, p.idesc, 1u);
+        if (leader) {
+          tc_mma_lohi<0>(tmem_d, a_lo, a_hi, b_lo, b_hi, idesc, (uint32_t)(kb != 0));
+          tc_mma_lohi<0>(tmem_d, a_lo + adv_a, a_hi, b_lo + adv_b, b_hi, idesc, 1u);
+          tc_mma_lohi<0>(tmem_d, a_lo + 2 * adv_a, a_hi, b_lo + 2 * adv_b, b_hi, idesc, 1u);
+          tc_mma_lohi<0>(tmem_d, a_lo + 3 * adv_a, a_hi, b_lo + 3 * adv_b, b_hi, idesc, 1u);
           tc_commit(smem_u32(&empty_bar[stage]));
-          a_lo += stage_adv; b_lo += stage_adv;
-          if (++stage == g.num_stages) { stage = 0; phase ^= 1u; a_lo = a_lo0; b_lo = b_lo0; }
         }
-        if (!ok) break;
-        tc_commit(smem_u32(&tfull_bar[acc]));
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1u;
+        __syncwarp();
+        a_lo += stage_adv; b_lo += stage_adv;
+        if (++stage == g.num_stages) { stage = 0; phase ^= 1u; a_lo = a_lo0; b_lo = b_lo0; }
       }
+      if (!ok) break;
+      if (leader) tc_commit(smem_u32(&tfull_bar[acc]));
+      __syncwarp();
+      acc ^= 1;
+      if (acc == 0) acc_phase ^= 1u;
     }
   } else {
     // ---------------- epilogue warps: TMEM lane quadrant = warp % 4, two warps per quadrant, each draining
