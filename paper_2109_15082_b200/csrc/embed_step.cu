@@ -6,19 +6,25 @@
 //            table's row steps and the LayerNorm parameters; the update re-quantizes the word table.
 // The word table is treated as a weight matrix with `vocab` output rows: its quantizer, straight-through
 // mask and fused AdamW + re-quantization are the kernels of the encoder matrices; LayerNorm, loss and
-// column reductions likewise.  New here: the gather (codes x row scale, exact), the scatter of the token
-// gradients into table rows (every token that gathered a row, added in token order: no atomics) and the
-// reductions over the batch for the position and token-type tables.  Nothing is allocated: the caller
-// brings every tensor and one workspace.
+// column reductions likewise.  New here: everything per token (both gathers, both LayerNorms, the loss, its
+// gradient through the LayerNorm) in one kernel, and everything that adds up the token gradients (rows of the
+// word table, sums over the batch for the position and token-type tables) in a second one, with fixed
+// summation orders.  Nothing is allocated: the caller brings every tensor and one workspace.
 #include <cmath>
 
 #include "../../include/mrem.h"
-#include "kernels.h"
+#include "optim.cuh"
 #include "vec.cuh"
 
 namespace mrem {
 
 namespace {
+
+__device__ __forceinline__ void note_token(unsigned* row_first, int* row_last, int* row_count, int id, int t) {
+  atomicMin(row_first + id, (unsigned)t);
+  atomicMax(row_last + id, t);
+  atomicAdd(row_count + id, 1);                                     // (starts at -1)
+}
 
 // y[t, :] = row(ids[t]) + pos[t % S, :] + type[type_ids[t], :], rounded as stored; one block of 128 threads per token.
 // With codes the row is scale[id] * codes[id, :] (the quantized table), else word[id, :].
@@ -27,7 +33,8 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
                                                         const float* __restrict__ scale, const float* __restrict__ pos,
                                                         const float* __restrict__ type, const int* __restrict__ ids,
                                                         const int* __restrict__ type_ids, int S, int H, int vocab, int n_types,
-                                                        T* __restrict__ y, int* __restrict__ status) {
+                                                        T* __restrict__ y, unsigned* row_first, int* row_last,
+                                                        int* row_count, int* __restrict__ status) {
   pdl_trigger();
   pdl_wait();
   const long long t = blockIdx.x;
@@ -37,6 +44,7 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
     id = min(max(id, 0), vocab - 1);
     tt = min(max(tt, 0), n_types - 1);
   }
+  if (threadIdx.x == 0 && row_first) note_token(row_first, row_last, row_count, id, (int)t);
   const int s = (int)(t % S);
   const float sc = codes ? scale[id] : 0.f;
   for (int c = threadIdx.x; c < H; c += blockDim.x) {
@@ -45,103 +53,401 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
   }
 }
 
-// Occurrence lists of the batch's ids, without sorting and without atomics.  Per token t (one thread each):
-//   lead[t] = index of the first token with the id of token t,  rank[t] = number of earlier tokens with that id.
-__global__ void __launch_bounds__(256) embed_lead_kernel(const int* __restrict__ ids, int M, int vocab, int* __restrict__ lead,
-                                                         int* __restrict__ rank) {
-  pdl_trigger();
-  pdl_wait();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= M) return;
-  const int id = min(max(ids[t], 0), vocab - 1);
-  int first = t, r = 0;
-  for (int i = t - 1; i >= 0; --i)
-    if (min(max(ids[i], 0), vocab - 1) == id) { first = i; ++r; }
-  lead[t] = first;
-  rank[t] = r;
-}
-// list = the tokens grouped by id (groups ordered by their first token, token order inside a group):
-//   position of token t = number of tokens whose group starts before t's group + rank[t];
-// for the first token of a group also start[t] = that position and count[t] = size of the group (count 0 elsewhere).
-__global__ void __launch_bounds__(256) embed_list_kernel(const int* __restrict__ lead, const int* __restrict__ rank, int M,
-                                                         int* __restrict__ list, int* __restrict__ start, int* __restrict__ count) {
-  pdl_trigger();
-  pdl_wait();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= M) return;
-  const int mine = lead[t];
-  int before = 0, same = 0;
-  for (int i = 0; i < M; ++i) {
-    const int l = lead[i];
-    before += l < mine;
-    same += l == mine;
+// Everything that happens to one token, one warp per token (rows up to 32 * V * ROW_NV wide, held in registers): both
+// gathers, both LayerNorms, the squared error, its gradient and the LayerNorm's backward: the operations of the separate
+// kernels (embed_sum, ln_fwd, loss, ln_bwd) in their order, without their intermediates' round trips through memory and
+// without six of their seven launches.  The first and the last token of every id and their number are noted (atomicMin /
+// atomicMax of an index, atomicAdd of 1: no dependence on scheduling); they say later which table rows were gathered at
+// all, who adds up a row's gradients, and how far to look.  One block more than the tokens need prepares the optimizer's
+// scalars beside them.
+constexpr int ROW_NV = 4;
+struct EmbedRow {
+  const float *t_word, *t_pos, *t_type, *t_g, *t_b;           // teacher tables and LayerNorm
+  const float *pos, *type, *ln_g, *ln_b;
+  const int8_t* codes; const float* scale;
+  const int *ids, *type_ids;
+  int S, H, vocab, n_types; long long M;
+  float eps, c;                                               // c: loss scale
+  int* status; unsigned* row_first; int *row_last, *row_count; unsigned* ticket;   // marks and ticket start as 0xffffffff
+  float *mean, *rstd, *loss_partial, *loss;
+  int* col_counters; int n_col_counters;
+  int row_blocks; OptimArgs optim;
+};
+
+template <int V>
+__device__ __forceinline__ void load_f32(const float* p, float* v) {
+#pragma unroll
+  for (int j = 0; j < V; j += 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p + j));
+    v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
   }
-  list[before + rank[t]] = t;
-  start[t] = before;
-  count[t] = mine == t ? same : 0;
 }
 
-// g_word[id, :] = sum over the tokens t with ids[t] == id of dy[t, :], in token order: the block of the first
-// token with an id adds that id's group of the list for its 128 columns (independent loads); rows no token gathered
-// keep the zeros the caller put there.
-template <typename T>
-__global__ void __launch_bounds__(128) embed_scatter_kernel(const T* __restrict__ dy, const int* __restrict__ ids,
-                                                            const int* __restrict__ list, const int* __restrict__ start,
-                                                            const int* __restrict__ count, int H, int vocab,
-                                                            float* __restrict__ g_word) {
+// Mean and 1 / sqrt(variance + eps) of a row held in registers.
+template <int V>
+__device__ __forceinline__ void row_stats(const float (&y)[ROW_NV][V], int lane, int H, float eps, float& mu, float& rs) {
+  float sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < ROW_NV; ++i)
+    if ((lane + 32 * i) * V < H) {
+#pragma unroll
+      for (int j = 0; j < V; ++j) sum += y[i][j];
+    }
+  mu = warp_sum(sum) / (float)H;
+  float sq = 0.f;
+#pragma unroll
+  for (int i = 0; i < ROW_NV; ++i)
+    if ((lane + 32 * i) * V < H) {
+#pragma unroll
+      for (int j = 0; j < V; ++j) sq += (y[i][j] - mu) * (y[i][j] - mu);
+    }
+  rs = 1.f / sqrtf(warp_sum(sq) / (float)H + eps);
+}
+
+template <typename T, int V>
+__global__ void __launch_bounds__(128) embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra,
+                                                        T* __restrict__ e_t, T* __restrict__ e_s, T* __restrict__ y_s,
+                                                        T* __restrict__ dsum, T* __restrict__ dy) {
   pdl_trigger();
   pdl_wait();
-  const int t0 = blockIdx.x, n = count[t0];
-  if (n == 0) return;                                               // block-uniform: not the first token of its id
-  const int c = blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= H) return;
-  const int id = min(max(ids[t0], 0), vocab - 1);
-  const int* grp = list + start[t0];
-  float acc = 0.f;
-  for (int j = 0; j < n; ++j) acc += to_f<T>(dy[(long long)grp[j] * H + c]);
-  g_word[(long long)id * H + c] = acc;
+  __shared__ float sh[32];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, H = p.H;
+  if ((int)blockIdx.x == p.row_blocks) {
+    if (threadIdx.x == 0) optim_prepare(p.optim);
+    return;
+  }
+  if (blockIdx.x == 0)                                        // tickets of the column reduction that follows
+    for (int i = threadIdx.x; i < p.n_col_counters; i += blockDim.x) p.col_counters[i] = 0;
+  float err = 0.f;
+  for (long long t = blockIdx.x * 4ll + wid; t < p.M; t += p.row_blocks * 4ll) {
+    int id = p.ids[t], tt = p.type_ids ? p.type_ids[t] : 0;
+    if (id < 0 || id >= p.vocab || tt < 0 || tt >= p.n_types) {   // recorded, then clamped: no out-of-range access
+      if (lane == 0) atomicCAS(p.status, 0, (int)DEV_BAD_INDEX);
+      id = min(max(id, 0), p.vocab - 1);
+      tt = min(max(tt, 0), p.n_types - 1);
+    }
+    if (lane == 0) note_token(p.row_first, p.row_last, p.row_count, id, (int)t);
+    const long long row = (long long)id * H, prow = (t % p.S) * (long long)H, trow = (long long)tt * H, base = t * H;
+    float et[ROW_NV][V], y[ROW_NV][V];                        // teacher row, student row, as stored before the LayerNorm
+    const float sc = p.scale[id];
+#pragma unroll
+    for (int i = 0; i < ROW_NV; ++i) {
+      const int c = (lane + 32 * i) * V;
+      if (c < H) {
+        float a[V], b[V];
+        load_f32<V>(p.t_word + row + c, et[i]);
+        load_f32<V>(p.t_pos + prow + c, a);
+        load_f32<V>(p.t_type + trow + c, b);
+#pragma unroll
+        for (int j = 0; j < V; ++j) et[i][j] = stored<T>(et[i][j] + a[j] + b[j]);
+        // (the student's position and token-type rows are written by a later kernel of this step: no read-only loads)
+#pragma unroll
+        for (int j = 0; j < V; j += 4) {
+          const float4 pa = *reinterpret_cast<const float4*>(p.pos + prow + c + j), ta = *reinterpret_cast<const float4*>(p.type + trow + c + j);
+          const char4 q = *reinterpret_cast<const char4*>(p.codes + row + c + j);
+          y[i][j] = stored<T>(sc * (float)q.x + pa.x + ta.x);
+          y[i][j + 1] = stored<T>(sc * (float)q.y + pa.y + ta.y);
+          y[i][j + 2] = stored<T>(sc * (float)q.z + pa.z + ta.z);
+          y[i][j + 3] = stored<T>(sc * (float)q.w + pa.w + ta.w);
+        }
+        store_vec<T, V>(y_s + base + c, y[i]);
+      }
+    }
+    float mu, rs;
+    row_stats<V>(et, lane, H, p.eps, mu, rs);
+#pragma unroll
+    for (int i = 0; i < ROW_NV; ++i) {
+      const int c = (lane + 32 * i) * V;
+      if (c < H) {
+        float g[V], b[V];
+        load_f32<V>(p.t_g + c, g);
+        load_f32<V>(p.t_b + c, b);
+#pragma unroll
+        for (int j = 0; j < V; ++j) et[i][j] = (et[i][j] - mu) * rs * g[j] + b[j];
+        store_vec<T, V>(e_t + base + c, et[i]);
+      }
+    }
+    row_stats<V>(y, lane, H, p.eps, mu, rs);
+    if (lane == 0) { p.mean[t] = mu; p.rstd[t] = rs; }
+    // the student's output, the squared error, its gradient and what of it enters the LayerNorm: et becomes that gradient
+    // times gamma, y the normalised row
+    float s1 = 0.f, s2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < ROW_NV; ++i) {
+      const int c = (lane + 32 * i) * V;
+      if (c < H) {
+        float g[V], d[V];
+        load_f32<V>(p.ln_g + c, g);
+        load_f32<V>(p.ln_b + c, d);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          y[i][j] = (y[i][j] - mu) * rs;
+          d[j] = y[i][j] * g[j] + d[j];
+        }
+        store_vec<T, V>(e_s + base + c, d);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          const float diff = stored<T>(d[j]) - stored<T>(et[i][j]);
+          err += diff * diff;
+          d[j] = stored<T>(2.f * p.c * diff);
+        }
+        if (extra) {
+          float x[V];
+          load_vec<T, V>(extra + base + c, x);
+#pragma unroll
+          for (int j = 0; j < V; ++j) d[j] = stored<T>(d[j] + x[j]);
+        }
+        store_vec<T, V>(dsum + base + c, d);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          et[i][j] = d[j] * g[j];
+          s1 += et[i][j];
+          s2 += et[i][j] * y[i][j];
+        }
+      }
+    }
+    s1 = warp_sum(s1) / (float)H;
+    s2 = warp_sum(s2) / (float)H;
+#pragma unroll
+    for (int i = 0; i < ROW_NV; ++i) {
+      const int c = (lane + 32 * i) * V;
+      if (c < H) {
+        float o[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) o[j] = rs * (et[i][j] - s1 - y[i][j] * s2);
+        store_vec<T, V>(dy + base + c, o);
+      }
+    }
+  }
+  // per-block errors, added in block order by the last block to arrive
+  err = block_sum(err, sh);
+  if (threadIdx.x == 0) {
+    p.loss_partial[blockIdx.x] = err;
+    if (!isfinite(err)) atomicCAS(p.status, 0, (int)DEV_NONFINITE);
+    __threadfence();
+    last = atomicAdd(p.ticket, 1u) + 2u == (unsigned)p.row_blocks;   // (starts at 0xffffffff)
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  float a = 0.f;
+  for (int i = threadIdx.x; i < p.row_blocks; i += blockDim.x) a += __ldcg(p.loss_partial + i);
+  a = block_sum(a, sh);
+  if (threadIdx.x == 0) *p.loss = a * p.c;
 }
 
-// g_pos[s, c] = sum_b dy[b, s, c] (rows of the table beyond seq get zero).
-template <typename T>
-__global__ void __launch_bounds__(256) embed_pos_kernel(const T* __restrict__ dy, int B, int S, int H, float* __restrict__ g_pos) {
-  pdl_trigger();
-  pdl_wait();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x, row = blockIdx.y;
-  if (c >= H) return;
-  float acc = 0.f;
-  if (row < S)
-    for (int b = 0; b < B; ++b) acc += to_f<T>(dy[((long long)b * S + row) * H + c]);
-  g_pos[(long long)row * H + c] = acc;
-}
-
-// Token-type table, two stages with fixed orders: partial[chunk, k, c] = sum over the chunk's tokens of type k (token
-// order), then g_type[k, c] = sum over the chunks in index order.
+// Every sum over the token gradients dy in one launch (256 threads a block), and AdamW on the small tensors as their sums
+// become complete:
+//   max_pos blocks: one position each, two half sums over the batch (even and odd sequences), then that row's update.
+//   TYPE_CHUNKS blocks per token type: one chunk of tokens each; the last chunk to finish adds the chunks in index order
+//     and updates the row.
+//   one block: update of the LayerNorm's parameters (their gradients come from the launch before).
+//   the rest, one warp per token and group of TAB_COLS columns: word table.  The warp of the FIRST token with an id adds the gradients of all tokens with
+//     it in token order: it compares 128 ids at a time up to the last one and keeps four rows' loads in flight.  A row
+//     gathered by more than WARP_MAX tokens is left to the whole block, its warps taking consecutive eighths of the tokens and
+//     the eight sums being added in warp order.  Warp w of block i has token w * blocks + i: frequent ids first appear among
+//     the first tokens, and would otherwise all meet in one block.
+// The former occurrence lists (one thread per token walking all the others, twice) alone took 300 us at 4096 tokens; this
+// kernel takes 30 us (32 x 128 tokens, hidden 1024; embed_row_kernel 30, the table update 170 of the step's 240).
 constexpr int TYPE_CHUNKS = 64;
-template <typename T>
-__global__ void __launch_bounds__(256) embed_type_partial_kernel(const T* __restrict__ dy, const int* __restrict__ type_ids,
-                                                                 long long M, int H, int n_types, float* __restrict__ partial) {
-  pdl_trigger();
-  pdl_wait();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x, chunk = blockIdx.y, k = blockIdx.z;
-  if (c >= H) return;
-  const long long per = (M + TYPE_CHUNKS - 1) / TYPE_CHUNKS, t0 = chunk * per, t1 = t0 + per < M ? t0 + per : M;
-  float acc = 0.f;
-  for (long long t = t0; t < t1; ++t) {
-    const int tt = type_ids ? min(max(type_ids[t], 0), n_types - 1) : 0;
-    if (tt == k) acc += to_f<T>(dy[t * H + c]);
-  }
-  partial[((long long)chunk * n_types + k) * H + c] = acc;
+constexpr int TAB_COLS = 512;                                 // columns a word-table block works on
+constexpr int WARP_MAX = 16;                                  // tokens of one id that a single warp adds up
+struct EmbedTables {
+  const int *ids, *type_ids; const unsigned* row_first; const int *row_last, *row_count; unsigned* type_ticket;
+  int B, S, H, vocab, n_types, max_pos, M;
+  float *g_word, *g_pos, *g_type, *type_partial;
+  const OptimScalars* sc;                                     // null: gradients only
+  AdamEntry pos, type, ln_g, ln_b;
+};
+
+__device__ __forceinline__ void adam_at(const AdamEntry& e, const OptimScalars& o, long long i, float g) {
+  float m = e.m[i], v = e.v[i];
+  e.p[i] = adam_one(e.p[i], g, m, v, o, e.wd, e.min_value);
+  e.m[i] = m;
+  e.v[i] = v;
 }
-__global__ void __launch_bounds__(256) embed_type_final_kernel(const float* __restrict__ partial, int H, int n_types,
-                                                               float* __restrict__ g_type) {
+
+// acc += the rows dy[t, c0 ..] of the tokens t in [b0, b1) whose (clamped) id is `id`, in token order, by one warp.
+template <typename T, int V, int NV>
+__device__ __forceinline__ void add_rows_of_id(const EmbedTables& p, const T* __restrict__ dy, int id, int b0, int b1, int c0, int lane,
+                                               float (&acc)[NV][V]) {
+  constexpr int FLY = sizeof(T) == 2 ? 4 : 2;                 // rows in flight
+  const int H = p.H;
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+#pragma unroll
+    for (int j = 0; j < V; ++j) acc[i][j] = 0.f;
+  for (int b = b0; b < b1; b += 128) {
+    int mine[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mine[k] = b + 32 * k + lane < b1 ? min(max(p.ids[b + 32 * k + lane], 0), p.vocab - 1) : -1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      unsigned hits = __ballot_sync(0xffffffffu, mine[k] == id);
+      while (hits) {
+        uint32_t r[FLY][NV][RawWords<T, V>::N];
+        const int n = min(__popc(hits), FLY);
+#pragma unroll
+        for (int f = 0; f < FLY; ++f) {
+          if (f < n) {
+            const T* src = dy + (long long)(b + 32 * k + __ffs(hits) - 1) * H;
+            hits &= hits - 1;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+              const int c = c0 + (lane + 32 * i) * V;
+              if (c < H) load_raw<T, V>(src + c, r[f][i]);
+            }
+          }
+        }
+#pragma unroll
+        for (int f = 0; f < FLY; ++f) {
+          if (f < n) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+              if (c0 + (lane + 32 * i) * V < H) {
+                float v[V];
+                widen_raw<T, V>(r[f][i], v);
+#pragma unroll
+                for (int j = 0; j < V; ++j) acc[i][j] += v[j];
+              }
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+template <typename T, int V>
+__global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_constant__ EmbedTables p, const T* __restrict__ dy) {
   pdl_trigger();
   pdl_wait();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
-  if (c >= H) return;
-  float acc = 0.f;
-  for (int chunk = 0; chunk < TYPE_CHUNKS; ++chunk) acc += partial[((long long)chunk * n_types + k) * H + c];
-  g_type[(long long)k * H + c] = acc;
+  __shared__ float red[8][TAB_COLS];
+  __shared__ int flag, group[8];
+  constexpr int NV = TAB_COLS / (32 * V);                     // vectors per lane in a pass
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, H = p.H;
+  const int n_sum = p.max_pos + TYPE_CHUNKS * p.n_types;
+  OptimScalars o{};
+  if (p.sc) o = *p.sc;
+  int blk = (int)blockIdx.x;
+  if (blk < n_sum) {
+    // sums over rows of dy: threads 0..127 take the even rows of the set, 128..255 the odd ones
+    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7;
+    const bool is_pos = blk < p.max_pos;
+    if (!is_pos) blk -= p.max_pos;
+    const int s = blk, k = blk / TYPE_CHUNKS, chunk = blk % TYPE_CHUNKS;
+    const int per = (p.M + TYPE_CHUNKS - 1) / TYPE_CHUNKS, t0 = chunk * per, t1 = min(p.M, t0 + per);
+    float* dst = is_pos ? p.g_pos + (long long)s * H : p.type_partial + ((long long)chunk * p.n_types + k) * H;
+    for (int c0 = 0; c0 < H; c0 += 128 * V) {
+      const int c = c0 + tx * V;
+      float acc[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) acc[j] = 0.f;
+      if (c < H && is_pos && s < p.S) {
+#pragma unroll 8
+        for (int b = ty; b < p.B; b += 2) {
+          float v[V];
+          load_vec<T, V>(dy + ((long long)b * p.S + s) * H + c, v);
+#pragma unroll
+          for (int j = 0; j < V; ++j) acc[j] += v[j];
+        }
+      } else if (c < H && !is_pos) {
+#pragma unroll 8
+        for (int t = t0 + ty; t < t1; t += 2) {
+          const int tt = p.type_ids ? min(max(p.type_ids[t], 0), p.n_types - 1) : 0;
+          float v[V];
+          load_vec<T, V>(dy + (long long)t * H + c, v);
+#pragma unroll
+          for (int j = 0; j < V; ++j) acc[j] += tt == k ? v[j] : 0.f;
+        }
+      }
+      if (ty == 1) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) red[j][tx] = acc[j];
+      }
+      __syncthreads();
+      if (ty == 0) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) red[j][tx] += acc[j];
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < 128 * V && c0 + i < H; i += 256) {
+        const float g = red[i % V][i / V];
+        dst[c0 + i] = g;
+        if (is_pos && p.sc) adam_at(p.pos, o, (long long)s * H + c0 + i, g);
+      }
+      __syncthreads();
+    }
+    if (is_pos) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + k, 1u) + 2u == (unsigned)TYPE_CHUNKS;   // (starts at 0xffffffff)
+    __syncthreads();
+    if (!flag) return;
+    __threadfence();
+    for (int c = threadIdx.x; c < H; c += 256) {
+      float acc = 0.f;
+#pragma unroll 8
+      for (int ch = 0; ch < TYPE_CHUNKS; ++ch) acc += __ldcg(p.type_partial + ((long long)ch * p.n_types + k) * H + c);
+      p.g_type[(long long)k * H + c] = acc;
+      if (p.sc) adam_at(p.type, o, (long long)k * H + c, acc);
+    }
+    return;
+  }
+  blk -= n_sum;
+  if (blk == 0) {
+    if (p.sc)
+      for (int c = threadIdx.x; c < H; c += 256) {
+        adam_at(p.ln_g, o, c, p.ln_g.g[c]);
+        adam_at(p.ln_b, o, c, p.ln_b.g[c]);
+      }
+    return;
+  }
+  const int nb = (p.M + 7) / 8, c0 = ((blk - 1) / nb) * TAB_COLS;
+  blk = (blk - 1) % nb;
+  const int tok = wid * nb + blk;
+  int mine = -1, count = 0;                                   // id whose row this warp's token is the first to gather
+  if (tok < p.M) {
+    const int id = min(max(p.ids[tok], 0), p.vocab - 1);
+    if (p.row_first[id] == (unsigned)tok) { mine = id; count = p.row_count[id] + 1; }
+  }
+  if (lane == 0) group[wid] = count > WARP_MAX ? mine : -1;
+  if (mine >= 0 && count <= WARP_MAX) {
+    const int end = count == 1 ? tok + 1 : p.row_last[mine] + 1;
+    float acc[NV][V];
+    add_rows_of_id<T, V, NV>(p, dy, mine, tok, end, c0, lane, acc);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = c0 + (lane + 32 * i) * V;
+      if (c < H) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4)
+          *reinterpret_cast<float4*>(p.g_word + (long long)mine * H + c + j) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+      }
+    }
+  }
+  __syncthreads();
+  for (int k = 0; k < 8; ++k) {
+    const int id = group[k];
+    if (id < 0) continue;
+    const int t0 = k * nb + blk, end = p.row_last[id] + 1, seg = (end - t0 + 7) / 8;
+    const int b0 = t0 + wid * seg, b1 = min(end, b0 + seg);
+    float acc[NV][V];
+    add_rows_of_id<T, V, NV>(p, dy, id, b0, b1, c0, lane, acc);
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+#pragma unroll
+      for (int j = 0; j < V; ++j) red[wid][(lane + 32 * i) * V + j] = acc[i][j];
+    __syncthreads();
+    for (int c = threadIdx.x; c < TAB_COLS && c0 + c < H; c += 256) {
+      float a = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) a += red[w][c];
+      p.g_word[(long long)id * H + c0 + c] = a;
+    }
+    __syncthreads();
+  }
 }
 
 struct Carve {                         // the workspace, cut the same way by the sizing call and by the step
@@ -155,8 +461,9 @@ struct EmbedScratch {
   long long col_plane;
   int* col_counters;
   int8_t* codes; int32_t* rowsum; float* scale;
-  OptimScalars* optim_sc; AdamEntry* table;
-  int *lead, *rank, *list, *start, *count; float* type_partial;
+  OptimScalars* optim_sc;
+  unsigned* marks; size_t mark_bytes;      // first and last token of every id and their number, then the loss and token-type tickets
+  float* type_partial;
   size_t bytes;
 };
 EmbedScratch carve(const mrem_embed_desc& d, long long max_tokens, void* base) {
@@ -174,10 +481,8 @@ EmbedScratch carve(const mrem_embed_desc& d, long long max_tokens, void* base) {
   s.rowsum = (int32_t*)A.take(sizeof(int32_t) * d.vocab);
   s.scale = (float*)A.take(sizeof(float) * d.vocab);
   s.optim_sc = (OptimScalars*)A.take(sizeof(OptimScalars));
-  s.table = (AdamEntry*)A.take(sizeof(AdamEntry) * 4);
-  s.lead = (int*)A.take(sizeof(int) * max_tokens); s.rank = (int*)A.take(sizeof(int) * max_tokens);
-  s.list = (int*)A.take(sizeof(int) * max_tokens); s.start = (int*)A.take(sizeof(int) * max_tokens);
-  s.count = (int*)A.take(sizeof(int) * max_tokens);
+  s.mark_bytes = sizeof(unsigned) * (3 * (size_t)d.vocab + 1 + d.n_types);
+  s.marks = (unsigned*)A.take(s.mark_bytes);
   s.type_partial = (float*)A.take(sizeof(float) * (size_t)TYPE_CHUNKS * d.n_types * d.hidden);
   s.bytes = (A.off + 255) & ~size_t(255);
   return s;
@@ -232,55 +537,72 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
 
   // Eq. 1 on the word table (only when the caller changed it or its steps since the last update)
   if (requantize) launch_quantize_weight(x->word, V, H, x->word_step, 1, d->e_bits, 0, s.codes, s.rowsum, s.scale, nullptr, dt, st);
-  // both embedding outputs
-#define MREM_EMB(T) do { \
-    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, x->t_word, (const int8_t*)nullptr, (const float*)nullptr, x->t_pos, x->t_type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_t, d_status); \
-    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, (const float*)x->word, (const int8_t*)s.codes, (const float*)s.scale, (const float*)x->pos, (const float*)x->type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_s, d_status); } while (0)
-  if (dt == 1) MREM_EMB(bf16); else MREM_EMB(float);
-#undef MREM_EMB
-  launch_layernorm_fwd(s.y_t, x->t_ln_g, x->t_ln_b, d->ln_eps, M, H, d_e_teacher, nullptr, nullptr, nullptr, 0, nullptr, nullptr, dt, st);
-  launch_layernorm_fwd(s.y_s, x->ln_g, x->ln_b, d->ln_eps, M, H, d_e_student, s.mean, s.rstd, nullptr, 0, nullptr, nullptr, dt, st);
-  // loss and its gradient
   const long long n = M * H;
   const float cc = d->loss_mean ? 1.f / (float)n : 1.f;
-  launch_loss(d_e_student, d_e_teacher, 1, n, cc, s.dE, s.loss_partial, d_status, dt, st);
-  launch_loss_finalize(s.loss_partial, 1, cc, d_loss, nullptr, st);
-  // LayerNorm backward and its parameter gradients
-  // (with a gradient arriving from the layers the embedding feeds, the LayerNorm sees the sum of the two)
   if (d_extra_grad && (reinterpret_cast<uintptr_t>(d_extra_grad) & 15)) return MREM_ERR_ALIGN;
-  launch_layernorm_bwd(s.dE, d_extra_grad, s.y_s, s.mean, s.rstd, x->ln_g, M, H, s.dy, d_extra_grad ? s.dsum : nullptr, dt, st);
-  if (cudaMemsetAsync(s.col_counters, 0, sizeof(int) * (H / 32 + 2), st) != cudaSuccess) return MREM_ERR_CUDA;
-  launch_col_reduce(d_extra_grad ? s.dsum : s.dE, H, s.y_s, s.mean, s.rstd, nullptr, 0, M, H, x->g_ln_b, x->g_ln_g, nullptr, s.col_scratch, s.col_plane,
+  if (cudaMemsetAsync(s.marks, 0xff, s.mark_bytes, st) != cudaSuccess) return MREM_ERR_CUDA;
+  unsigned* row_first = s.marks;
+  int *row_last = (int*)(s.marks + V), *row_count = row_last + V;
+  unsigned *loss_ticket = s.marks + 3 * (size_t)V, *type_ticket = loss_ticket + 1;
+  bool aligned = true;                                     // 16-byte accesses of the tables' rows
+  const float* const rows[] = {x->t_word, x->t_pos, x->t_type, x->t_ln_g, x->t_ln_b, x->pos, x->type, x->ln_g, x->ln_b};
+  for (const float* q : rows) aligned = aligned && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+  void* dsum = s.dsum;                                     // the gradient the LayerNorm sees
+  OptimArgs oa{};
+  if (o) oa = OptimArgs{s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay};
+  if (H <= 32 * (dt == 1 ? 8 : 4) * ROW_NV && aligned) {
+    // the row fits a warp's registers: everything per token in one kernel
+    const int row_blocks = (int)((M + 3) / 4 < RED_BLOCKS ? (M + 3) / 4 : RED_BLOCKS);
+    const EmbedRow er{x->t_word, x->t_pos, x->t_type, x->t_ln_g, x->t_ln_b, x->pos, x->type, x->ln_g, x->ln_b, s.codes, s.scale, d_ids, d_type_ids,
+                      (int)seq, H, V, (int)d->n_types, M, d->ln_eps, cc, d_status, row_first, row_last, row_count, loss_ticket,
+                      s.mean, s.rstd, s.loss_partial, d_loss, s.col_counters, H / 32 + 2, row_blocks, oa};
+    const unsigned grid = (unsigned)(row_blocks + (o ? 1 : 0));
+    Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)), 0, st);
+    if (dt == 1)
+      launch_k(embed_row_kernel<bf16, 8>, grid, 128, 0, st, er, (const bf16*)d_extra_grad, (bf16*)d_e_teacher, (bf16*)d_e_student, (bf16*)s.y_s, (bf16*)s.dsum, (bf16*)s.dy);
+    else
+      launch_k(embed_row_kernel<float, 4>, grid, 128, 0, st, er, (const float*)d_extra_grad, (float*)d_e_teacher, (float*)d_e_student, (float*)s.y_s, (float*)s.dsum, (float*)s.dy);
+  } else {
+    // wide rows: both embedding sums, the two LayerNorms, the loss and the LayerNorm backward as kernels of their own
+#define MREM_EMB(T) do { \
+    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, x->t_word, (const int8_t*)nullptr, (const float*)nullptr, x->t_pos, x->t_type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_t, (unsigned*)nullptr, (int*)nullptr, (int*)nullptr, d_status); \
+    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, (const float*)x->word, (const int8_t*)s.codes, (const float*)s.scale, (const float*)x->pos, (const float*)x->type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_s, row_first, row_last, row_count, d_status); } while (0)
+    if (dt == 1) MREM_EMB(bf16); else MREM_EMB(float);
+#undef MREM_EMB
+    launch_layernorm_fwd(s.y_t, x->t_ln_g, x->t_ln_b, d->ln_eps, M, H, d_e_teacher, nullptr, nullptr, nullptr, 0, nullptr, nullptr, dt, st);
+    launch_layernorm_fwd(s.y_s, x->ln_g, x->ln_b, d->ln_eps, M, H, d_e_student, s.mean, s.rstd, nullptr, 0, nullptr, nullptr, dt, st);
+    launch_loss(d_e_student, d_e_teacher, 1, n, cc, s.dE, s.loss_partial, d_status, dt, st);
+    launch_loss_finalize(s.loss_partial, 1, cc, d_loss, nullptr, st);
+    // (with a gradient arriving from the layers the embedding feeds, the LayerNorm sees the sum of the two)
+    launch_layernorm_bwd(s.dE, d_extra_grad, s.y_s, s.mean, s.rstd, x->ln_g, M, H, s.dy, d_extra_grad ? s.dsum : nullptr, dt, st);
+    if (cudaMemsetAsync(s.col_counters, 0, sizeof(int) * (H / 32 + 2), st) != cudaSuccess) return MREM_ERR_CUDA;
+    if (!d_extra_grad) dsum = s.dE;
+    if (o) launch_optim_prepare(s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay, st);
+  }
+  launch_col_reduce(dsum, H, s.y_s, s.mean, s.rstd, nullptr, 0, M, H, x->g_ln_b, x->g_ln_g, nullptr, s.col_scratch, s.col_plane,
                     s.col_counters, dt, st);
-  // position / token-type tables: sums over the batch; word table: every token's gradient into the row it gathered
-  if (cudaMemsetAsync(x->g_word, 0, sizeof(float) * (size_t)V * H, st) != cudaSuccess) return MREM_ERR_CUDA;
-  launch_k(embed_lead_kernel, (unsigned)((M + 255) / 256), 256, 0, st, d_ids, (int)M, V, s.lead, s.rank);
-  launch_k(embed_list_kernel, (unsigned)((M + 255) / 256), 256, 0, st, (const int*)s.lead, (const int*)s.rank, (int)M, s.list, s.start, s.count);
-  const dim3 gcol((H + 255) / 256), gscat((unsigned)M, (H + 127) / 128);
-#define MREM_EMB_BWD(T) do { \
-    launch_k(embed_pos_kernel<T>, dim3(gcol.x, d->max_pos), 256, 0, st, (const T*)s.dy, (int)batch, (int)seq, H, x->g_pos); \
-    launch_k(embed_type_partial_kernel<T>, dim3(gcol.x, TYPE_CHUNKS, d->n_types), 256, 0, st, (const T*)s.dy, d_type_ids, M, H, (int)d->n_types, s.type_partial); \
-    launch_k(embed_scatter_kernel<T>, gscat, 128, 0, st, (const T*)s.dy, d_ids, (const int*)s.list, (const int*)s.start, (const int*)s.count, H, V, x->g_word); } while (0)
-  if (dt == 1) MREM_EMB_BWD(bf16); else MREM_EMB_BWD(float);
-#undef MREM_EMB_BWD
-  launch_k(embed_type_final_kernel, dim3(gcol.x, d->n_types), 256, 0, st, (const float*)s.type_partial, H, (int)d->n_types, x->g_type);
+  // word, position and token-type tables: sums of the token gradients.  Rows of the word table that no token gathered are
+  // cleared by the update (row_first says which they are), without one here.
+  if (!o && cudaMemsetAsync(x->g_word, 0, sizeof(float) * (size_t)V * H, st) != cudaSuccess) return MREM_ERR_CUDA;
+  const EmbedTables tb{d_ids, d_type_ids, row_first, row_last, row_count, type_ticket, (int)batch, (int)seq, H, V, (int)d->n_types,
+                       (int)d->max_pos, (int)M, x->g_word, x->g_pos, x->g_type, s.type_partial, o ? s.optim_sc : nullptr,
+                       {x->pos, x->g_pos, x->m_pos, x->v_pos, 0, 1.f, -INFINITY}, {x->type, x->g_type, x->m_type, x->v_type, 0, 1.f, -INFINITY},
+                       {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, 0, 0.f, -INFINITY}, {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, 0, 0.f, -INFINITY}};
+  const unsigned tgrid = (unsigned)(d->max_pos + (long long)TYPE_CHUNKS * d->n_types + 1 + ((M + 7) / 8) * ((H + TAB_COLS - 1) / TAB_COLS));
+  {
+    Scope sc("embed_tables", (double)M * H * 3.0 * (dt == 1 ? 2.0 : 4.0), 0, st);
+    if (dt == 1) launch_k(embed_tables_kernel<bf16, 8>, tgrid, 256, 0, st, tb, (const bf16*)s.dy);
+    else launch_k(embed_tables_kernel<float, 4>, tgrid, 256, 0, st, tb, (const float*)s.dy);
+  }
   if (!o) {
     // gradients only: the word table's straight-through mask and its row-step gradients, left in g_word / g_word_step
     launch_ste_weight(x->word, x->word_step, 1, d->e_bits, 0, x->g_word, V, H, x->g_word_step, st);
     return cudaGetLastError() == cudaSuccess ? MREM_OK : MREM_ERR_CUDA;
   }
-  // update: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one pass;
-  // the small tensors through the table kernel (embedding tables decayed like weight matrices, LayerNorm not)
-  launch_optim_prepare(s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay, st);
+  // update of the word table: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one
+  // pass (the small tensors, the other embedding tables decayed like weight matrices, LayerNorm not, are updated above)
   launch_fused_weight_update(x->word, x->g_word, x->m_word, x->v_word, x->word_step, nullptr, x->m_word_step, x->v_word_step, s.optim_sc,
-                             V, H, d->e_bits, 0, 1, 1, s.codes, s.rowsum, s.scale, nullptr, dt, st);
-  const AdamEntry host[4] = {
-      {x->pos, x->g_pos, x->m_pos, x->v_pos, (long long)d->max_pos * H, 1.f, -INFINITY},
-      {x->type, x->g_type, x->m_type, x->v_type, (long long)d->n_types * H, 1.f, -INFINITY},
-      {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, H, 0.f, -INFINITY},
-      {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, H, 0.f, -INFINITY}};
-  if (cudaMemcpyAsync(s.table, host, sizeof(host), cudaMemcpyHostToDevice, st) != cudaSuccess) return MREM_ERR_CUDA;
-  launch_adamw_table(s.table, 4, (long long)(d->max_pos + d->n_types + 2) * H, s.optim_sc, st);
+                             V, H, d->e_bits, 0, 1, 1, s.codes, s.rowsum, s.scale, nullptr, dt, st, row_first);
   return cudaGetLastError() == cudaSuccess ? MREM_OK : MREM_ERR_CUDA;
 }
 

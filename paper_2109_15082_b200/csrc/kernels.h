@@ -167,6 +167,8 @@ void launch_effective_bias(const float* b, const float* beta, const float* wscal
 // bc = 1 - beta^t; lr_bc1 = lr / bc1, rsqrt_bc2 = 1 / sqrt(bc2)
 struct OptimScalars { float lr, beta1, beta2, eps, bc1, bc2, weight_decay, lr_bc1, rsqrt_bc2; };
 struct AdamEntry { float* p; const float* g; float* m; float* v; long long n; float wd; float min_value; };   // wd: 1 = decayed
+// What optim_prepare (optim.cuh) needs: where the scalars go, the device step counter, and the caller's numbers.
+struct OptimArgs { OptimScalars* out; int* d_t; int host_t; float lr0; int total; float beta1, beta2, eps, weight_decay; };
 // Computes the scalars of this step on the device: t = ++(*d_t) (or host_t when >= 1),
 // lr = lr0 * (1 - (t-1)/total) when total > 0 else lr0.
 void launch_optim_prepare(OptimScalars* d_out, int* d_t, int host_t, float lr0, int total_steps, float beta1,
@@ -176,11 +178,12 @@ void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total
 
 // Fused per-row update of a weight matrix and its per-row steps: step gradient (or ds_in when the
 // gradients were already masked), AdamW on step and weights, re-quantization (codes, row sums,
-// scale, dequantized row).
-void launch_fused_weight_update(float* w, const float* g, float* m, float* v, float* steps, const float* ds_in,
+// scale, dequantized row).  row_used (may be null): one word per row, 0xffffffff where no gradient arrived; such a row's
+// g is taken as zero without being read, and written as zero (grid 0 only).
+void launch_fused_weight_update(float* w, float* g, float* m, float* v, float* steps, const float* ds_in,
                                 float* m_s, float* v_s, const OptimScalars* sc, int rows, int cols, int bits, int grid,
                                 int train_w, int train_s, int8_t* codes, int32_t* rowsum, float* scale, void* what,
-                                int dt, cudaStream_t st);
+                                int dt, cudaStream_t st, const unsigned* row_used = nullptr);
 
 // ---- step-size initialisation
 // Per-row max|w| or mean|w| -> steps (per row, or one value when !per_row: two passes).

@@ -312,24 +312,10 @@ __global__ void effective_bias_kernel(const float* __restrict__ b, const float* 
 }
 
 // ------------------------------------------------------------------ AdamW
-__global__ void optim_prepare_kernel(OptimScalars* out, int* d_t, int host_t, float lr0, int total, float b1, float b2,
-                                     float eps, float wd) {
+__global__ void optim_prepare_kernel(const __grid_constant__ OptimArgs a) {
   pdl_trigger();
   pdl_wait();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int t = host_t >= 1 ? host_t : (*d_t + 1);
-  *d_t = t;
-  OptimScalars o;
-  o.lr = total > 0 ? lr0 * fmaxf(1.f - (float)(t - 1) / (float)total, 0.f) : lr0;
-  o.beta1 = b1;
-  o.beta2 = b2;
-  o.eps = eps;
-  o.weight_decay = wd;
-  o.bc1 = (float)(1.0 - pow((double)b1, (double)t));
-  o.bc2 = (float)(1.0 - pow((double)b2, (double)t));
-  o.lr_bc1 = (float)((double)o.lr / (1.0 - pow((double)b1, (double)t)));
-  o.rsqrt_bc2 = (float)(1.0 / sqrt(1.0 - pow((double)b2, (double)t)));
-  *out = o;
+  if (threadIdx.x == 0 && blockIdx.x == 0) optim_prepare(a);
 }
 
 __global__ void __launch_bounds__(256) adamw_table_kernel(const AdamEntry* __restrict__ table,
@@ -460,7 +446,7 @@ void launch_effective_bias(const float* b, const float* beta, const float* wscal
 
 void launch_optim_prepare(OptimScalars* d_out, int* d_t, int host_t, float lr0, int total_steps, float beta1,
                           float beta2, float eps, float weight_decay, cudaStream_t st) {
-  launch_k(optim_prepare_kernel, 1, 32, 0, st, d_out, d_t, host_t, lr0, total_steps, beta1, beta2, eps, weight_decay);
+  launch_k(optim_prepare_kernel, 1, 32, 0, st, OptimArgs{d_out, d_t, host_t, lr0, total_steps, beta1, beta2, eps, weight_decay});
 }
 void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, const OptimScalars* d_sc,
                         cudaStream_t st) {

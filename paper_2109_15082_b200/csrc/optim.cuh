@@ -13,6 +13,24 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   return y;
 }
 
+// The scalars of one optimizer step (one thread): t = ++(*d_t), or host_t when >= 1; lr decayed linearly when total > 0.
+__device__ __forceinline__ void optim_prepare(const OptimArgs& a) {
+  const int t = a.host_t >= 1 ? a.host_t : (*a.d_t + 1);
+  *a.d_t = t;
+  const double bc1 = 1.0 - pow((double)a.beta1, (double)t), bc2 = 1.0 - pow((double)a.beta2, (double)t);
+  OptimScalars o;
+  o.lr = a.total > 0 ? a.lr0 * fmaxf(1.f - (float)(t - 1) / (float)a.total, 0.f) : a.lr0;
+  o.beta1 = a.beta1;
+  o.beta2 = a.beta2;
+  o.eps = a.eps;
+  o.weight_decay = a.weight_decay;
+  o.bc1 = (float)bc1;
+  o.bc2 = (float)bc2;
+  o.lr_bc1 = (float)((double)o.lr / bc1);
+  o.rsqrt_bc2 = (float)(1.0 / sqrt(bc2));
+  *a.out = o;
+}
+
 // p <- max(p * (1 - lr*wd) - lr * (m/bc1) / (sqrt(v/bc2) + eps), min_value); m, v updated in place.
 __device__ __forceinline__ float adam_one(float p, float g, float& m, float& v, const OptimScalars& o, float wd_on,
                                           float min_value) {

@@ -49,13 +49,15 @@ __device__ __forceinline__ void store_what4<bf16>(bf16* p, float a, float b, flo
 // NT threads per row, NV float4 vectors per thread kept in registers: (256, 1) for rows up to 1024 wide,
 // (512, 2) up to 4096; wider rows are re-read.
 // GRID (the weight grid, 0: Eq. 1's integers, 1: half-integer 2-bit levels) is a template parameter: the per-weight code
-// then holds one of the two rules, not both under predicates.
-template <typename T, int NV, int NT, int GRID>
+// then holds one of the two rules, not both under predicates.  SPARSE: row_used says which rows got a gradient at all (an
+// embedding table); its own variant, because the dense one is at the register limit of its occupancy.
+template <typename T, int NV, int NT, int GRID, bool SPARSE>
 __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_kernel(
-    float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
+    float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
     float* __restrict__ steps, const float* __restrict__ ds_in, float* __restrict__ m_s, float* __restrict__ v_s,
     const OptimScalars* __restrict__ sc, int cols, int bits, int train_w, int train_s,
-    int8_t* __restrict__ codes, int32_t* __restrict__ rowsum, float* __restrict__ scale, T* __restrict__ what) {
+    int8_t* __restrict__ codes, int32_t* __restrict__ rowsum, float* __restrict__ scale, T* __restrict__ what,
+    const unsigned* __restrict__ row_used) {
   pdl_trigger();
   pdl_wait();
   constexpr int grid = GRID;
@@ -63,6 +65,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
   __shared__ int shi[32];
   __shared__ float s_new_sh;
   const int row = blockIdx.x;
+  // a row marked 0xffffffff got no gradient: g is not read, and is cleared here instead of by a pass before this one
+  const bool no_grad = SPARSE && row_used[row] == 0xffffffffu;
   const OptimScalars o = *sc;
   const float s_old = steps[row];
   const float r_old = __frcp_rn(s_old);
@@ -73,7 +77,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
   const int nvec = cols / 4;                                   // cols is a multiple of 16
   const bool cached = nvec <= NV * NT;
   const float4* w4 = reinterpret_cast<const float4*>(w + base);
-  const float4* g4 = reinterpret_cast<const float4*>(g + base);
+  float4* g4 = reinterpret_cast<float4*>(g + base);
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 wr[NV], gr[NV], mr[NV], vr[NV];
   const float4* m4c = reinterpret_cast<const float4*>(m + base);
   const float4* v4c = reinterpret_cast<const float4*>(v + base);
@@ -85,7 +90,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
     for (int i = 0; i < NV; ++i) {
       const int c = threadIdx.x + i * NT;
       if (c < nvec) {
-        wr[i] = w4[c]; gr[i] = g4[c];
+        wr[i] = w4[c];
+        if (no_grad) { gr[i] = zero4; g4[c] = zero4; } else gr[i] = g4[c];
         if (train_w) { mr[i] = m4c[c]; vr[i] = v4c[c]; }
       }
     }
@@ -105,7 +111,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
   }
   if (!cached) {
     for (int c = threadIdx.x; c < nvec; c += NT) {
-      const float4 wv = w4[c], d = g4[c];
+      if (no_grad) g4[c] = zero4;
+      const float4 wv = w4[c], d = no_grad ? zero4 : g4[c];
       bool in;
       ds = step_grad_acc(ds, wv.x, d.x, s_old, r_old, qmax, grid, in);
       ds = step_grad_acc(ds, wv.y, d.y, s_old, r_old, qmax, grid, in);
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
   } else {
     for (int c = threadIdx.x; c < nvec; c += NT) {
       const float4 wv = w4[c];
-      float4 d = g4[c];
+      float4 d = no_grad ? zero4 : g4[c];
       if (!ds_in) {
         bool in;
         float lvl;
@@ -189,13 +196,13 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 6 : 2) fused_weight_update_ker
 
 }  // namespace
 
-void launch_fused_weight_update(float* w, const float* g, float* m, float* v, float* steps, const float* ds_in,
+void launch_fused_weight_update(float* w, float* g, float* m, float* v, float* steps, const float* ds_in,
                                 float* m_s, float* v_s, const OptimScalars* sc, int rows, int cols, int bits, int grid,
                                 int train_w, int train_s, int8_t* codes, int32_t* rowsum, float* scale, void* what,
-                                int dt, cudaStream_t st) {
+                                int dt, cudaStream_t st, const unsigned* row_used) {
   Scope scope("fused_weight_update", (double)rows * cols * (29.0 + (what ? (dt == 1 ? 2.0 : 4.0) : 0.0)), 0, st);
-#define MREM_FWU_G(T, NV, NT, G) launch_k(fused_weight_update_kernel<T, NV, NT, G>, rows, NT, 0, st, w, g, m, v, steps, ds_in, m_s, v_s, sc, cols, bits, train_w, train_s, codes, rowsum, scale, (T*)what)
-#define MREM_FWU(T, NV, NT) do { if (grid == 0) MREM_FWU_G(T, NV, NT, 0); else MREM_FWU_G(T, NV, NT, 1); } while (0)
+#define MREM_FWU_G(T, NV, NT, G, SP) launch_k(fused_weight_update_kernel<T, NV, NT, G, SP>, rows, NT, 0, st, w, g, m, v, steps, ds_in, m_s, v_s, sc, cols, bits, train_w, train_s, codes, rowsum, scale, (T*)what, row_used)
+#define MREM_FWU(T, NV, NT) do { if (grid != 0) MREM_FWU_G(T, NV, NT, 1, false); else if (row_used) MREM_FWU_G(T, NV, NT, 0, true); else MREM_FWU_G(T, NV, NT, 0, false); } while (0)
   if (dt == 1) { if (cols <= 1024) MREM_FWU(bf16, 1, 256); else MREM_FWU(bf16, 2, 512); }
   else { if (cols <= 1024) MREM_FWU(float, 1, 256); else MREM_FWU(float, 2, 512); }
 #undef MREM_FWU

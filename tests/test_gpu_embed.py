@@ -88,6 +88,36 @@ def test_embedding_step_matches_the_oracle(act_dtype, e_bits, sizes):
     assert abs(loss_after - r2["loss"]) / r2["loss"] < 2e-2
 
 
+# row widths on both sides of what a warp holds (1024 bf16, 512 float32), token counts that are no multiple of a block's
+# eight, every token on one id, every token on its own; tolerances as above
+@pytest.mark.parametrize("act_dtype,H,batch,seq,kind", [("bf16", 16, 1, 8, "zipf"), ("bf16", 1024, 3, 11, "same"), ("bf16", 1040, 3, 11, "zipf"),
+                                                        ("f32", 512, 2, 9, "distinct"), ("f32", 528, 2, 9, "same"), ("bf16", 192, 7, 47, "same")])
+def test_embedding_sums_at_the_edges_of_their_kernels(act_dtype, H, batch, seq, kind):
+    e, desc, teacher, student, step, ids, tt = _problem(act_dtype, 4, H=H, batch=batch, seq=seq)
+    if kind == "same":
+        ids = np.full_like(ids, 7)
+    elif kind == "distinct":
+        ids = np.ascontiguousarray(np.arange(ids.size, dtype=np.int32).reshape(ids.shape)[::-1] * 3)
+    d_ids, d_tt = torch.from_numpy(ids).to(e.device), torch.from_numpy(tt).to(e.device)
+    r = O.embed_loss_backward(desc, teacher, student, step, 4, ids, tt)
+    for g in e.g.values():
+        g.fill_(float("nan"))                                            # every entry has to be written
+    loss = float(e.step(d_ids, d_tt, None)[0])
+    assert abs(loss - r["loss"]) <= 2e-2 * r["loss"] and int(e.status[0]) == 0
+    for k in ("word", "pos", "type", "ln_g", "ln_b", "word_step"):
+        assert rel(e.g[k].cpu().numpy(), r["grads"][k]) < 2e-2, k
+    kept = {k: e.g[k].clone() for k in ("pos", "type", "ln_g", "ln_b")}
+    e.g["word"].fill_(float("nan"))
+    e.step(d_ids, d_tt, B.make_optim(step=1, lr=1e-3))
+    used = np.zeros(e.V, bool)
+    used[ids.reshape(-1)] = True
+    g = e.g["word"].cpu().numpy()
+    assert np.isfinite(g).all() and not g[~used].any()                   # with an update: the unmasked sums, zero elsewhere
+    for k, v in kept.items():
+        assert torch.equal(e.g[k], v), k
+        assert np.abs(e.s[k].cpu().numpy() - student[k]).max() > 0, k    # and they were updated
+
+
 def test_embedding_step_rejects_and_reports_bad_input():
     e, desc, teacher, student, step, ids, tt = _problem("bf16", 4, V=64, H=32, P=16, batch=2, seq=8)
     d_ids, d_tt = torch.from_numpy(ids).to(e.device), torch.from_numpy(tt).to(e.device)
