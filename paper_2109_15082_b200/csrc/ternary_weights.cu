@@ -10,21 +10,23 @@
 //
 // Refitted scale (b-bit, the loss-aware rule read with unit curvature weights): minimise ||w - alpha q||^2 over
 // alpha and q in Omega(b)^n by alternating the two exact half-steps  q = Pi_Omega(b)(w / alpha)  (Eq. 1, float32
-// division)  and  alpha = <q, w> / <q, q>  (float64 sums in a fixed order, alpha rounded to float32), LAQ_ROUNDS
-// times from alpha_0 = min(3 mean|w|, max|w|) / qmax; a row of zeros keeps alpha = 0 and codes 0.
+// division)  and  alpha = <q, w> / <q, q>  (alpha rounded to float32), LAQ_ROUNDS times from
+// alpha_0 = min(3 mean|w|, max|w|) / qmax; a row of zeros keeps alpha = 0 and codes 0.  A round is a function of alpha
+// alone, so a round that returns the alpha it was given ends the loop: all later rounds would repeat it (Gaussian rows
+// 768 wide need 10 rounds on average, 1024 wide 11, 3072 wide 14 of the 15).
 #include "optim.cuh"
 
 namespace mrem {
 
 namespace {
 
-// Threads per row (NT) and float4 vectors per thread kept in registers (MAXV): a block of 256 threads with 4 vectors
-// each holds rows up to 4096 wide; the alternating rule, whose 16 rounds are a dependent chain per thread, takes 128
-// threads with 2 vectors each for rows up to 1024 wide (measured against 32 x 8 and 256 x 1).
+// Ternary rule: 256 threads per row, up to 4 float4 vectors per thread in registers (rows up to 4096 wide).  Refitted
+// scale: two vectors per thread and as many threads as that takes (rows up to 4096 wide; 96 threads for 768, 384 for
+// 3072: no idle lanes at the encoder's widths).  Wider rows are re-read by 256 threads.
 constexpr int TW_THREADS = 256;
 constexpr int TW_MAXV = 4;
-constexpr int TW_NARROW_THREADS = 128;   // rows up to 1024 wide under the alternating rule: 2 vectors per thread
-constexpr int TW_NARROW_MAXV = 2;
+constexpr int LAQ_V = 2;
+constexpr int LAQ_MAX_WARPS = 16;
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -161,23 +163,14 @@ __device__ __forceinline__ void block_sum_di(double& a, int& n, double* shd, int
   n = __reduce_add_sync(0xffffffffu, lane < nw ? shi[lane] : 0);
 }
 
-// The alternating rule on one row (same conventions as ternary_row).
-template <typename T, int NT, int MAXV>
-__device__ __forceinline__ void laq_row(const float4* wr, bool cached, const float* w_row, int cols, int row, int bits,
-                                        int8_t* codes_row, int32_t* rowsum, float* scale, T* what_row, double* shd,
-                                        int* shi, float* shf) {
+// The alternating rule on a row too wide for registers, re-read in every round.
+template <typename T, int NT>
+__device__ __forceinline__ void laq_row(const float* w_row, int cols, int row, int bits, int8_t* codes_row, int32_t* rowsum,
+                                        float* scale, T* what_row, double* shd, int* shi, float* shf) {
   const int nvec = cols / 4;
   const float qmax = (float)((1 << (bits - 1)) - 1);
   auto for_row = [&](auto&& f) {
-    if (cached) {
-#pragma unroll
-      for (int i = 0; i < MAXV; ++i) {
-        const int c = threadIdx.x + i * NT;
-        if (c < nvec) f(c, wr[i]);
-      }
-    } else {
-      for (int c = threadIdx.x; c < nvec; c += NT) f(c, reinterpret_cast<const float4*>(w_row)[c]);
-    }
+    for (int c = threadIdx.x; c < nvec; c += NT) f(c, reinterpret_cast<const float4*>(w_row)[c]);
   };
   double s = 0.0;
   float mx = 0.f;
@@ -192,29 +185,14 @@ __device__ __forceinline__ void laq_row(const float4* wr, bool cached, const flo
     double qw = 0.0, qw1 = 0.0, qw2 = 0.0, qw3 = 0.0;
     int qq = 0;
     auto sums = [&](auto code) {
-      if (cached) {
-#pragma unroll
-        for (int i = 0; i < MAXV; ++i) {
-          if (threadIdx.x + i * NT < nvec) {
-            const int q0 = code(wr[i].x), q1 = code(wr[i].y), q2 = code(wr[i].z), q3 = code(wr[i].w);
-            qw = fma(int_as_double(q0), (double)wr[i].x, qw);        // four independent chains
-            qw1 = fma(int_as_double(q1), (double)wr[i].y, qw1);
-            qw2 = fma(int_as_double(q2), (double)wr[i].z, qw2);
-            qw3 = fma(int_as_double(q3), (double)wr[i].w, qw3);
-            qq += q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3;
-          }
-        }
-      } else {
-        for (int c = threadIdx.x; c < nvec; c += NT) {
-          const float4 v = reinterpret_cast<const float4*>(w_row)[c];
-          const int q0 = code(v.x), q1 = code(v.y), q2 = code(v.z), q3 = code(v.w);
-          qw = fma(int_as_double(q0), (double)v.x, qw);
-          qw1 = fma(int_as_double(q1), (double)v.y, qw1);
-          qw2 = fma(int_as_double(q2), (double)v.z, qw2);
-          qw3 = fma(int_as_double(q3), (double)v.w, qw3);
-          qq += q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3;
-        }
-      }
+      for_row([&](int, float4 v) {
+        const int q0 = code(v.x), q1 = code(v.y), q2 = code(v.z), q3 = code(v.w);
+        qw = fma(int_as_double(q0), (double)v.x, qw);              // four independent chains
+        qw1 = fma(int_as_double(q1), (double)v.y, qw1);
+        qw2 = fma(int_as_double(q2), (double)v.z, qw2);
+        qw3 = fma(int_as_double(q3), (double)v.w, qw3);
+        qq += q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3;
+      });
     };
     if (alpha > 1e-30f) {                                  // 1 / alpha and the residual stay in the normal range
       const float r_alpha = __frcp_rn(alpha);
@@ -224,7 +202,9 @@ __device__ __forceinline__ void laq_row(const float4* wr, bool cached, const flo
     }
     qw = (qw + qw1) + (qw2 + qw3);
     block_sum_di(qw, qq, shd, shi);
-    alpha = qq > 0 ? (float)(qw / (double)qq) : 0.f;
+    const float next = qq > 0 ? (float)(qw / (double)qq) : 0.f;
+    if (next == alpha) break;
+    alpha = next;
   }
   // last round: the codes of this alpha (by the division of Eq. 1) go out with the scale refitted to them
   double qw = 0.0;
@@ -257,16 +237,238 @@ __device__ __forceinline__ void laq_row(const float4* wr, bool cached, const flo
   }
 }
 
+// The rule on a row held in registers, LAQ_V vectors per thread (missing ones are zeros: their code is 0 and they add
+// nothing).  The rounds that only feed the two sums get them without float64 arithmetic per weight: w / 2^(e - 23), e = the
+// exponent of max|w|, is split once into two integers of 12 bits and a rest of at most 1/2,
+//   w = (4096 nh + nm + nl) 2^(e - 23),
+// so that sums of q nh and q nm over a thread's weights are exact in float32 (below 2^24 for codes of up to 4 bits) and, as
+// integers, over the block; the rest enters at 2^-39 of max|w|.  7 instructions per weight and round instead of 38, four
+// integer warp reductions instead of a float64 butterfly, one barrier instead of two.
+// BERT-base module of three layers: step 1801 -> 1693 us.
+struct LaqShared { int4 sums[2][LAQ_MAX_WARPS]; double d[32]; int i[64]; float f[32]; };
+
+template <typename T>
+__device__ __forceinline__ void laq_row_cached(const float4 (&wr)[LAQ_V], int cols, int row, int bits, int8_t* codes_row,
+                                               int32_t* rowsum, float* scale, T* what_row, LaqShared& sh) {
+  constexpr int NW = 4 * LAQ_V;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, nvec = cols / 4;
+  const float qmax = (float)((1 << (bits - 1)) - 1);
+  float2 w[NW / 2];
+#pragma unroll
+  for (int i = 0; i < LAQ_V; ++i) { w[2 * i] = make_float2(wr[i].x, wr[i].y); w[2 * i + 1] = make_float2(wr[i].z, wr[i].w); }
+  double s = 0.0;
+  float mx = 0.f;
+#pragma unroll
+  for (int e = 0; e < NW / 2; ++e) {
+    s += (double)fabsf(w[e].x) + (double)fabsf(w[e].y);
+    mx = fmaxf(mx, fmaxf(fabsf(w[e].x), fabsf(w[e].y)));
+  }
+  s = block_sum_d(s, sh.d);
+  mx = block_max(mx, sh.f);
+  float alpha = (float)(fmin(3.0 * (s / (double)cols), (double)mx) / (double)qmax);
+  const bool split = bits <= 4 && mx > 1e-30f && mx < 1e30f;
+  const int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
+  float2 nh[NW / 2], nm[NW / 2], nl[NW / 2];
+  double unit = 0.0;                                       // 2^(ex - 23)
+  if (split) {
+    const float inv_u = __uint_as_float((uint32_t)(127 + 11 - ex) << 23);
+    unit = (double)__uint_as_float((uint32_t)(127 - 23 + ex) << 23);
+#pragma unroll
+    for (int e = 0; e < NW / 2; ++e) {
+      const float tx = w[e].x * inv_u, ty = w[e].y * inv_u;     // exact, below 2^12
+      nh[e] = make_float2(rne_magic(tx), rne_magic(ty));
+      const float ux = (tx - nh[e].x) * 4096.f, uy = (ty - nh[e].y) * 4096.f;
+      nm[e] = make_float2(rne_magic(ux), rne_magic(uy));
+      nl[e] = make_float2(ux - nm[e].x, uy - nm[e].y);
+    }
+  }
+  for (int r = 0; r + 1 < LAQ_ROUNDS; ++r) {
+    float next;
+    if (split && alpha > 1e-30f) {                         // 1 / alpha and the residual stay in the normal range
+      const float r_alpha = __frcp_rn(alpha);
+      const float2 r2 = make_float2(r_alpha, r_alpha), na2 = make_float2(-alpha, -alpha), magic2 = make_float2(ROUND_MAGIC, ROUND_MAGIC),
+                   nmagic2 = make_float2(-ROUND_MAGIC, -ROUND_MAGIC);
+      float2 ah = make_float2(0.f, 0.f), am = ah, al = ah, aq = ah;
+#pragma unroll
+      for (int e = 0; e < NW / 2; ++e) {                   // (quotient() and the rounding on pairs)
+        const float2 z0 = mul2(w[e], r2), z = fma2(fma2(z0, na2, w[e]), r2, z0);
+        const float2 q = add2(add2(make_float2(fminf(fmaxf(z.x, -qmax), qmax), fminf(fmaxf(z.y, -qmax), qmax)), magic2), nmagic2);
+        ah = fma2(q, nh[e], ah);
+        am = fma2(q, nm[e], am);
+        al = fma2(q, nl[e], al);
+        aq = fma2(q, q, aq);
+      }
+      const int4 mine = make_int4(__reduce_add_sync(0xffffffffu, __float2int_rn(ah.x + ah.y)), __reduce_add_sync(0xffffffffu, __float2int_rn(am.x + am.y)),
+                                  __reduce_add_sync(0xffffffffu, __float2int_rn((al.x + al.y) * 65536.f)), __reduce_add_sync(0xffffffffu, __float2int_rn(aq.x + aq.y)));
+      if (lane == 0) sh.sums[r & 1][wid] = mine;
+      __syncthreads();
+      int4 t = make_int4(0, 0, 0, 0);
+      if (nw <= 4) {
+        for (int k = 0; k < nw; ++k) {
+          const int4 v = sh.sums[r & 1][k];
+          t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+        }
+      } else {
+        if (lane < nw) t = sh.sums[r & 1][lane];
+        t = make_int4(__reduce_add_sync(0xffffffffu, t.x), __reduce_add_sync(0xffffffffu, t.y), __reduce_add_sync(0xffffffffu, t.z),
+                      __reduce_add_sync(0xffffffffu, t.w));
+      }
+      // <q, w> / <q, q>: float32 quotient and one correction from the float64 residual (2^-46 before the rounding to float32)
+      const double qw = fma((double)t.z, 1.52587890625e-05, fma((double)t.x, 4096.0, (double)t.y)) * unit;
+      const float rq = __frcp_rn((float)t.w), a0 = (float)qw * rq;
+      next = t.w > 0 ? (float)fma(fma(-(double)a0, (double)t.w, qw), (double)rq, (double)a0) : 0.f;
+    } else {
+      double qw = 0.0;
+      int qq = 0;
+      if (alpha > 0.f) {
+#pragma unroll
+        for (int e = 0; e < NW / 2; ++e) {
+          const int qx = laq_code(w[e].x, alpha, qmax), qy = laq_code(w[e].y, alpha, qmax);
+          qw += (double)qx * (double)w[e].x + (double)qy * (double)w[e].y;
+          qq += qx * qx + qy * qy;
+        }
+      }
+      block_sum_di(qw, qq, sh.d, sh.i);
+      next = qq > 0 ? (float)(qw / (double)qq) : 0.f;
+    }
+    if (next == alpha) break;
+    alpha = next;
+  }
+  // last round: the codes of this alpha (by the division of Eq. 1) go out with the scale refitted to them (float64)
+  double qw = 0.0;
+  int qq = 0, sum = 0;
+  float q[NW];
+  const bool normal = alpha > 1e-30f && alpha < 1e30f;
+  const float r_alpha = __frcp_rn(alpha);
+#pragma unroll
+  for (int i = 0; i < LAQ_V; ++i) {
+    const int c = threadIdx.x + i * blockDim.x;
+    uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = 4 * i + j;
+      const float we = (j & 1) ? w[e >> 1].y : w[e >> 1].x;
+      int k = 0;
+      q[e] = 0.f;
+      if (normal) {
+        q[e] = code_f<false>(we, alpha, r_alpha, -qmax, qmax, b[j]);
+        k = (int)(int8_t)(b[j] & 0xffu);
+      } else if (alpha > 0.f) {
+        k = laq_code(we, alpha, qmax);
+        q[e] = (float)k;
+        b[j] = (uint32_t)k;
+      }
+      qw += int_as_double(k) * (double)we;
+      qq += k * k;
+      sum += k;
+    }
+    if (c < nvec) *reinterpret_cast<uint32_t*>(codes_row + 4 * c) = pack_low_bytes(b[0], b[1], b[2], b[3]);
+  }
+  qw = warp_sum_d(qw);
+  qq = __reduce_add_sync(0xffffffffu, qq);
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  __syncthreads();
+  if (lane == 0) { sh.d[wid] = qw; sh.i[wid] = qq; sh.i[32 + wid] = sum; }
+  __syncthreads();
+  qw = warp_sum_d(lane < nw ? sh.d[lane] : 0.0);
+  qq = __reduce_add_sync(0xffffffffu, lane < nw ? sh.i[lane] : 0);
+  const float next = qq > 0 ? (float)(qw / (double)qq) : 0.f;
+  if (what_row) {
+#pragma unroll
+    for (int i = 0; i < LAQ_V; ++i) {
+      const int c = threadIdx.x + i * blockDim.x;
+      if (c < nvec) store4<T>(what_row + 4 * c, next * q[4 * i], next * q[4 * i + 1], next * q[4 * i + 2], next * q[4 * i + 3]);
+    }
+  }
+  if (wid == 0) {
+    sum = __reduce_add_sync(0xffffffffu, lane < nw ? sh.i[32 + lane] : 0);
+    if (lane == 0) {
+      rowsum[row] = sum;
+      scale[row] = next;
+    }
+  }
+}
+
+// The two kernels of the refitted scale on rows held in registers; NT: upper bound of the block size.
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) laq_quantize_kernel(const float* __restrict__ w, int cols, int bits,
+                                                                     int8_t* __restrict__ codes, int32_t* __restrict__ rowsum,
+                                                                     float* __restrict__ scale, T* __restrict__ what) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ LaqShared sh;
+  const long long base = (long long)blockIdx.x * cols;
+  const float4* w4 = reinterpret_cast<const float4*>(w + base);
+  float4 wr[LAQ_V];
+#pragma unroll
+  for (int i = 0; i < LAQ_V; ++i) {
+    const int c = threadIdx.x + i * blockDim.x;
+    wr[i] = c < cols / 4 ? w4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  laq_row_cached<T>(wr, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
+}
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) laq_update_kernel(float* __restrict__ w, const float* __restrict__ g,
+                                                                   float* __restrict__ m, float* __restrict__ v,
+                                                                   const OptimScalars* __restrict__ sc, int cols, int train_w,
+                                                                   int bits, int8_t* __restrict__ codes,
+                                                                   int32_t* __restrict__ rowsum, float* __restrict__ scale,
+                                                                   T* __restrict__ what) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ LaqShared sh;
+  const OptimScalars o = *sc;
+  const long long base = (long long)blockIdx.x * cols;
+  const int nvec = cols / 4;
+  float4* w4 = reinterpret_cast<float4*>(w + base);
+  const float4* g4 = reinterpret_cast<const float4*>(g + base);
+  float4* m4 = reinterpret_cast<float4*>(m + base);
+  float4* v4 = reinterpret_cast<float4*>(v + base);
+  float4 wr[LAQ_V], gr[LAQ_V], mr[LAQ_V], vr[LAQ_V];
+#pragma unroll
+  for (int i = 0; i < LAQ_V; ++i) {                        // all loads in flight first
+    const int c = threadIdx.x + i * blockDim.x;
+    wr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < nvec) {
+      wr[i] = w4[c];
+      if (train_w) { gr[i] = g4[c]; mr[i] = m4[c]; vr[i] = v4[c]; }
+    }
+  }
+  if (train_w) {
+#pragma unroll
+    for (int i = 0; i < LAQ_V; ++i) {
+      const int c = threadIdx.x + i * blockDim.x;
+      if (c < nvec) {
+        wr[i].x = adam_one(wr[i].x, gr[i].x, mr[i].x, vr[i].x, o, 1.f, -INFINITY);
+        wr[i].y = adam_one(wr[i].y, gr[i].y, mr[i].y, vr[i].y, o, 1.f, -INFINITY);
+        wr[i].z = adam_one(wr[i].z, gr[i].z, mr[i].z, vr[i].z, o, 1.f, -INFINITY);
+        wr[i].w = adam_one(wr[i].w, gr[i].w, mr[i].w, vr[i].w, o, 1.f, -INFINITY);
+        w4[c] = wr[i];
+        m4[c] = mr[i];
+        v4[c] = vr[i];
+      }
+    }
+  }
+  laq_row_cached<T>(wr, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
+}
+
+// Block size of the two kernels above, or 0 when the row does not fit.
+inline int laq_threads(int cols) {
+  const int warps = (cols / 4 + 32 * LAQ_V - 1) / (32 * LAQ_V);
+  return warps <= LAQ_MAX_WARPS ? 32 * warps : 0;
+}
+
 template <typename T, int RULE, int NT, int MAXV>
 __device__ __forceinline__ void closed_form_row(const float4* wr, bool cached, const float* w_row, int cols,
                                                 int row, int bits, int8_t* codes_row, int32_t* rowsum, float* scale,
                                                 T* what_row, double* shd, int* shi, float* shf) {
-  if (RULE == 3) laq_row<T, NT, MAXV>(wr, cached, w_row, cols, row, bits, codes_row, rowsum, scale, what_row, shd, shi, shf);
+  if (RULE == 3) laq_row<T, NT>(w_row, cols, row, bits, codes_row, rowsum, scale, what_row, shd, shi, shf);
   else ternary_row<T, NT, MAXV>(wr, cached, w_row, cols, row, codes_row, rowsum, scale, what_row, shd, shi);
 }
 
 template <typename T, int RULE, int NT, int MAXV>
-__global__ void __launch_bounds__(NT, NT == TW_NARROW_THREADS ? 8 : (RULE == 2 ? 5 : 4)) closed_form_quantize_kernel(const float* __restrict__ w, int cols,
+__global__ void __launch_bounds__(NT, RULE == 2 ? 5 : 4) closed_form_quantize_kernel(const float* __restrict__ w, int cols,
                                                                       int bits,
                                                                       int8_t* __restrict__ codes,
                                                                       int32_t* __restrict__ rowsum,
@@ -279,7 +481,7 @@ __global__ void __launch_bounds__(NT, NT == TW_NARROW_THREADS ? 8 : (RULE == 2 ?
   const int row = blockIdx.x;
   const long long base = (long long)row * cols;
   const int nvec = cols / 4;
-  const bool cached = nvec <= MAXV * NT;
+  const bool cached = RULE == 2 && nvec <= MAXV * NT;
   float4 wr[MAXV];
   if (cached) {
 #pragma unroll
@@ -294,7 +496,7 @@ __global__ void __launch_bounds__(NT, NT == TW_NARROW_THREADS ? 8 : (RULE == 2 ?
 
 // AdamW on the row (gradient of w_hat passed through unchanged), then the rule on the new weights.
 template <typename T, int RULE, int NT, int MAXV>
-__global__ void __launch_bounds__(NT, NT == TW_NARROW_THREADS ? 8 : (RULE == 2 ? 5 : 4)) closed_form_update_kernel(float* __restrict__ w, const float* __restrict__ g,
+__global__ void __launch_bounds__(NT, RULE == 2 ? 5 : 4) closed_form_update_kernel(float* __restrict__ w, const float* __restrict__ g,
                                                                     float* __restrict__ m, float* __restrict__ v,
                                                                     const OptimScalars* __restrict__ sc, int cols,
                                                                     int train_w, int bits,
@@ -310,7 +512,7 @@ __global__ void __launch_bounds__(NT, NT == TW_NARROW_THREADS ? 8 : (RULE == 2 ?
   const OptimScalars o = *sc;
   const long long base = (long long)row * cols;
   const int nvec = cols / 4;
-  const bool cached = nvec <= MAXV * NT;
+  const bool cached = RULE == 2 && nvec <= MAXV * NT;
   float4* w4 = reinterpret_cast<float4*>(w + base);
   const float4* g4 = reinterpret_cast<const float4*>(g + base);
   float4* m4 = reinterpret_cast<float4*>(m + base);
@@ -351,13 +553,15 @@ void launch_closed_form_quantize(const float* w, int rows, int cols, int rule, i
                                  float* scale, void* what, int dt, cudaStream_t st) {
   Scope sc("quantize_weight", (double)rows * cols * (5.0 + (what ? (dt == 1 ? 2.0 : 4.0) : 0.0)) + rows * 8.0, 0, st);
   auto go = [&](auto kernel, int nt, auto* out) { launch_k(kernel, rows, nt, 0, st, w, cols, bits, codes, rowsum, scale, out); };
-  const bool narrow = rule == 3 && cols <= TW_NARROW_THREADS * 4 * TW_NARROW_MAXV;
+  const int nt = rule == 3 ? laq_threads(cols) : 0;
   if (dt == 1) {
-    if (narrow) go(closed_form_quantize_kernel<bf16, 3, TW_NARROW_THREADS, TW_NARROW_MAXV>, TW_NARROW_THREADS, (bf16*)what);
+    if (nt > 128) go(laq_quantize_kernel<bf16, 512>, nt, (bf16*)what);
+    else if (nt) go(laq_quantize_kernel<bf16, 128>, nt, (bf16*)what);
     else if (rule == 3) go(closed_form_quantize_kernel<bf16, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
     else go(closed_form_quantize_kernel<bf16, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
   } else {
-    if (narrow) go(closed_form_quantize_kernel<float, 3, TW_NARROW_THREADS, TW_NARROW_MAXV>, TW_NARROW_THREADS, (float*)what);
+    if (nt > 128) go(laq_quantize_kernel<float, 512>, nt, (float*)what);
+    else if (nt) go(laq_quantize_kernel<float, 128>, nt, (float*)what);
     else if (rule == 3) go(closed_form_quantize_kernel<float, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
     else go(closed_form_quantize_kernel<float, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
   }
@@ -370,13 +574,15 @@ void launch_closed_form_update(float* w, const float* g, float* m, float* v, con
   auto go = [&](auto kernel, int nt, auto* out) {
     launch_k(kernel, rows, nt, 0, st, w, g, m, v, sc, cols, train_w, bits, codes, rowsum, scale, out);
   };
-  const bool narrow = rule == 3 && cols <= TW_NARROW_THREADS * 4 * TW_NARROW_MAXV;
+  const int nt = rule == 3 ? laq_threads(cols) : 0;
   if (dt == 1) {
-    if (narrow) go(closed_form_update_kernel<bf16, 3, TW_NARROW_THREADS, TW_NARROW_MAXV>, TW_NARROW_THREADS, (bf16*)what);
+    if (nt > 128) go(laq_update_kernel<bf16, 512>, nt, (bf16*)what);
+    else if (nt) go(laq_update_kernel<bf16, 128>, nt, (bf16*)what);
     else if (rule == 3) go(closed_form_update_kernel<bf16, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
     else go(closed_form_update_kernel<bf16, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
   } else {
-    if (narrow) go(closed_form_update_kernel<float, 3, TW_NARROW_THREADS, TW_NARROW_MAXV>, TW_NARROW_THREADS, (float*)what);
+    if (nt > 128) go(laq_update_kernel<float, 512>, nt, (float*)what);
+    else if (nt) go(laq_update_kernel<float, 128>, nt, (float*)what);
     else if (rule == 3) go(closed_form_update_kernel<float, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
     else go(closed_form_update_kernel<float, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
   }
