@@ -1,114 +1,72 @@
-// Fused attention backward of the student for one (batch, head) per CTA on sm_100a, sequences up
-// to 128 tokens, head size 64.  Inputs: the gradient of the context, the codes of Q, K, V, the stored
-// probabilities P and the pre-quantization Q, K, V.  One kernel does what otherwise takes four
-// batched products, the softmax backward and three straight-through kernels:
-//   dP_hat = s_v * dctx V_q^T                      (tcgen05, accumulators in TMEM)
-//   STE of the P quantizer, softmax backward dS = P * (dP - sum_j dP P), by 256 threads (two per
-//     query row) reading TMEM; P_hat codes and dS are written to swizzled shared memory
-//   dV_hat = s_p * P_q^T dctx,  dQ_hat = s_k/sqrt(d) * dS K_q,  dK_hat = s_q/sqrt(d) * dS^T Q_q
-//     (three tcgen05 products; the same shared-memory tile serves as K-major A operand of one
-//     product and as MN-major A operand of another, so nothing is transposed; the codes of P and
-//     dS share one tile, dQ and dK take over the TMEM columns of dP, so two CTAs fit on an SM)
-//   STE of the Q, K, V quantizers on the way out, with their step-size gradients.
-// Step-size gradients leave as one partial sum per CTA and site (summed later in CTA order).
-// All waits are time-bounded.
-#include "gemm.h"
-#include "kernels.h"
-#include "tc_ptx.cuh"
-
-#include <type_traits>
+// Fused attention backward of the student on sm_100a, sequences up to 128 tokens, head size 64: one (batch, head) per CTA.
+// Inputs: the gradient of the quantized context, the context and Q, K, V before quantization, the codes of Q, K, V, and per
+// query row the two numbers the forward pass left of its softmax (maximum, 1 / sum).  One kernel does what otherwise takes
+// five batched products, the softmax and its backward and four straight-through kernels:
+//   STE of the context's quantizer: dctx (in place in its operand tile)
+//   S = Q_q K_q^T and dP_hat = s_v dctx V_q^T                       (tcgen05, accumulators in TMEM)
+//   P from S exactly as the forward pass formed it (bit for bit: the products of codes are exact), its codes, the STE of its
+//     quantizer, dS = P * (dP - sum_j dP P): two threads per query row reading TMEM; codes of P and dS go to shared memory
+//   dV_hat = s_p P_q^T dctx,  dQ_hat = s_k/sqrt(d) dS K_q,  dK_hat = s_q/sqrt(d) dS^T Q_q
+//     (three tcgen05 products; the same shared-memory tile serves as K-major A operand of one product and as MN-major A
+//     operand of another, so nothing is transposed)
+//   STE of the Q, K, V quantizers on the way out.
+// Step-size gradients leave as one partial sum per CTA and site (summed later in CTA order).  All waits are time-bounded.
+//
+// What bounds it: a CTA is a serial chain of small steps, so what counts is their latency.  The probabilities are recomputed
+// (6 instructions per score) instead of written by the forward pass and read twice by lanes that each own a row (32 lines per
+// load: 4,900 of the kernel's 40,000 cycles, and 33 MB per launch at 32 x 16 x 128 x 128); the values before quantization come
+// in and the gradients go out through operand tiles that are no longer needed (TMA); tests for clipped values are made once
+// per warp and chunk.  32 x 16 heads x 128 x 128: 50 + 8 us (kernel, STE of the context) -> 29 us.
+// Shared memory: Q, K, V, dctx tiles of 16 KB and one of 32 KB that is the context, then the codes of P, then dS; the V tile
+// becomes V before quantization -> dV out -> K before quantization -> dK out, the dctx tile Q before quantization -> dQ out.
+// TMEM (256 columns, two CTAs per SM): dP | S; dV takes the place of S, dQ and dK that of dP.
+#include "attention_bwd.cuh"
 
 namespace mrem {
+
+using namespace att;
 
 namespace {
 
 constexpr int ATB_THREADS = 288;          // warp 0: TMA + MMA issue; warps 1..8: row work, two threads per row
-constexpr int HD = 64;
-// TMEM columns: dP in 0..127; once dS has been formed from it, dQ and dK take its place
-constexpr int TMEM_DP = 0, TMEM_DV = 128, TMEM_DQ = 0, TMEM_DK = 64, TMEM_ALLOC = 256;
+constexpr int TMEM_DP = 0, TMEM_S = 128, TMEM_DV = 128, TMEM_DQ = 0, TMEM_DK = 64, TMEM_ALLOC = 256;
 
 struct AttnBwdParams {
   int S, h, B, H;
-  int n16;                   // S rounded up to 16
-  int n_kb;                  // 64-wide blocks covering S
   float inv_sqrt_d;
-  const float *s_q, *s_k, *s_v, *s_p;
-  float q_lo, q_hi;          // code range of the symmetric Q/K/V sites
-  float p_lo, p_hi;          // code range of the P site
-  const bf16* P;             // [B, h, S, S]
-  const bf16* qkv;           // [B*S, 3H] values before quantization
-  bf16* dqkv;                // [B*S, 3H] out
-  float *part_q, *part_k, *part_v, *part_p;   // [red_slots] each: one partial per CTA, the rest zeroed
+  const float *s_q, *s_k, *s_v, *s_p, *s_c;
+  const float* alpha;        // score scale of the forward pass
+  const int* len;            // [B] valid keys (clamped)
+  const float2* stat;        // [B, h, S] (alpha log2(e) max, 1 / sum)
+  float q_hi;                // code range -q_hi .. q_hi of the symmetric Q / K / V / context sites
+  float p_hi;                // upper end of the code range of the P site (probabilities are not negative)
+  float *part_q, *part_k, *part_v, *part_p, *part_c;   // [red_slots] each: one partial per CTA, the rest zeroed
   int red_slots;
   int* status;
   unsigned long long wait_ns;  // limit of each wait on an mbarrier
 };
 
-__device__ __forceinline__ void ld16(const void* p, uint32_t* w) {
-  const uint4 u = *reinterpret_cast<const uint4*>(p);
-  w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
-}
-__device__ __forceinline__ void st16(void* p, const uint32_t* w) {
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-__device__ __forceinline__ float2 unpack2(uint32_t w) {
-  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
-}
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
+struct AttnBwdMaps { CUtensorMap codes, raw, dctx, ctx, out; };
 
-// The epilogue of one gradient: scale the accumulator, apply the straight-through mask of the site's
-// quantizer, store 32 head columns of one token, return this thread's share of the step-size gradient.
-__device__ __forceinline__ float ste_store(const uint32_t* a, bool row_ok, const bf16* x, bf16* out, float scale,
-                                           float step, float lo, float hi) {
-  float acc = 0.f;
-  const float r_step = __frcp_rn(step);
-  if (row_ok) {
-    uint32_t xw[16], ow[16];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) ld16(x + t * 8, xw + 4 * t);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float2 xv = unpack2(xw[j]);
-      const float g0 = scale * __uint_as_float(a[2 * j]), g1 = scale * __uint_as_float(a[2 * j + 1]);
-      const float z0 = quotient(xv.x, step, r_step), z1 = quotient(xv.y, step, r_step);
-      const float c0 = fminf(fmaxf(z0, lo), hi), c1 = fminf(fmaxf(z1, lo), hi);
-      const bool in0 = c0 == z0, in1 = c1 == z1;              // inside the code range
-      const float q0 = rne_magic(c0), q1 = rne_magic(c1);
-      acc += g0 * (in0 ? q0 - z0 : q0) + g1 * (in1 ? q1 - z1 : q1);
-      ow[j] = pack2(in0 ? g0 : 0.f, in1 ? g1 : 0.f);
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) st16(out + t * 8, ow + 4 * t);
-  }
-  return acc;
-}
-
-__global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __grid_constant__ CUtensorMap map_codes,
-                                                                       const __grid_constant__ CUtensorMap map_dctx,
+__global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __grid_constant__ AttnBwdMaps maps,
                                                                        const __grid_constant__ AttnBwdParams p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full, bar_a, bar_p, bar_b, bar_s, bar_o;
+  enum { B_CODES, B_CTX, B_STE, B_A, B_RV, B_P, B_B, B_RQ, B_S, B_O, B_RK, N_BARS };
+  __shared__ __align__(8) uint64_t bars[N_BARS];
   __shared__ uint32_t tmem_slot;
   __shared__ float red_dot[2][128];
-  __shared__ float red_part[8][4];
+  __shared__ float red_part[8][5];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int head = blockIdx.x, b = blockIdx.y;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  // sX holds the codes of P (A operand of the dV product) first and dS (A operand of dQ and dK) afterwards
   const uint32_t sQ = base, sK = sQ + 16384, sV = sK + 16384, sD = sV + 16384, sX = sD + 16384;
-  uint8_t* gX = smem_raw + (sX - smem_u32(smem_raw));
+  uint8_t* const g0 = smem_raw + (base - smem_u32(smem_raw));
+  uint8_t *const gV = g0 + (sV - base), *const gD = g0 + (sD - base), *const gX = g0 + (sX - base);
+  auto bar = [&](int i) { return smem_u32(&bars[i]); };
   pdl_trigger();
 
   if (threadIdx.x == 0) {
-    mbar_init(smem_u32(&bar_full), 1);
-    mbar_init(smem_u32(&bar_a), 1);
-    mbar_init(smem_u32(&bar_p), 256);
-    mbar_init(smem_u32(&bar_b), 1);
-    mbar_init(smem_u32(&bar_s), 256);
-    mbar_init(smem_u32(&bar_o), 1);
+    for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_STE || i == B_P || i == B_S) ? 256 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -122,176 +80,233 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
   tc_fence_after();
   pdl_wait();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
-  const int ksteps = p.n16 / 16;
+  const int len = p.len[b];
+  const int n_valid = (len + 31) / 32, n_chunks = (p.S + 31) / 32;        // 32-key chunks with a valid key, with any key
+  const int q_steps = (p.S + 15) / 16, k_steps = (len + 15) / 16;
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint32_t bar = smem_u32(&bar_full);
-      mbar_expect_tx(bar, 4u * 16384u);
-      tma_load_4d(sD, &map_dctx, bar, 0, 0, head, b);
-      tma_load_4d(sV, &map_codes, bar, 0, 0, 2 * p.h + head, b);
-      tma_load_4d(sK, &map_codes, bar, 0, 0, p.h + head, b);
-      tma_load_4d(sQ, &map_codes, bar, 0, 0, head, b);
-      bool ok = mbar_wait(bar, 0, p.wait_ns);
+      mbar_expect_tx(bar(B_CTX), 2u * 16384u);
+      tma_load_4d(sD, &maps.dctx, bar(B_CTX), 0, 0, head, b);
+      tma_load_4d(sX, &maps.ctx, bar(B_CTX), 0, 0, head, b);
+      mbar_expect_tx(bar(B_CODES), 3u * 16384u);
+      tma_load_4d(sQ, &maps.codes, bar(B_CODES), 0, 0, head, b);
+      tma_load_4d(sK, &maps.codes, bar(B_CODES), 0, 0, p.h + head, b);
+      tma_load_4d(sV, &maps.codes, bar(B_CODES), 0, 0, 2 * p.h + head, b);
+      bool ok = mbar_wait(bar(B_CODES), 0, p.wait_ns);
       if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_TMA);
       tc_fence_after();
-      if (ok) {      // dP_hat [queries x keys] = dctx [q x d] * V_q^T
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n16 >> 3) << 17) | (8u << 24);
+      const uint32_t f32 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
+      const uint32_t id_s = f32 | ((uint32_t)(n_valid * 32 >> 3) << 17);
+      if (ok)        // S [queries x keys] = Q_q [q x d] * K_q^T
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          tc_mma<0>(tmem + TMEM_DP, smem_desc(sD + k * 32, 16u, 1024u), smem_desc(sV + k * 32, 16u, 1024u), idesc, (uint32_t)(k != 0));
-      }
-      tc_commit(smem_u32(&bar_a));
-      const uint32_t f = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HD >> 3) << 17) | (8u << 24);
+          tc_mma<0>(tmem + TMEM_S, smem_desc(sQ + k * 32, 16u, 1024u), smem_desc(sK + k * 32, 16u, 1024u), id_s, (uint32_t)(k != 0));
+      ok = mbar_wait(bar(B_STE), 0, p.wait_ns) && ok;
+      tc_fence_after();
+      if (ok)        // dP_hat [queries x keys] = dctx [q x d] * V_q^T
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          tc_mma<0>(tmem + TMEM_DP, smem_desc(sD + k * 32, 16u, 1024u), smem_desc(sV + k * 32, 16u, 1024u), id_s, (uint32_t)(k != 0));
+      tc_commit(bar(B_A));
+      ok = mbar_wait(bar(B_A), 0, p.wait_ns) && ok;
+      mbar_expect_tx(bar(B_RV), 16384u);                       // the V tile is free: V before quantization
+      tma_load_4d(sV, &maps.raw, bar(B_RV), 0, 0, 2 * p.h + head, b);
+      const uint32_t f = f32 | ((uint32_t)(HD >> 3) << 17);
       const uint32_t id_tt = f | (1u << 15) | (1u << 16);     // A and B MN-major
       const uint32_t id_nt = f | (1u << 16);                  // A K-major, B MN-major
-      ok = ok && mbar_wait(smem_u32(&bar_p), 0, p.wait_ns);
-      if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_EPI);
+      ok = mbar_wait(bar(B_P), 0, p.wait_ns) && ok;
       tc_fence_after();
       if (ok)
-        for (int ks = 0; ks < ksteps; ++ks)       // dV_hat [keys x d] = P_q^T [keys x q] * dctx [q x d]
+#pragma unroll 1
+        for (int ks = 0; ks < q_steps; ++ks)      // dV_hat [keys x d] = P_q^T [keys x q] * dctx [q x d]
           tc_mma<0>(tmem + TMEM_DV, smem_desc(sX + ks * 2048, 16384u, 1024u), smem_desc(sD + ks * 2048, 8192u, 1024u), id_tt, (uint32_t)(ks != 0));
-      tc_commit(smem_u32(&bar_b));
-      ok = ok && mbar_wait(smem_u32(&bar_s), 0, p.wait_ns);
+      tc_commit(bar(B_B));
+      ok = mbar_wait(bar(B_B), 0, p.wait_ns) && ok;
+      mbar_expect_tx(bar(B_RQ), 16384u);                       // the dctx tile is free: Q before quantization
+      tma_load_4d(sD, &maps.raw, bar(B_RQ), 0, 0, head, b);
+      ok = mbar_wait(bar(B_S), 0, p.wait_ns) && ok;
       if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_EPI);
       tc_fence_after();
       if (ok) {
-        for (int ks = 0; ks < ksteps; ++ks)       // dQ_hat [q x d] = dS [q x keys] * K_q [keys x d]
+#pragma unroll 1
+        for (int ks = 0; ks < k_steps; ++ks)      // dQ_hat [q x d] = dS [q x keys] * K_q [keys x d]
           tc_mma<0>(tmem + TMEM_DQ, smem_desc(sX + (ks >> 2) * 16384 + (ks & 3) * 32, 16u, 1024u), smem_desc(sK + ks * 2048, 8192u, 1024u), id_nt, (uint32_t)(ks != 0));
-        for (int ks = 0; ks < ksteps; ++ks)       // dK_hat [keys x d] = dS^T [keys x q] * Q_q [q x d]
+#pragma unroll 1
+        for (int ks = 0; ks < q_steps; ++ks)      // dK_hat [keys x d] = dS^T [keys x q] * Q_q [q x d]
           tc_mma<0>(tmem + TMEM_DK, smem_desc(sX + ks * 2048, 16384u, 1024u), smem_desc(sQ + ks * 2048, 8192u, 1024u), id_tt, (uint32_t)(ks != 0));
       }
-      tc_commit(smem_u32(&bar_o));
+      tc_commit(bar(B_O));
     }
   } else {
     const int quad = warp & 3, half = (warp - 1) >> 2;
-    const int r = quad * 32 + lane;                       // row of the tile: a query for dP/dS/dQ, a key for dK/dV
+    const int r = quad * 32 + lane;                       // row of the tile: a query for S / dP / dS / dQ, a key for dK / dV
     const bool row_ok = r < p.S;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const float s_p = *p.s_p, s_v = *p.s_v, s_q = *p.s_q, s_k = *p.s_k;
-    const float r_p = __frcp_rn(s_p);
-    const int n_chunks = (p.S + 31) / 32;
-    const long long prow = (((long long)b * p.h + head) * p.S + r) * p.S;
-    float ds_p = 0.f;
-    bool got = mbar_wait(smem_u32(&bar_a), 0, p.wait_ns);
+    const float s_p = *p.s_p, s_v = *p.s_v, s_q = *p.s_q, s_k = *p.s_k, s_c = *p.s_c;
+    float2 st = make_float2(0.f, 0.f);                    // rows beyond the sequence: P = 0
+    if (row_ok) st = p.stat[((long long)b * p.h + head) * p.S + r];
+    const float alpha2 = *p.alpha * 1.4426950408889634f;
+    bool got = mbar_wait(bar(B_CTX), 0, p.wait_ns);
+    // ---- STE of the context's quantizer, 32 of the row's 64 columns per thread, in place
+    float ds_c;
+    {
+      uint32_t d[16], x[16];
+      tile_load(gD, r, half, d);
+      tile_load(gX, r, half, x);
+      ds_c = ste32(x, [&](int j) { return unpack2(d[j]); }, s_c, p.q_hi, range_limit(s_c, p.q_hi));
+      tile_store(gD, r, half, x);                         // (bf16 gradients pass or become zero: nothing is rounded again)
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive(bar(B_STE));
+    got = mbar_wait(bar(B_A), 0, p.wait_ns) && got;
     tc_fence_after();
-    // ---- pass A: STE of the P quantizer, row dot product, the codes of P into the operand tile
-    float dot = 0.f;
-    for (int c = half; c < 2 * p.n_kb; c += 2) {
-      uint32_t cw[16];
-      if (c < n_chunks) {                   // warp-uniform: the TMEM accesses below are warp-collective
-        uint32_t a[32], pw[16];
-        tmem_ld32(trow + TMEM_DP + (uint32_t)(c * 32), a);
-        const int ncol = row_ok ? p.S - c * 32 : 0;
+    // ---- pass A: P as the forward pass formed it, its codes into the operand tile, STE of its quantizer, row dot product
+    const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p),
+                 magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
+    const float lim_p = range_limit(s_p, p.p_hi);
+    // the row's largest probability is 1 / sum, rounded as stored: one test per warp tells whether anything clips
+    const bool clips = !__all_sync(0xffffffffu, __bfloat162float(__float2bfloat16_rn(st.y)) <= lim_p);
+    // this thread's probabilities, two chunks of 32; the loops over them stay rolled, the chunks rotate through the registers
+    // (the kernel's code is executed once per CTA: with everything unrolled it was 130 KB, and a third of the stalls were
+    //  instruction fetches)
+    uint32_t pw0[16], pw1[16];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          if (t * 8 < ncol) ld16(p.P + prow + c * 32 + t * 8, pw + 4 * t);
-          else { pw[4 * t] = pw[4 * t + 1] = pw[4 * t + 2] = pw[4 * t + 3] = 0u; }
-        }
-        // FULL: every lane's 32 keys lie inside the sequence (the common case), no per-element bounds
-        auto chunk = [&](auto full_tag) {
-          constexpr bool FULL = decltype(full_tag)::value;
+    for (int j = 0; j < 16; ++j) pw1[j] = 0u;
+    float2 dot2 = both(0.f), dsp2 = both(0.f);
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+      const int c = half + 2 * i;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) pw0[j] = pw1[j];
+      if (c >= n_chunks) continue;                        // (warp-uniform: TMEM accesses are warp-collective)
+      uint32_t cw[16];
+      if (c < n_valid) {
+        const int ncol = len - c * 32;                    // below 32 only in the last chunk
+        {
+          uint32_t a[32];
+          tmem_ld32(trow + TMEM_S + (uint32_t)(c * 32), a);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const float2 pv = unpack2(pw[j]);
-            float d0 = s_v * __uint_as_float(a[2 * j]), d1 = s_v * __uint_as_float(a[2 * j + 1]);
-            const float z0 = quotient(pv.x, s_p, r_p), z1 = quotient(pv.y, s_p, r_p);
-            const float c0 = fminf(fmaxf(z0, p.p_lo), p.p_hi), c1 = fminf(fmaxf(z1, p.p_lo), p.p_hi);
-            const bool in0 = c0 == z0, in1 = c1 == z1;            // inside the code range
-            const float q0 = rne_magic(c0), q1 = rne_magic(c1);
-            const bool v0 = FULL || 2 * j < ncol, v1 = FULL || 2 * j + 1 < ncol;      // inside the sequence (row and key)
-            if (v0) ds_p += d0 * (in0 ? q0 - z0 : q0);
-            if (v1) ds_p += d1 * (in1 ? q1 - z1 : q1);
-            d0 = (in0 && v0) ? d0 : 0.f;
-            d1 = (in1 && v1) ? d1 : 0.f;
-            dot += d0 * pv.x + d1 * pv.y;
-            a[2 * j] = __float_as_uint(d0);
-            a[2 * j + 1] = __float_as_uint(d1);
-            cw[j] = pack2(v0 ? q0 : 0.f, v1 ? q1 : 0.f);
+            const float2 t = fma2(acc2(a, j), alpha22, nmx2);
+            float2 v = mul2(make_float2(exp2_approx(t.x), exp2_approx(t.y)), inv2);
+            if (ncol < 32) { v.x = 2 * j < ncol ? v.x : 0.f; v.y = 2 * j + 1 < ncol ? v.y : 0.f; }
+            pw1[j] = pack2(v);
           }
-        };
-        if (__all_sync(0xffffffffu, ncol >= 32)) chunk(std::true_type{}); else chunk(std::false_type{});
-        tmem_st32(trow + TMEM_DP + (uint32_t)(c * 32), a);        // masked dP kept in place for pass B
+        }
+        uint32_t a[32];
+        tmem_ld32(trow + TMEM_DP + (uint32_t)(c * 32), a);
+        if (!clips) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float2 pv = unpack2(pw1[j]), d = mul2(acc2(a, j), sv2);
+            const float2 z0 = mul2(pv, r2), z = fma2(fma2(z0, ns2, pv), r2, z0);
+            const float2 q = add2(add2(z, magic2), nmagic2);
+            dsp2 = fma2(d, fma2(z, m1, q), dsp2);
+            dot2 = fma2(d, pv, dot2);
+            cw[j] = pack2(q);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float2 pv = unpack2(pw1[j]);
+            float2 d = mul2(acc2(a, j), sv2);
+            const float2 z0 = mul2(pv, r2), z = fma2(fma2(z0, ns2, pv), r2, z0);
+            const bool in0 = pv.x <= lim_p, in1 = pv.y <= lim_p;
+            const float2 q = add2(add2(make_float2(fminf(z.x, p.p_hi), fminf(z.y, p.p_hi)), magic2), nmagic2);
+            dsp2 = fma2(d, make_float2(in0 ? q.x - z.x : q.x, in1 ? q.y - z.y : q.y), dsp2);
+            d = make_float2(in0 ? d.x : 0.f, in1 ? d.y : 0.f);
+            dot2 = fma2(d, pv, dot2);
+            cw[j] = pack2(q);
+          }
+        }
       } else {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) cw[j] = 0u;
+        for (int j = 0; j < 16; ++j) pw1[j] = cw[j] = 0u;
       }
-      uint8_t* rowp = gX + (c >> 1) * 16384 + r * 128;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) st16(rowp + ((((c & 1) * 4 + t) ^ (r & 7)) * 16), cw + 4 * t);
+      tile_store(gX + (c >> 1) * 16384, r, c & 1, cw);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
-    mbar_arrive(smem_u32(&bar_p));
-    red_dot[half][r] = dot;
+    mbar_arrive(bar(B_P));
+    red_dot[half][r] = dot2.x + dot2.y;
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    dot = red_dot[0][r] + red_dot[1][r];
-    // ---- pass B: dS = P * (dP - dot), held in registers until the dV product has consumed the codes of P
-    uint32_t sw[2][16];
-#pragma unroll
+    const float2 ndot2 = both(-(red_dot[0][r] + red_dot[1][r]));
+    // ---- pass B: dS = P * (dP - dot), in place of P, held in registers until the dV product has consumed the codes of P
+#pragma unroll 1
     for (int i = 0; i < 2; ++i) {
       const int c = half + 2 * i;
-      if (c < n_chunks) {
-        uint32_t a[32], pw[16];
+      if (c < n_valid) {
+        uint32_t a[32];
         tmem_ld32(trow + TMEM_DP + (uint32_t)(c * 32), a);
-        const int ncol = row_ok ? p.S - c * 32 : 0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          if (t * 8 < ncol) ld16(p.P + prow + c * 32 + t * 8, pw + 4 * t);
-          else { pw[4 * t] = pw[4 * t + 1] = pw[4 * t + 2] = pw[4 * t + 3] = 0u; }
-        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const float2 pv = unpack2(pw[j]);
-          sw[i][j] = pack2(pv.x * (__uint_as_float(a[2 * j]) - dot), pv.y * (__uint_as_float(a[2 * j + 1]) - dot));
+          const float2 pv = unpack2(pw0[j]);
+          float2 d = mul2(acc2(a, j), sv2);
+          if (clips) d = make_float2(pv.x <= lim_p ? d.x : 0.f, pv.y <= lim_p ? d.y : 0.f);
+          pw0[j] = pack2(mul2(pv, add2(d, ndot2)));
         }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) sw[i][j] = 0u;
       }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) { const uint32_t t = pw0[j]; pw0[j] = pw1[j]; pw1[j] = t; }
     }
-    got = mbar_wait(smem_u32(&bar_b), 0, p.wait_ns) && got;
+    got = mbar_wait(bar(B_B), 0, p.wait_ns) && got;
     tc_fence_after();
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int c = half + 2 * i;
-      if (c < 2 * p.n_kb) {
-        uint8_t* rowp = gX + (c >> 1) * 16384 + r * 128;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) st16(rowp + ((((c & 1) * 4 + t) ^ (r & 7)) * 16), sw[i] + 4 * t);
-      }
-    }
+    if (half < n_chunks) tile_store(gX, r, half, pw0);
+    if (half + 2 < n_chunks) tile_store(gX + 16384, r, half, pw1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
-    mbar_arrive(smem_u32(&bar_s));
-    // ---- the three gradients: STE of the Q, K, V quantizers, 32 of the 64 head columns per thread
-    const long long grow = ((long long)b * p.S + r) * 3 * p.H + head * HD + half * 32;
-    uint32_t a[32];
-    tmem_ld32(trow + (uint32_t)(TMEM_DV + half * 32), a);           // complete since bar_b
-    const float ds_v = ste_store(a, row_ok, p.qkv + grow + 2 * p.H, p.dqkv + grow + 2 * p.H, s_p, s_v, p.q_lo, p.q_hi);
-    got = mbar_wait(smem_u32(&bar_o), 0, p.wait_ns) && got;
-    if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
-    tc_fence_after();
-    tmem_ld32(trow + (uint32_t)(TMEM_DQ + half * 32), a);
-    const float ds_q = ste_store(a, row_ok, p.qkv + grow, p.dqkv + grow, p.inv_sqrt_d * s_k, s_q, p.q_lo, p.q_hi);
-    tmem_ld32(trow + (uint32_t)(TMEM_DK + half * 32), a);
-    const float ds_k = ste_store(a, row_ok, p.qkv + grow + p.H, p.dqkv + grow + p.H, p.inv_sqrt_d * s_q, s_k, p.q_lo, p.q_hi);
+    mbar_arrive(bar(B_S));
+    // ---- the three gradients: STE of the Q, K, V quantizers, 32 of the 64 head columns per thread, in place in the tile
+    // that holds the values before quantization, then one tiled store (rows beyond the sequence are clipped)
+    float ds_v = 0.f, ds_q = 0.f, ds_k = 0.f;
+#pragma unroll 1
+    for (int g = 0; g < 3; ++g) {                          // V, Q, K
+      const float step = g == 0 ? s_v : (g == 1 ? s_q : s_k), scale = g == 0 ? s_p : p.inv_sqrt_d * (g == 1 ? s_k : s_q);
+      uint8_t* const tile = g == 1 ? gD : gV;
+      got = mbar_wait(bar(g == 0 ? B_RV : (g == 1 ? B_RQ : B_RK)), 0, p.wait_ns) && got;
+      if (g == 1) { got = mbar_wait(bar(B_O), 0, p.wait_ns) && got; tc_fence_after(); }
+      uint32_t a[32], x[16];
+      tmem_ld32(trow + (uint32_t)((g == 0 ? TMEM_DV : (g == 1 ? TMEM_DQ : TMEM_DK)) + half * 32), a);
+      tile_load(tile, r, half, x);
+      const float2 sc2 = both(scale);
+      float ds = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, step, p.q_hi, range_limit(step, p.q_hi));
+      tile_store(tile, r, half, x);
+      fence_async_shared();
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      ds = row_ok ? ds : 0.f;
+      ds_v = g == 0 ? ds : ds_v; ds_q = g == 1 ? ds : ds_q; ds_k = g == 2 ? ds : ds_k;
+      if (threadIdx.x == 32) {
+        tma_store_4d(&maps.out, g == 1 ? sD : sV, 0, 0, (g == 0 ? 2 * p.h : (g == 1 ? 0 : p.h)) + head, b);
+        tma_store_commit();
+        if (g == 0) {
+          tma_store_wait_read<0>();                        // dV has left the tile: K before quantization
+          mbar_expect_tx(bar(B_RK), 16384u);
+          tma_load_4d(sV, &maps.raw, bar(B_RK), 0, 0, p.h + head, b);
+        }
+      }
+    }
     tc_fence_before();
+    if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
     // ---- one partial per CTA and site, added in a fixed order
-    const float w_p = warp_sum(ds_p), w_q = warp_sum(ds_q), w_k = warp_sum(ds_k), w_v = warp_sum(ds_v);
-    if (lane == 0) { red_part[warp - 1][0] = w_p; red_part[warp - 1][1] = w_q; red_part[warp - 1][2] = w_k; red_part[warp - 1][3] = w_v; }
+    const float w[5] = {warp_sum(dsp2.x + dsp2.y), warp_sum(ds_q), warp_sum(ds_k), warp_sum(ds_v), warp_sum(ds_c)};
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) red_part[warp - 1][i] = w[i];
+    }
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (warp == 1 && lane < 4) {
+    if (warp == 1 && lane < 5) {
       float t = 0.f;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) t += red_part[w][lane];
-      float* dst = lane == 0 ? p.part_p : (lane == 1 ? p.part_q : (lane == 2 ? p.part_k : p.part_v));
+      for (int k = 0; k < 8; ++k) t += red_part[k][lane];
+      float* dst = lane == 0 ? p.part_p : (lane == 1 ? p.part_q : (lane == 2 ? p.part_k : (lane == 3 ? p.part_v : p.part_c)));
       dst[b * p.h + head] = t;
     }
     if (head == 0 && b == 0)             // the slots no CTA owns
       for (int i = p.B * p.h + (int)threadIdx.x - 32; i < p.red_slots; i += 256) {
-        p.part_p[i] = 0.f; p.part_q[i] = 0.f; p.part_k[i] = 0.f; p.part_v[i] = 0.f;
+        p.part_p[i] = 0.f; p.part_q[i] = 0.f; p.part_k[i] = 0.f; p.part_v[i] = 0.f; p.part_c[i] = 0.f;
       }
+    if (threadIdx.x == 32) tma_store_wait_all();
   }
   __syncthreads();
   if (warp == 0) {
@@ -303,31 +318,32 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
 }  // namespace
 
 bool attention_bwd_supported(int S, int head_dim, int dt, int batch_heads) {
-  return dt == 1 && head_dim == HD && S % 8 == 0 && S <= 128 && batch_heads <= RED_BLOCKS;
+  return dt == 1 && head_dim == HD && S % 8 == 0 && S <= 384 && batch_heads <= RED_BLOCKS;
 }
 
-int launch_attention_bwd(const void* qkv_codes, const void* qkv, const void* P, const void* dctx, int B, int S, int h,
-                         int H, const float* s_q, const float* s_k, const float* s_v, const float* s_p, int q_lo,
-                         int q_hi, int p_lo, int p_hi, void* dqkv, float* part_q, float* part_k, float* part_v,
-                         float* part_p, int* status, cudaStream_t st) {
+int launch_attention_bwd(const AttentionBwd& a, cudaStream_t st) {
+  if (a.S > 128) return launch_attention_bwd_long(a, st);
   AttnBwdParams p;
-  p.S = S; p.h = h; p.B = B; p.H = H;
-  p.n16 = (S + 15) / 16 * 16;
-  p.n_kb = (S + 63) / 64;
+  p.S = a.S; p.h = a.h; p.B = a.B; p.H = a.H;
   p.inv_sqrt_d = 1.f / sqrtf((float)HD);
-  p.s_q = s_q; p.s_k = s_k; p.s_v = s_v; p.s_p = s_p;
-  p.q_lo = (float)q_lo; p.q_hi = (float)q_hi; p.p_lo = (float)p_lo; p.p_hi = (float)p_hi;
-  p.P = (const bf16*)P; p.qkv = (const bf16*)qkv; p.dqkv = (bf16*)dqkv;
-  p.part_q = part_q; p.part_k = part_k; p.part_v = part_v; p.part_p = part_p;
+  p.s_q = a.s_q; p.s_k = a.s_k; p.s_v = a.s_v; p.s_p = a.s_p; p.s_c = a.s_c;
+  p.alpha = a.alpha; p.len = a.len; p.stat = a.stat;
+  p.q_hi = (float)a.q_hi; p.p_hi = (float)a.p_hi;
+  p.part_q = a.part_q; p.part_k = a.part_k; p.part_v = a.part_v; p.part_p = a.part_p; p.part_c = a.part_c;
   p.red_slots = RED_BLOCKS;
-  p.status = status;
+  p.status = a.status;
   p.wait_ns = g_wait_limit_ns;
-  CUtensorMap mc, md;
-  OperandDesc oc{qkv_codes, 3LL * H, HD, (long long)S * 3 * H, 0};
-  int rc = make_operand_map(&mc, oc, 2, S, HD, 3 * h, B, 128, HD);
-  if (rc != GEMM_OK) return rc;
-  OperandDesc od{dctx, (long long)H, HD, (long long)S * H, 0};
-  rc = make_operand_map(&md, od, 2, S, HD, h, B, 128, HD);
+  // tensor maps over [tokens, 3H] and [tokens, H] tensors: (64 of a head, S rows, head slots, B)
+  AttnBwdMaps m;
+  const long long S = a.S;
+  auto map = [&](CUtensorMap* out, const void* ptr, int slots) {
+    return make_operand_map(out, OperandDesc{ptr, (long long)slots * HD, HD, S * slots * HD, 0}, 2, a.S, HD, slots, a.B, 128, HD);
+  };
+  int rc = map(&m.codes, a.qkv_codes, 3 * a.h);
+  if (rc == GEMM_OK) rc = map(&m.raw, a.qkv, 3 * a.h);
+  if (rc == GEMM_OK) rc = map(&m.out, a.dqkv, 3 * a.h);
+  if (rc == GEMM_OK) rc = map(&m.dctx, a.dctx, a.h);
+  if (rc == GEMM_OK) rc = map(&m.ctx, a.ctx, a.h);
   if (rc != GEMM_OK) return rc;
   const int smem = 1024 + 4 * 16384 + 32768;      // two CTAs per SM
   static bool attr_set = false;
@@ -335,8 +351,8 @@ int launch_attention_bwd(const void* qkv_codes, const void* qkv, const void* P, 
     if (cudaFuncSetAttribute(attention_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GEMM_ERR_CUDA;
     attr_set = true;
   }
-  Scope sc("attention_bwd_tcgen05", 8.0 * B * h * (double)S * S * HD, 1, st);
-  if (launch_k(attention_bwd_kernel, dim3(h, B), ATB_THREADS, smem, st, mc, md, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  Scope sc("attention_bwd_tcgen05", 10.0 * a.B * a.h * (double)S * S * HD, 1, st);
+  if (launch_k(attention_bwd_kernel, dim3(a.h, a.B), ATB_THREADS, smem, st, m, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }
 

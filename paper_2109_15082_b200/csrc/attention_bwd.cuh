@@ -1,0 +1,85 @@
+// Pieces shared by the attention backward kernels: pairs of values, rows of swizzled operand tiles, the straight-through
+// pass of a symmetric quantizer over 32 values of a row.
+#pragma once
+#include "gemm.h"
+#include "kernels.h"
+#include "tc_ptx.cuh"
+
+namespace mrem {
+namespace att {
+
+constexpr int HD = 64;                    // head size
+
+__device__ __forceinline__ void ld16(const void* p, uint32_t* w) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
+}
+__device__ __forceinline__ void st16(void* p, const uint32_t* w) {
+  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ float2 unpack2(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
+__device__ __forceinline__ uint32_t pack2(float2 v) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 acc2(const uint32_t* a, int j) { return make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])); }
+
+// The largest non-negative bfloat16 value whose quotient by `step` is within the code range (quotient() is monotonic, and
+// for bfloat16 values the IEEE division): |x| <= this is the straight-through mask.
+__device__ __forceinline__ float range_limit(float step, float hi) {
+  const float r = __frcp_rn(step);
+  const uint32_t b = __float_as_uint(hi * step) >> 16;
+  float lim = __uint_as_float((b - 1u) << 16);
+  if (quotient(__uint_as_float(b << 16), step, r) <= hi) lim = __uint_as_float(b << 16);
+  if (quotient(__uint_as_float((b + 1u) << 16), step, r) <= hi) lim = __uint_as_float((b + 1u) << 16);
+  return lim;
+}
+
+// Straight-through pass of one symmetric quantizer over 32 values of a row: x (bf16 pairs before quantization, replaced by the
+// masked gradient as bf16 pairs), g(j) = the incoming gradient of pair j.  Returns the sum of the step-size terms.
+template <class G>
+__device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi, float lim) {
+  const float2 r2 = both(__frcp_rn(step)), ns2 = both(-step), magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
+  __nv_bfloat162 mx = __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[0]));
+#pragma unroll
+  for (int j = 1; j < 16; ++j) mx = __hmax2(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[j])));
+  const float2 m = __bfloat1622float2(mx);
+  float2 ds = both(0.f);
+  if (__all_sync(0xffffffffu, fmaxf(m.x, m.y) <= lim)) {       // nothing clipped in the whole warp
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float2 xv = unpack2(x[j]), gv = g(j);
+      const float2 z0 = mul2(xv, r2), z = fma2(fma2(z0, ns2, xv), r2, z0);
+      const float2 q = add2(add2(z, magic2), nmagic2);
+      ds = fma2(gv, fma2(z, m1, q), ds);
+      x[j] = pack2(gv);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float2 xv = unpack2(x[j]);
+      float2 gv = g(j);
+      const float2 z0 = mul2(xv, r2), z = fma2(fma2(z0, ns2, xv), r2, z0);
+      const bool in0 = fabsf(xv.x) <= lim, in1 = fabsf(xv.y) <= lim;
+      const float2 c = make_float2(fminf(fmaxf(z.x, -hi), hi), fminf(fmaxf(z.y, -hi), hi));
+      const float2 q = add2(add2(c, magic2), nmagic2);
+      ds = fma2(gv, make_float2(in0 ? q.x - z.x : q.x, in1 ? q.y - z.y : q.y), ds);
+      x[j] = pack2(make_float2(in0 ? gv.x : 0.f, in1 ? gv.y : 0.f));
+    }
+  }
+  return ds.x + ds.y;
+}
+
+// 32 columns (64 bytes) of a row of a 128-byte-swizzled tile of 128 rows x 128 bytes
+__device__ __forceinline__ void tile_load(const uint8_t* tile, int r, int half, uint32_t* w) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) ld16(tile + r * 128 + (((half * 4 + t) ^ (r & 7)) * 16), w + 4 * t);
+}
+__device__ __forceinline__ void tile_store(uint8_t* tile, int r, int half, const uint32_t* w) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) st16(tile + r * 128 + (((half * 4 + t) ^ (r & 7)) * 16), w + 4 * t);
+}
+
+}  // namespace att
+}  // namespace mrem

@@ -1,0 +1,554 @@
+// Fused attention backward of the student for 129 to 384 tokens (head size 64), two kernels:
+//   attention_bwd_q_kernel   one 128-query block of one head per CTA: STE of the context's quantizer (the masked gradient is
+//                            also written for the second kernel), P from the scores, the row sums of dP P, dQ
+//   attention_bwd_kv_kernel  one 128-key block of one head per CTA: dK and dV, accumulated in TMEM over the queries in chunks of
+//                            64, from TRANSPOSED score tiles (keys in the lanes), so that the codes of P^T and dS^T are
+//                            plain K-major operands
+// The probabilities are formed again from the codes of Q and K and the forward pass's row statistics in both (bit for bit
+// what the forward pass used), so nothing of size seq x seq is ever written: the kernel-per-operation path moves eleven such
+// tensors through memory (75 MB each at 16 x 16 x 384 x 384).  dP is formed twice; the products are far from the limit.
+// The CTAs of one head form a cluster that adds its step-size partials through distributed shared memory in rank order.
+// All waits are time-bounded.
+//
+// What bounds them: the arithmetic on the scores, about 15 + 15 issue slots each.  The query kernel keeps a whole row block of
+// scores in TMEM (384 of 512 columns, one CTA per SM) and therefore runs four threads per row; the key kernel needs 256
+// columns and 103 KB, two CTAs per SM.  16 x 16 heads x 384 x 384: the products, softmax backward and STE passes took 190 us
+// and the forward pass 35 us more for writing P and its codes; now 95 + 68 us.
+#include "attention_bwd.cuh"
+
+namespace mrem {
+
+using namespace att;
+
+namespace {
+
+struct LongParams {
+  int S, h, B;
+  float inv_sqrt_d;
+  const float *s_q, *s_k, *s_v, *s_p, *s_c;
+  const float* alpha;
+  const int* len;
+  const float2* stat;
+  float* dot;                // [B, h, S] row sums of dP P
+  float q_hi, p_hi;
+  float *part_q, *part_k, *part_v, *part_p, *part_c;
+  int red_slots;
+  int* status;
+  unsigned long long wait_ns;
+};
+
+// Adds `n` per-CTA sums (the same array in every CTA, filled before the call) over the CTAs of the cluster, in rank order, in
+// the first CTA; all threads of all CTAs call it.
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void store_remote(float* local, uint32_t rank, float v) {
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(local)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+// ------------------------------------------------------------------ queries
+constexpr int Q_THREADS = 544;            // warp 0: TMA + MMA issue; 16 warps, four threads per query row
+struct QMaps { CUtensorMap codes, raw, dctx, ctx, dctx_out, out; };
+
+__global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __grid_constant__ QMaps maps, const __grid_constant__ LongParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  enum { B_CTX, B_QK, B_V, B_STE, B_A, B_P, B_B, B_RQ, B_S, B_O, N_BARS };
+  __shared__ __align__(8) uint64_t bars[N_BARS];
+  __shared__ uint32_t tmem_slot;
+  __shared__ float red_dot[4][128];
+  __shared__ float red_part[16][3];
+  __shared__ float cta_part[3][3];                         // [cluster rank][site]
+  constexpr int TMEM_DQ = 384;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int qb = blockIdx.x, head = blockIdx.y, b = blockIdx.z, q0 = qb * 128;
+  const int n_box = (p.S + 127) / 128;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  // X (dS, up to six blocks of 64 keys) starts where V was; the context sits behind V before
+  const uint32_t sQ = base, sD = sQ + 16384, sK = sD + 16384, sX = sK + n_box * 16384, sV = sX, sC = sV + n_box * 16384;
+  uint8_t* const g0 = smem_raw + (base - smem_u32(smem_raw));
+  uint8_t *const gD = g0 + (sD - base), *const gX = g0 + (sX - base), *const gC = g0 + (sC - base);
+  auto bar = [&](int i) { return smem_u32(&bars[i]); };
+  pdl_trigger();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_STE || i == B_P || i == B_S) ? 512 : 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait();
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  const int len = p.len[b], n_valid = (len + 31) / 32;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const int boxes = (len + 127) / 128;
+      mbar_expect_tx(bar(B_CTX), 2u * 16384u);
+      tma_load_4d(sD, &maps.dctx, bar(B_CTX), 0, q0, head, b);
+      tma_load_4d(sC, &maps.ctx, bar(B_CTX), 0, q0, head, b);
+      mbar_expect_tx(bar(B_QK), 16384u * (uint32_t)(1 + boxes));
+      tma_load_4d(sQ, &maps.codes, bar(B_QK), 0, q0, head, b);
+#pragma unroll 1
+      for (int i = 0; i < boxes; ++i) tma_load_4d(sK + i * 16384, &maps.codes, bar(B_QK), 0, i * 128, p.h + head, b);
+      mbar_expect_tx(bar(B_V), 16384u * (uint32_t)boxes);
+#pragma unroll 1
+      for (int i = 0; i < boxes; ++i) tma_load_4d(sV + i * 16384, &maps.codes, bar(B_V), 0, i * 128, 2 * p.h + head, b);
+      const uint32_t f32 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
+      auto scores = [&](uint32_t a, uint32_t keys) {       // [128 x valid keys] = A [128 x d] * keys^T, at most 256 keys a piece
+#pragma unroll 1
+        for (int n0 = 0; n0 < n_valid * 32; n0 += 256) {
+          const uint32_t id = f32 | ((uint32_t)(min(256, n_valid * 32 - n0) >> 3) << 17);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            tc_mma<0>(tmem + (uint32_t)n0, smem_desc(a + k * 32, 16u, 1024u), smem_desc(keys + n0 * 128 + k * 32, 16u, 1024u), id, (uint32_t)(k != 0));
+        }
+      };
+      bool ok = mbar_wait(bar(B_QK), 0, p.wait_ns);
+      if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_TMA);
+      tc_fence_after();
+      if (ok) scores(sQ, sK);
+      tc_commit(bar(B_A));
+      ok = mbar_wait(bar(B_STE), 0, p.wait_ns) && ok;
+      if (ok) tma_store_4d(&maps.dctx_out, sD, 0, q0, head, b);     // the masked context gradient, for the key kernel
+      tma_store_commit();
+      ok = mbar_wait(bar(B_V), 0, p.wait_ns) && ok;
+      ok = mbar_wait(bar(B_P), 0, p.wait_ns) && ok;
+      tc_fence_after();
+      if (ok) scores(sD, sV);                              // dP_hat, over the scores
+      tc_commit(bar(B_B));
+      ok = mbar_wait(bar(B_B), 0, p.wait_ns) && ok;
+      tma_store_wait_read<0>();
+      mbar_expect_tx(bar(B_RQ), 16384u);                   // the dctx tile is free: Q before quantization
+      tma_load_4d(sD, &maps.raw, bar(B_RQ), 0, q0, head, b);
+      ok = mbar_wait(bar(B_S), 0, p.wait_ns) && ok;
+      if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_EPI);
+      tc_fence_after();
+      if (ok)
+#pragma unroll 1
+        for (int ks = 0; ks < (len + 15) / 16; ++ks)       // dQ_hat [q x d] = dS [q x keys] * K_q [keys x d]
+          tc_mma<0>(tmem + TMEM_DQ, smem_desc(sX + (ks >> 2) * 16384 + (ks & 3) * 32, 16u, 1024u), smem_desc(sK + ks * 2048, 8192u, 1024u),
+                    f32 | (1u << 16) | ((uint32_t)(HD >> 3) << 17), (uint32_t)(ks != 0));
+      tc_commit(bar(B_O));
+      tma_store_wait_all();
+    }
+  } else {
+    const int quad = warp & 3, part = (warp - 1) >> 2;
+    const int r = quad * 32 + lane, q = q0 + r;
+    const bool row_ok = q < p.S;
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const float s_p = *p.s_p, s_v = *p.s_v, s_q = *p.s_q, s_k = *p.s_k, s_c = *p.s_c;
+    const long long srow = ((long long)b * p.h + head) * p.S + q;
+    float2 st = make_float2(0.f, 0.f);                     // rows beyond the sequence: P = 0
+    if (row_ok) st = p.stat[srow];
+    const float alpha2 = *p.alpha * 1.4426950408889634f;
+    bool got = mbar_wait(bar(B_CTX), 0, p.wait_ns);
+    float ds_c = 0.f, ds_q = 0.f;
+    if (part < 2) {                                        // STE of the context's quantizer, 32 columns per thread, in place
+      uint32_t d[16], x[16];
+      tile_load(gD, r, part, d);
+      tile_load(gC, r, part, x);
+      ds_c = ste32(x, [&](int j) { return unpack2(d[j]); }, s_c, p.q_hi, range_limit(s_c, p.q_hi));
+      tile_store(gD, r, part, x);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive(bar(B_STE));
+    got = mbar_wait(bar(B_A), 0, p.wait_ns) && got;
+    tc_fence_after();
+    const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p),
+                 magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
+    const float lim_p = range_limit(s_p, p.p_hi);
+    const bool clips = !__all_sync(0xffffffffu, __bfloat162float(__float2bfloat16_rn(st.y)) <= lim_p);   // largest P of the row: 1 / sum
+    // ---- this thread's probabilities: chunks part, part + 4, part + 8 of 32 keys
+    // (rolled loops, the chunks rotating through the registers: see attention_bwd.cu)
+    uint32_t pw0[16], pw1[16], pw2[16];
+    auto rotate = [&](const uint32_t* w) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) { const uint32_t t = w[j]; pw0[j] = pw1[j]; pw1[j] = pw2[j]; pw2[j] = t; }
+    };
+#pragma unroll
+    for (int j = 0; j < 16; ++j) pw1[j] = pw2[j] = 0u;
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      const int c = part + 4 * i;
+      rotate(pw2);
+      if (c >= n_valid) continue;
+      const int ncol = len - c * 32;
+      uint32_t a[32];
+      tmem_ld32(trow + (uint32_t)(c * 32), a);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 t = fma2(acc2(a, j), alpha22, nmx2);
+        float2 v = mul2(make_float2(exp2_approx(t.x), exp2_approx(t.y)), inv2);
+        if (ncol < 32) { v.x = 2 * j < ncol ? v.x : 0.f; v.y = 2 * j + 1 < ncol ? v.y : 0.f; }
+        pw2[j] = pack2(v);
+      }
+    }
+    tc_fence_before();
+    mbar_arrive(bar(B_P));
+    got = mbar_wait(bar(B_B), 0, p.wait_ns) && got;
+    tc_fence_after();
+    // ---- STE of P's quantizer and the row sums
+    float2 dot2 = both(0.f), dsp2 = both(0.f);
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      const int c = part + 4 * i;
+      if (c >= n_valid) { rotate(pw0); continue; }
+      uint32_t a[32];
+      tmem_ld32(trow + (uint32_t)(c * 32), a);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 pv = unpack2(pw0[j]);
+        float2 d = mul2(acc2(a, j), sv2);
+        const float2 z0 = mul2(pv, r2), z = fma2(fma2(z0, ns2, pv), r2, z0);
+        if (!clips) {
+          const float2 qv = add2(add2(z, magic2), nmagic2);
+          dsp2 = fma2(d, fma2(z, m1, qv), dsp2);
+        } else {
+          const bool in0 = pv.x <= lim_p, in1 = pv.y <= lim_p;
+          const float2 qv = add2(add2(make_float2(fminf(z.x, p.p_hi), fminf(z.y, p.p_hi)), magic2), nmagic2);
+          dsp2 = fma2(d, make_float2(in0 ? qv.x - z.x : qv.x, in1 ? qv.y - z.y : qv.y), dsp2);
+          d = make_float2(in0 ? d.x : 0.f, in1 ? d.y : 0.f);
+        }
+        dot2 = fma2(d, pv, dot2);
+      }
+      rotate(pw0);
+    }
+    red_dot[part][r] = dot2.x + dot2.y;
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    const float dot = (red_dot[0][r] + red_dot[1][r]) + (red_dot[2][r] + red_dot[3][r]);
+    if (part == 0 && row_ok) p.dot[srow] = dot;
+    const float2 ndot2 = both(-dot);
+    // ---- dS = P * (dP - dot) into the operand tile (V, under it, has been consumed by dP's product)
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      const int c = part + 4 * i;
+      if (c >= n_valid) break;
+      uint32_t a[32], w[16];
+      tmem_ld32(trow + (uint32_t)(c * 32), a);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 pv = unpack2(pw0[j]);
+        float2 d = mul2(acc2(a, j), sv2);
+        if (clips) d = make_float2(pv.x <= lim_p ? d.x : 0.f, pv.y <= lim_p ? d.y : 0.f);
+        w[j] = pack2(mul2(pv, add2(d, ndot2)));
+      }
+      tile_store(gX + (c >> 1) * 16384, r, c & 1, w);
+      rotate(pw0);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    mbar_arrive(bar(B_S));
+    // ---- dQ: STE of Q's quantizer, in place in the tile that holds Q before quantization
+    got = mbar_wait(bar(B_RQ), 0, p.wait_ns) && got;
+    got = mbar_wait(bar(B_O), 0, p.wait_ns) && got;
+    tc_fence_after();
+    if (part < 2) {
+      uint32_t a[32], x[16];
+      tmem_ld32(trow + (uint32_t)(TMEM_DQ + part * 32), a);
+      tile_load(gD, r, part, x);
+      const float2 sc2 = both(p.inv_sqrt_d * s_k);
+      ds_q = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, s_q, p.q_hi, range_limit(s_q, p.q_hi));
+      tile_store(gD, r, part, x);
+      if (!row_ok) ds_q = 0.f;
+    }
+    fence_async_shared();
+    tc_fence_before();
+    if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
+    const float w[3] = {warp_sum(dsp2.x + dsp2.y), warp_sum(ds_q), warp_sum(ds_c)};
+    if (lane == 0) { red_part[warp - 1][0] = w[0]; red_part[warp - 1][1] = w[1]; red_part[warp - 1][2] = w[2]; }
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    if (threadIdx.x == 32) { tma_store_4d(&maps.out, sD, 0, q0, head, b); tma_store_commit(); }
+    if (warp == 1 && lane < 3) {
+      float t = 0.f;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) t += red_part[k][lane];
+      store_remote(&cta_part[cluster_rank()][lane], 0, t);
+    }
+    if (threadIdx.x == 32) tma_store_wait_all();
+  }
+  __syncthreads();
+  cluster_sync();
+  if (qb == 0 && threadIdx.x < 3) {
+    float t = 0.f;
+    for (int k = 0; k < (int)gridDim.x; ++k) t += cta_part[k][threadIdx.x];
+    float* dst = threadIdx.x == 0 ? p.part_p : (threadIdx.x == 1 ? p.part_q : p.part_c);
+    dst[b * p.h + head] = t;
+  }
+  if (qb == 0 && head == 0 && b == 0)                      // the slots no head owns
+    for (int i = p.B * p.h + (int)threadIdx.x; i < p.red_slots; i += Q_THREADS) { p.part_p[i] = 0.f; p.part_q[i] = 0.f; p.part_c[i] = 0.f; }
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ keys and values
+constexpr int KV_THREADS = 288;           // warp 0: TMA + MMA issue; 8 warps, two threads per key, 32 of a chunk's 64 queries each
+struct KvMaps { CUtensorMap codes, codes64, raw, dctx64, out; };
+
+__global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const __grid_constant__ KvMaps maps, const __grid_constant__ LongParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  enum { B_KV, B_F0, B_F1, B_A, B_P, B_W, B_RAW, N_BARS };
+  __shared__ __align__(8) uint64_t bars[N_BARS];
+  __shared__ uint32_t tmem_slot;
+  __shared__ float red_part[8][2];
+  __shared__ float cta_part[3][2];
+  constexpr int TMEM_S = 0, TMEM_DP = 64, TMEM_DV = 128, TMEM_DK = 192;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kb = blockIdx.x, head = blockIdx.y, b = blockIdx.z, k0 = kb * 128;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t sK = base, sV = sK + 16384, sC = sV + 16384 /* two buffers of Q | dctx chunks */, sP = sC + 32768, sS = sP + 16384;
+  uint8_t* const g0 = smem_raw + (base - smem_u32(smem_raw));
+  uint8_t *const gK = g0, *const gV = g0 + (sV - base), *const gP = g0 + (sP - base), *const gS = g0 + (sS - base);
+  float4* const qstat = reinterpret_cast<float4*>(g0 + (sS - base) + 16384);   // per query: -max, 1 / sum, -dot
+  auto bar = [&](int i) { return smem_u32(&bars[i]); };
+  pdl_trigger();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), i == B_P ? 256 : 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(256) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait();
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  const int len = p.len[b], n_q = (p.S + 63) / 64;
+  const bool active = k0 < len;                            // a block of padded keys has zero gradients
+  const float s_p = *p.s_p, lim_p = range_limit(s_p, p.p_hi);
+  bool over = false;
+  if (active)
+    for (int i = threadIdx.x; i < n_q * 64; i += KV_THREADS) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);          // queries beyond the sequence: P = 0
+      if (i < p.S) {
+        const long long at = ((long long)b * p.h + head) * p.S + i;
+        const float2 st = p.stat[at];
+        v = make_float4(-st.x, st.y, -p.dot[at], 0.f);
+      }
+      over = over || __bfloat162float(__float2bfloat16_rn(v.y)) > lim_p;   // the largest P of the query's row
+      qstat[i] = v;
+    }
+  const bool clips = __syncthreads_or(over);
+
+  if (warp == 0) {
+    if (lane == 0 && active) {
+      const uint32_t f32 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
+      const uint32_t id_s = f32 | (8u << 17), id_g = f32 | (8u << 17) | (1u << 16);     // N = 64; B K-major / MN-major
+      auto load_chunk = [&](int c) {
+        const uint32_t dst = sC + (c & 1) * 16384, fb = bar(B_F0 + (c & 1));
+        mbar_expect_tx(fb, 16384u);
+        tma_load_4d(dst, &maps.codes64, fb, 0, c * 64, head, b);
+        tma_load_4d(dst + 8192, &maps.dctx64, fb, 0, c * 64, head, b);
+      };
+      mbar_expect_tx(bar(B_KV), 2u * 16384u);
+      tma_load_4d(sK, &maps.codes, bar(B_KV), 0, k0, p.h + head, b);
+      tma_load_4d(sV, &maps.codes, bar(B_KV), 0, k0, 2 * p.h + head, b);
+      load_chunk(0);
+      if (n_q > 1) load_chunk(1);
+      bool ok = mbar_wait(bar(B_KV), 0, p.wait_ns);
+#pragma unroll 1
+      for (int c = 0; c <= n_q; ++c) {
+        if (c > 0) { ok = mbar_wait(bar(B_P), (uint32_t)((c - 1) & 1), p.wait_ns) && ok; tc_fence_after(); }
+        if (c < n_q) {                                     // S^T and dP^T of chunk c: [128 keys x 64 queries]
+          ok = mbar_wait(bar(B_F0 + (c & 1)), (uint32_t)((c >> 1) & 1), p.wait_ns) && ok;
+          tc_fence_after();
+          const uint32_t q = sC + (c & 1) * 16384, d = q + 8192;
+          if (ok)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              tc_mma<0>(tmem + TMEM_S, smem_desc(sK + k * 32, 16u, 1024u), smem_desc(q + k * 32, 16u, 1024u), id_s, (uint32_t)(k != 0));
+              tc_mma<0>(tmem + TMEM_DP, smem_desc(sV + k * 32, 16u, 1024u), smem_desc(d + k * 32, 16u, 1024u), id_s, (uint32_t)(k != 0));
+            }
+          tc_commit(bar(B_A));
+        }
+        if (c > 0) {                                       // dV += P_q^T dctx, dK += dS^T Q_q of chunk c - 1
+          const uint32_t q = sC + ((c - 1) & 1) * 16384, d = q + 8192;
+          if (ok)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+              tc_mma<0>(tmem + TMEM_DV, smem_desc(sP + ks * 32, 16u, 1024u), smem_desc(d + ks * 2048, 8192u, 1024u), id_g, (uint32_t)(c > 1 || ks != 0));
+              tc_mma<0>(tmem + TMEM_DK, smem_desc(sS + ks * 32, 16u, 1024u), smem_desc(q + ks * 2048, 8192u, 1024u), id_g, (uint32_t)(c > 1 || ks != 0));
+            }
+          tc_commit(bar(B_W));
+          if (c + 1 < n_q) {                               // the buffer of chunk c - 1 is free once those products have run
+            ok = mbar_wait(bar(B_W), (uint32_t)((c - 1) & 1), p.wait_ns) && ok;
+            load_chunk(c + 1);
+          }
+        }
+        if (c == n_q - 1) {                                // the codes of K and V are not needed any more: the values before quantization
+          ok = mbar_wait(bar(B_A), (uint32_t)(c & 1), p.wait_ns) && ok;
+          mbar_expect_tx(bar(B_RAW), 2u * 16384u);
+          tma_load_4d(sV, &maps.raw, bar(B_RAW), 0, k0, 2 * p.h + head, b);
+          tma_load_4d(sK, &maps.raw, bar(B_RAW), 0, k0, p.h + head, b);
+        }
+      }
+      if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_EPI);
+    }
+  } else {
+    const int quad = warp & 3, half = (warp - 1) >> 2;
+    const int r = quad * 32 + lane, key = k0 + r;
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    float ds_v = 0.f, ds_k = 0.f;
+    if (active) {
+      const float s_v = *p.s_v, s_q = *p.s_q, s_k = *p.s_k;
+      const float alpha2 = *p.alpha * 1.4426950408889634f, keep = key < len ? 1.f : 0.f;
+      const float2 alpha22 = both(alpha2), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p), magic2 = both(ROUND_MAGIC),
+                   nmagic2 = both(-ROUND_MAGIC);
+      bool got = true;
+#pragma unroll 1
+      for (int c = 0; c < n_q; ++c) {
+        got = mbar_wait(bar(B_A), (uint32_t)(c & 1), p.wait_ns) && got;
+        tc_fence_after();
+        uint32_t pw[16], w[16];
+        const float4* st = qstat + c * 64 + half * 32;
+        {
+          uint32_t a[32];
+          tmem_ld32(trow + (uint32_t)(TMEM_S + half * 32), a);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float4 s0 = st[2 * j], s1 = st[2 * j + 1];
+            const float2 t = fma2(acc2(a, j), alpha22, make_float2(s0.x, s1.x));
+            const float2 v = mul2(make_float2(exp2_approx(t.x), exp2_approx(t.y)), make_float2(s0.y, s1.y));
+            pw[j] = pack2(make_float2(keep != 0.f ? v.x : 0.f, keep != 0.f ? v.y : 0.f));
+          }
+        }
+        uint32_t a[32];
+        tmem_ld32(trow + (uint32_t)(TMEM_DP + half * 32), a);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float2 pv = unpack2(pw[j]);
+          float2 d = mul2(acc2(a, j), sv2);
+          const float2 z0 = mul2(pv, r2);
+          float2 z = fma2(fma2(z0, ns2, pv), r2, z0);
+          if (clips) {
+            d = make_float2(pv.x <= lim_p ? d.x : 0.f, pv.y <= lim_p ? d.y : 0.f);
+            z = make_float2(fminf(z.x, p.p_hi), fminf(z.y, p.p_hi));
+          }
+          w[j] = pack2(mul2(pv, add2(d, make_float2(st[2 * j].z, st[2 * j + 1].z))));
+          pw[j] = pack2(add2(add2(z, magic2), nmagic2));
+        }
+        if (c > 0) {                                       // the products of the chunk before have read the two tiles
+          got = mbar_wait(bar(B_W), (uint32_t)((c - 1) & 1), p.wait_ns) && got;
+          tc_fence_after();
+        }
+        tile_store(gP, r, half, pw);
+        tile_store(gS, r, half, w);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_fence_before();
+        mbar_arrive(bar(B_P));
+      }
+      got = mbar_wait(bar(B_W), (uint32_t)((n_q - 1) & 1), p.wait_ns) && got;
+      got = mbar_wait(bar(B_RAW), 0, p.wait_ns) && got;
+      tc_fence_after();
+#pragma unroll 1
+      for (int g = 0; g < 2; ++g) {                        // V, K: in place in the tile that holds the values before quantization
+        const float step = g == 0 ? s_v : s_k;
+        uint8_t* const tile = g == 0 ? gV : gK;
+        uint32_t a[32], x[16];
+        tmem_ld32(trow + (uint32_t)((g == 0 ? TMEM_DV : TMEM_DK) + half * 32), a);
+        tile_load(tile, r, half, x);
+        const float2 sc2 = both(g == 0 ? s_p : p.inv_sqrt_d * s_q);
+        float ds = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, step, p.q_hi, range_limit(step, p.q_hi));
+        tile_store(tile, r, half, x);
+        ds = key < p.S ? ds : 0.f;
+        if (g == 0) ds_v = ds; else ds_k = ds;
+      }
+      tc_fence_before();
+      if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
+    } else {
+      uint32_t z[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) z[j] = 0u;
+      tile_store(gV, r, half, z);
+      tile_store(gK, r, half, z);
+    }
+    fence_async_shared();
+    const float w0 = warp_sum(ds_v), w1 = warp_sum(ds_k);
+    if (lane == 0) { red_part[warp - 1][0] = w0; red_part[warp - 1][1] = w1; }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (threadIdx.x == 32) {
+      tma_store_4d(&maps.out, sV, 0, k0, 2 * p.h + head, b);
+      tma_store_4d(&maps.out, sK, 0, k0, p.h + head, b);
+      tma_store_commit();
+    }
+    if (warp == 1 && lane < 2) {
+      float t = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) t += red_part[k][lane];
+      store_remote(&cta_part[cluster_rank()][lane], 0, t);
+    }
+    if (threadIdx.x == 32) tma_store_wait_all();
+  }
+  __syncthreads();
+  cluster_sync();
+  if (kb == 0 && threadIdx.x < 2) {
+    float t = 0.f;
+    for (int k = 0; k < (int)gridDim.x; ++k) t += cta_part[k][threadIdx.x];
+    (threadIdx.x == 0 ? p.part_v : p.part_k)[b * p.h + head] = t;
+  }
+  if (kb == 0 && head == 0 && b == 0)
+    for (int i = p.B * p.h + (int)threadIdx.x; i < p.red_slots; i += KV_THREADS) { p.part_v[i] = 0.f; p.part_k[i] = 0.f; }
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+  }
+}
+
+}  // namespace
+
+int launch_attention_bwd_long(const AttentionBwd& a, cudaStream_t st) {
+  LongParams p;
+  p.S = a.S; p.h = a.h; p.B = a.B;
+  p.inv_sqrt_d = 1.f / sqrtf((float)HD);
+  p.s_q = a.s_q; p.s_k = a.s_k; p.s_v = a.s_v; p.s_p = a.s_p; p.s_c = a.s_c;
+  p.alpha = a.alpha; p.len = a.len; p.stat = a.stat; p.dot = a.dot;
+  p.q_hi = (float)a.q_hi; p.p_hi = (float)a.p_hi;
+  p.part_q = a.part_q; p.part_k = a.part_k; p.part_v = a.part_v; p.part_p = a.part_p; p.part_c = a.part_c;
+  p.red_slots = RED_BLOCKS;
+  p.status = a.status;
+  p.wait_ns = g_wait_limit_ns;
+  const long long S = a.S;
+  auto map = [&](CUtensorMap* out, const void* ptr, int slots, int rows) {     // (64 of a head, S rows, head slots, B)
+    return make_operand_map(out, OperandDesc{ptr, (long long)slots * HD, HD, S * slots * HD, 0}, 2, a.S, HD, slots, a.B, rows, HD);
+  };
+  QMaps mq;
+  KvMaps mk;
+  int rc = map(&mq.codes, a.qkv_codes, 3 * a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mq.raw, a.qkv, 3 * a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mq.dctx, a.dctx, a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mq.ctx, a.ctx, a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mq.dctx_out, a.dctx_masked, a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mq.out, a.dqkv, 3 * a.h, 128);
+  if (rc == GEMM_OK) rc = map(&mk.codes64, a.qkv_codes, 3 * a.h, 64);
+  if (rc == GEMM_OK) rc = map(&mk.dctx64, a.dctx_masked, a.h, 64);
+  if (rc != GEMM_OK) return rc;
+  mk.codes = mq.codes; mk.raw = mq.raw; mk.out = mq.out;
+  const int n_box = (a.S + 127) / 128, n_kb = (a.S + 63) / 64;
+  const int smem_q = 1024 + 16384 * (2 + n_box + n_kb), smem_k = 1024 + 6 * 16384 + n_kb * 64 * (int)sizeof(float4);
+  static bool attr_set = false;
+  if (!attr_set) {
+    if (cudaFuncSetAttribute(attention_bwd_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + 16384 * 11) != cudaSuccess ||
+        cudaFuncSetAttribute(attention_bwd_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + 6 * 16384 + 6144) != cudaSuccess)
+      return GEMM_ERR_CUDA;
+    attr_set = true;
+  }
+  const dim3 grid(n_box, a.h, a.B);
+  Scope sc("attention_bwd_tcgen05", 14.0 * a.B * a.h * (double)S * S * HD, 1, st);
+  if (launch_cluster(attention_bwd_q_kernel, grid, Q_THREADS, smem_q, st, n_box, mq, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  if (launch_cluster(attention_bwd_kv_kernel, grid, KV_THREADS, smem_k, st, n_box, mk, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
+}
+
+}  // namespace mrem

@@ -42,6 +42,7 @@ struct AttnParams {
   bf16* ctx;                 // [B*S, H]
   int8_t* ctx_q8;            // [B*S, H]
   bf16* ctx_qt;              // [B*S, H]
+  AttentionStats stats;      // for the backward pass (null members: none)
   int* status;
   unsigned long long wait_ns;  // limit of each wait on an mbarrier
 };
@@ -196,6 +197,10 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
       for (int k = 1; k < TPR; ++k) sum += red[1][k][r];
     }
     const float inv_sum = __frcp_rn(sum);
+    if (p.stats.row && part == 0) {
+      if (row_ok) p.stats.row[((long long)b * p.h + head) * p.S + q] = make_float2(mx2, inv_sum);
+      if (r == 0 && qb == 0 && head == 0) { p.stats.len[b] = len; if (b == 0) *p.stats.alpha = alpha; }
+    }
     const float2 inv2 = make_float2(inv_sum, inv_sum), r2 = make_float2(r_ps, r_ps), ns2 = make_float2(-ps, -ps);
     const float2 magic2 = make_float2(ROUND_MAGIC, ROUND_MAGIC), nmagic2 = make_float2(-ROUND_MAGIC, -ROUND_MAGIC);
     const long long prow = (((long long)b * p.h + head) * p.S + q) * p.S;
@@ -279,7 +284,7 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
           if ((j & 2) == 0) c8[j >> 2] = two; else c8[j >> 2] |= two << 16;
         }
       }
-      if (row_ok) {
+      if (row_ok && p.ctx) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) store16(p.ctx + crow + hh * 32 + t * 8, w + 4 * t);
         if constexpr (QUANT) {
@@ -320,7 +325,7 @@ bool attention_fwd_supported(int S, int head_dim, int dt) { return dt == 1 && he
 int launch_attention_fwd(const void* qkv, int B, int S, int h, int H, const int* valid_len, float alpha_const,
                          const float* a_p0, const float* a_p1, const float* c_p0, const float* c_p1,
                          const float* p_step, int p_lo, int p_hi, void* P, void* P_qt, void* ctx, const float* c_step,
-                         int c_qmax, int8_t* ctx_q8, void* ctx_qt, int* status, cudaStream_t st) {
+                         int c_qmax, int8_t* ctx_q8, void* ctx_qt, int* status, cudaStream_t st, const AttentionStats* stats) {
   AttnParams p;
   p.S = S; p.h = h; p.B = B; p.H = H;
   int cols = 64;
@@ -331,6 +336,7 @@ int launch_attention_fwd(const void* qkv, int B, int S, int h, int H, const int*
   p.p_step = p_step; p.p_lo = (float)p_lo; p.p_hi = (float)p_hi;
   p.c_step = c_step; p.c_qmax = (float)c_qmax;
   p.P = (bf16*)P; p.P_qt = (bf16*)P_qt; p.ctx = (bf16*)ctx; p.ctx_q8 = ctx_q8; p.ctx_qt = (bf16*)ctx_qt;
+  p.stats = stats ? *stats : AttentionStats{nullptr, nullptr, nullptr};
   p.status = status;
   p.wait_ns = g_wait_limit_ns;
   // one map over the [tokens, 3H] tensor: (64 of a head, S rows, 3h head slots, B)

@@ -68,22 +68,37 @@ void launch_softmax_fwd(const float* scores, const int* valid_len, int B, int h,
 // Fused attention forward on the tensor cores (bf16 storage, head size 64, seq <= 384, seq % 8 == 0):
 // scores, masked softmax, quantizer of the probabilities, context product and (student) the context's
 // codes in one kernel.  Returns a GemmRc.  Null p_step / c_step: no quantizer; null P: the probabilities are
-// not written (a full-precision pass whose probabilities nobody reads); null P_qt: their codes are not written.
+// not written (nobody reads them); null P_qt: their codes are not written; null ctx: only the probabilities.
+// stats (may be null): what the backward pass needs to form the probabilities again, bit for bit: the score scale, the
+// clamped valid lengths and per query row alpha log2(e) max and 1 / sum.
+struct AttentionStats { float* alpha; int* len; float2* row; };
 bool attention_fwd_supported(int S, int head_dim, int dt);
 int launch_attention_fwd(const void* qkv, int B, int S, int h, int H, const int* valid_len, float alpha_const,
                          const float* a_p0, const float* a_p1, const float* c_p0, const float* c_p1,
                          const float* p_step, int p_lo, int p_hi, void* P, void* P_qt, void* ctx, const float* c_step,
-                         int c_qmax, int8_t* ctx_q8, void* ctx_qt, int* status, cudaStream_t st);
+                         int c_qmax, int8_t* ctx_q8, void* ctx_qt, int* status, cudaStream_t st,
+                         const AttentionStats* stats = nullptr);
 
-// Fused attention backward of the student on the tensor cores (bf16 storage, head size 64, seq <= 128,
-// seq % 8 == 0, batch * heads <= RED_BLOCKS): from the context gradient to the masked gradients of
-// the pre-quantization Q, K, V ([B*S, 3H]) with the step-size partials of the Q, K, V, P sites
-// (RED_BLOCKS slots each; unused slots are zeroed).  Returns a GemmRc.
+// Fused attention backward of the student on the tensor cores (bf16 storage, head size 64, seq <= 384,
+// seq % 8 == 0, batch * heads <= RED_BLOCKS; one kernel up to 128 tokens, two above): from the gradient of the quantized context to the masked gradients of
+// the pre-quantization Q, K, V ([B*S, 3H]) with the step-size partials of the Q, K, V, P and context sites
+// (RED_BLOCKS slots each; unused slots are zeroed).  The probabilities are formed again from the codes of Q and K and the
+// forward pass's row statistics.  Returns a GemmRc.
+struct AttentionBwd {
+  const void *qkv_codes, *qkv;            // [B*S, 3H] codes and values before quantization
+  const void *ctx, *dctx;                 // [B*S, H] context before quantization, gradient of the quantized context
+  int B, S, h, H;
+  const float *s_q, *s_k, *s_v, *s_p, *s_c;
+  const float* alpha; const int* len; const float2* stat;   // AttentionStats of the forward pass
+  int q_hi, p_hi;                         // code ranges: -q_hi .. q_hi (Q, K, V, context), .. p_hi (P)
+  void* dqkv;                             // [B*S, 3H] out
+  void* dctx_masked; float* dot;          // scratch above 128 tokens: [B*S, H] and [B, h, S]
+  float *part_q, *part_k, *part_v, *part_p, *part_c;
+  int* status;
+};
 bool attention_bwd_supported(int S, int head_dim, int dt, int batch_heads);
-int launch_attention_bwd(const void* qkv_codes, const void* qkv, const void* P, const void* dctx, int B, int S, int h,
-                         int H, const float* s_q, const float* s_k, const float* s_v, const float* s_p, int q_lo,
-                         int q_hi, int p_lo, int p_hi, void* dqkv, float* part_q, float* part_k, float* part_v,
-                         float* part_p, int* status, cudaStream_t st);
+int launch_attention_bwd(const AttentionBwd& a, cudaStream_t st);
+int launch_attention_bwd_long(const AttentionBwd& a, cudaStream_t st);    // 129 .. 384 tokens
 
 // ---- loss (Eq. 3)
 // partial[l][block] = sum (f_hat - f)^2 over the block's share; dF = 2 c (f_hat - f).

@@ -105,6 +105,7 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->t_y1 = A.take(M * H * es); c->t_a = A.take(M * H * es); c->t_g = A.take(M * F * es);
   c->t_y2 = A.take(M * H * es);
   c->scores = (float*)A.take(PS * sizeof(float));
+  c->att_dot = (float*)A.take(sizeof(float) * d.max_batch * d.n_heads * d.max_seq);
   c->x_mix = A.take(M * H * es);
   c->dF = A.take((size_t)L * M * H * es);
   c->d_y2 = A.take(M * H * es); c->d_ghat = A.take(M * F * es); c->d_u = A.take(M * F * es);
@@ -123,6 +124,8 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
     s.x_q8 = (int8_t*)A.take(M * H); s.x_qt = A.take(M * H * es);
     s.qkv = A.take(M * 3 * H * es); s.qkv_qt = A.take(M * 3 * H * es);
     s.P = A.take(PS * es); s.P_qt = A.take(PS * es);
+    s.p_alpha = (float*)A.take(sizeof(float)); s.p_len = (int*)A.take(sizeof(int) * d.max_batch);
+    s.p_stat = (float2*)A.take(sizeof(float2) * d.max_batch * d.n_heads * d.max_seq); s.p_kept = false;
     s.ctx = A.take(M * H * es); s.ctx_q8 = (int8_t*)A.take(M * H); s.ctx_qt = A.take(M * H * es);
     s.y1 = A.take(M * H * es); s.mean1 = (float*)A.take(M * 4); s.rstd1 = (float*)A.take(M * 4);
     s.a = A.take(M * H * es); s.a_q8 = (int8_t*)A.take(M * H); s.a_qt = A.take(M * H * es);
@@ -397,7 +400,14 @@ int32_t mrem_get_activation(mrem_ctx* c, int32_t role, int32_t layer, int32_t wh
     if (which >= 0 && which < MREM_ACT_COUNT) p = t[which];
   } else if (role == MREM_STUDENT) {
     if (!c->have_student) return fail(c, MREM_ERR_ORDER, "get_activation: no student pass to read");
-    const LayerStash& s = c->stash[layer];
+    LayerStash& s = c->stash[layer];
+    if (which == MREM_ACT_P && !s.p_kept) {            // formed again with the forward pass's own scale, lengths and arithmetic
+      const int H = c->d.hidden;
+      if (launch_attention_fwd(s.qkv_qt, c->cur_batch, c->cur_seq, c->d.n_heads, H, s.p_len, 1.f, s.p_alpha, nullptr, nullptr, nullptr, nullptr,
+                               0, 0, s.P, nullptr, nullptr, nullptr, 0, nullptr, nullptr, c->status, c->stream) != GEMM_OK)
+        return fail(c, MREM_ERR_CUDA, "get_activation: launch failed");
+      s.p_kept = true;
+    }
     const void* t[MREM_ACT_COUNT] = {s.qkv, s.P, s.ctx, s.y1, s.a, s.u, s.y2};
     if (which >= 0 && which < MREM_ACT_COUNT) p = t[which];
   } else {

@@ -26,7 +26,9 @@ struct WeightBuf {                      // quantized form of one weight matrix
 struct LayerStash {                     // what the student forward keeps for the backward
   int8_t* x_q8; void* x_qt;
   void* qkv; void* qkv_qt;
-  void* P; void* P_qt;
+  void* P; void* P_qt;                  // kernel-per-operation backward only; else formed again from what follows
+  float* p_alpha; int* p_len; float2* p_stat;   // AttentionStats
+  bool p_kept;                          // the last forward pass wrote P
   void* ctx; int8_t* ctx_q8; void* ctx_qt;
   void* y1; float* mean1; float* rstd1;
   void* a; int8_t* a_q8; void* a_qt;
@@ -87,6 +89,7 @@ struct mrem_ctx {
   // shared scratch
   void *t_qkv, *t_P, *t_ctx, *t_y1, *t_a, *t_g, *t_y2;   // teacher activations
   float* scores;
+  float* att_dot;                                       // [B, h, S] row sums of the attention backward
   void* x_mix;                                          // Eq. 4 input of the student
   void* dF;                                             // [L, M, H] loss gradients
   void *d_y2, *d_ghat, *d_u, *d_ahat, *d_a, *d_y1, *d_ctxhat, *d_ctx, *d_phat, *d_s, *d_qkvhat, *d_qkv, *d_xhat,

@@ -212,17 +212,20 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
     launch_quantize_act3(s.qkv, c->dt, M, H, 3 * H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], rx.lo, rx.hi, s.qkv_qt,
                          3 * H, c->stream);
     if (attention_fwd_supported(S, hd, c->dt)) {
-      // (the single-kernel attention backward takes the codes of the probabilities from the probabilities themselves:
-      //  they are written out only for the kernel-per-operation backward)
-      const bool codes_needed = !(c->fused_attention_bwd && attention_bwd_supported(S, hd, c->dt, B * h));
+      // (the single-kernel attention backward forms the probabilities again from the codes of Q and K and the row
+      //  statistics: they and their codes are written out only for the kernel-per-operation backward)
+      s.p_kept = !(c->fused_attention_bwd && attention_bwd_supported(S, hd, c->dt, B * h));
+      const AttentionStats stats{s.p_alpha, s.p_len, s.p_stat};
       r.note(launch_attention_fwd(s.qkv_qt, B, S, h, H, len, 1.f / sqrtf((float)hd), b.a_steps[S_Q], b.a_steps[S_K],
-                                  b.a_steps[S_P], b.a_steps[S_V], b.a_steps[S_P], rp.lo, rp.hi, s.P, codes_needed ? s.P_qt : nullptr, s.ctx,
-                                  b.a_steps[S_C], rx.hi, s.ctx_q8, s.ctx_qt, c->status, c->stream),
+                                  b.a_steps[S_P], b.a_steps[S_V], b.a_steps[S_P], rp.lo, rp.hi, s.p_kept ? s.P : nullptr,
+                                  s.p_kept ? s.P_qt : nullptr, s.ctx, b.a_steps[S_C], rx.hi, s.ctx_q8, s.ctx_qt, c->status, c->stream,
+                                  s.p_kept ? nullptr : &stats),
              "attention launch failed");
     } else {
       r.gemm(view(s.qkv_qt, 3 * H, 0, hd, (long long)S * 3 * H), view(r.at(s.qkv_qt, H), 3 * H, 0, hd, (long long)S * 3 * H),
              S, S, hd, h, B,
              Epi(c->scores, OUT_F32, S, (long long)S * S, (long long)h * S * S).alpha(1.f / sqrtf((float)hd), b.a_steps[S_Q], b.a_steps[S_K]).e);
+      s.p_kept = true;
       launch_softmax_fwd(c->scores, len, B, h, S, s.P, b.a_steps[S_P], nullptr, rp.lo, rp.hi, s.P_qt, c->dt, c->stream);
       r.gemm(view(s.P_qt, S, 0, (long long)S * S, (long long)h * S * S), view(r.at(s.qkv_qt, 2 * H), 3 * H, 1, hd, (long long)S * 3 * H),
              S, hd, S, h, B, Epi(s.ctx, ok, H, hd, (long long)S * H).alpha(1.f, b.a_steps[S_P], b.a_steps[S_V]).e);
@@ -380,15 +383,16 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
                       c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
     r.gemm(view(q.d_y1, H), weights(w[W_O].what, H, 1), (int)M, H, H, 1, 1, Epi(c->d_ctxhat, ok, H).e);
     rw.defer(view(q.d_y1, H, 1), view(s.ctx_qt, H, 1), H, H, (int)M, Epi(g.p[MREM_WO], OUT_F32, H).alpha(1.f, b.a_steps[S_C]).e);
-    launch_ste_act(s.ctx, H, c->d_ctxhat, H, nullptr, 0, c->d_ctx, H, M, H, b.a_steps[S_C], nullptr, rx.lo, rx.hi,
-                   part + S_C * RED_BLOCKS, nullptr, c->dt, st);
     // attention:  ctx = P_hat V_hat,  P = softmax(Q_hat K_hat^T / sqrt(d))
-    if (c->fused_attention_bwd && attention_bwd_supported(S, hd, c->dt, B * h)) {
-      r.note(launch_attention_bwd(s.qkv_qt, s.qkv, s.P, c->d_ctx, B, S, h, H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V],
-                                  b.a_steps[S_P], rx.lo, rx.hi, rp.lo, rp.hi, q.d_qkv, part + S_Q * RED_BLOCKS,
-                                  part + S_K * RED_BLOCKS, part + S_V * RED_BLOCKS, part + S_P * RED_BLOCKS, c->status, st),
-             "attention backward launch failed");
+    if (!s.p_kept) {
+      const AttentionBwd ab{s.qkv_qt, s.qkv, s.ctx, c->d_ctxhat, B, S, h, H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], b.a_steps[S_P],
+                            b.a_steps[S_C], s.p_alpha, s.p_len, s.p_stat, rx.hi, rp.hi, q.d_qkv, c->d_ctx, c->att_dot,
+                            part + S_Q * RED_BLOCKS,
+                            part + S_K * RED_BLOCKS, part + S_V * RED_BLOCKS, part + S_P * RED_BLOCKS, part + S_C * RED_BLOCKS, c->status};
+      r.note(launch_attention_bwd(ab, st), "attention backward launch failed");
     } else {
+      launch_ste_act(s.ctx, H, c->d_ctxhat, H, nullptr, 0, c->d_ctx, H, M, H, b.a_steps[S_C], nullptr, rx.lo, rx.hi,
+                     part + S_C * RED_BLOCKS, nullptr, c->dt, st);
       r.gemm(view(c->d_ctx, H, 0, hd, (long long)S * H), view(r.at(s.qkv_qt, 2 * H), 3 * H, 0, hd, sQKV), S, S, hd, h, B,
              Epi(c->d_phat, ok, S, sSS, sHSS).alpha(1.f, b.a_steps[S_V]).e);
       r.gemm(view(s.P_qt, S, 1, sSS, sHSS), view(c->d_ctx, H, 1, hd, (long long)S * H), S, hd, S, h, B,
