@@ -278,25 +278,19 @@ __device__ __forceinline__ void drain_chunks(const Epilogue& e, uint32_t taddr, 
                                              const float* cv, long long off, bool row_ok, uint32_t* res0, const StoreCtx& sx,
                                              int n) {
   const bool pipelined_res = OUT == OUT_BF16 && EpiFlags<MODE>(e).res;
-  uint32_t ra[32], rb2[32], res1[16];
-  tmem_ld32_issue(taddr, ra);
-  for (int c = 0; c < nchunks; c += 2) {
+  // one copy of the chunk's code: the loop stays rolled and the residual in flight moves to the front (a second copy, for
+  // registers that alternate, is 250 more instructions for every launch to fetch)
+  uint32_t acc[32], res1[16];
+#pragma unroll 1
+  for (int c = 0; c < nchunks; ++c) {
+    tmem_ld32_issue(taddr + 32u * (uint32_t)c, acc);
+    if (pipelined_res && c + 1 < nchunks) fetch_res_bf16(e, off + 32 * (c + 1), row_ok, res1);
     tmem_ld_wait();
-    tmem_ld_pin(ra);
-    const bool more1 = c + 1 < nchunks;
-    if (more1) {
-      tmem_ld32_issue(taddr + 32u * (uint32_t)(c + 1), rb2);
-      if (pipelined_res) fetch_res_bf16(e, off + 32 * (c + 1), row_ok, res1);
-    }
-    finish_chunk<KIND, OUT, MODE>(e, ra, res0, alpha, rb, cv + 32 * c, off + 32 * c, row_ok, sx, n + 32 * c);
-    if (more1) {
-      tmem_ld_wait();
-      tmem_ld_pin(rb2);
-      if (c + 2 < nchunks) {
-        tmem_ld32_issue(taddr + 32u * (uint32_t)(c + 2), ra);
-        if (pipelined_res) fetch_res_bf16(e, off + 32 * (c + 2), row_ok, res0);
-      }
-      finish_chunk<KIND, OUT, MODE>(e, rb2, res1, alpha, rb, cv + 32 * (c + 1), off + 32 * (c + 1), row_ok, sx, n + 32 * (c + 1));
+    tmem_ld_pin(acc);
+    finish_chunk<KIND, OUT, MODE>(e, acc, res0, alpha, rb, cv + 32 * c, off + 32 * c, row_ok, sx, n + 32 * c);
+    if (pipelined_res) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) res0[j] = res1[j];
     }
   }
 }
