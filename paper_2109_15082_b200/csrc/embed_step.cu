@@ -601,8 +601,9 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   }
   // update of the word table: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one
   // pass (the small tensors, the other embedding tables decayed like weight matrices, LayerNorm not, are updated above)
-  launch_fused_weight_update(x->word, x->g_word, x->m_word, x->v_word, x->word_step, nullptr, x->m_word_step, x->v_word_step, s.optim_sc,
-                             V, H, d->e_bits, 0, 1, 1, s.codes, s.rowsum, s.scale, nullptr, dt, st, row_first);
+  const RowUpdate table{x->word, x->g_word, x->m_word, x->v_word, x->word_step, x->m_word_step, x->v_word_step, nullptr,
+                        s.codes, s.rowsum, s.scale, nullptr, V, H};
+  launch_fused_weight_update(&table, 1, s.optim_sc, d->e_bits, 0, 1, 1, dt, st, row_first);
   return cudaGetLastError() == cudaSuccess ? MREM_OK : MREM_ERR_CUDA;
 }
 

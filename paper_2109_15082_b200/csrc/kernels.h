@@ -191,13 +191,20 @@ void launch_optim_prepare(OptimScalars* d_out, int* d_t, int host_t, float lr0, 
 void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, const OptimScalars* d_sc,
                         cudaStream_t st);
 
-// Fused per-row update of a weight matrix and its per-row steps: step gradient (or ds_in when the
+// Fused per-row update of weight matrices and their per-row steps: step gradient (or ds_in when the
 // gradients were already masked), AdamW on step and weights, re-quantization (codes, row sums,
 // scale, dequantized row).  row_used (may be null): one word per row, 0xffffffff where no gradient arrived; such a row's
-// g is taken as zero without being read, and written as zero (grid 0 only).
-void launch_fused_weight_update(float* w, float* g, float* m, float* v, float* steps, const float* ds_in,
-                                float* m_s, float* v_s, const OptimScalars* sc, int rows, int cols, int bits, int grid,
-                                int train_w, int train_s, int8_t* codes, int32_t* rowsum, float* scale, void* what,
+// g is taken as zero without being read, and written as zero (grid 0 and one matrix only).
+struct RowUpdate {
+  float *w, *g, *m, *v;                // latent weights, their gradient, moments: rows x cols
+  float *steps, *m_s, *v_s;            // one step per row, its moments
+  const float* ds_in;                  // step gradients, when g is masked already; else null
+  int8_t* codes; int32_t* rowsum; float* scale; void* what;
+  int rows, cols;
+};
+constexpr int MAX_ROW_UPDATES = 4;
+// `n` matrices (at most MAX_ROW_UPDATES) in one launch.
+void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
                                 int dt, cudaStream_t st, const unsigned* row_used = nullptr);
 
 // ---- step-size initialisation

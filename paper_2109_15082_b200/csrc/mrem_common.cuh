@@ -185,9 +185,10 @@ __device__ __forceinline__ float rne_magic(float z) { uint32_t b; return rne_mag
 // gives, at a fraction of its instructions; returned as a float, with the bit pattern that carries its low byte.
 // r_s = RN(1 / s).  The three-instruction quotient is within one ulp of the correctly rounded one (1.5e-5 at |z| <= 255),
 // so the two can round to different integers only when the quotient lies that close to a half-integer: any value within
-// 2^-10 of one is decided by the division instruction instead (about one element in a thousand).  A quotient beyond the
+// HALF_WINDOW (twice that) of one is decided by the division instruction instead, about one element in 16000.  A quotient beyond the
 // range is clipped to the same bound by both.  EXACT_QUOTIENT: the numerator is a bfloat16 value, for which the quotient
 // IS the correctly rounded one (see quotient()) and no second look is needed.
+constexpr float HALF_WINDOW = 3.0517578125e-5f;
 template <bool EXACT_QUOTIENT>
 __device__ __forceinline__ float code_f(float n, float s, float r_s, float lo, float hi, uint32_t& bits) {
   // (the first product is kept inside [lo - 1, hi + 1]: unchanged wherever the code is not simply a bound, and a
@@ -196,7 +197,7 @@ __device__ __forceinline__ float code_f(float n, float s, float r_s, float lo, f
   float zc = fminf(fmaxf(__fmaf_rn(__fmaf_rn(-z0, s, n), r_s, z0), lo), hi);
   float q = rne_magic(zc, bits);
   if constexpr (!EXACT_QUOTIENT) {
-    if (fabsf(fabsf(zc - q) - 0.5f) < 9.765625e-4f) {
+    if (fabsf(fabsf(zc - q) - 0.5f) < HALF_WINDOW) {
       zc = fminf(fmaxf(__fdiv_rn(n, s), lo), hi);
       q = rne_magic(zc, bits);
     }

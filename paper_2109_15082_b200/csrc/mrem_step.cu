@@ -257,24 +257,24 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
   return cudaGetLastError() == cudaSuccess ? MREM_OK : fail(c, MREM_ERR_CUDA, "student forward: launch failed");
 }
 
-// The fused update of one layer's four matrices and their row steps (Algorithm 2: Update(w), Update(s)).
-void enqueue_matrix_update(mrem_ctx* c, int l, int k, cudaStream_t st) {
+// The fused update of `n` of one layer's matrices, from index k0 on, and their row steps (Algorithm 2: Update(w), Update(s)).
+void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st) {
   const mrem_module_desc& d = c->d;
   const int train_w = (d.trainable_mask & MREM_TRAIN_WEIGHTS) != 0, train_s = (d.trainable_mask & MREM_TRAIN_W_STEPS) != 0;
-  const int pid = kMatParam[k];
-  WeightBuf& w = c->wq[l][k];
   LayerGrad& g = c->grad[l];
-  if (closed_form_weights(d)) {
-    launch_closed_form_update(c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->optim_sc, w.rows, w.cols, train_w,
-                              d.w_grid, d.w_bits, w.codes, w.rowsum, w.scale, w.what, c->dt, st);
-    return;
+  RowUpdate mats[N_WMAT];
+  static_assert(N_WMAT <= MAX_ROW_UPDATES, "a layer's matrices go in one launch");
+  for (int i = 0; i < n; ++i) {
+    const int k = k0 + i, pid = kMatParam[k];
+    WeightBuf& w = c->wq[l][k];
+    if (closed_form_weights(d))
+      launch_closed_form_update(c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->optim_sc, w.rows, w.cols, train_w,
+                                d.w_grid, d.w_bits, w.codes, w.rowsum, w.scale, w.what, c->dt, st);
+    else
+      mats[i] = RowUpdate{c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->bind[l].w_steps[k], g.m_ws[k], g.v_ws[k],
+                          c->w_ste_done ? g.ws[k] : nullptr, w.codes, w.rowsum, w.scale, w.what, w.rows, w.cols};
   }
-  launch_fused_weight_update(c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->bind[l].w_steps[k],
-                             c->w_ste_done ? g.ws[k] : nullptr, g.m_ws[k], g.v_ws[k], c->optim_sc, w.rows, w.cols,
-                             d.w_bits, d.w_grid, train_w, train_s, w.codes, w.rowsum, w.scale, w.what, c->dt, st);
-}
-void enqueue_matrix_updates(mrem_ctx* c, int l, cudaStream_t st) {
-  for (int k = 0; k < N_WMAT; ++k) enqueue_matrix_update(c, l, k, st);
+  if (!closed_form_weights(d)) launch_fused_weight_update(mats, n, c->optim_sc, d.w_bits, d.w_grid, train_w, train_s, c->dt, st);
 }
 
 // ------------------------------------------------------------------ backward
@@ -427,7 +427,7 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
     // the side stream is done with this layer's copy of the gradient buffers once the grouped products have run
     if (two_streams && cudaEventRecord(c->ev_layer[l & 1], side) != cudaSuccess) sync_failed = true;
     // nothing below reads what the update writes: the latent weights, moments, row steps and this layer's codes
-    if (update_as_you_go) enqueue_matrix_updates(c, l, side);
+    if (update_as_you_go) enqueue_matrix_updates(c, l, 0, N_WMAT, side);
   }
   // step-size and offset gradients of every layer's activation quantizers: the per-block partial sums the
   // kernels above left, added in index order (one launch for the whole module; only the update reads them)
@@ -577,7 +577,7 @@ int32_t mrem_step(mrem_ctx* c, const mrem_optim* o) {
   if (d.w_step_per_row) {
     // every tensor but the matrices and their steps, then one fused pass per matrix
     launch_adamw_table(c->adam_rest, c->rest_entries, c->rest_elems, c->optim_sc, c->stream);
-    for (int l = 0; l < d.n_layers; ++l) enqueue_matrix_updates(c, l, c->stream);
+    for (int l = 0; l < d.n_layers; ++l) enqueue_matrix_updates(c, l, 0, N_WMAT, c->stream);
   } else {
     if (!c->w_ste_done) {
       for (int l = 0; l < d.n_layers; ++l)
@@ -684,7 +684,7 @@ int32_t mrem_rem_step(mrem_ctx* c, int32_t layer, int32_t tensor_id, const void*
     // update: the matrix and its steps (which also re-quantizes it), the input quantizer's step and offset
     launch_optim_prepare(c->optim_sc, c->t_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps,
                          o->weight_decay, st);
-    enqueue_matrix_update(c, layer, k, st);
+    enqueue_matrix_updates(c, layer, k, 1, st);
     if (d.trainable_mask & MREM_TRAIN_A_STEPS) {
       AdamEntry host[2];
       int ne = 0;

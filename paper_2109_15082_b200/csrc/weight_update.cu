@@ -1,4 +1,4 @@
-// Fused update of one weight matrix and its per-row quantization steps (Algorithm 2:
+// Fused update of weight matrices and their per-row quantization steps (Algorithm 2:
 // Update(w), Update(s)), one block per output row and ONE pass over the row's state:
 //   1. straight-through factors of the weight quantizer at the old (w, s): the step
 //      gradient ds = sum_k dW_hat * d w_hat / d s (fixed-order block sum),
@@ -16,21 +16,6 @@ namespace mrem {
 
 namespace {
 
-
-// Code of Eq. 1 and the same value as a float.  Integer grid: the sum with 1.5 * 2^23 holds the code in its
-// low mantissa bits (two's complement), so neither direction goes through the conversion unit.
-__device__ __forceinline__ int weight_code(float w, float s, float r_s, float qmax, int grid, float& qf) {
-  if (grid == 0) {      // the exact code without the division instruction (code_f); r_s = RN(1 / s)
-    uint32_t bits;
-    qf = code_f<false>(w, s, r_s, -qmax, qmax, bits);
-    return (int)(int8_t)(bits & 0xffu);
-  }
-  const float z = __fdiv_rn(w, s);
-  const int q = 2 * (int)fminf(fmaxf(floorf(z), -2.f), 1.f) + 1;
-  qf = (float)q;
-  return q;
-}
-
 template <typename T>
 __device__ __forceinline__ void store_what4(T* p, float a, float b, float c, float d);
 template <>
@@ -46,171 +31,260 @@ __device__ __forceinline__ void store_what4<bf16>(bf16* p, float a, float b, flo
   *reinterpret_cast<uint2*>(p) = t;
 }
 
-// One block of NT threads per row, NV float4 vectors per thread kept in registers: (256, 1) for rows up to 1024 wide,
-// (512, 2) up to 4096; wider rows are re-read.  Rows of at most three quarters of that (768 and 3072, the widths of a 768
-// wide encoder) get three quarters of the threads: the others would only wait in the barriers, and a third more blocks fit
-// on an SM.  30522 x 768 table: update 148 -> 125 us, step 190 -> 167 us; 3 x 72 tokens, hidden 768: step 656 -> 640 us.
+// Pairs of weights: the arithmetic below is the scalar one of optim.cuh and code_f, two elements per instruction where the
+// hardware has the form.
+__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 quotient2(float2 x, float2 neg_s, float2 r_s) {        // quotient() of both
+  const float2 z0 = mul2(x, r_s);
+  return fma2(fma2(z0, neg_s, x), r_s, z0);
+}
+__device__ __forceinline__ float2 clamp2(float2 z, float b) {
+  return make_float2(fminf(fmaxf(z.x, -b), b), fminf(fmaxf(z.y, -b), b));
+}
+// The step gradient's terms of two elements (step_grad_acc), and which gradients pass.
+template <int GRID>
+__device__ __forceinline__ float2 step_grad2(float2 acc, float2 w, float2 d, float2 neg_s, float2 r_s, float qmax, bool& in0, bool& in1) {
+  const float2 z = quotient2(w, neg_s, r_s);
+  float2 level;
+  if (GRID == 0) {
+    const float2 zc = clamp2(z, qmax);
+    in0 = zc.x == z.x; in1 = zc.y == z.y;
+    level = add2(add2(zc, splat(RINT_MAGIC)), splat(-RINT_MAGIC));
+  } else {                                                     // clamp(floor(z), -2, 1) + 0.5 without the conversion unit
+    in0 = z.x >= -2.f && z.x < 2.f; in1 = z.y >= -2.f && z.y < 2.f;
+    level.x = z.x < 0.f ? (z.x < -1.f ? -1.5f : -0.5f) : (z.x >= 1.f ? 1.5f : 0.5f);
+    level.y = z.y < 0.f ? (z.y < -1.f ? -1.5f : -0.5f) : (z.y >= 1.f ? 1.5f : 0.5f);
+  }
+  const float2 inside = make_float2(in0 ? -z.x : 0.f, in1 ? -z.y : 0.f);
+  return fma2(d, add2(level, inside), acc);
+}
+__device__ __noinline__ float exact_quotient(float x, float s) { return __fdiv_rn(x, s); }      // rare: kept out of line
+struct Adam2 { float2 b1, ob1, b2, ob2, rsq, eps, neg_lr, decay; };
+__device__ __forceinline__ float2 adam2(float2 p, float2 g, float2& m, float2& v, const Adam2& a) {      // adam_one of both
+  m = fma2(a.b1, m, mul2(a.ob1, g));
+  v = fma2(a.b2, v, mul2(mul2(a.ob2, g), g));
+  const float2 denom = fma2(make_float2(sqrt_approx(v.x), sqrt_approx(v.y)), a.rsq, a.eps), num = mul2(a.neg_lr, m);
+  return add2(mul2(p, a.decay), make_float2(__fdividef(num.x, denom.x), __fdividef(num.y, denom.y)));
+}
+
+struct UpdateParams {
+  RowUpdate mat[MAX_ROW_UPDATES];
+  int row_end[MAX_ROW_UPDATES];        // running row count: matrix i owns the blocks [row_end[i - 1], row_end[i])
+  int n, bits, train_w, train_s;
+  const OptimScalars* sc;
+  const unsigned* row_used;
+};
+
+// One block of NT threads per row, NV float4 vectors of w, g, m and v per thread in registers; rows wider than the widest
+// variant holds are re-read by it.  The matrices of a layer whose rows take the same variant go in one launch.
+// The kernel moves 31 bytes a weight and should be bound by that, but was bound by the issue slots (71 % busy, DRAM at 39 %):
+// with one float4 per thread, the two block sums, the step's own update behind a barrier and the scalars cost each thread as
+// much as its four weights.  So: few threads per row, every thread forms the row's new step itself, and the arithmetic runs
+// on pairs.  Measured: a layer of 1024 x 4096 shapes 87 -> 74 us (floor 59), its three 1024-wide matrices 56 -> 47 us in one
+// launch; 30522 x 1024 table 165 -> 136 us (7.1 TB/s), 30522 x 768 128 -> 116 us.
+// Variants (X(index, NT, NV, blocks per SM)), by the widest row they hold: 16 weights a thread keep the most bytes in flight
+// (1024 wide: 64 x 4 vectors 136 us, 128 x 2 144 us, 256 x 1 152 us for that table), but 64 x 3 for 768 wide rows, with
+// the same ten blocks on an SM, does not (128 us; 96 x 2 at 62 registers 116 us).
+#define UPD_VARIANTS(X) X(0, 96, 2, 10) X(1, 64, 4, 10) X(2, 128, 4, 5) X(3, 192, 4, 3) X(4, 256, 4, 2)
+constexpr int UPD_WIDEST = 4;
 // GRID (the weight grid, 0: Eq. 1's integers, 1: half-integer 2-bit levels) is a template parameter: the per-weight code
 // then holds one of the two rules, not both under predicates.  SPARSE: row_used says which rows got a gradient at all (an
-// embedding table); its own variant, because the dense one is at the register limit of its occupancy.
-template <typename T, int NV, int NT, int GRID, bool SPARSE>
-__global__ void __launch_bounds__(NT, NT == 192 ? 8 : (NT == 256 ? 6 : 2)) fused_weight_update_kernel(
-    float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-    float* __restrict__ steps, const float* __restrict__ ds_in, float* __restrict__ m_s, float* __restrict__ v_s,
-    const OptimScalars* __restrict__ sc, int cols, int bits, int train_w, int train_s,
-    int8_t* __restrict__ codes, int32_t* __restrict__ rowsum, float* __restrict__ scale, T* __restrict__ what,
-    const unsigned* __restrict__ row_used) {
+// embedding table, one matrix per launch: its pointers stay at fixed places of the parameters, 235 -> 204 us for the step).
+template <typename T, int NV, int NT, int BLOCKS, int GRID, bool SPARSE>
+__global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const __grid_constant__ UpdateParams P) {
   pdl_trigger();
   pdl_wait();
-  constexpr int grid = GRID;
-  __shared__ float sh[32];
-  __shared__ int shi[32];
-  __shared__ float s_new_sh;
-  const int row = blockIdx.x;
+  constexpr int NW = NT / 32;
+  constexpr bool WIDE = NT == 256;                             // the variant that also takes rows beyond its registers
+  __shared__ float ds_sh[NW];
+  __shared__ int sum_sh[NW];
+  int mi = 0;
+  if (!SPARSE)
+    while (mi + 1 < P.n && (int)blockIdx.x >= P.row_end[mi]) ++mi;
+  const RowUpdate& M = P.mat[mi];
+  const int row = (int)blockIdx.x - (mi ? P.row_end[mi - 1] : 0), t = threadIdx.x;
+  const int train_w = P.train_w, train_s = P.train_s;
   // a row marked 0xffffffff got no gradient: g is not read, and is cleared here instead of by a pass before this one
-  const bool no_grad = SPARSE && row_used[row] == 0xffffffffu;
-  const OptimScalars o = *sc;
-  const float s_old = steps[row];
-  const float r_old = __frcp_rn(s_old);
-  float ms_pre = 0.f, vs_pre = 0.f;
-  if (threadIdx.x == 0 && train_s) { ms_pre = m_s[row]; vs_pre = v_s[row]; }
-  const float qmax = (float)((1 << (bits - 1)) - 1);
-  const long long base = (long long)row * cols;
-  const int nvec = cols / 4;                                   // cols is a multiple of 16
-  const bool cached = nvec <= NV * NT;
-  const float4* w4 = reinterpret_cast<const float4*>(w + base);
-  float4* g4 = reinterpret_cast<float4*>(g + base);
+  const bool no_grad = SPARSE && P.row_used[row] == 0xffffffffu;
+  const long long base = (long long)row * M.cols;
+  const int nvec = M.cols / 4;                                 // cols is a multiple of 16
+  const bool cached = !WIDE || nvec <= NV * NT;
+  float4* w4 = reinterpret_cast<float4*>(M.w + base);
+  float4* g4 = reinterpret_cast<float4*>(M.g + base);
+  float4* m4 = reinterpret_cast<float4*>(M.m + base);
+  float4* v4 = reinterpret_cast<float4*>(M.v + base);
+  T* const what = M.what ? reinterpret_cast<T*>(M.what) + base : nullptr;
+  int8_t* const codes = M.codes + base;
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 wr[NV], gr[NV], mr[NV], vr[NV];
-  const float4* m4c = reinterpret_cast<const float4*>(m + base);
-  const float4* v4c = reinterpret_cast<const float4*>(v + base);
-  // 1. step gradient of this row; the masked gradient is kept for step 3.  The moments are fetched now
-  //    as well, so that their latency hides behind the reduction and the step's own update.
-  float ds = 0.f;
+  // everything is fetched before the first use: the moments' latency hides behind the reduction and the step's update
   if (cached) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int c = threadIdx.x + i * NT;
+      const int c = t + i * NT;
+      wr[i] = gr[i] = mr[i] = vr[i] = zero4;
       if (c < nvec) {
         wr[i] = w4[c];
-        if (no_grad) { gr[i] = zero4; g4[c] = zero4; } else gr[i] = g4[c];
-        if (train_w) { mr[i] = m4c[c]; vr[i] = v4c[c]; }
+        if (no_grad) g4[c] = zero4; else gr[i] = g4[c];
+        if (train_w) { mr[i] = m4[c]; vr[i] = v4[c]; }
       }
     }
   }
+  const OptimScalars o = *P.sc;
+  const float s_old = M.steps[row];
+  float ms = 0.f, vs = 0.f;
+  if (train_s) { ms = M.m_s[row]; vs = M.v_s[row]; }
+  const float qmax = (float)((1 << (P.bits - 1)) - 1);
+  const bool masked = M.ds_in != nullptr;                      // gradients were masked and reduced before (same arithmetic)
+  // 1. step gradient of this row; the masked gradient is kept for step 3
+  const float2 ns_old = splat(-s_old), r_old = splat(__frcp_rn(s_old));
+  float2 ds2 = splat(0.f);
+  auto ste = [&](float4 wv, float4 d) {
+    bool a, b, e, f;
+    ds2 = step_grad2<GRID>(ds2, make_float2(wv.x, wv.y), make_float2(d.x, d.y), ns_old, r_old, qmax, a, b);
+    ds2 = step_grad2<GRID>(ds2, make_float2(wv.z, wv.w), make_float2(d.z, d.w), ns_old, r_old, qmax, e, f);
+    return make_float4(a || masked ? d.x : 0.f, b || masked ? d.y : 0.f, e || masked ? d.z : 0.f, f || masked ? d.w : 0.f);
+  };
+  if (cached) {
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const int c = threadIdx.x + i * NT;
-    if (cached && c < nvec) {
-      bool in;
-      float4 d = gr[i];
-      ds = step_grad_acc(ds, wr[i].x, d.x, s_old, r_old, qmax, grid, in); d.x = (in || ds_in) ? d.x : 0.f;
-      ds = step_grad_acc(ds, wr[i].y, d.y, s_old, r_old, qmax, grid, in); d.y = (in || ds_in) ? d.y : 0.f;
-      ds = step_grad_acc(ds, wr[i].z, d.z, s_old, r_old, qmax, grid, in); d.z = (in || ds_in) ? d.z : 0.f;
-      ds = step_grad_acc(ds, wr[i].w, d.w, s_old, r_old, qmax, grid, in); d.w = (in || ds_in) ? d.w : 0.f;
-      gr[i] = d;
-    }
-  }
-  if (!cached) {
-    for (int c = threadIdx.x; c < nvec; c += NT) {
+    for (int i = 0; i < NV; ++i) gr[i] = ste(wr[i], gr[i]);    // (a vector beyond the row has a zero gradient)
+  } else {
+    for (int c = t; c < nvec; c += NT) {
       if (no_grad) g4[c] = zero4;
-      const float4 wv = w4[c], d = no_grad ? zero4 : g4[c];
-      bool in;
-      ds = step_grad_acc(ds, wv.x, d.x, s_old, r_old, qmax, grid, in);
-      ds = step_grad_acc(ds, wv.y, d.y, s_old, r_old, qmax, grid, in);
-      ds = step_grad_acc(ds, wv.z, d.z, s_old, r_old, qmax, grid, in);
-      ds = step_grad_acc(ds, wv.w, d.w, s_old, r_old, qmax, grid, in);
+      ste(w4[c], no_grad ? zero4 : g4[c]);
     }
   }
-  ds = block_sum(ds, sh);
-  if (ds_in) ds = ds_in[row];          // gradients were masked and reduced before (same arithmetic)
-  // 2. the row's step (its moments were fetched before the reduction)
-  if (threadIdx.x == 0) {
-    float s_new = s_old;
-    if (train_s) {
-      float ms = ms_pre, vs = vs_pre;
-      s_new = adam_one(s_old, ds, ms, vs, o, 0.f, 1e-8f);
-      m_s[row] = ms;
-      v_s[row] = vs;
-      steps[row] = s_new;
-    }
-    s_new_sh = s_new;
-  }
+  float ds = warp_sum(ds2.x + ds2.y);
+  if ((threadIdx.x & 31) == 0) ds_sh[threadIdx.x >> 5] = ds;
   __syncthreads();
-  const float s_new = s_new_sh, r_new = __frcp_rn(s_new);
-  const float sc_new = grid == 0 ? s_new : 0.5f * s_new;
+  ds = ds_sh[0];
+#pragma unroll
+  for (int i = 1; i < NW; ++i) ds += ds_sh[i];
+  if (masked) ds = M.ds_in[row];
+  // 2. the row's step, formed by every thread
+  const float s_new = train_s ? adam_one(s_old, ds, ms, vs, o, 0.f, 1e-8f) : s_old;
+  const float sc_new = GRID == 0 ? s_new : 0.5f * s_new;
   // 3 + 4. weights, then their new codes
-  float4* wo = reinterpret_cast<float4*>(w + base);
-  float4* m4 = reinterpret_cast<float4*>(m + base);
-  float4* v4 = reinterpret_cast<float4*>(v + base);
-  int sum = 0;
+  const float2 ns_new = splat(-s_new), r_new = splat(__frcp_rn(s_new));
+  const Adam2 ad = {splat(o.beta1), splat(__fsub_rn(1.f, o.beta1)), splat(o.beta2), splat(__fsub_rn(1.f, o.beta2)),
+                    splat(o.rsqrt_bc2), splat(o.eps), splat(-o.lr_bc1), splat(__fsub_rn(1.f, __fmul_rn(o.lr, o.weight_decay)))};
+  float2 sum2 = splat(0.f);                                    // codes are whole numbers: exact in any order
   auto update = [&](int c, float4 wv, float4 d, float4 mm, float4 vv) {
+    float2 wa = make_float2(wv.x, wv.y), wb = make_float2(wv.z, wv.w);
     if (train_w) {
-      wv.x = adam_one(wv.x, d.x, mm.x, vv.x, o, 1.f, -INFINITY);
-      wv.y = adam_one(wv.y, d.y, mm.y, vv.y, o, 1.f, -INFINITY);
-      wv.z = adam_one(wv.z, d.z, mm.z, vv.z, o, 1.f, -INFINITY);
-      wv.w = adam_one(wv.w, d.w, mm.w, vv.w, o, 1.f, -INFINITY);
-      wo[c] = wv;
-      m4[c] = mm;
-      v4[c] = vv;
+      float2 ma = make_float2(mm.x, mm.y), mb = make_float2(mm.z, mm.w), va = make_float2(vv.x, vv.y), vb = make_float2(vv.z, vv.w);
+      wa = adam2(wa, make_float2(d.x, d.y), ma, va, ad);
+      wb = adam2(wb, make_float2(d.z, d.w), mb, vb, ad);
+      w4[c] = make_float4(wa.x, wa.y, wb.x, wb.y);
+      m4[c] = make_float4(ma.x, ma.y, mb.x, mb.y);
+      v4[c] = make_float4(va.x, va.y, vb.x, vb.y);
     }
-    float f0, f1, f2, f3;
-    const int q0 = weight_code(wv.x, s_new, r_new, qmax, grid, f0), q1 = weight_code(wv.y, s_new, r_new, qmax, grid, f1);
-    const int q2 = weight_code(wv.z, s_new, r_new, qmax, grid, f2), q3 = weight_code(wv.w, s_new, r_new, qmax, grid, f3);
-    *reinterpret_cast<uint32_t*>(codes + base + 4 * c) =
-        (uint32_t)(q0 & 0xff) | ((uint32_t)(q1 & 0xff) << 8) | ((uint32_t)(q2 & 0xff) << 16) | ((uint32_t)(q3 & 0xff) << 24);
-    if (what) store_what4<T>(what + base + 4 * c, sc_new * f0, sc_new * f1, sc_new * f2, sc_new * f3);
-    sum += q0 + q1 + q2 + q3;
+    float2 fa, fb;
+    uint32_t b0, b1, b2, b3;
+    if (GRID == 0) {      // the exact code without the division instruction (code_f), one look at the half-integers for all four
+      auto code_quotient = [&](float2 x) {                     // (a first product that overflows ends on its sign's bound)
+        const float2 z0 = clamp2(mul2(x, r_new), qmax + 1.f);
+        return clamp2(fma2(fma2(z0, ns_new, x), r_new, z0), qmax);
+      };
+      float2 za = code_quotient(wa), zb = code_quotient(wb);
+      auto round2 = [&]() {
+        const float2 ta = add2(za, splat(ROUND_MAGIC)), tb = add2(zb, splat(ROUND_MAGIC));
+        fa = add2(ta, splat(-ROUND_MAGIC)); fb = add2(tb, splat(-ROUND_MAGIC));
+        b0 = __float_as_uint(ta.x); b1 = __float_as_uint(ta.y); b2 = __float_as_uint(tb.x); b3 = __float_as_uint(tb.y);
+      };
+      round2();
+      const float2 ea = fma2(fa, splat(-1.f), za), eb = fma2(fb, splat(-1.f), zb);
+      const float near = fminf(fminf(fabsf(fabsf(ea.x) - 0.5f), fabsf(fabsf(ea.y) - 0.5f)),
+                               fminf(fabsf(fabsf(eb.x) - 0.5f), fabsf(fabsf(eb.y) - 0.5f)));
+      if (near < HALF_WINDOW) {
+        za = clamp2(make_float2(exact_quotient(wa.x, s_new), exact_quotient(wa.y, s_new)), qmax);
+        zb = clamp2(make_float2(exact_quotient(wb.x, s_new), exact_quotient(wb.y, s_new)), qmax);
+        round2();
+      }
+    } else {
+      // 2 clamp(floor(w / s), -2, 1) + 1: a quotient of floats rounds to 1 or more exactly when w >= s, and to less than -1
+      // exactly when -w > s (the neighbours of s are further than half an ulp of 1 away from it, relatively)
+      auto level = [&](float x) { return x < 0.f ? (-x > s_new ? -3.f : -1.f) : (x >= s_new ? 3.f : 1.f); };
+      fa = make_float2(level(wa.x), level(wa.y)); fb = make_float2(level(wb.x), level(wb.y));
+      const float2 ta = add2(fa, splat(ROUND_MAGIC)), tb = add2(fb, splat(ROUND_MAGIC));
+      b0 = __float_as_uint(ta.x); b1 = __float_as_uint(ta.y); b2 = __float_as_uint(tb.x); b3 = __float_as_uint(tb.y);
+    }
+    *reinterpret_cast<uint32_t*>(codes + 4 * c) = pack_low_bytes(b0, b1, b2, b3);
+    const float2 ha = mul2(splat(sc_new), fa), hb = mul2(splat(sc_new), fb);
+    if (what) store_what4<T>(what + 4 * c, ha.x, ha.y, hb.x, hb.y);
+    sum2 = add2(sum2, add2(fa, fb));
   };
   if (cached) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int c = threadIdx.x + i * NT;
+      const int c = t + i * NT;
       if (c < nvec) update(c, wr[i], gr[i], mr[i], vr[i]);
     }
   } else {
-    for (int c = threadIdx.x; c < nvec; c += NT) {
+    for (int c = t; c < nvec; c += NT) {
       const float4 wv = w4[c];
-      float4 d = no_grad ? zero4 : g4[c];
-      if (!ds_in) {
-        bool in;
-        float lvl;
-        weight_ste(quotient(wv.x, s_old, r_old), qmax, grid, in, lvl); d.x = in ? d.x : 0.f;
-        weight_ste(quotient(wv.y, s_old, r_old), qmax, grid, in, lvl); d.y = in ? d.y : 0.f;
-        weight_ste(quotient(wv.z, s_old, r_old), qmax, grid, in, lvl); d.z = in ? d.z : 0.f;
-        weight_ste(quotient(wv.w, s_old, r_old), qmax, grid, in, lvl); d.w = in ? d.w : 0.f;
-      }
-      update(c, wv, d, train_w ? m4[c] : make_float4(0, 0, 0, 0), train_w ? v4[c] : make_float4(0, 0, 0, 0));
+      update(c, wv, ste(wv, no_grad ? zero4 : g4[c]), train_w ? m4[c] : zero4, train_w ? v4[c] : zero4);
     }
   }
-  sum = warp_sum_i(sum);
-  if ((threadIdx.x & 31) == 0) shi[threadIdx.x >> 5] = sum;
+  const int sum = __reduce_add_sync(0xffffffffu, (int)sum2.x + (int)sum2.y);
+  if ((threadIdx.x & 31) == 0) sum_sh[threadIdx.x >> 5] = sum;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    int t = threadIdx.x < (blockDim.x >> 5) ? shi[threadIdx.x] : 0;
-    t = warp_sum_i(t);
-    if (threadIdx.x == 0) {
-      rowsum[row] = t;
-      scale[row] = sc_new;
+  if (t == 0) {
+    int total = 0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) total += sum_sh[i];
+    M.rowsum[row] = total;
+    M.scale[row] = sc_new;
+    if (train_s) {
+      M.m_s[row] = ms;
+      M.v_s[row] = vs;
+      M.steps[row] = s_new;
     }
   }
 }
 
+template <typename T, int NV, int NT, int BLOCKS>
+void launch_rows(const UpdateParams& p, int grid, cudaStream_t st) {
+  const int rows = p.row_end[p.n - 1];
+  if (grid != 0) launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 1, false>, rows, NT, 0, st, p);
+  else if (p.row_used) launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 0, true>, rows, NT, 0, st, p);
+  else launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 0, false>, rows, NT, 0, st, p);
+}
+template <typename T>
+void launch_variant(int variant, const UpdateParams& p, int grid, cudaStream_t st) {
+#define MREM_UPD(I, NT, NV, BLOCKS) case I: launch_rows<T, NV, NT, BLOCKS>(p, grid, st); break;
+  switch (variant) { UPD_VARIANTS(MREM_UPD) }
+#undef MREM_UPD
+}
+int variant_of(int cols) {
+#define MREM_UPD(I, NT, NV, BLOCKS) if (cols <= NT * NV * 4) return I;
+  UPD_VARIANTS(MREM_UPD)
+#undef MREM_UPD
+  return UPD_WIDEST;
+}
+
 }  // namespace
 
-void launch_fused_weight_update(float* w, float* g, float* m, float* v, float* steps, const float* ds_in,
-                                float* m_s, float* v_s, const OptimScalars* sc, int rows, int cols, int bits, int grid,
-                                int train_w, int train_s, int8_t* codes, int32_t* rowsum, float* scale, void* what,
+void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
                                 int dt, cudaStream_t st, const unsigned* row_used) {
-  Scope scope("fused_weight_update", (double)rows * cols * (29.0 + (what ? (dt == 1 ? 2.0 : 4.0) : 0.0)), 0, st);
-#define MREM_FWU_G(T, NV, NT, G, SP) launch_k(fused_weight_update_kernel<T, NV, NT, G, SP>, rows, NT, 0, st, w, g, m, v, steps, ds_in, m_s, v_s, sc, cols, bits, train_w, train_s, codes, rowsum, scale, (T*)what, row_used)
-#define MREM_FWU(T, NV, NT) do { if (grid != 0) MREM_FWU_G(T, NV, NT, 1, false); else if (row_used) MREM_FWU_G(T, NV, NT, 0, true); else MREM_FWU_G(T, NV, NT, 0, false); } while (0)
-#define MREM_FWU_T(T) do { if (cols > 512 && cols <= 768) MREM_FWU(T, 1, 192); else if (cols <= 1024) MREM_FWU(T, 1, 256); \
-    else if (cols > 2048 && cols <= 3072) MREM_FWU(T, 2, 384); else MREM_FWU(T, 2, 512); } while (0)
-  if (dt == 1) MREM_FWU_T(bf16); else MREM_FWU_T(float);
-#undef MREM_FWU_T
-#undef MREM_FWU
-#undef MREM_FWU_G
+  unsigned done = 0;
+  for (int i = 0; i < n; ++i) {
+    if (done >> i & 1u) continue;
+    UpdateParams p = {};
+    p.bits = bits; p.train_w = train_w; p.train_s = train_s; p.sc = sc; p.row_used = row_used;
+    const int variant = variant_of(mats[i].cols);
+    double bytes = 0;
+    int rows = 0;
+    for (int j = i; j < n; ++j) {                              // the matrices of one variant go in one launch
+      if (variant_of(mats[j].cols) != variant) continue;
+      done |= 1u << j;
+      p.mat[p.n] = mats[j];
+      p.row_end[p.n++] = rows += mats[j].rows;
+      bytes += (double)mats[j].rows * mats[j].cols * (29.0 + (mats[j].what ? (dt == 1 ? 2.0 : 4.0) : 0.0));
+    }
+    Scope scope("fused_weight_update", bytes, 0, st);
+    if (dt == 1) launch_variant<bf16>(variant, p, grid, st); else launch_variant<float>(variant, p, grid, st);
+  }
 }
 
 }  // namespace mrem
