@@ -63,7 +63,6 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
   uint8_t* const g0 = smem_raw + (base - smem_u32(smem_raw));
   uint8_t *const gV = g0 + (sV - base), *const gD = g0 + (sD - base), *const gX = g0 + (sX - base);
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
-  pdl_trigger();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_STE || i == B_P || i == B_S) ? 256 : 1);
@@ -79,6 +78,7 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
   __syncthreads();
   tc_fence_after();
   pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const int len = p.len[b];
   const int n_valid = (len + 31) / 32, n_chunks = (p.S + 31) / 32;        // 32-key chunks with a valid key, with any key

@@ -71,7 +71,6 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
   uint8_t* const g0 = smem_raw + (base - smem_u32(smem_raw));
   uint8_t *const gD = g0 + (sD - base), *const gX = g0 + (sX - base), *const gC = g0 + (sC - base);
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_STE || i == B_P || i == B_S) ? 512 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -85,6 +84,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
   __syncthreads();
   tc_fence_after();
   pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const int len = p.len[b], n_valid = (len + 31) / 32;
 
@@ -310,7 +310,6 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
   uint8_t *const gK = g0, *const gV = g0 + (sV - base), *const gP = g0 + (sP - base), *const gS = g0 + (sS - base);
   float4* const qstat = reinterpret_cast<float4*>(g0 + (sS - base) + 16384);   // per query: -max, 1 / sum, -dot
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), i == B_P ? 256 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -324,6 +323,7 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
   __syncthreads();
   tc_fence_after();
   pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const int len = p.len[b], n_q = (p.S + 63) / 64;
   const bool active = k0 < len;                            // a block of padded keys has zero gradients

@@ -68,7 +68,6 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
   // P takes the place of Q and K once the scores are in TMEM
   const uint32_t sV = base, sP = sV + n_box * 16384, sQ = sP, sK = sQ + 16384;
   uint8_t* gP = smem_raw + (sP - smem_u32(smem_raw));        // generic pointer to the P operand tile
-  pdl_trigger();
 
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar_qk), 1);
@@ -89,6 +88,7 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
   __syncthreads();
   tc_fence_after();
   pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   int len = p.valid_len ? p.valid_len[b] : p.S;
   len = len < 1 ? 1 : (len > p.S ? p.S : len);

@@ -35,8 +35,8 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
                                                         const int* __restrict__ type_ids, int S, int H, int vocab, int n_types,
                                                         T* __restrict__ y, unsigned* row_first, int* row_last,
                                                         int* row_count, int* __restrict__ status) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const long long t = blockIdx.x;
   int id = ids[t], tt = type_ids ? type_ids[t] : 0;
   if (id < 0 || id >= vocab || tt < 0 || tt >= n_types) {          // recorded, then clamped: no out-of-range access
@@ -108,8 +108,8 @@ template <typename T, int V>
 __global__ void __launch_bounds__(128) embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra,
                                                         T* __restrict__ e_t, T* __restrict__ e_s, T* __restrict__ y_s,
                                                         T* __restrict__ dsum, T* __restrict__ dy) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   __shared__ int last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, H = p.H;
@@ -321,8 +321,8 @@ __device__ __forceinline__ void add_rows_of_id(const EmbedTables& p, const T* __
 
 template <typename T, int V>
 __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_constant__ EmbedTables p, const T* __restrict__ dy) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][TAB_COLS];
   __shared__ int flag, group[8];
   constexpr int NV = TAB_COLS / (32 * V);                     // vectors per lane in a pass

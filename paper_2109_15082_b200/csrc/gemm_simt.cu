@@ -23,8 +23,8 @@ __device__ __forceinline__ float load_op(const OperandDesc& o, long long base, i
 }
 
 __global__ void __launch_bounds__(256) simt_gemm_kernel(const SimtParams p) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sa[TK][TS + 1];
   __shared__ float sb[TK][TS + 1];
   const int z = blockIdx.z, b0 = z % p.g.nb0, b1 = z / p.g.nb0;

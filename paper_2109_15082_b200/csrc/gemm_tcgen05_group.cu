@@ -46,7 +46,6 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int total_tiles = g.tile_end[g.n - 1];
-  pdl_trigger();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < g.num_stages; ++s) {
@@ -114,6 +113,7 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
           if (++stage == g.num_stages) { stage = 0; phase ^= 1u; }
         }
       }
+      pdl_trigger();                     // see tc_gemm_kernel
       if (!ok) {
         // let the copies already in flight land before the CTA may exit
         for (int s = 0; s < g.num_stages; ++s) {

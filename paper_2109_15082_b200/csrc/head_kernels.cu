@@ -21,8 +21,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) head_pool_kernel(const T* __restrict__ f_s, const T* __restrict__ f_t, long long seq_stride,
                                                         int B, int H, const float* __restrict__ wp, const float* __restrict__ bp,
                                                         float* __restrict__ pooled) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ float cls[];                                    // [HV][H]
   const int v0 = blockIdx.y * HV, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int idx = threadIdx.x; idx < HV * H; idx += blockDim.x) {
@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(256) head_logits_kernel(const float* __restric
                                                           const float* __restrict__ wc, const float* __restrict__ bc, float cc,
                                                           float* __restrict__ part, float* __restrict__ logits,
                                                           float* __restrict__ dpre) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float z_s[64], z_t[64], dz[64];
   const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const float* ps = pooled + (long long)b * H;
@@ -94,8 +94,8 @@ __global__ void __launch_bounds__(256) head_logits_kernel(const float* __restric
 template <typename T>
 __global__ void __launch_bounds__(256) head_back_kernel(const float* __restrict__ dpre, int B, int H, const float* __restrict__ wp,
                                                         long long seq_stride, T* __restrict__ dF) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ float sm[];                                     // dp[HV][H], then red[4][HV][64]
   float* dp = sm;
   float* red = sm + HV * H;
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(256) head_back_kernel(const float* __restrict_
 
 __global__ void head_loss_final_kernel(const float* __restrict__ part, int B, float cc, float* __restrict__ loss_total,
                                        float* __restrict__ logit_loss) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     float acc = 0.f;
     for (int b = 0; b < B; ++b) acc += part[b];

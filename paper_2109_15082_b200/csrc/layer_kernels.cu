@@ -21,8 +21,8 @@ template <typename T, int V>
 __global__ void __launch_bounds__(256) loss_kernel(const T* __restrict__ fh, const T* __restrict__ f,
                                                    long long n, float c, T* __restrict__ dF,
                                                    float* __restrict__ partial, int* __restrict__ status) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const long long base = (long long)blockIdx.y * n;
   float acc = 0.f;
@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(256) loss_kernel(const T* __restrict__ fh, con
 }
 __global__ void loss_final_kernel(const float* __restrict__ partial, int n_layers, int nb, float c,
                                   float* __restrict__ total, float* __restrict__ per_layer) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   float tot = 0.f;
   for (int l = 0; l < n_layers; ++l) {
@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(256) ste_act_kernel(const T* __restrict__ x, l
                                                       const float* __restrict__ step,
                                                       const float* __restrict__ offset, float lo, float hi,
                                                       float* __restrict__ part_s, float* __restrict__ part_o) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const float s = *step, r_s = __frcp_rn(s);
   const bool has_off = offset != nullptr;
@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(256) gelu_bwd_kernel(const T* __restrict__ u, 
                                                        const float* __restrict__ offset, float lo, float hi,
                                                        int quantized, float* __restrict__ part_s,
                                                        float* __restrict__ part_o) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const float s = quantized ? *step : 1.f, r_s = __frcp_rn(s);
   const bool has_off = offset != nullptr;
@@ -174,8 +174,8 @@ __global__ void __launch_bounds__(256) gelu_bwd_colsum_kernel(const T* __restric
                                                               float* __restrict__ part_o, int n_slots,
                                                               float* __restrict__ bias_grad, float* __restrict__ scratch,
                                                               int* __restrict__ counters) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int BC = GB_TX * V;                              // columns per block
   __shared__ float sh[32];
   __shared__ float cs[GB_TY][BC + 1];
@@ -261,8 +261,8 @@ __global__ void __launch_bounds__(256) gelu_bwd_colsum_kernel(const T* __restric
 __global__ void __launch_bounds__(256) ste_weight_kernel(const float* __restrict__ w, const float* __restrict__ steps,
                                                          int per_row, int bits, int grid, float* __restrict__ dw,
                                                          int cols, float* __restrict__ ds_rows) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const int row = blockIdx.x;
   const float s = steps[per_row ? row : 0];
@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(256) ste_weight_kernel(const float* __restrict
 }
 
 __global__ void __launch_bounds__(256) reduce_table_kernel(const ReduceEntry* __restrict__ table) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const ReduceEntry e = table[blockIdx.x];
   float a = 0.f;
@@ -297,31 +297,31 @@ __global__ void __launch_bounds__(256) reduce_table_kernel(const ReduceEntry* __
 }
 
 __global__ void scale_vec_kernel(const float* __restrict__ in, const float* __restrict__ scale, float* __restrict__ out, int n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = scale[0] * in[i];
 }
 __global__ void effective_bias_kernel(const float* __restrict__ b, const float* __restrict__ beta,
                                       const float* __restrict__ wscale, const int32_t* __restrict__ rowsum,
                                       float* __restrict__ beff, int n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) beff[i] = b[i] + beta[0] * wscale[i] * (float)rowsum[i];
 }
 
 // ------------------------------------------------------------------ AdamW
 __global__ void optim_prepare_kernel(const __grid_constant__ OptimArgs a) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0 && blockIdx.x == 0) optim_prepare(a);
 }
 
 __global__ void __launch_bounds__(256) adamw_table_kernel(const AdamEntry* __restrict__ table,
                                                           const OptimScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const AdamEntry e = table[blockIdx.y];
   const OptimScalars o = *sc;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < e.n; i += (long long)gridDim.x * blockDim.x) {
@@ -422,8 +422,8 @@ void launch_ste_weight(const float* w, const float* steps, int per_row, int bits
 // (event processing, launch and drain of a grid) and therefore what every traced duration contains on top of the
 // kernel's own run time.
 __global__ void empty_kernel() {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
 }
 void launch_trace_calibration(int n, cudaStream_t st) {
   for (int i = 0; i < n; ++i) {

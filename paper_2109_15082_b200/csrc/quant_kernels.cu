@@ -16,8 +16,8 @@ __global__ void __launch_bounds__(256) quantize_weight_kernel(const float* __res
                                                               int grid, int8_t* __restrict__ codes,
                                                               int32_t* __restrict__ rowsum, float* __restrict__ scale,
                                                               T* __restrict__ what) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ int sh[32];
   const int row = blockIdx.x;
   const float s = steps[per_row ? row : 0];
@@ -62,8 +62,8 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const T* __restrict__
                                                            T* __restrict__ qt, long long ld_qt, int seg_cols,
                                                            const float* __restrict__ step1,
                                                            const float* __restrict__ step2) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   // seg_cols > 0: three column segments of that width (a multiple of V), each with its own step
   const float s0 = *step, s1 = seg_cols ? *step1 : s0, s2 = seg_cols ? *step2 : s0;
   const float r0 = __frcp_rn(s0), r1 = __frcp_rn(s1), r2 = __frcp_rn(s2);
@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(256) quantize_act_rows_kernel(const T* __restr
                                                                 T* __restrict__ qt, long long ld_qt, int seg_cols,
                                                                 const float* __restrict__ step1,
                                                                 const float* __restrict__ step2) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const float s0 = *step, s1 = seg_cols ? *step1 : s0, s2 = seg_cols ? *step2 : s0;
   const float r0 = __frcp_rn(s0), r1 = __frcp_rn(s1), r2 = __frcp_rn(s2);
   const bool has_off = offset != nullptr;
@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(256) quantize_act_rows_kernel(const T* __restr
 template <typename T, int V>
 __global__ void __launch_bounds__(256) mix_kernel(const T* __restrict__ f, const T* __restrict__ fh, float lam,
                                                   T* __restrict__ out, long long n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; i < n; i += (long long)gridDim.x * blockDim.x * V) {
     float a[V], b[V];
     load_vec<T, V>(f + i, a);
@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(256) gelu_quant_kernel(const T* __restrict__ u
                                                          const float* __restrict__ step,
                                                          const float* __restrict__ offset, float lo, float hi,
                                                          int8_t* __restrict__ q8, T* __restrict__ qt) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const float s = *step, r_s = __frcp_rn(s);
   const bool has_off = offset != nullptr;
   const float off = has_off ? *offset : 0.f;
@@ -180,8 +180,8 @@ __global__ void __launch_bounds__(256) gelu_quant_kernel(const T* __restrict__ u
 // stat[row] = max|w| (rule 0) or mean|w| (rule 1) of one row; per_row: steps[row] = stat/qmax | stat.
 __global__ void __launch_bounds__(256) weight_row_stat_kernel(const float* __restrict__ w, int cols, int rule,
                                                               float* __restrict__ stat) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const float* wr = w + (long long)blockIdx.x * cols;
   float acc = 0.f;
@@ -194,8 +194,8 @@ __global__ void __launch_bounds__(256) weight_row_stat_kernel(const float* __res
 }
 __global__ void weight_steps_from_stat_kernel(const float* __restrict__ stat, int rows, int cols, int per_row,
                                               int rule, float qmax, float* __restrict__ steps) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (per_row) {
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
       const float v = rule == 0 ? __fdiv_rn(stat[r], qmax) : __fdiv_rn(stat[r], (float)cols);
@@ -212,8 +212,8 @@ __global__ void weight_steps_from_stat_kernel(const float* __restrict__ stat, in
 template <typename T>
 __global__ void __launch_bounds__(256) minmax_kernel(const T* __restrict__ x, long long ld, long long rows, int cols,
                                                      float* __restrict__ part) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   float lo = INFINITY, hi = -INFINITY;
   const long long total = rows * cols;
@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(256) minmax_kernel(const T* __restrict__ x, lo
   }
 }
 __global__ void minmax_final_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     float lo = INFINITY, hi = -INFINITY;
     for (int i = 0; i < n; ++i) {
@@ -244,8 +244,8 @@ __global__ void minmax_final_kernel(const float* __restrict__ part, int n, float
   }
 }
 __global__ void step_from_minmax_kernel(const float* __restrict__ mm, int mode, float qmax, float* step, float* offset) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     float s, o = 0.f;
     if (mode == 0) s = __fdiv_rn(fmaxf(fabsf(mm[0]), fabsf(mm[1])), qmax);
@@ -258,8 +258,8 @@ __global__ void step_from_minmax_kernel(const float* __restrict__ mm, int mode, 
 
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ src, const int* __restrict__ idx,
                                                           long long row_vecs, uint4* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const uint4* s = src + (long long)idx[blockIdx.y] * row_vecs;
   uint4* o = out + (long long)blockIdx.y * row_vecs;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < row_vecs; i += (long long)gridDim.x * blockDim.x)
@@ -267,16 +267,16 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
 }
 
 __global__ void __launch_bounds__(256) widen_bf16_kernel(const bf16* __restrict__ src, float* __restrict__ dst, long long n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     dst[i] = __bfloat162float(src[i]);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) narrow_kernel(const float* __restrict__ src, T* __restrict__ dst, long long n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     dst[i] = from_f<T>(src[i]);
 }

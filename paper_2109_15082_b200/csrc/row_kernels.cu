@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(128) ln_fwd_kernel(const T* __restrict__ y, co
                                                      int cols, T* __restrict__ out, float* __restrict__ mean,
                                                      float* __restrict__ rstd, const float* __restrict__ step,
                                                      float qmax, int8_t* __restrict__ q8, T* __restrict__ qt) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long row = blockIdx.x * 4ll + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -141,8 +141,8 @@ __global__ void __launch_bounds__(128) ln_bwd_kernel(const T* __restrict__ dout,
                                                      const float* __restrict__ rstd, const float* __restrict__ gamma,
                                                      long long rows, int cols, T* __restrict__ dy,
                                                      T* __restrict__ dsum) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long row = blockIdx.x * 4ll + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(128, 7) ln_bwd_ste_kernel(const T* __restrict_
                                                          const float* __restrict__ rstd, const float* __restrict__ gamma,
                                                          long long rows, int cols, T* __restrict__ dy,
                                                          T* __restrict__ dsum, float* __restrict__ part_s, int n_slots) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[4];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const float s = *step, r_s = __frcp_rn(s);
@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict_
                                                             float* __restrict__ out0, float* __restrict__ out1,
                                                             float* __restrict__ out2, float* __restrict__ scratch,
                                                             long long plane, int* __restrict__ counters) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int BC = COLRED_CT * V;                        // columns per block
   __shared__ float sh[3][COLRED_RT][BC + 1];
   __shared__ int is_last;
@@ -401,8 +401,8 @@ __global__ void __launch_bounds__(128) softmax_fwd_kernel(const float* __restric
                                                           const float* __restrict__ step,
                                                           const float* __restrict__ offset, float lo, float hi,
                                                           T* __restrict__ qt) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long row = blockIdx.x * 4ll + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -474,8 +474,8 @@ __global__ void __launch_bounds__(256) softmax_bwd_kernel(const T* __restrict__ 
                                                           T* __restrict__ dS, long long rows, int S,
                                                           const float* __restrict__ step, float lo, float hi,
                                                           int quantized, float* __restrict__ part_s) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float sh[32];
   const int lane = threadIdx.x & 31;
   const long long warp0 = blockIdx.x * 8ll + (threadIdx.x >> 5), nwarps = gridDim.x * 8ll;

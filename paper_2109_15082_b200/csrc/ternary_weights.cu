@@ -394,8 +394,8 @@ template <typename T, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) laq_quantize_kernel(const float* __restrict__ w, int cols, int bits,
                                                                      int8_t* __restrict__ codes, int32_t* __restrict__ rowsum,
                                                                      float* __restrict__ scale, T* __restrict__ what) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ LaqShared sh;
   const long long base = (long long)blockIdx.x * cols;
   const float4* w4 = reinterpret_cast<const float4*>(w + base);
@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) laq_update_kernel(float* __rest
                                                                    int bits, int8_t* __restrict__ codes,
                                                                    int32_t* __restrict__ rowsum, float* __restrict__ scale,
                                                                    T* __restrict__ what) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ LaqShared sh;
   const OptimScalars o = *sc;
   const long long base = (long long)blockIdx.x * cols;
@@ -473,8 +473,8 @@ __global__ void __launch_bounds__(NT, RULE == 2 ? 5 : 4) closed_form_quantize_ke
                                                                       int8_t* __restrict__ codes,
                                                                       int32_t* __restrict__ rowsum,
                                                                       float* __restrict__ scale, T* __restrict__ what) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double shd[64];
   __shared__ int shi[32];
   __shared__ float shf[32];
@@ -503,8 +503,8 @@ __global__ void __launch_bounds__(NT, RULE == 2 ? 5 : 4) closed_form_update_kern
                                                                     int8_t* __restrict__ codes,
                                                                     int32_t* __restrict__ rowsum,
                                                                     float* __restrict__ scale, T* __restrict__ what) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double shd[64];
   __shared__ int shi[32];
   __shared__ float shf[32];

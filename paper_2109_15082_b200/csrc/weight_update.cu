@@ -92,8 +92,8 @@ constexpr int UPD_WIDEST = 4;
 // embedding table, one matrix per launch: its pointers stay at fixed places of the parameters, 235 -> 204 us for the step).
 template <typename T, int NV, int NT, int BLOCKS, int GRID, bool SPARSE>
 __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const __grid_constant__ UpdateParams P) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int NW = NT / 32;
   constexpr bool WIDE = NT == 256;                             // the variant that also takes rows beyond its registers
   __shared__ float ds_sh[NW];
