@@ -181,15 +181,19 @@ void launch_effective_bias(const float* b, const float* beta, const float* wscal
 // ---- optimizer (AdamW)
 // bc = 1 - beta^t; lr_bc1 = lr / bc1, rsqrt_bc2 = 1 / sqrt(bc2)
 struct OptimScalars { float lr, beta1, beta2, eps, bc1, bc2, weight_decay, lr_bc1, rsqrt_bc2; };
-struct AdamEntry { float* p; const float* g; float* m; float* v; long long n; float wd; float min_value; };   // wd: 1 = decayed
+// wd: 1 = decayed.  part (may be null): RED_BLOCKS partial sums of the one gradient element, for launches that form it
+// themselves; p null: nothing to update.
+struct AdamEntry { float* p; float* g; float* m; float* v; long long n; float wd; float min_value; const float* part = nullptr; };
 // What optim_prepare (optim.cuh) needs: where the scalars go, the device step counter, and the caller's numbers.
 struct OptimArgs { OptimScalars* out; int* d_t; int host_t; float lr0; int total; float beta1, beta2, eps, weight_decay; };
 // Computes the scalars of this step on the device: t = ++(*d_t) (or host_t when >= 1),
 // lr = lr0 * (1 - (t-1)/total) when total > 0 else lr0.
 void launch_optim_prepare(OptimScalars* d_out, int* d_t, int host_t, float lr0, int total_steps, float beta1,
                           float beta2, float eps, float weight_decay, cudaStream_t st);
-void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, const OptimScalars* d_sc,
-                        cudaStream_t st);
+// max_n: elements of the longest entry.  sum_parts: the gradients of entries with `part` are the sums of their partials (formed
+// and written by this launch), else they are already there.
+void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, long long max_n, bool sum_parts,
+                        const OptimScalars* d_sc, cudaStream_t st);
 
 // Fused per-row update of weight matrices and their per-row steps: step gradient (or ds_in when the
 // gradients were already masked), AdamW on step and weights, re-quantization (codes, row sums,

@@ -318,12 +318,22 @@ __global__ void optim_prepare_kernel(const __grid_constant__ OptimArgs a) {
   if (threadIdx.x == 0 && blockIdx.x == 0) optim_prepare(a);
 }
 
-__global__ void __launch_bounds__(256) adamw_table_kernel(const AdamEntry* __restrict__ table,
+__global__ void __launch_bounds__(256) adamw_table_kernel(const AdamEntry* __restrict__ table, int sum_parts,
                                                           const OptimScalars* __restrict__ sc) {
   pdl_wait();
   pdl_trigger();
+  __shared__ float sh[32];
   const AdamEntry e = table[blockIdx.y];
   const OptimScalars o = *sc;
+  if (sum_parts && e.part) {                                   // as reduce_table_kernel does
+    if (blockIdx.x) return;
+    float a = 0.f;
+    for (int i = threadIdx.x; i < RED_BLOCKS; i += blockDim.x) a += e.part[i];
+    a = block_sum(a, sh);
+    if (threadIdx.x == 0) *e.g = a;
+    __syncthreads();
+  }
+  if (!e.p) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < e.n; i += (long long)gridDim.x * blockDim.x) {
     float m = e.m[i], v = e.v[i];
     e.p[i] = adam_one(e.p[i], e.g[i], m, v, o, e.wd, e.min_value);
@@ -448,12 +458,14 @@ void launch_optim_prepare(OptimScalars* d_out, int* d_t, int host_t, float lr0, 
                           float beta2, float eps, float weight_decay, cudaStream_t st) {
   launch_k(optim_prepare_kernel, 1, 32, 0, st, OptimArgs{d_out, d_t, host_t, lr0, total_steps, beta1, beta2, eps, weight_decay});
 }
-void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, const OptimScalars* d_sc,
-                        cudaStream_t st) {
+void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total_elems, long long max_n, bool sum_parts,
+                        const OptimScalars* d_sc, cudaStream_t st) {
   if (n_entries <= 0) return;
   Scope sc("adamw", (double)total_elems * 28.0, 0, st);
-  dim3 grid(64, n_entries);
-  launch_k(adamw_table_kernel, grid, 256, 0, st, d_table, d_sc);
+  // four elements a thread where the entries are vectors: most blocks of a wider grid would find nothing to do
+  const long long want = (max_n + 1023) / 1024;
+  dim3 grid((unsigned)(want < 1 ? 1 : (want < 64 ? want : 64)), n_entries);
+  launch_k(adamw_table_kernel, grid, 256, 0, st, d_table, (int)sum_parts, d_sc);
 }
 
 }  // namespace mrem

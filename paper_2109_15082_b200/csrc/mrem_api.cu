@@ -209,15 +209,24 @@ int build_tables(mrem_ctx* c) {
       if ((d.act_asym_sites & 2) && b.a_off[7])
         { adam.push_back({b.a_off[7], g.off + 7, g.m_off + 7, g.v_off + 7, 1, 0.f, -INFINITY}); rest.push_back(adam.back()); }
     }
+    // the scalars' gradients are sums of partials; those that are not trained are only formed
+    for (int site = 0; site <= N_SITES; ++site) {
+      float* const grad = site < N_SITES ? g.a + site : g.off + 7;
+      AdamEntry* e = nullptr;
+      for (AdamEntry& r : rest) if (r.g == grad) e = &r;
+      if (!e) { rest.push_back({nullptr, grad, nullptr, nullptr, 0, 0.f, 0.f}); e = &rest.back(); }
+      e->part = s.part + site * RED_BLOCKS;
+    }
   }
   if (cudaMemcpyAsync(c->reduce_table, red.data(), sizeof(ReduceEntry) * red.size(), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
     return fail(c, MREM_ERR_CUDA, "table upload failed");
   c->adam_entries = (int)adam.size();
   c->adam_elems = 0;
-  for (const AdamEntry& e : adam) c->adam_elems += e.n;
+  c->adam_longest = 0;
+  for (const AdamEntry& e : adam) { c->adam_elems += e.n; if (e.n > c->adam_longest) c->adam_longest = e.n; }
   c->rest_entries = (int)rest.size();
-  c->rest_elems = 0;
-  for (const AdamEntry& e : rest) c->rest_elems += e.n;
+  c->rest_elems = c->rest_longest = 0;
+  for (const AdamEntry& e : rest) { c->rest_elems += e.n; if (e.n > c->rest_longest) c->rest_longest = e.n; }
   if (!rest.empty() && cudaMemcpyAsync(c->adam_rest, rest.data(), sizeof(AdamEntry) * rest.size(), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
     return fail(c, MREM_ERR_CUDA, "table upload failed");
   if (cudaMemcpyAsync(c->adam_table, adam.data(), sizeof(AdamEntry) * adam.size(), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)

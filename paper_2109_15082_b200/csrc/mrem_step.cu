@@ -280,12 +280,11 @@ void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st) 
 // ------------------------------------------------------------------ backward
 // Two streams: the weight-gradient products (tensor-core bound, results needed only by the update) are
 // issued on the side stream and run under the main stream's element-wise and row kernels (memory bound);
-// the main stream waits for them before the next layer reuses the gradient buffers they read.  With
-// `update_as_you_go` (per-row steps; the optimizer scalars of this step are already on the device) each
-// layer's matrices are also updated on the side stream as soon as their gradients are complete.  The main
-// stream joins the side stream before returning.  While kernels are being timed one by one (tracing) all
-// of it stays on the main stream.
-int student_backward(mrem_ctx* c, bool update_as_you_go) {
+// the main stream waits for them before the next layer reuses the gradient buffers they read.  With `o` (per-row steps)
+// the whole update happens here as well: each layer's matrices on the side stream as soon as their gradients are
+// complete, everything else at the end.  The main stream joins the side stream before returning.  While kernels are
+// being timed one by one (tracing) all of it stays on the main stream.
+int student_backward(mrem_ctx* c, const mrem_optim* o) {
   const mrem_module_desc& d = c->d;
   const int H = d.hidden, F = d.ffn, h = d.n_heads, hd = H / h, B = c->cur_batch, S = c->cur_seq;
   const long long M = (long long)B * S;
@@ -303,6 +302,12 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
     if (two_streams && (cudaEventRecord(c->ev_join, side) != cudaSuccess || cudaStreamWaitEvent(c->stream, c->ev_join, 0) != cudaSuccess))
       sync_failed = true;
   };
+  if (o) {
+    fork();
+    launch_optim_prepare(c->optim_sc, c->t_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps,
+                         o->weight_decay, side);
+  }
+  const bool halves = M <= 2048;
   const int ok = r.okind();
   const float inv_sqrt_d = 1.f / sqrtf((float)hd);
   // Buffers the side stream reads, two copies used by alternate layers: the main stream starts the layer below while
@@ -381,6 +386,15 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
     fork();
     launch_col_reduce(q.d_a, H, s.y1, s.mean1, s.rstd1, q.d_y1, H, M, H, g.p[MREM_LN1_B], g.p[MREM_LN1_G], g.p[MREM_BO],
                       c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
+    // Up to 2048 tokens the feed-forward half's weight-gradient products go now: their update (two thirds of the layer's
+    // weights) runs under the attention half, and the last layer leaves less of it for the end (3 x 72 tokens: step 506 -> 501
+    // us, 8 x 256: 1038 -> 1020).  With more tokens the products take longer than the updates, and one launch for all four
+    // is the better one (32 x 128: 1325 -> 1317, with refitted scales 1474 -> 1460).
+    // (The products that read these two matrices are behind the fork above.)
+    if (halves) {
+      rw.flush_deferred();
+      if (o) enqueue_matrix_updates(c, l, W_1, 2, side);
+    }
     r.gemm(view(q.d_y1, H), weights(w[W_O].what, H, 1), (int)M, H, H, 1, 1, Epi(c->d_ctxhat, ok, H).e);
     rw.defer(view(q.d_y1, H, 1), view(s.ctx_qt, H, 1), H, H, (int)M, Epi(g.p[MREM_WO], OUT_F32, H).alpha(1.f, b.a_steps[S_C]).e);
     // attention:  ctx = P_hat V_hat,  P = softmax(Q_hat K_hat^T / sqrt(d))
@@ -411,7 +425,7 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
     launch_col_reduce(q.d_qkv, 3 * H, nullptr, nullptr, nullptr, nullptr, 0, M, 3 * H, g.p[MREM_BQKV], nullptr, nullptr, c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
     r.gemm(view(q.d_qkv, 3 * H), weights(w[W_QKV].what, H, 1), (int)M, H, 3 * H, 1, 1, Epi(c->d_xhat, ok, H).e);
     rw.defer(view(q.d_qkv, 3 * H, 1), view(s.x_qt, H, 1), 3 * H, H, (int)M, Epi(g.p[MREM_WQKV], OUT_F32, H).alpha(1.f, b.a_steps[S_X]).e);
-    rw.flush_deferred();                              // the layer's four weight-gradient products, one launch
+    rw.flush_deferred();                              // the weight-gradient products that are left
     if (fuse_ln && l > 0) {
       // left to the LayerNorm backward of the layer below, which reads d_xhat and d_y1 before anything overwrites them
       pending.x = x_in; pending.add = q.d_y1; pending.step = b.a_steps[S_X]; pending.part = part + S_X * RED_BLOCKS;
@@ -426,12 +440,18 @@ int student_backward(mrem_ctx* c, bool update_as_you_go) {
     //  or on demand by mrem_get_grad)
     // the side stream is done with this layer's copy of the gradient buffers once the grouped products have run
     if (two_streams && cudaEventRecord(c->ev_layer[l & 1], side) != cudaSuccess) sync_failed = true;
-    // nothing below reads what the update writes: the latent weights, moments, row steps and this layer's codes
-    if (update_as_you_go) enqueue_matrix_updates(c, l, 0, N_WMAT, side);
+    if (o) {
+      if (l == 0) join();                             // (the products that read the activation steps as scales are behind this)
+      fork();                                         // the input gradient's product reads Wqkv's dequantized values
+      // nothing below reads what the update writes: the latent weights, moments, row steps and this layer's codes
+      enqueue_matrix_updates(c, l, 0, halves ? W_1 : N_WMAT, side);
+    }
   }
-  // step-size and offset gradients of every layer's activation quantizers: the per-block partial sums the
-  // kernels above left, added in index order (one launch for the whole module; only the update reads them)
-  launch_reduce_table(c->reduce_table, c->reduce_per_layer * d.n_layers, c->stream);
+  // step-size and offset gradients of every layer's activation quantizers are the per-block partial sums the kernels above
+  // left, added in index order: one launch for the whole module, which with `o` also updates everything but the matrices
+  // (beside the last matrices' update)
+  if (o) launch_adamw_table(c->adam_rest, c->rest_entries, c->rest_elems, c->rest_longest, true, c->optim_sc, c->stream);
+  else launch_reduce_table(c->reduce_table, c->reduce_per_layer * d.n_layers, c->stream);
   join();
   c->have_input_grad = true;           // layer 0's straight-through pass wrote it to carry[0]
   if (sync_failed) return fail(c, MREM_ERR_CUDA, "backward: stream fork/join failed");
@@ -533,7 +553,7 @@ int32_t mrem_module_backward(mrem_ctx* c) {
   for (int l = 0; l < c->d.n_layers; ++l)
     for (int k = 0; k < N_WMAT; ++k) if (!c->bind[l].w_steps[k] && !closed_form_weights(c->d)) return fail(c, MREM_ERR_ORDER, "backward: weight steps not bound");
   if (c->tables_dirty) { const int rc = build_tables(c); if (rc != MREM_OK) return rc; }
-  const int rc = student_backward(c, false);
+  const int rc = student_backward(c, nullptr);
   if (rc != MREM_OK) return rc;
   c->have_grads = true;
   c->w_ste_done = false;
@@ -553,12 +573,9 @@ int32_t mrem_backward_and_step(mrem_ctx* c, const mrem_optim* o) {
   for (int l = 0; l < c->d.n_layers; ++l)
     for (int k = 0; k < N_WMAT; ++k) if (!c->bind[l].w_steps[k] && !closed_form_weights(c->d)) return fail(c, MREM_ERR_ORDER, "backward: weight steps not bound");
   if (c->tables_dirty) { const int rc = build_tables(c); if (rc != MREM_OK) return rc; }
-  launch_optim_prepare(c->optim_sc, c->t_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps,
-                       o->weight_decay, c->stream);
   c->w_ste_done = false;
-  const int rc = student_backward(c, true);
+  const int rc = student_backward(c, o);
   if (rc != MREM_OK) return rc;
-  launch_adamw_table(c->adam_rest, c->rest_entries, c->rest_elems, c->optim_sc, c->stream);
   if (cudaGetLastError() != cudaSuccess) return fail(c, MREM_ERR_CUDA, "step: launch failed");
   c->have_grads = false; c->have_loss = false; c->have_student = false; c->have_teacher = false;
   c->codes_fresh = true;
@@ -576,7 +593,7 @@ int32_t mrem_step(mrem_ctx* c, const mrem_optim* o) {
   const mrem_module_desc& d = c->d;
   if (d.w_step_per_row) {
     // every tensor but the matrices and their steps, then one fused pass per matrix
-    launch_adamw_table(c->adam_rest, c->rest_entries, c->rest_elems, c->optim_sc, c->stream);
+    launch_adamw_table(c->adam_rest, c->rest_entries, c->rest_elems, c->rest_longest, false, c->optim_sc, c->stream);
     for (int l = 0; l < d.n_layers; ++l) enqueue_matrix_updates(c, l, 0, N_WMAT, c->stream);
   } else {
     if (!c->w_ste_done) {
@@ -588,7 +605,7 @@ int32_t mrem_step(mrem_ctx* c, const mrem_optim* o) {
           launch_reduce_table(c->reduce_table + (size_t)l * c->reduce_per_layer + N_SITES + 1 + k, 1, c->stream);
         }
     }
-    launch_adamw_table(c->adam_table, c->adam_entries, c->adam_elems, c->optim_sc, c->stream);
+    launch_adamw_table(c->adam_table, c->adam_entries, c->adam_elems, c->adam_longest, false, c->optim_sc, c->stream);
   }
   if (cudaGetLastError() != cudaSuccess) return fail(c, MREM_ERR_CUDA, "step: launch failed");
   c->have_grads = false; c->have_loss = false; c->have_student = false; c->have_teacher = false;
@@ -692,7 +709,7 @@ int32_t mrem_rem_step(mrem_ctx* c, int32_t layer, int32_t tensor_id, const void*
       if (ar.asym) host[ne++] = AdamEntry{b.a_off[site], g.off + site, g.m_off + site, g.v_off + site, 1, 0.f, -INFINITY};
       if (cudaMemcpyAsync(c->rem_table, host, sizeof(AdamEntry) * ne, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return fail(c, MREM_ERR_CUDA, "rem_step: table upload failed");
-      launch_adamw_table(c->rem_table, ne, ne, c->optim_sc, st);
+      launch_adamw_table(c->rem_table, ne, ne, 1, false, c->optim_sc, st);
     }
   }
   if (r.rc != MREM_OK) return r.rc;
