@@ -70,7 +70,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, const uint32_t
     return;
   }
   float v[32];
-  const float rb = e.row_bias ? e.row_bias[row] : 0.f;
+  const float rb = row_term(e, row);
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     const int n = min(col0 + j, p.N - 1);

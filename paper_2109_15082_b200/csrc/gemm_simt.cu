@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(const SimtParams p) {
       const int n = n0 + tx * 4 + j;
       if (n >= p.g.N) continue;
       float v = acc[i][j] * (e.col_scale ? alpha * e.col_scale[n] : alpha);
-      v += (e.col_bias ? e.col_bias[n] : 0.f) + (e.row_bias ? e.row_bias[m] : 0.f);
+      v += (e.col_bias ? e.col_bias[n] : 0.f) + row_term(e, m);
       if (e.residual) v += reinterpret_cast<const float*>(e.residual)[row_off + n];
       if (e.act == 1) v = gelu_erf(v);
       reinterpret_cast<float*>(e.out)[row_off + n] = v;

@@ -210,7 +210,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (direct && col_begin < p.N) nfull = min((p.N - col_begin) >> 5, cols_per_warp >> 5);
       uint32_t res0[16];
       if (nfull > 0 && res_bf16) fetch_res_bf16(e, row_off + col_begin, row_ok, res0);   // in flight during the wait
-      const float rb = (e.row_bias && row_ok) ? e.row_bias[row] : 0.f;
+      const float rb = row_ok ? row_term(e, row) : 0.f;
       float* cv = col_terms[warp - 2];
       if (nfull > 0) stage_col_terms<MODE>(e, cv, alpha, col_begin, cols_per_warp, p.N, lane);   // before the wait as well
       // every lane polls; the decision is made warp-uniform before any .sync.aligned instruction

@@ -190,7 +190,7 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
       const bool row_ok = row < p.M;
       const long long row_off = (long long)t.b0 * e.c_b0 + (long long)t.b1 * e.c_b1 + (long long)row * e.ldc;
       const int nfull = col_begin < p.N ? min((p.N - col_begin) >> 5, cols_per_warp >> 5) : 0;   // N % 32 == 0 (host)
-      const float rb = (e.row_bias && row_ok) ? e.row_bias[row] : 0.f;
+      const float rb = row_ok ? row_term(e, row) : 0.f;
       const bool got = mbar_wait_or_abort(smem_u32(&tfull_bar[acc]), acc_phase, vabort, g.p[0].wait_ns);
       if (!__all_sync(0xffffffffu, got)) {
         if (lane == 0 && !*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);

@@ -56,9 +56,12 @@ void launch_layernorm_fwd(const void* y, const float* gamma, const float* beta, 
                           void* out, float* mean, float* rstd, const float* step, int qmax, int8_t* q8, void* qt,
                           int dt, cudaStream_t st);
 
-// g = stored(gelu(u)); codes of g (asymmetric when offset != null) as int8/uint8 and storage-type numbers.
+// The bias of a product whose left operand carries an offset beta: beff[i] = b[i] + beta * wscale[i] * rowsum[i] (b null: 0).
+struct EffectiveBias { const float *b, *wscale; const int32_t* rowsum; float* beff; int n; };
+// g = stored(gelu(u)); codes of g (asymmetric when offset != null) as int8/uint8 and storage-type numbers.  eb (may be null,
+// needs an offset): the effective bias of the product that reads the codes, on the way.
 void launch_gelu_quant(const void* u, long long n, const float* step, const float* offset, int lo, int hi,
-                       int8_t* q8, void* qt, int dt, cudaStream_t st);
+                       int8_t* q8, void* qt, int dt, cudaStream_t st, const EffectiveBias* eb = nullptr);
 
 // P = softmax(scores) over the last axis with keys >= valid_len[b] masked out; scores fp32
 // [B, h, S, S]; optional codes of P as storage-type numbers.
@@ -102,8 +105,10 @@ int launch_attention_bwd_long(const AttentionBwd& a, cudaStream_t st);    // 129
 
 // ---- loss (Eq. 3)
 // partial[l][block] = sum (f_hat - f)^2 over the block's share; dF = 2 c (f_hat - f).
+// totals (may be null): the block that finishes last adds the partials as well; `counter` is zero before and after.
+struct LossTotals { int* counter; float* total; float* per_layer; };
 void launch_loss(const void* f_hat, const void* f, int n_layers, long long n_per_layer, float c, void* dF,
-                 float* partial, int* status, int dt, cudaStream_t st);
+                 float* partial, int* status, int dt, cudaStream_t st, const LossTotals* totals = nullptr);
 void launch_loss_finalize(const float* partial, int n_layers, float c, float* loss_total, float* loss_per_layer,
                           cudaStream_t st);
 
@@ -172,9 +177,7 @@ struct ReduceEntry { const float* src; int count; float* dst; };
 void launch_trace_calibration(int n, cudaStream_t st);
 void launch_reduce_table(const ReduceEntry* d_table, int n_entries, cudaStream_t st);
 
-// out[i] = scale[0] * in[i]  (small vectors)
-void launch_scale_vec(const float* in, const float* scale, float* out, int n, cudaStream_t st);
-// beff[n] = b[n] + beta[0] * wscale[n] * rowsum[n]
+// beff[n] = b[n] + beta[0] * wscale[n] * rowsum[n]  (b null: 0)
 void launch_effective_bias(const float* b, const float* beta, const float* wscale, const int32_t* rowsum, float* beff,
                            int n, cudaStream_t st);
 

@@ -17,13 +17,17 @@ __device__ __forceinline__ float qz(float x, float s, float r_s, float off, bool
 __device__ __forceinline__ int qcode(float z, float lo, float hi) { return __float2int_rn(fminf(fmaxf(z, lo), hi)); }
 
 // ------------------------------------------------------------------ loss (Eq. 3) and its gradient
+// `counter` not null: the block that finishes last (ticket) adds every layer's partials in index order and the layers in
+// order, so the totals do not depend on which block that is; a launch of its own for that was 5 us on the step's chain.
 template <typename T, int V>
 __global__ void __launch_bounds__(256) loss_kernel(const T* __restrict__ fh, const T* __restrict__ f,
                                                    long long n, float c, T* __restrict__ dF,
-                                                   float* __restrict__ partial, int* __restrict__ status) {
+                                                   float* __restrict__ partial, int* __restrict__ status,
+                                                   int* __restrict__ counter, float* __restrict__ total, float* __restrict__ per_layer) {
   pdl_wait();
   pdl_trigger();
   __shared__ float sh[32];
+  __shared__ int is_last;
   const long long base = (long long)blockIdx.y * n;
   float acc = 0.f;
   for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; i < n; i += (long long)gridDim.x * blockDim.x * V) {
@@ -42,6 +46,32 @@ __global__ void __launch_bounds__(256) loss_kernel(const T* __restrict__ fh, con
   if (threadIdx.x == 0) {
     partial[blockIdx.y * gridDim.x + blockIdx.x] = acc;
     if (!isfinite(acc) && status) atomicCAS(status, 0, (int)DEV_NONFINITE);
+    is_last = 0;
+    if (counter) {
+      __threadfence();
+      is_last = atomicAdd(counter, 1) == (int)(gridDim.x * gridDim.y) - 1;
+    }
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = gridDim.x, n_layers = gridDim.y;
+  float tot = 0.f;
+  for (int l0 = 0; l0 < n_layers; l0 += 8) {                   // a layer per warp
+    const int l = l0 + warp;
+    float a = 0.f;
+    if (l < n_layers) {
+      for (int i = lane; i < nb; i += 32) a += __ldcg(partial + l * nb + i);
+      a = warp_sum(a) * c;
+      if (lane == 0) { sh[warp] = a; if (per_layer) per_layer[l] = a; }
+    }
+    __syncthreads();
+    for (int k = 0; k < 8 && l0 + k < n_layers; ++k) tot += sh[k];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (total) *total = tot;
+    *counter = 0;                                              // ready for the next launch
   }
 }
 __global__ void loss_final_kernel(const float* __restrict__ partial, int n_layers, int nb, float c,
@@ -296,19 +326,13 @@ __global__ void __launch_bounds__(256) reduce_table_kernel(const ReduceEntry* __
   if (threadIdx.x == 0) *e.dst = a;
 }
 
-__global__ void scale_vec_kernel(const float* __restrict__ in, const float* __restrict__ scale, float* __restrict__ out, int n) {
-  pdl_wait();
-  pdl_trigger();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = scale[0] * in[i];
-}
 __global__ void effective_bias_kernel(const float* __restrict__ b, const float* __restrict__ beta,
                                       const float* __restrict__ wscale, const int32_t* __restrict__ rowsum,
                                       float* __restrict__ beff, int n) {
   pdl_wait();
   pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) beff[i] = b[i] + beta[0] * wscale[i] * (float)rowsum[i];
+  if (i < n) beff[i] = (b ? b[i] : 0.f) + beta[0] * wscale[i] * (float)rowsum[i];
 }
 
 // ------------------------------------------------------------------ AdamW
@@ -357,15 +381,21 @@ inline bool al16(const void* p) { return p == nullptr || (reinterpret_cast<uintp
   } while (0)
 
 void launch_loss(const void* f_hat, const void* f, int n_layers, long long n_per_layer, float c, void* dF,
-                 float* partial, int* status, int dt, cudaStream_t st) {
+                 float* partial, int* status, int dt, cudaStream_t st, const LossTotals* totals) {
   Scope sc("recon_loss", (double)n_layers * n_per_layer * 3 * (dt == 1 ? 2.0 : 4.0), 0, st);
-  dim3 grid(RED_BLOCKS, n_layers);
+  const LossTotals t = totals ? *totals : LossTotals{nullptr, nullptr, nullptr};
   MREM_DT(dt, T, {
     constexpr int V = 16 / (int)sizeof(T);
-    if (n_per_layer % V == 0 && al16(f_hat) && al16(f) && al16(dF))
-      launch_k(loss_kernel<T, V>, grid, 256, 0, st, (const T*)f_hat, (const T*)f, n_per_layer, c, (T*)dF, partial, status);
-    else
-      launch_k(loss_kernel<T, 1>, grid, 256, 0, st, (const T*)f_hat, (const T*)f, n_per_layer, c, (T*)dF, partial, status);
+    const bool vec = n_per_layer % V == 0 && al16(f_hat) && al16(f) && al16(dF);
+    long long blocks = RED_BLOCKS;                             // (what launch_loss_finalize expects)
+    if (totals) {                                              // one wave over all layers, and none for a block without work
+      const long long work = (n_per_layer / (vec ? V : 1) + 255) / 256, wave = RED_BLOCKS / n_layers;
+      blocks = work < wave ? work : wave;
+      if (blocks < 1) blocks = 1;
+    }
+    dim3 grid((unsigned)blocks, n_layers);
+    if (vec) launch_k(loss_kernel<T, V>, grid, 256, 0, st, (const T*)f_hat, (const T*)f, n_per_layer, c, (T*)dF, partial, status, t.counter, t.total, t.per_layer);
+    else launch_k(loss_kernel<T, 1>, grid, 256, 0, st, (const T*)f_hat, (const T*)f, n_per_layer, c, (T*)dF, partial, status, t.counter, t.total, t.per_layer);
   });
 }
 void launch_loss_finalize(const float* partial, int n_layers, float c, float* loss_total, float* loss_per_layer,
@@ -446,9 +476,6 @@ void launch_reduce_table(const ReduceEntry* d_table, int n_entries, cudaStream_t
   if (n_entries > 0) launch_k(reduce_table_kernel, n_entries, 256, 0, st, d_table);
 }
 
-void launch_scale_vec(const float* in, const float* scale, float* out, int n, cudaStream_t st) {
-  launch_k(scale_vec_kernel, (n + 255) / 256, 256, 0, st, in, scale, out, n);
-}
 void launch_effective_bias(const float* b, const float* beta, const float* wscale, const int32_t* rowsum, float* beff,
                            int n, cudaStream_t st) {
   launch_k(effective_bias_kernel, (n + 255) / 256, 256, 0, st, b, beta, wscale, rowsum, beff, n);

@@ -75,6 +75,7 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->minmax = (float*)A.take(256);
   c->d_loss_e2e = (float*)A.take(256);
   c->loss_partial = (float*)A.take(sizeof(float) * RED_BLOCKS * L);
+  c->loss_counter = (int*)A.take(256);
   c->head_scratch = (float*)A.take(sizeof(float) * head_scratch_floats(d.max_batch, H));
   c->col_plane = (long long)COL_CHUNKS * (3 * H > F ? 3 * H : F);
   c->col_scratch = (float*)A.take(sizeof(float) * 3 * c->col_plane);
@@ -83,8 +84,6 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->gb_scratch = (float*)A.take(sizeof(float) * c->gb_floats);
   c->gb_n_counters = F / 32 + 2;
   c->gb_counters = (int*)A.take(sizeof(int) * c->gb_n_counters);
-  c->rowbias = (float*)A.take(sizeof(float) * (3 * H > F ? 3 * H : F));
-  c->alt_rowbias = (float*)A.take(sizeof(float) * (3 * H > F ? 3 * H : F));
   c->reduce_per_layer = N_SITES + 1 + N_WMAT;
   c->reduce_table = (ReduceEntry*)A.take(sizeof(ReduceEntry) * c->reduce_per_layer * L);
   c->adam_table = (AdamEntry*)A.take(sizeof(AdamEntry) * (MREM_N_PARAMS + N_WMAT + N_SITES + 1) * L);

@@ -255,7 +255,7 @@ __device__ __forceinline__ float gelu_erf_grad(float u) {
 // ---------------------------------------------------------------- GEMM interface (both back ends)
 enum OutKind : int { OUT_F32 = 0, OUT_BF16 = 1, OUT_I32 = 2 };
 
-// out[b][m][n] = act( alpha * col_scale[n] * acc + col_bias[n] + row_bias[m] + residual[b][m][n] )
+// out[b][m][n] = act( alpha * col_scale[n] * acc + col_bias[n] + row_scale * row_bias[m] + residual[b][m][n] )
 // alpha = alpha_const * (*alpha_p0) * (*alpha_p1)   (null pointers count as 1)
 struct Epilogue {
   void* out;
@@ -269,7 +269,11 @@ struct Epilogue {
   const float* col_scale;      // [N] or null
   const float* col_bias;       // [N] or null
   const float* row_bias;       // [M] or null
+  const float* row_scale;      // one value, or null: 1
 };
+__device__ __forceinline__ float row_term(const Epilogue& e, int row) {
+  return e.row_bias ? (e.row_scale ? *e.row_scale : 1.f) * e.row_bias[row] : 0.f;
+}
 
 // One operand of C[m,n] = sum_k A[m,k] * B[n,k].  `mn_contig` = 1 when the operand is
 // stored with its M (or N) index contiguous and k strided, 0 when k is contiguous.

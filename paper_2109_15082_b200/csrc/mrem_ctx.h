@@ -101,12 +101,10 @@ struct mrem_ctx {
   long long gb_floats = 0;               // (its own: column reductions of the side stream run at the same time)
   int* gb_counters = nullptr;
   int gb_n_counters = 0;
-  float* rowbias;
   // second copy of the backward buffers the side stream reads (layers alternate between the two copies, so the
   // main stream may start the layer below while the side stream still works on this one)
   void *alt_d_y2 = nullptr, *alt_d_sum = nullptr, *alt_d_u = nullptr, *alt_d_a = nullptr, *alt_d_y1 = nullptr, *alt_d_qkv = nullptr;
-  float* alt_rowbias = nullptr;
-  float* loss_partial;
+  float* loss_partial;  int* loss_counter;
   float* head_scratch = nullptr;         // pooled vectors, gradient and per-sequence errors of the output-logit term
   float* minmax;
   int* status;

@@ -37,7 +37,7 @@ struct Epi {                       // shorthand builder of an Epilogue
   Epi& alpha(float a, const float* p0 = nullptr, const float* p1 = nullptr) { e.alpha_const = a; e.alpha_p0 = p0; e.alpha_p1 = p1; return *this; }
   Epi& colscale(const float* p) { e.col_scale = p; return *this; }
   Epi& colbias(const float* p) { e.col_bias = p; return *this; }
-  Epi& rowbias(const float* p) { e.row_bias = p; return *this; }
+  Epi& rowbias(const float* p, const float* scale) { e.row_bias = p; e.row_scale = scale; return *this; }
   Epi& residual(const void* p) { e.residual = p; return *this; }
   Epi& gelu() { e.act = 1; return *this; }
 };
@@ -237,12 +237,10 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
                          b.a_steps[S_A], rx.hi, s.a_q8, s.a_qt, c->dt, c->stream);
     r.gemm_i8(s.a_q8, 0, w[W_1].codes, (int)M, F, H,
               Epi(s.u, ok, F).alpha(1.f, b.a_steps[S_A]).colscale(w[W_1].scale).colbias(b.student[MREM_B1]).e);
-    launch_gelu_quant(s.u, M * F, b.a_steps[S_G], rg.asym ? b.a_off[S_G] : nullptr, rg.lo, rg.hi, s.g_q8, s.g_qt, c->dt, c->stream);
-    const float* bias2 = b.student[MREM_B2];
-    if (rg.asym) {
-      launch_effective_bias(b.student[MREM_B2], b.a_off[S_G], w[W_2].scale, w[W_2].rowsum, w[W_2].beff, H, c->stream);
-      bias2 = w[W_2].beff;
-    }
+    const EffectiveBias eb{b.student[MREM_B2], w[W_2].scale, w[W_2].rowsum, w[W_2].beff, H};
+    launch_gelu_quant(s.u, M * F, b.a_steps[S_G], rg.asym ? b.a_off[S_G] : nullptr, rg.lo, rg.hi, s.g_q8, s.g_qt, c->dt, c->stream,
+                      rg.asym ? &eb : nullptr);
+    const float* bias2 = rg.asym ? w[W_2].beff : b.student[MREM_B2];
     r.gemm_i8(s.g_q8, rg.asym ? 1 : 0, w[W_2].codes, (int)M, H, F,
               Epi(s.y2, ok, H).alpha(1.f, b.a_steps[S_G]).colscale(w[W_2].scale).colbias(bias2).residual(s.a).e);
     if (l + 1 < d.n_layers)
@@ -313,9 +311,9 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
   // Buffers the side stream reads, two copies used by alternate layers: the main stream starts the layer below while
   // the side stream still reduces and multiplies this layer's gradients, and waits (ev_layer) only before it
   // overwrites the copy of the layer two above.
-  struct SideBufs { void *d_y2, *d_sum, *d_u, *d_a, *d_y1, *d_qkv; float* rowbias; };
-  const SideBufs copies[2] = {{c->d_y2, c->d_sum, c->d_u, c->d_a, c->d_y1, c->d_qkv, c->rowbias},
-                              {c->alt_d_y2, c->alt_d_sum, c->alt_d_u, c->alt_d_a, c->alt_d_y1, c->alt_d_qkv, c->alt_rowbias}};
+  struct SideBufs { void *d_y2, *d_sum, *d_u, *d_a, *d_y1, *d_qkv; };
+  const SideBufs copies[2] = {{c->d_y2, c->d_sum, c->d_u, c->d_a, c->d_y1, c->d_qkv},
+                              {c->alt_d_y2, c->alt_d_sum, c->alt_d_u, c->alt_d_a, c->alt_d_y1, c->alt_d_qkv}};
   const void* carry = nullptr;
   // the straight-through passes that feed a LayerNorm's backward run inside it where the row fits its registers
   const bool fuse_ln = layernorm_bwd_ste_supported(H, c->dt);
@@ -359,7 +357,7 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
     {
       Epi e(g.p[MREM_W2], OUT_F32, F);
       e.alpha(1.f, b.a_steps[S_G]);
-      if (rg.asym) { launch_scale_vec(g.p[MREM_B2], b.a_off[S_G], q.rowbias, H, side); e.rowbias(q.rowbias); }
+      if (rg.asym) e.rowbias(g.p[MREM_B2], b.a_off[S_G]);
       rw.defer(view(q.d_y2, H, 1), view(s.g_qt, F, 1), H, F, (int)M, e.e);
     }
     // (the bias gradient of FFN1, the column sums of d_u, rides along where the vector path applies)
@@ -527,8 +525,8 @@ int32_t mrem_recon_loss(mrem_ctx* c, float* loss_total, float* loss_per_layer) {
   if (!c->have_teacher || !c->have_student) return fail(c, MREM_ERR_ORDER, "recon_loss: needs a teacher and a student forward of the same batch");
   const long long n = (long long)c->cur_batch * c->cur_seq * c->d.hidden;
   const float cc = (c->d.loss_mean ? 1.f / (float)n : 1.f) * c->loss_share;
-  launch_loss(c->s_out, c->t_out, c->d.n_layers, n, cc, c->dF, c->loss_partial, c->status, c->dt, c->stream);
-  launch_loss_finalize(c->loss_partial, c->d.n_layers, cc, loss_total, loss_per_layer, c->stream);
+  const LossTotals totals{c->loss_counter, loss_total, loss_per_layer};
+  launch_loss(c->s_out, c->t_out, c->d.n_layers, n, cc, c->dF, c->loss_partial, c->status, c->dt, c->stream, &totals);
   if (c->head.wp) {
     // last module of the model: the output-logit term, its gradient added to the last layer's loss gradient
     const int L = c->d.n_layers, C = c->head.n_classes;
@@ -669,24 +667,22 @@ int32_t mrem_rem_step(mrem_ctx* c, int32_t layer, int32_t tensor_id, const void*
   Epi fe(y, ok, N);
   fe.alpha(1.f, step).colscale(w.scale);
   if (ar.asym) {
-    if (cudaMemsetAsync(c->alt_rowbias, 0, sizeof(float) * N, st) != cudaSuccess) return fail(c, MREM_ERR_CUDA, "rem_step: memset failed");
-    launch_effective_bias(c->alt_rowbias, off, w.scale, w.rowsum, w.beff, N, st);
+    launch_effective_bias(nullptr, off, w.scale, w.rowsum, w.beff, N, st);
     fe.colbias(w.beff);
   }
   r.gemm_i8(q8, ar.asym ? 1 : 0, w.codes, (int)M, N, K, fe.e);
   // loss and its gradient
   const long long n = M * N;
   const float cc = d.loss_mean ? 1.f / (float)n : 1.f;
-  launch_loss(y, target, 1, n, cc, dy, c->loss_partial, c->status, c->dt, st);
-  launch_loss_finalize(c->loss_partial, 1, cc, d_loss, nullptr, st);
+  const LossTotals totals{c->loss_counter, d_loss, nullptr};
+  launch_loss(y, target, 1, n, cc, dy, c->loss_partial, c->status, c->dt, st, &totals);
   // d l / d w_hat = dy^T a_hat, a_hat = step * codes (+ offset: a row bias of offset * column sums of dy)
   Epi we(g.p[tensor_id], OUT_F32, K);
   we.alpha(1.f, step);
   if (ar.asym) {
     launch_col_reduce(dy, N, nullptr, nullptr, nullptr, nullptr, 0, M, N, g.p[bias_id], nullptr, nullptr, c->col_scratch, c->col_plane,
                       c->col_counters, c->dt, st);
-    launch_scale_vec(g.p[bias_id], off, c->rowbias, N, st);
-    we.rowbias(c->rowbias);
+    we.rowbias(g.p[bias_id], off);
   }
   r.gemm(view(dy, N, 1), view(qt, K, 1), N, K, (int)M, 1, 1, we.e);
   // d l / d a_hat = dy w_hat, then the straight-through factors of the input quantizer

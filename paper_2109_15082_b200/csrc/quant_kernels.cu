@@ -151,12 +151,15 @@ template <typename T, int V>
 __global__ void __launch_bounds__(256) gelu_quant_kernel(const T* __restrict__ u, long long n,
                                                          const float* __restrict__ step,
                                                          const float* __restrict__ offset, float lo, float hi,
-                                                         int8_t* __restrict__ q8, T* __restrict__ qt) {
+                                                         int8_t* __restrict__ q8, T* __restrict__ qt,
+                                                         const __grid_constant__ EffectiveBias eb) {
   pdl_wait();
   pdl_trigger();
   const float s = *step, r_s = __frcp_rn(s);
   const bool has_off = offset != nullptr;
   const float off = has_off ? *offset : 0.f;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < eb.n; i += gridDim.x * blockDim.x)
+    eb.beff[i] = eb.b[i] + off * eb.wscale[i] * (float)eb.rowsum[i];
   for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; i < n; i += (long long)gridDim.x * blockDim.x * V) {
     float v[V];
     load_vec<T, V>(u + i, v);
@@ -369,17 +372,18 @@ void launch_mix(const void* f, const void* f_hat, float lam, void* out, long lon
 }
 
 void launch_gelu_quant(const void* u, long long n, const float* step, const float* offset, int lo, int hi,
-                       int8_t* q8, void* qt, int dt, cudaStream_t st) {
+                       int8_t* q8, void* qt, int dt, cudaStream_t st, const EffectiveBias* eb) {
   if (n <= 0) return;
+  const EffectiveBias bias = eb ? *eb : EffectiveBias{nullptr, nullptr, nullptr, nullptr, 0};
   Scope sc("gelu_quant", (double)n * ((dt == 1 ? 2.0 : 4.0) * (qt ? 2 : 1) + (q8 ? 1 : 0)), 0, st);
   if (dt == 1) {
     const bool v = n % 8 == 0 && vec_ok<bf16>(u, 8, 8) && vec_ok<bf16>(qt, 8, 8) && (reinterpret_cast<uintptr_t>(q8) % 8) == 0;
-    if (v) launch_k(gelu_quant_kernel<bf16, 8>, grid_for(n / 8), 256, 0, st, (const bf16*)u, n, step, offset, (float)lo, (float)hi, q8, (bf16*)qt);
-    else launch_k(gelu_quant_kernel<bf16, 1>, grid_for(n), 256, 0, st, (const bf16*)u, n, step, offset, (float)lo, (float)hi, q8, (bf16*)qt);
+    if (v) launch_k(gelu_quant_kernel<bf16, 8>, grid_for(n / 8), 256, 0, st, (const bf16*)u, n, step, offset, (float)lo, (float)hi, q8, (bf16*)qt, bias);
+    else launch_k(gelu_quant_kernel<bf16, 1>, grid_for(n), 256, 0, st, (const bf16*)u, n, step, offset, (float)lo, (float)hi, q8, (bf16*)qt, bias);
   } else {
     const bool v = n % 4 == 0 && vec_ok<float>(u, 4, 4) && vec_ok<float>(qt, 4, 4) && (reinterpret_cast<uintptr_t>(q8) % 4) == 0;
-    if (v) launch_k(gelu_quant_kernel<float, 4>, grid_for(n / 4), 256, 0, st, (const float*)u, n, step, offset, (float)lo, (float)hi, q8, (float*)qt);
-    else launch_k(gelu_quant_kernel<float, 1>, grid_for(n), 256, 0, st, (const float*)u, n, step, offset, (float)lo, (float)hi, q8, (float*)qt);
+    if (v) launch_k(gelu_quant_kernel<float, 4>, grid_for(n / 4), 256, 0, st, (const float*)u, n, step, offset, (float)lo, (float)hi, q8, (float*)qt, bias);
+    else launch_k(gelu_quant_kernel<float, 1>, grid_for(n), 256, 0, st, (const float*)u, n, step, offset, (float)lo, (float)hi, q8, (float*)qt, bias);
   }
 }
 
