@@ -334,10 +334,15 @@ namespace {
 // not hidden.  A step of a narrow tile is cheaper, but far from proportionally (the A tile is re-fetched
 // for every column block and the shared-memory traffic per flop grows), so wide tiles win unless they
 // leave most SMs idle.
-int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count) {
+// `splits` > 1: that many CTAs share each tile's inner dimension (tc_gemm_split_kernel), worth the exchange of partial sums where
+// the tiles are few and the inner dimension is long.  Alone / shared, us: 216 x 768 x 3072 17.0 / 9.5 (int8 codes 10.4 / 7.4),
+// 216 x 768 x 2304 13.5 / 8.6, 512 x 768 x 3072 17.3 / 11.8, 1024 x 1024 x 4096 22.9 / 17.1, 128 x 1024 x 1024 7.8 / 6.9,
+// 216 x 768 x 768 6.7 / 6.3; on the other side of the line 512 x 1024 x 1024 8.2 / 9.2, 1024 x 1024 x 1024 8.5 / 8.8.
+int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count, bool can_split, int* splits) {
   const int m_tiles = (M + BLOCK_M - 1) / BLOCK_M;
   int best = 64;
   double best_cost = 1e30;
+  *splits = 1;
   for (int bn = 64; bn <= 256; bn *= 2) {
     if (bn > 64 && bn / 2 >= N) break;
     const long long tiles = (long long)m_tiles * ((N + bn - 1) / bn) * batches;
@@ -346,6 +351,12 @@ int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count) {
     const double epi_us = bn == 64 ? 0.5 : (bn == 128 ? 1.0 : 2.0);
     const double cost = (double)waves * (k_blocks * step_us + epi_us);
     if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+    for (int s = 2; s <= 4 && can_split && bn <= 128; s *= 2) {
+      if (tiles * s > (s == 2 ? sm_count - 4 : sm_count - 20) || k_blocks < 4 * s) continue;      // all clusters at once
+      const double exchange_us = 1.5 + 0.012 * (double)(tiles * s);
+      const double split_cost = (double)((k_blocks + s - 1) / s) * step_us + epi_us / s + exchange_us;
+      if (split_cost < best_cost - 1e-9) { best_cost = split_cost; best = bn; *splits = s; }
+    }
   }
   return best;
 }
@@ -359,7 +370,9 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
   if (kind == 1 && (A.mn_contig || B.mn_contig)) return GEMM_ERR_ARG;
   TcParams p;
   p.M = g.M; p.N = g.N; p.K = g.K; p.nb0 = g.nb0; p.nb1 = g.nb1;
-  p.block_n = block_n > 0 ? block_n : pick_block_n(g.M, g.N, (g.K + 128 / es - 1) / (128 / es), g.nb0 * g.nb1, sm_count);
+  int splits = 1;
+  p.block_n = block_n > 0 ? block_n : pick_block_n(g.M, g.N, (g.K + 128 / es - 1) / (128 / es), g.nb0 * g.nb1, sm_count,
+                                                   tc_gemm_split_eligible(kind, g, epi), &splits);
   if (p.block_n != 64 && p.block_n != 128 && p.block_n != 256) return GEMM_ERR_ARG;
   p.block_k = 128 / es;
   p.m_tiles = (g.M + BLOCK_M - 1) / BLOCK_M;
@@ -440,6 +453,7 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
              A.mn_contig ? "T" : "N", B.mn_contig ? "N" : "T", g.nb0 * g.nb1);
     return std::string(buf);
   }, 2.0 * g.M * g.N * (double)g.K * g.nb0 * g.nb1, 1, stream, 0);
+  if (splits > 1) return tc_gemm_split_launch(kind, ma, mb, mc, p, splits, stream);
   if (launch_k(kern, grid, GEMM_THREADS, smem, stream, ma, mb, mc, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }
