@@ -216,7 +216,10 @@ __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* 
     }
     if (f.act) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j]);
+      for (int j = 0; j < 32; j += 2) {
+        const float2 t = gelu_erf2(make_float2(v[j], v[j + 1]));
+        v[j] = t.x; v[j + 1] = t.y;
+      }
     }
     uint32_t o[16];
 #pragma unroll

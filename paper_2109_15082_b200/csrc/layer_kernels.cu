@@ -147,6 +147,47 @@ __global__ void __launch_bounds__(256) ste_act_kernel(const T* __restrict__ x, l
 }
 
 // ------------------------------------------------------------------ GELU backward with the STE of its output quantizer
+// d <- d * 1[inside] * gelu'(u) of V elements; their parts of the step and offset gradients go to ds and dofs.  Without an
+// offset `off` is 0 (x - 0 = x).  Bound by instruction issue (73 % busy, DRAM at 25 %): the arithmetic runs on pairs.
+template <typename T, int V>
+__device__ __forceinline__ void gelu_bwd_vec(const float* u, float* d, float s, float r_s, float off, float lo, float hi, int quantized,
+                                             float& ds, float& dofs) {
+  if constexpr (V == 1) {
+    float tail, ex;
+    gelu_parts(u[0], tail, ex);
+    if (quantized) {
+      const float z = quotient(__fsub_rn(stored<T>(gelu_from_tail(u[0], tail)), off), s, r_s);
+      const bool in = z >= lo && z <= hi;
+      ds += d[0] * (rne_magic(fminf(fmaxf(z, lo), hi)) - (in ? z : 0.f));
+      dofs += in ? 0.f : d[0];
+      d[0] = in ? d[0] : 0.f;
+    }
+    d[0] *= gelu_grad_from_parts(u[0], tail, ex);
+  } else {
+    float2 ds2 = splat(0.f), dofs2 = splat(0.f);
+    const float2 neg_s = splat(-s), r2 = splat(r_s), neg_off = splat(-off);
+#pragma unroll
+    for (int j = 0; j < V; j += 2) {
+      const float2 x = make_float2(u[j], u[j + 1]);
+      float2 neg_abs, tail, ex, dv = make_float2(d[j], d[j + 1]);
+      gelu_parts2(x, neg_abs, tail, ex);
+      if (quantized) {
+        const float2 z = quotient2(add2(stored2<T>(gelu_from_tail2(x, neg_abs, tail)), neg_off), neg_s, r2), zc = clamp2(z, lo, hi);
+        const bool in0 = zc.x == z.x, in1 = zc.y == z.y;
+        uint32_t b0, b1;
+        ds2 = fma2(dv, add2(rne_magic2(zc, b0, b1), make_float2(in0 ? -z.x : 0.f, in1 ? -z.y : 0.f)), ds2);
+        const float2 pass = make_float2(in0 ? dv.x : 0.f, in1 ? dv.y : 0.f);
+        dofs2 = add2(dofs2, fma2(pass, splat(-1.f), dv));
+        dv = pass;
+      }
+      dv = mul2(dv, gelu_grad_from_parts2(x, tail, ex));
+      d[j] = dv.x; d[j + 1] = dv.y;
+    }
+    ds += ds2.x + ds2.y;
+    dofs += dofs2.x + dofs2.y;
+  }
+}
+
 template <typename T, int V>
 __global__ void __launch_bounds__(256) gelu_bwd_kernel(const T* __restrict__ u, const T* __restrict__ dghat,
                                                        T* __restrict__ du, long long n,
@@ -158,26 +199,13 @@ __global__ void __launch_bounds__(256) gelu_bwd_kernel(const T* __restrict__ u, 
   pdl_trigger();
   __shared__ float sh[32];
   const float s = quantized ? *step : 1.f, r_s = __frcp_rn(s);
-  const bool has_off = offset != nullptr;
-  const float off = has_off ? *offset : 0.f;
+  const float off = offset ? *offset : 0.f;
   float ds = 0.f, dofs = 0.f;
   for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; i < n; i += (long long)gridDim.x * blockDim.x * V) {
     float uv[V], d[V];
     load_vec<T, V>(u + i, uv);
     load_vec<T, V>(dghat + i, d);
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-      float tail, ex;
-      gelu_parts(uv[j], tail, ex);
-      if (quantized) {
-        const float z = qz(stored<T>(gelu_from_tail(uv[j], tail)), s, r_s, off, has_off);
-        const bool in = z >= lo && z <= hi;
-        ds += d[j] * (rne_magic(fminf(fmaxf(z, lo), hi)) - (in ? z : 0.f));
-        dofs += in ? 0.f : d[j];
-        d[j] = in ? d[j] : 0.f;
-      }
-      d[j] *= gelu_grad_from_parts(uv[j], tail, ex);
-    }
+    gelu_bwd_vec<T, V>(uv, d, s, r_s, off, lo, hi, quantized, ds, dofs);
     store_vec<T, V>(du + i, d);
   }
   ds = block_sum(ds, sh);
@@ -194,6 +222,8 @@ __global__ void __launch_bounds__(256) gelu_bwd_kernel(const T* __restrict__ u, 
 // its rows in row order, the block adds its 16 row lanes in index order, and the last block to finish a column group
 // (ticket counter) adds the chunks' partials in index order, so the sums do not depend on scheduling.  Block b = y *
 // gridDim.x + x leaves its partial step / offset gradient in slot b; slots from the grid size up to n_slots are zeroed.
+// 4096 x 4096: 34 -> 33 us on pairs, -> 30 with the next row's operands fetched ahead and one wave of blocks instead of two
+// (4096 x 3072: 26 -> 24 for the last); 15 us is its traffic.
 constexpr int GB_TX = 16, GB_TY = 16;
 template <typename T, int V>
 __global__ void __launch_bounds__(256) gelu_bwd_colsum_kernel(const T* __restrict__ u, const T* __restrict__ dghat,
@@ -211,8 +241,7 @@ __global__ void __launch_bounds__(256) gelu_bwd_colsum_kernel(const T* __restric
   __shared__ float cs[GB_TY][BC + 1];
   __shared__ int is_last;
   const float s = quantized ? *step : 1.f, r_s = __frcp_rn(s);
-  const bool has_off = offset != nullptr;
-  const float off = has_off ? *offset : 0.f;
+  const float off = offset ? *offset : 0.f;
   const int tx = threadIdx.x % GB_TX, ty = threadIdx.x / GB_TX;
   const int c = blockIdx.x * BC + tx * V;
   const int chunks = gridDim.y;
@@ -223,24 +252,21 @@ __global__ void __launch_bounds__(256) gelu_bwd_colsum_kernel(const T* __restric
   for (int j = 0; j < V; ++j) acc[j] = 0.f;
   float ds = 0.f, dofs = 0.f;
   if (c < cols) {
+    // the next row's operands are on their way while this one's are worked on
+    uint32_t un[RawWords<T, V>::N], dn[RawWords<T, V>::N];
+    if (r0 + ty < r1) { load_raw<T, V>(u + (r0 + ty) * cols + c, un); load_raw<T, V>(dghat + (r0 + ty) * cols + c, dn); }
+#pragma unroll 1
     for (long long r = r0 + ty; r < r1; r += GB_TY) {
       const long long i = r * cols + c;
       float uv[V], d[V];
-      load_vec<T, V>(u + i, uv);
-      load_vec<T, V>(dghat + i, d);
+      widen_raw<T, V>(un, uv);
+      widen_raw<T, V>(dn, d);
+      if (r + GB_TY < r1) { load_raw<T, V>(u + i + GB_TY * cols, un); load_raw<T, V>(dghat + i + GB_TY * cols, dn); }
+      gelu_bwd_vec<T, V>(uv, d, s, r_s, off, lo, hi, quantized, ds, dofs);
 #pragma unroll
-      for (int j = 0; j < V; ++j) {
-        float tail, ex;
-        gelu_parts(uv[j], tail, ex);
-        if (quantized) {
-          const float z = qz(stored<T>(gelu_from_tail(uv[j], tail)), s, r_s, off, has_off);
-          const bool in = z >= lo && z <= hi;
-          ds += d[j] * (rne_magic(fminf(fmaxf(z, lo), hi)) - (in ? z : 0.f));
-          dofs += in ? 0.f : d[j];
-          d[j] = in ? d[j] : 0.f;
-        }
-        d[j] *= gelu_grad_from_parts(uv[j], tail, ex);
-        acc[j] += d[j];
+      for (int j = 0; j < V; j += 2) {
+        const float2 t = add2(make_float2(acc[j], acc[j + 1]), make_float2(d[j], d[j + 1]));
+        acc[j] = t.x; acc[j + 1] = t.y;
       }
       store_vec<T, V>(du + i, d);
     }
@@ -426,7 +452,7 @@ bool launch_gelu_bwd_colsum(const void* u, const void* dghat, void* du, long lon
     constexpr int V = 16 / (int)sizeof(T);
     constexpr int BC = GB_TX * V;
     const int col_blocks = (cols + BC - 1) / BC;
-    long long chunks = RED_BLOCKS / col_blocks;                       // the grid fills the RED_BLOCKS partial-sum slots
+    long long chunks = RED_BLOCKS / 2 / col_blocks;                   // one wave of four blocks per SM
     if (chunks > (rows + GB_TY - 1) / GB_TY) chunks = (rows + GB_TY - 1) / GB_TY;
     if (chunks > scratch_floats / cols) chunks = scratch_floats / cols;
     if (cols % V == 0 && al16(u) && al16(dghat) && al16(du) && chunks >= 1 && col_blocks <= n_counters && col_blocks <= RED_BLOCKS) {

@@ -87,6 +87,10 @@ template <> __device__ __forceinline__ bf16 from_f<bf16>(float v) { return __flo
 
 // value of v after a round trip through storage type T
 template <typename T> __device__ __forceinline__ float stored(float v) { return to_f<T>(from_f<T>(v)); }
+template <typename T> __device__ __forceinline__ float2 stored2(float2 v) {
+  if constexpr (sizeof(T) == 4) return v;
+  else return __bfloat1622float2(__floats2bfloat162_rn(v.x, v.y));
+}
 
 // ---------------------------------------------------------------- reductions
 __device__ __forceinline__ float warp_sum(float v) {
@@ -203,7 +207,7 @@ __device__ __forceinline__ float code_f(float n, float s, float r_s, float lo, f
   float zc = fminf(fmaxf(__fmaf_rn(__fmaf_rn(-z0, s, n), r_s, z0), lo), hi);
   float q = rne_magic(zc, bits);
   if constexpr (!EXACT_QUOTIENT) {
-    if (fabsf(fabsf(zc - q) - 0.5f) < HALF_WINDOW) {
+    if (fabsf(zc - q) > 0.5f - HALF_WINDOW) {
       zc = fminf(fmaxf(__fdiv_rn(n, s), lo), hi);
       q = rne_magic(zc, bits);
     }
@@ -217,6 +221,51 @@ __device__ __forceinline__ int code_of(float n, float s, float r_s, float lo, fl
 // low bytes of four words -> one word (byte i from b_i)
 __device__ __forceinline__ uint32_t pack_low_bytes(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
   return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+}
+
+__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 clamp2(float2 z, float lo, float hi) { return make_float2(fminf(fmaxf(z.x, lo), hi), fminf(fmaxf(z.y, lo), hi)); }
+// quotient() of two: neg_s = -s, r_s = RN(1 / s)
+__device__ __forceinline__ float2 quotient2(float2 x, float2 neg_s, float2 r_s) {
+  const float2 z0 = mul2(x, r_s);
+  return fma2(fma2(z0, neg_s, x), r_s, z0);
+}
+__device__ __forceinline__ float2 rne_magic2(float2 z, uint32_t& b0, uint32_t& b1) {
+  const float2 t = add2(z, splat(ROUND_MAGIC));
+  b0 = __float_as_uint(t.x);
+  b1 = __float_as_uint(t.y);
+  return add2(t, splat(-ROUND_MAGIC));
+}
+static __device__ __noinline__ float exact_quotient(float x, float s) { return __fdiv_rn(x, s); }      // rare: kept out of line
+// code_f of N (even) numerators, in place, with one look at the half-integers for all of them.
+template <bool EXACT_QUOTIENT, int N>
+__device__ __forceinline__ void codes_f(float* n, float s, float r_s, float lo, float hi, uint32_t* bits) {
+  const float2 neg_s = splat(-s), r2 = splat(r_s);
+  float2 q[N / 2];
+  float off_center = 0.f;
+#pragma unroll
+  for (int j = 0; j < N / 2; ++j) {
+    const float2 x = make_float2(n[2 * j], n[2 * j + 1]), z0 = clamp2(mul2(x, r2), lo - 1.f, hi + 1.f);
+    const float2 z = clamp2(fma2(fma2(z0, neg_s, x), r2, z0), lo, hi);
+    q[j] = rne_magic2(z, bits[2 * j], bits[2 * j + 1]);
+    if (!EXACT_QUOTIENT) {
+      const float2 e = fma2(q[j], splat(-1.f), z);
+      off_center = fmaxf(off_center, fmaxf(fabsf(e.x), fabsf(e.y)));
+    }
+  }
+  if (!EXACT_QUOTIENT && off_center > 0.5f - HALF_WINDOW) {
+#pragma unroll
+    for (int j = 0; j < N / 2; ++j)
+      q[j] = rne_magic2(clamp2(make_float2(exact_quotient(n[2 * j], s), exact_quotient(n[2 * j + 1], s)), lo, hi), bits[2 * j], bits[2 * j + 1]);
+  }
+#pragma unroll
+  for (int j = 0; j < N / 2; ++j) { n[2 * j] = q[j].x; n[2 * j + 1] = q[j].y; }
+}
+
+template <bool EXACT_QUOTIENT, int N>
+__device__ __forceinline__ void codes_of(float* n, float s, float r_s, float lo, float hi, uint32_t* bits) {      // one or an even number
+  if constexpr (N == 1) n[0] = code_f<EXACT_QUOTIENT>(n[0], s, r_s, lo, hi, bits[0]);
+  else codes_f<EXACT_QUOTIENT, N>(n, s, r_s, lo, hi, bits);
 }
 
 // GELU(u) = u * Phi(u) with the erf form.  erf(x) = 1 - (a1 t + ... + a5 t^5) exp(-x^2), t = 1/(1 + p x), x >= 0
@@ -245,6 +294,30 @@ __device__ __forceinline__ float gelu_erf(float u) {
 __device__ __forceinline__ float gelu_grad_from_parts(float u, float tail, float ex) {
   const float cdf = u >= 0.f ? 1.f - tail : tail;
   return fmaf(u, ex * 0.39894228040143268f, cdf);             // exp(-u^2/2) / sqrt(2 pi)
+}
+// The same of two values, operation by operation (neg_abs = -|u|).
+__device__ __forceinline__ void gelu_parts2(float2 u, float2& neg_abs, float2& tail, float2& ex) {
+  neg_abs = make_float2(-fabsf(u.x), -fabsf(u.y));
+  const float2 a = mul2(mul2(u, u), splat(-0.72134752044448170f));
+  ex = make_float2(exp2_approx(a.x), exp2_approx(a.y));
+  const float2 den = fma2(splat(-0.23164189f), neg_abs, splat(1.f)), t = make_float2(rcp_approx(den.x), rcp_approx(den.y));
+  float2 poly = fma2(splat(0.5307027145f), t, splat(-0.7265760135f));
+  poly = fma2(poly, t, splat(0.7107068705f));
+  poly = fma2(poly, t, splat(-0.142248368f));
+  poly = fma2(poly, t, splat(0.127414796f));
+  tail = mul2(mul2(poly, t), ex);
+}
+__device__ __forceinline__ float2 gelu_from_tail2(float2 u, float2 neg_abs, float2 tail) {
+  return fma2(neg_abs, tail, make_float2(fmaxf(u.x, 0.f), fmaxf(u.y, 0.f)));
+}
+__device__ __forceinline__ float2 gelu_erf2(float2 u) {
+  float2 neg_abs, tail, ex;
+  gelu_parts2(u, neg_abs, tail, ex);
+  return gelu_from_tail2(u, neg_abs, tail);
+}
+__device__ __forceinline__ float2 gelu_grad_from_parts2(float2 u, float2 tail, float2 ex) {
+  const float2 upper = fma2(tail, splat(-1.f), splat(1.f));
+  return fma2(u, mul2(ex, splat(0.39894228040143268f)), make_float2(u.x >= 0.f ? upper.x : tail.x, u.y >= 0.f ? upper.y : tail.y));
 }
 __device__ __forceinline__ float gelu_erf_grad(float u) {
   float tail, ex;

@@ -114,7 +114,8 @@ __global__ void __launch_bounds__(128) ln_fwd_kernel(const T* __restrict__ y, co
     if (step) {
       uint32_t b[V];
 #pragma unroll
-      for (int j = 0; j < V; ++j) o[j] = code_f<sizeof(T) == 2>(stored<T>(o[j]), s, r_s, -qmax, qmax, b[j]);   // bfloat16-valued numerators are exact
+      for (int j = 0; j < V; ++j) o[j] = stored<T>(o[j]);
+      codes_of<sizeof(T) == 2, V>(o, s, r_s, -qmax, qmax, b);                   // bfloat16-valued numerators are exact
       if (q8) store_code_bytes<V>(q8 + row * cols + c, b);
       if (qt) store_vec<T, V>(qt + row * cols + c, o);
     }

@@ -33,21 +33,13 @@ __device__ __forceinline__ void store_what4<bf16>(bf16* p, float a, float b, flo
 
 // Pairs of weights: the arithmetic below is the scalar one of optim.cuh and code_f, two elements per instruction where the
 // hardware has the form.
-__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float2 quotient2(float2 x, float2 neg_s, float2 r_s) {        // quotient() of both
-  const float2 z0 = mul2(x, r_s);
-  return fma2(fma2(z0, neg_s, x), r_s, z0);
-}
-__device__ __forceinline__ float2 clamp2(float2 z, float b) {
-  return make_float2(fminf(fmaxf(z.x, -b), b), fminf(fmaxf(z.y, -b), b));
-}
 // The step gradient's terms of two elements (step_grad_acc), and which gradients pass.
 template <int GRID>
 __device__ __forceinline__ float2 step_grad2(float2 acc, float2 w, float2 d, float2 neg_s, float2 r_s, float qmax, bool& in0, bool& in1) {
   const float2 z = quotient2(w, neg_s, r_s);
   float2 level;
   if (GRID == 0) {
-    const float2 zc = clamp2(z, qmax);
+    const float2 zc = clamp2(z, -qmax, qmax);
     in0 = zc.x == z.x; in1 = zc.y == z.y;
     level = add2(add2(zc, splat(RINT_MAGIC)), splat(-RINT_MAGIC));
   } else {                                                     // clamp(floor(z), -2, 1) + 0.5 without the conversion unit
@@ -58,7 +50,6 @@ __device__ __forceinline__ float2 step_grad2(float2 acc, float2 w, float2 d, flo
   const float2 inside = make_float2(in0 ? -z.x : 0.f, in1 ? -z.y : 0.f);
   return fma2(d, add2(level, inside), acc);
 }
-__device__ __noinline__ float exact_quotient(float x, float s) { return __fdiv_rn(x, s); }      // rare: kept out of line
 struct Adam2 { float2 b1, ob1, b2, ob2, rsq, eps, neg_lr, decay; };
 __device__ __forceinline__ float2 adam2(float2 p, float2 g, float2& m, float2& v, const Adam2& a) {      // adam_one of both
   m = fma2(a.b1, m, mul2(a.ob1, g));
@@ -165,7 +156,7 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
   const float s_new = train_s ? adam_one(s_old, ds, ms, vs, o, 0.f, 1e-8f) : s_old;
   const float sc_new = GRID == 0 ? s_new : 0.5f * s_new;
   // 3 + 4. weights, then their new codes
-  const float2 ns_new = splat(-s_new), r_new = splat(__frcp_rn(s_new));
+  const float2 r_new = splat(__frcp_rn(s_new));
   const Adam2 ad = {splat(o.beta1), splat(__fsub_rn(1.f, o.beta1)), splat(o.beta2), splat(__fsub_rn(1.f, o.beta2)),
                     splat(o.rsqrt_bc2), splat(o.eps), splat(-o.lr_bc1), splat(__fsub_rn(1.f, __fmul_rn(o.lr, o.weight_decay)))};
   float2 sum2 = splat(0.f);                                    // codes are whole numbers: exact in any order
@@ -181,26 +172,12 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
     }
     float2 fa, fb;
     uint32_t b0, b1, b2, b3;
-    if (GRID == 0) {      // the exact code without the division instruction (code_f), one look at the half-integers for all four
-      auto code_quotient = [&](float2 x) {                     // (a first product that overflows ends on its sign's bound)
-        const float2 z0 = clamp2(mul2(x, r_new), qmax + 1.f);
-        return clamp2(fma2(fma2(z0, ns_new, x), r_new, z0), qmax);
-      };
-      float2 za = code_quotient(wa), zb = code_quotient(wb);
-      auto round2 = [&]() {
-        const float2 ta = add2(za, splat(ROUND_MAGIC)), tb = add2(zb, splat(ROUND_MAGIC));
-        fa = add2(ta, splat(-ROUND_MAGIC)); fb = add2(tb, splat(-ROUND_MAGIC));
-        b0 = __float_as_uint(ta.x); b1 = __float_as_uint(ta.y); b2 = __float_as_uint(tb.x); b3 = __float_as_uint(tb.y);
-      };
-      round2();
-      const float2 ea = fma2(fa, splat(-1.f), za), eb = fma2(fb, splat(-1.f), zb);
-      const float near = fminf(fminf(fabsf(fabsf(ea.x) - 0.5f), fabsf(fabsf(ea.y) - 0.5f)),
-                               fminf(fabsf(fabsf(eb.x) - 0.5f), fabsf(fabsf(eb.y) - 0.5f)));
-      if (near < HALF_WINDOW) {
-        za = clamp2(make_float2(exact_quotient(wa.x, s_new), exact_quotient(wa.y, s_new)), qmax);
-        zb = clamp2(make_float2(exact_quotient(wb.x, s_new), exact_quotient(wb.y, s_new)), qmax);
-        round2();
-      }
+    if (GRID == 0) {
+      float q[4] = {wa.x, wa.y, wb.x, wb.y};
+      uint32_t bits[4];
+      codes_f<false, 4>(q, s_new, r_new.x, -qmax, qmax, bits);
+      fa = make_float2(q[0], q[1]); fb = make_float2(q[2], q[3]);
+      b0 = bits[0]; b1 = bits[1]; b2 = bits[2]; b3 = bits[3];
     } else {
       // 2 clamp(floor(w / s), -2, 1) + 1: a quotient of floats rounds to 1 or more exactly when w >= s, and to less than -1
       // exactly when -w > s (the neighbours of s are further than half an ulp of 1 away from it, relatively)
