@@ -181,6 +181,7 @@ __device__ __forceinline__ void fetch_res_bf16(const Epilogue& e, long long off,
 template <int KIND, int OUT, int MODE>
 __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* r, const uint32_t* res, float alpha, float rb,
                                              const float* cv, long long off, bool row_ok, const StoreCtx& sx, int n) {
+  constexpr bool ROW_BIAS = MODE < 0 || (MODE & 16) != 0;      // (epilogue_mode: the bf16 variants have none)
   if (OUT == OUT_I32) {
     if (row_ok) {
       int* out = reinterpret_cast<int*>(e.out) + off;
@@ -192,26 +193,31 @@ __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* 
   const EpiFlags<MODE> f(e);
   float v[32];
 #pragma unroll
-  for (int j = 0; j < 32; j += 4) {
-    float4 sc = make_float4(alpha, alpha, alpha, alpha), bi = make_float4(rb, rb, rb, rb);
+  for (int j = 0; j < 32; j += 4) {                            // pairs: the epilogue's warps are few and their instructions count
+    float4 sc = make_float4(alpha, alpha, alpha, alpha);
     if (f.scale) sc = *reinterpret_cast<const float4*>(cv + j);
+    float2 a = make_float2((KIND == 1) ? (float)(int)r[j] : __uint_as_float(r[j]), (KIND == 1) ? (float)(int)r[j + 1] : __uint_as_float(r[j + 1]));
+    float2 b = make_float2((KIND == 1) ? (float)(int)r[j + 2] : __uint_as_float(r[j + 2]), (KIND == 1) ? (float)(int)r[j + 3] : __uint_as_float(r[j + 3]));
+    const float2 sa = make_float2(sc.x, sc.y), sb = make_float2(sc.z, sc.w);
     if (f.bias) {
       const float4 t = *reinterpret_cast<const float4*>(cv + COLVEC + j);
-      bi.x += t.x; bi.y += t.y; bi.z += t.z; bi.w += t.w;
+      float2 ta = make_float2(t.x, t.y), tb = make_float2(t.z, t.w);
+      if (ROW_BIAS) { ta = add2(ta, splat(rb)); tb = add2(tb, splat(rb)); }
+      a = fma2(a, sa, ta); b = fma2(b, sb, tb);
+    } else if (ROW_BIAS) {
+      a = fma2(a, sa, splat(rb)); b = fma2(b, sb, splat(rb));
+    } else {
+      a = mul2(a, sa); b = mul2(b, sb);
     }
-    const float a0 = (KIND == 1) ? (float)(int)r[j] : __uint_as_float(r[j]);
-    const float a1 = (KIND == 1) ? (float)(int)r[j + 1] : __uint_as_float(r[j + 1]);
-    const float a2 = (KIND == 1) ? (float)(int)r[j + 2] : __uint_as_float(r[j + 2]);
-    const float a3 = (KIND == 1) ? (float)(int)r[j + 3] : __uint_as_float(r[j + 3]);
-    v[j] = a0 * sc.x + bi.x; v[j + 1] = a1 * sc.y + bi.y; v[j + 2] = a2 * sc.z + bi.z; v[j + 3] = a3 * sc.w + bi.w;
+    v[j] = a.x; v[j + 1] = a.y; v[j + 2] = b.x; v[j + 3] = b.y;
   }
   if (OUT == OUT_BF16) {
     if (f.res) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&res[j]));
-        v[2 * j] += t.x;
-        v[2 * j + 1] += t.y;
+        const float2 t = add2(make_float2(v[2 * j], v[2 * j + 1]), __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&res[j])));
+        v[2 * j] = t.x;
+        v[2 * j + 1] = t.y;
       }
     }
     if (f.act) {
@@ -336,12 +342,12 @@ __device__ __forceinline__ void drain_dispatch(const Epilogue& e, uint32_t taddr
 
 // The epilogue variant a launch takes: bf16 outputs with one of the term sets the encoder uses, and plain fp32
 // outputs (the weight gradients), get a kernel compiled for exactly those terms (bit 0 column scale, bit 1
-// column bias, bit 2 residual, bit 3 GELU, bit 4 fp32 output; alpha and the row bias are always applied);
+// column bias, bit 2 residual, bit 3 GELU, bit 4 fp32 output; alpha is always applied, the row bias with bit 4);
 // everything else runs the variant that reads them at run time (-1).
 inline int epilogue_mode(int kind, const Epilogue& e) {
   const int mode = (e.col_scale ? 1 : 0) | (e.col_bias ? 2 : 0) | (e.residual ? 4 : 0) | (e.act == 1 ? 8 : 0);
   if (e.out_kind == OUT_F32) return (kind == 0 && mode == 0) ? 16 : -1;
-  if (e.out_kind != OUT_BF16) return -1;
+  if (e.out_kind != OUT_BF16 || e.row_bias) return -1;
   if (kind == 0) return (mode == 0 || mode == 2 || mode == 6 || mode == 10) ? mode : -1;
   return (mode == 3 || mode == 7) ? mode : -1;
 }
