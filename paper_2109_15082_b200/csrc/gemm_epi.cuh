@@ -349,7 +349,7 @@ inline int epilogue_mode(int kind, const Epilogue& e) {
   if (e.out_kind == OUT_F32) return (kind == 0 && mode == 0) ? 16 : -1;
   if (e.out_kind != OUT_BF16 || e.row_bias) return -1;
   if (kind == 0) return (mode == 0 || mode == 2 || mode == 6 || mode == 10) ? mode : -1;
-  return (mode == 3 || mode == 7) ? mode : -1;
+  return (mode == 1 || mode == 3 || mode == 7) ? mode : -1;
 }
 
 // True when rows of out (and residual) start on 32-byte boundaries for every row, batch and 32-column chunk,

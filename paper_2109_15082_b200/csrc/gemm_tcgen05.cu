@@ -433,7 +433,7 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
   typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
   static const struct { int kind, mode; Kern fn; } variants[] = {
       {0, -1, tc_gemm_kernel<0, -1>}, {0, 0, tc_gemm_kernel<0, 0>}, {0, 2, tc_gemm_kernel<0, 2>}, {0, 6, tc_gemm_kernel<0, 6>},
-      {0, 10, tc_gemm_kernel<0, 10>}, {0, 16, tc_gemm_kernel<0, 16>}, {1, -1, tc_gemm_kernel<1, -1>}, {1, 3, tc_gemm_kernel<1, 3>}, {1, 7, tc_gemm_kernel<1, 7>}};
+      {0, 10, tc_gemm_kernel<0, 10>}, {0, 16, tc_gemm_kernel<0, 16>}, {1, -1, tc_gemm_kernel<1, -1>}, {1, 1, tc_gemm_kernel<1, 1>}, {1, 3, tc_gemm_kernel<1, 3>}, {1, 7, tc_gemm_kernel<1, 7>}};
   constexpr int n_variants = sizeof(variants) / sizeof(variants[0]);
   static bool attr_set[n_variants] = {};
   const int mode = epilogue_mode(kind, epi);

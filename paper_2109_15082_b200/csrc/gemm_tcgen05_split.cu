@@ -230,7 +230,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
 typedef void (*SplitKern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams, int);
 const struct { int kind, mode; SplitKern fn; } kVariants[] = {
     {0, 0, tc_gemm_split_kernel<0, 0>}, {0, 2, tc_gemm_split_kernel<0, 2>}, {0, 6, tc_gemm_split_kernel<0, 6>},
-    {0, 10, tc_gemm_split_kernel<0, 10>}, {0, 16, tc_gemm_split_kernel<0, 16>}, {1, -1, tc_gemm_split_kernel<1, -1>}, {1, 3, tc_gemm_split_kernel<1, 3>}, {1, 7, tc_gemm_split_kernel<1, 7>}};
+    {0, 10, tc_gemm_split_kernel<0, 10>}, {0, 16, tc_gemm_split_kernel<0, 16>}, {1, -1, tc_gemm_split_kernel<1, -1>}, {1, 1, tc_gemm_split_kernel<1, 1>}, {1, 3, tc_gemm_split_kernel<1, 3>}, {1, 7, tc_gemm_split_kernel<1, 7>}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 constexpr int SPLIT_STAGES = 6;
 

@@ -88,7 +88,6 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->reduce_table = (ReduceEntry*)A.take(sizeof(ReduceEntry) * c->reduce_per_layer * L);
   c->adam_table = (AdamEntry*)A.take(sizeof(AdamEntry) * (MREM_N_PARAMS + N_WMAT + N_SITES + 1) * L);
   c->adam_rest = (AdamEntry*)A.take(sizeof(AdamEntry) * (MREM_N_PARAMS + N_WMAT + N_SITES + 1) * L);
-  c->rem_table = (AdamEntry*)A.take(sizeof(AdamEntry) * 2);
   c->h2d_xt = A.take(M * H * es);
   c->h2d_xs = A.take(M * H * es);
   c->h2d_len = (int32_t*)A.take(sizeof(int32_t) * d.max_batch);
@@ -173,6 +172,7 @@ int build_tables(mrem_ctx* c) {
   const int L = d.n_layers;
   std::vector<ReduceEntry> red;
   std::vector<AdamEntry> adam, rest;
+  c->rest_site.assign((size_t)L * (N_SITES + 1), 0);
   for (int l = 0; l < L; ++l) {
     LayerStash& s = c->stash[l];
     LayerGrad& g = c->grad[l];
@@ -215,6 +215,7 @@ int build_tables(mrem_ctx* c) {
       for (AdamEntry& r : rest) if (r.g == grad) e = &r;
       if (!e) { rest.push_back({nullptr, grad, nullptr, nullptr, 0, 0.f, 0.f}); e = &rest.back(); }
       e->part = s.part + site * RED_BLOCKS;
+      c->rest_site[(size_t)l * (N_SITES + 1) + site] = (int)(e - rest.data());
     }
   }
   if (cudaMemcpyAsync(c->reduce_table, red.data(), sizeof(ReduceEntry) * red.size(), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
