@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
   const float s_new = train_s ? adam_one(s_old, ds, ms, vs, o, 0.f, 1e-8f) : s_old;
   const float sc_new = GRID == 0 ? s_new : 0.5f * s_new;
   // 3 + 4. weights, then their new codes
-  const float2 r_new = splat(__frcp_rn(s_new));
+  const float2 ns_new = splat(-s_new), r_new = splat(__frcp_rn(s_new));
   const Adam2 ad = {splat(o.beta1), splat(__fsub_rn(1.f, o.beta1)), splat(o.beta2), splat(__fsub_rn(1.f, o.beta2)),
                     splat(o.rsqrt_bc2), splat(o.eps), splat(-o.lr_bc1), splat(__fsub_rn(1.f, __fmul_rn(o.lr, o.weight_decay)))};
   float2 sum2 = splat(0.f);                                    // codes are whole numbers: exact in any order
@@ -172,12 +172,19 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
     }
     float2 fa, fb;
     uint32_t b0, b1, b2, b3;
-    if (GRID == 0) {
-      float q[4] = {wa.x, wa.y, wb.x, wb.y};
-      uint32_t bits[4];
-      codes_f<false, 4>(q, s_new, r_new.x, -qmax, qmax, bits);
-      fa = make_float2(q[0], q[1]); fb = make_float2(q[2], q[3]);
-      b0 = bits[0]; b1 = bits[1]; b2 = bits[2]; b3 = bits[3];
+    if (GRID == 0) {      // codes_f, written out: as a call the loads of a row were scheduled worse (30522 x 1024 table, step 205 -> 232 us)
+      auto code_quotient = [&](float2 x) {                     // (a first product that overflows ends on its sign's bound)
+        const float2 z0 = clamp2(mul2(x, r_new), -qmax - 1.f, qmax + 1.f);
+        return clamp2(fma2(fma2(z0, ns_new, x), r_new, z0), -qmax, qmax);
+      };
+      float2 za = code_quotient(wa), zb = code_quotient(wb);
+      fa = rne_magic2(za, b0, b1); fb = rne_magic2(zb, b2, b3);
+      const float2 ea = fma2(fa, splat(-1.f), za), eb = fma2(fb, splat(-1.f), zb);
+      if (fmaxf(fmaxf(fabsf(ea.x), fabsf(ea.y)), fmaxf(fabsf(eb.x), fabsf(eb.y))) > 0.5f - HALF_WINDOW) {
+        za = clamp2(make_float2(exact_quotient(wa.x, s_new), exact_quotient(wa.y, s_new)), -qmax, qmax);
+        zb = clamp2(make_float2(exact_quotient(wb.x, s_new), exact_quotient(wb.y, s_new)), -qmax, qmax);
+        fa = rne_magic2(za, b0, b1); fb = rne_magic2(zb, b2, b3);
+      }
     } else {
       // 2 clamp(floor(w / s), -2, 1) + 1: a quotient of floats rounds to 1 or more exactly when w >= s, and to less than -1
       // exactly when -w > s (the neighbours of s are further than half an ulp of 1 away from it, relatively)
