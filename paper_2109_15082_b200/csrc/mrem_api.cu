@@ -409,13 +409,14 @@ int32_t mrem_get_activation(mrem_ctx* c, int32_t role, int32_t layer, int32_t wh
     if (which >= 0 && which < MREM_ACT_COUNT) p = t[which];
   } else if (role == MREM_STUDENT) {
     if (!c->have_student) return fail(c, MREM_ERR_ORDER, "get_activation: no student pass to read");
-    LayerStash& s = c->stash[layer];
-    if (which == MREM_ACT_P && !s.p_kept) {            // formed again with the forward pass's own scale, lengths and arithmetic
+    const LayerStash& s = c->stash[layer];
+    // formed again with the forward pass's own scale, lengths and arithmetic (the codes are not: the backward pass goes on
+    // forming both itself)
+    if (which == MREM_ACT_P && !s.p_kept) {
       const int H = c->d.hidden;
       if (launch_attention_fwd(s.qkv_qt, c->cur_batch, c->cur_seq, c->d.n_heads, H, s.p_len, 1.f, s.p_alpha, nullptr, nullptr, nullptr, nullptr,
                                0, 0, s.P, nullptr, nullptr, nullptr, 0, nullptr, nullptr, c->status, c->stream) != GEMM_OK)
         return fail(c, MREM_ERR_CUDA, "get_activation: launch failed");
-      s.p_kept = true;
     }
     const void* t[MREM_ACT_COUNT] = {s.qkv, s.P, s.ctx, s.y1, s.a, s.u, s.y2};
     if (which >= 0 && which < MREM_ACT_COUNT) p = t[which];

@@ -43,3 +43,28 @@ def test_attention_at_the_edges_of_its_tiles(seq, lens):
             assert not a[i, :, :, n:].any() and torch.allclose(a[i].float().sum(-1), torch.ones((), device=m.device), atol=2 ** -8 * 2)
     finally:
         p.close()
+
+
+# one kernel, two kernels
+@pytest.mark.parametrize("seq", [72, 200])
+def test_reading_the_probabilities_leaves_the_backward_pass_alone(seq):
+    """The fused path forms the probabilities when they are read, without their codes: the gradients that follow are the same bits."""
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=2)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002)
+    try:
+        m = p.m
+
+        def gradient(read):
+            m.quantize_weights()
+            m.forward_teacher(p.xd, p.vld, wl.batch, seq)
+            m.forward_student(p.xd, p.vld, wl.batch, seq)
+            if read:
+                m.activation(B.STUDENT, 0, B.ACT_P, (wl.batch, wl.n_heads, seq, seq))
+            m.recon_loss()
+            m.backward()
+            return m.grad(0, B.WQKV, (3 * wl.hidden, wl.hidden)).clone()
+
+        a = gradient(False)
+        assert a.any() and torch.equal(a, gradient(True))
+    finally:
+        p.close()
