@@ -376,6 +376,44 @@ def test_graph_replay_and_host_step_equal_eager():
     assert results[0][0][2] != results[0][0][0]
 
 
+@pytest.mark.parametrize("lam", [0.35, 1.0])
+def test_teacher_forced_graph_replay_and_host_step_equal_eager(lam):
+    """The captured step runs the two forward passes side by side under teacher forcing too: the bits of the eager sequence."""
+    wl, kw = CASES["bf16_small"]
+    opt = B.make_optim(lr=1e-4, step=0, decay_total_steps=10)
+    results = []
+    side = torch.cuda.Stream()
+    for mode in ("eager", "graph", "host"):
+        with torch.cuda.stream(side):
+            p = Problem(wl, **kw)
+            try:
+                m = p.m
+                losses = []
+                if mode == "graph":
+                    side.synchronize()
+                    B.mrem_graph_capture_step(m.ctx, p.xtd, p.xd, lam, p.vld, wl.batch, wl.seq, m.t_out, m.s_out, m.loss, opt)
+                h_xt, h_xs = (x.cpu().contiguous().pin_memory() for x in (p.xtd, p.xd))
+                h_len = torch.from_numpy(p.vl).pin_memory()
+                for _ in range(3):
+                    if mode == "eager":
+                        p.run_gpu(lam=lam, same_input=False)
+                        m.step(opt)
+                        losses.append(float(m.loss[0]))
+                    elif mode == "graph":
+                        B.mrem_graph_launch(m.ctx)
+                        torch.cuda.synchronize()
+                        losses.append(float(m.loss[0]))
+                    else:
+                        losses.append(B.mrem_recon_step_host(m.ctx, h_xt, h_xs, h_len, wl.batch, wl.seq, lam, opt))
+                torch.cuda.synchronize()
+                assert m.poll_status() == 0
+                results.append((losses, m.student_numpy()[0]["W1"].copy()))
+            finally:
+                p.close()
+    for losses, w1 in results[1:]:
+        assert losses == results[0][0] and np.array_equal(w1, results[0][1])
+
+
 def test_state_export_import_resumes_bitwise():
     wl, kw = CASES["bf16_small"]
     opt = B.make_optim(lr=1e-4, step=0, decay_total_steps=8)
