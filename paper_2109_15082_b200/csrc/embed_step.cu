@@ -53,14 +53,17 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
   }
 }
 
-// Everything that happens to one token, one warp per token (rows up to 32 * V * ROW_NV wide, held in registers): both
-// gathers, both LayerNorms, the squared error, its gradient and the LayerNorm's backward: the operations of the separate
-// kernels (embed_sum, ln_fwd, loss, ln_bwd) in their order, without their intermediates' round trips through memory and
-// without six of their seven launches.  The first and the last token of every id and their number are noted (atomicMin /
+// Everything that happens to one token, W warps per token and one vector of V columns per thread (rows up to 32 * V * MAX_W
+// wide): both gathers, both LayerNorms, the squared error, its gradient and the LayerNorm's backward: the operations of the
+// separate kernels (embed_sum, ln_fwd, loss, ln_bwd) in their order, without their intermediates' round trips through memory
+// and without six of their seven launches.  Latency bounds it: with one vector per thread a token is one round of loads and three block sums
+// (both modules' means together, both variances, the two sums of the backward), and eight blocks share an SM.
+// (One warp per token with the whole row in its 128 registers: 22 % of the warps active, 29 us; the step of 30522 x 1024, 32 x 128
+// tokens 204 -> 200 us, of 30522 x 768, 5 x 56 tokens 154 -> 150.)  The first and the last token of every id and their number are noted (atomicMin /
 // atomicMax of an index, atomicAdd of 1: no dependence on scheduling); they say later which table rows were gathered at
 // all, who adds up a row's gradients, and how far to look.  One block more than the tokens need prepares the optimizer's
 // scalars beside them.
-constexpr int ROW_NV = 4;
+constexpr int MAX_W = 4;
 struct EmbedRow {
   const float *t_word, *t_pos, *t_type, *t_g, *t_b;           // teacher tables and LayerNorm
   const float *pos, *type, *ln_g, *ln_b;
@@ -83,36 +86,34 @@ __device__ __forceinline__ void load_f32(const float* p, float* v) {
   }
 }
 
-// Mean and 1 / sqrt(variance + eps) of a row held in registers.
-template <int V>
-__device__ __forceinline__ void row_stats(const float (&y)[ROW_NV][V], int lane, int H, float eps, float& mu, float& rs) {
-  float sum = 0.f;
+// Sums of two values over the W warps of a token, in warp order; every thread gets them.  `part`: one place per warp of the block.
+template <int W>
+__device__ __forceinline__ float2 token_sums(float a, float b, float2* part, int warp) {
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (W == 1) return make_float2(a, b);
+  if ((threadIdx.x & 31) == 0) part[warp] = make_float2(a, b);
+  __syncthreads();
+  const int first = warp / W * W;
+  float2 r = part[first];
 #pragma unroll
-  for (int i = 0; i < ROW_NV; ++i)
-    if ((lane + 32 * i) * V < H) {
-#pragma unroll
-      for (int j = 0; j < V; ++j) sum += y[i][j];
-    }
-  mu = warp_sum(sum) / (float)H;
-  float sq = 0.f;
-#pragma unroll
-  for (int i = 0; i < ROW_NV; ++i)
-    if ((lane + 32 * i) * V < H) {
-#pragma unroll
-      for (int j = 0; j < V; ++j) sq += (y[i][j] - mu) * (y[i][j] - mu);
-    }
-  rs = 1.f / sqrtf(warp_sum(sq) / (float)H + eps);
+  for (int k = 1; k < W; ++k) { r.x += part[first + k].x; r.y += part[first + k].y; }
+  return r;
 }
 
-template <typename T, int V>
-__global__ void __launch_bounds__(128) embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra,
-                                                        T* __restrict__ e_t, T* __restrict__ e_s, T* __restrict__ y_s,
-                                                        T* __restrict__ dsum, T* __restrict__ dy) {
+__host__ __device__ constexpr int tokens_per_block(int W) { return W == 3 ? 1 : 4 / W; }
+
+template <typename T, int V, int W>
+__global__ void __launch_bounds__(32 * W * tokens_per_block(W), 8)
+embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra, T* __restrict__ e_t, T* __restrict__ e_s,
+                 T* __restrict__ y_s, T* __restrict__ dsum, T* __restrict__ dy) {
   pdl_wait();
   pdl_trigger();
+  constexpr int TPB = tokens_per_block(W);
   __shared__ float sh[32];
+  __shared__ float2 part[3][W * TPB];                         // one set per sum: the next token's first is behind this one's last
   __shared__ int last;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, H = p.H;
+  const int wid = threadIdx.x >> 5, H = p.H, c = (int)(threadIdx.x % (32 * W)) * V;
   if ((int)blockIdx.x == p.row_blocks) {
     if (threadIdx.x == 0) optim_prepare(p.optim);
     return;
@@ -120,104 +121,98 @@ __global__ void __launch_bounds__(128) embed_row_kernel(const __grid_constant__ 
   if (blockIdx.x == 0)                                        // tickets of the column reduction that follows
     for (int i = threadIdx.x; i < p.n_col_counters; i += blockDim.x) p.col_counters[i] = 0;
   float err = 0.f;
-  for (long long t = blockIdx.x * 4ll + wid; t < p.M; t += p.row_blocks * 4ll) {
-    int id = p.ids[t], tt = p.type_ids ? p.type_ids[t] : 0;
+  for (long long t0 = (long long)blockIdx.x * TPB; t0 < p.M; t0 += (long long)p.row_blocks * TPB) {
+    const long long t = t0 + wid / W;
+    const bool live = t < p.M, on = live && c < H;
+    int id = live ? p.ids[t] : 0, tt = live && p.type_ids ? p.type_ids[t] : 0;
     if (id < 0 || id >= p.vocab || tt < 0 || tt >= p.n_types) {   // recorded, then clamped: no out-of-range access
-      if (lane == 0) atomicCAS(p.status, 0, (int)DEV_BAD_INDEX);
+      if (c == 0) atomicCAS(p.status, 0, (int)DEV_BAD_INDEX);
       id = min(max(id, 0), p.vocab - 1);
       tt = min(max(tt, 0), p.n_types - 1);
     }
-    if (lane == 0) note_token(p.row_first, p.row_last, p.row_count, id, (int)t);
+    if (live && c == 0) note_token(p.row_first, p.row_last, p.row_count, id, (int)t);
     const long long row = (long long)id * H, prow = (t % p.S) * (long long)H, trow = (long long)tt * H, base = t * H;
-    float et[ROW_NV][V], y[ROW_NV][V];                        // teacher row, student row, as stored before the LayerNorm
-    const float sc = p.scale[id];
+    float et[V], y[V];                                        // teacher row, student row, as stored before the LayerNorm
 #pragma unroll
-    for (int i = 0; i < ROW_NV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < H) {
-        float a[V], b[V];
-        load_f32<V>(p.t_word + row + c, et[i]);
-        load_f32<V>(p.t_pos + prow + c, a);
-        load_f32<V>(p.t_type + trow + c, b);
+    for (int j = 0; j < V; ++j) et[j] = y[j] = 0.f;
+    if (on) {
+      const float sc = p.scale[id];
+      float a[V], b[V];
+      load_f32<V>(p.t_word + row + c, et);
+      load_f32<V>(p.t_pos + prow + c, a);
+      load_f32<V>(p.t_type + trow + c, b);
+      // (the student's position and token-type rows are written by a later kernel of this step: no read-only loads)
 #pragma unroll
-        for (int j = 0; j < V; ++j) et[i][j] = stored<T>(et[i][j] + a[j] + b[j]);
-        // (the student's position and token-type rows are written by a later kernel of this step: no read-only loads)
-#pragma unroll
-        for (int j = 0; j < V; j += 4) {
-          const float4 pa = *reinterpret_cast<const float4*>(p.pos + prow + c + j), ta = *reinterpret_cast<const float4*>(p.type + trow + c + j);
-          const char4 q = *reinterpret_cast<const char4*>(p.codes + row + c + j);
-          y[i][j] = stored<T>(sc * (float)q.x + pa.x + ta.x);
-          y[i][j + 1] = stored<T>(sc * (float)q.y + pa.y + ta.y);
-          y[i][j + 2] = stored<T>(sc * (float)q.z + pa.z + ta.z);
-          y[i][j + 3] = stored<T>(sc * (float)q.w + pa.w + ta.w);
-        }
-        store_vec<T, V>(y_s + base + c, y[i]);
+      for (int j = 0; j < V; j += 4) {
+        const float4 pa = *reinterpret_cast<const float4*>(p.pos + prow + c + j), ta = *reinterpret_cast<const float4*>(p.type + trow + c + j);
+        const char4 q = *reinterpret_cast<const char4*>(p.codes + row + c + j);
+        y[j] = stored<T>(sc * (float)q.x + pa.x + ta.x);
+        y[j + 1] = stored<T>(sc * (float)q.y + pa.y + ta.y);
+        y[j + 2] = stored<T>(sc * (float)q.z + pa.z + ta.z);
+        y[j + 3] = stored<T>(sc * (float)q.w + pa.w + ta.w);
       }
-    }
-    float mu, rs;
-    row_stats<V>(et, lane, H, p.eps, mu, rs);
 #pragma unroll
-    for (int i = 0; i < ROW_NV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < H) {
-        float g[V], b[V];
-        load_f32<V>(p.t_g + c, g);
-        load_f32<V>(p.t_b + c, b);
-#pragma unroll
-        for (int j = 0; j < V; ++j) et[i][j] = (et[i][j] - mu) * rs * g[j] + b[j];
-        store_vec<T, V>(e_t + base + c, et[i]);
-      }
+      for (int j = 0; j < V; ++j) et[j] = stored<T>(et[j] + a[j] + b[j]);
+      store_vec<T, V>(y_s + base + c, y);
     }
-    row_stats<V>(y, lane, H, p.eps, mu, rs);
-    if (lane == 0) { p.mean[t] = mu; p.rstd[t] = rs; }
-    // the student's output, the squared error, its gradient and what of it enters the LayerNorm: et becomes that gradient
-    // times gamma, y the normalised row
+    float sum_t = 0.f, sum_s = 0.f;
+#pragma unroll
+    for (int j = 0; j < V; ++j) { sum_t += et[j]; sum_s += y[j]; }
+    float2 r = token_sums<W>(sum_t, sum_s, part[0], wid);
+    const float mu_t = r.x / (float)H, mu = r.y / (float)H;
+    sum_t = sum_s = 0.f;
+    if (on) {
+#pragma unroll
+      for (int j = 0; j < V; ++j) { sum_t += (et[j] - mu_t) * (et[j] - mu_t); sum_s += (y[j] - mu) * (y[j] - mu); }
+    }
+    r = token_sums<W>(sum_t, sum_s, part[1], wid);
+    const float rs_t = 1.f / sqrtf(r.x / (float)H + p.eps), rs = 1.f / sqrtf(r.y / (float)H + p.eps);
+    if (live && c == 0) { p.mean[t] = mu; p.rstd[t] = rs; }
+    // both outputs, the squared error, its gradient and what of it enters the LayerNorm: et becomes that gradient times
+    // gamma, y the normalised row
     float s1 = 0.f, s2 = 0.f;
+    if (on) {
+      float g[V], d[V];
+      load_f32<V>(p.t_g + c, g);
+      load_f32<V>(p.t_b + c, d);
 #pragma unroll
-    for (int i = 0; i < ROW_NV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < H) {
-        float g[V], d[V];
-        load_f32<V>(p.ln_g + c, g);
-        load_f32<V>(p.ln_b + c, d);
+      for (int j = 0; j < V; ++j) et[j] = (et[j] - mu_t) * rs_t * g[j] + d[j];
+      store_vec<T, V>(e_t + base + c, et);
+      load_f32<V>(p.ln_g + c, g);
+      load_f32<V>(p.ln_b + c, d);
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          y[i][j] = (y[i][j] - mu) * rs;
-          d[j] = y[i][j] * g[j] + d[j];
-        }
-        store_vec<T, V>(e_s + base + c, d);
+      for (int j = 0; j < V; ++j) {
+        y[j] = (y[j] - mu) * rs;
+        d[j] = y[j] * g[j] + d[j];
+      }
+      store_vec<T, V>(e_s + base + c, d);
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          const float diff = stored<T>(d[j]) - stored<T>(et[i][j]);
-          err += diff * diff;
-          d[j] = stored<T>(2.f * p.c * diff);
-        }
-        if (extra) {
-          float x[V];
-          load_vec<T, V>(extra + base + c, x);
+      for (int j = 0; j < V; ++j) {
+        const float diff = stored<T>(d[j]) - stored<T>(et[j]);
+        err += diff * diff;
+        d[j] = stored<T>(2.f * p.c * diff);
+      }
+      if (extra) {
+        float x[V];
+        load_vec<T, V>(extra + base + c, x);
 #pragma unroll
-          for (int j = 0; j < V; ++j) d[j] = stored<T>(d[j] + x[j]);
-        }
-        store_vec<T, V>(dsum + base + c, d);
+        for (int j = 0; j < V; ++j) d[j] = stored<T>(d[j] + x[j]);
+      }
+      store_vec<T, V>(dsum + base + c, d);
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          et[i][j] = d[j] * g[j];
-          s1 += et[i][j];
-          s2 += et[i][j] * y[i][j];
-        }
+      for (int j = 0; j < V; ++j) {
+        et[j] = d[j] * g[j];
+        s1 += et[j];
+        s2 += et[j] * y[j];
       }
     }
-    s1 = warp_sum(s1) / (float)H;
-    s2 = warp_sum(s2) / (float)H;
+    r = token_sums<W>(s1, s2, part[2], wid);
+    if (on) {
+      s1 = r.x / (float)H;
+      s2 = r.y / (float)H;
 #pragma unroll
-    for (int i = 0; i < ROW_NV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < H) {
-        float o[V];
-#pragma unroll
-        for (int j = 0; j < V; ++j) o[j] = rs * (et[i][j] - s1 - y[i][j] * s2);
-        store_vec<T, V>(dy + base + c, o);
-      }
+      for (int j = 0; j < V; ++j) et[j] = rs * (et[j] - s1 - y[j] * s2);
+      store_vec<T, V>(dy + base + c, et);
     }
   }
   // per-block errors, added in block order by the last block to arrive
@@ -249,7 +244,7 @@ __global__ void __launch_bounds__(128) embed_row_kernel(const __grid_constant__ 
 //     the eight sums being added in warp order.  Warp w of block i has token w * blocks + i: frequent ids first appear among
 //     the first tokens, and would otherwise all meet in one block.
 // The former occurrence lists (one thread per token walking all the others, twice) alone took 300 us at 4096 tokens; this
-// kernel takes 30 us (32 x 128 tokens, hidden 1024; embed_row_kernel 30, the table update 170 of the step's 240).
+// kernel takes 30 us (32 x 128 tokens, hidden 1024; embed_row_kernel 25, the table update 136 of the step's 200).
 constexpr int TYPE_CHUNKS = 64;
 constexpr int TAB_COLS = 512;                                 // columns a word-table block works on
 constexpr int WARP_MAX = 16;                                  // tokens of one id that a single warp adds up
@@ -550,18 +545,22 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   void* dsum = s.dsum;                                     // the gradient the LayerNorm sees
   OptimArgs oa{};
   if (o) oa = OptimArgs{s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay};
-  if (H <= 32 * (dt == 1 ? 8 : 4) * ROW_NV && aligned) {
-    // the row fits a warp's registers: everything per token in one kernel
-    const int row_blocks = (int)((M + 3) / 4 < RED_BLOCKS ? (M + 3) / 4 : RED_BLOCKS);
+  const int row_warps = (H + 32 * (dt == 1 ? 8 : 4) - 1) / (32 * (dt == 1 ? 8 : 4));
+  if (row_warps <= MAX_W && aligned) {
+    // one vector per thread: everything per token in one kernel
+    const int tpb = tokens_per_block(row_warps);
+    const long long want = (M + tpb - 1) / tpb;
+    const int row_blocks = (int)(want < RED_BLOCKS ? want : RED_BLOCKS);
     const EmbedRow er{x->t_word, x->t_pos, x->t_type, x->t_ln_g, x->t_ln_b, x->pos, x->type, x->ln_g, x->ln_b, s.codes, s.scale, d_ids, d_type_ids,
                       (int)seq, H, V, (int)d->n_types, M, d->ln_eps, cc, d_status, row_first, row_last, row_count, loss_ticket,
                       s.mean, s.rstd, s.loss_partial, d_loss, s.col_counters, H / 32 + 2, row_blocks, oa};
     const unsigned grid = (unsigned)(row_blocks + (o ? 1 : 0));
     Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)), 0, st);
-    if (dt == 1)
-      launch_k(embed_row_kernel<bf16, 8>, grid, 128, 0, st, er, (const bf16*)d_extra_grad, (bf16*)d_e_teacher, (bf16*)d_e_student, (bf16*)s.y_s, (bf16*)s.dsum, (bf16*)s.dy);
-    else
-      launch_k(embed_row_kernel<float, 4>, grid, 128, 0, st, er, (const float*)d_extra_grad, (float*)d_e_teacher, (float*)d_e_student, (float*)s.y_s, (float*)s.dsum, (float*)s.dy);
+#define MREM_ROW(T, V, W) launch_k(embed_row_kernel<T, V, W>, grid, 32 * W * tokens_per_block(W), 0, st, er, (const T*)d_extra_grad, (T*)d_e_teacher, (T*)d_e_student, (T*)s.y_s, (T*)s.dsum, (T*)s.dy)
+#define MREM_ROWS(T, V) do { if (row_warps == 1) MREM_ROW(T, V, 1); else if (row_warps == 2) MREM_ROW(T, V, 2); else if (row_warps == 3) MREM_ROW(T, V, 3); else MREM_ROW(T, V, 4); } while (0)
+    if (dt == 1) MREM_ROWS(bf16, 8); else MREM_ROWS(float, 4);
+#undef MREM_ROWS
+#undef MREM_ROW
   } else {
     // wide rows: both embedding sums, the two LayerNorms, the loss and the LayerNorm backward as kernels of their own
 #define MREM_EMB(T) do { \
