@@ -244,7 +244,8 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 //     the eight sums being added in warp order.  Warp w of block i has token w * blocks + i: frequent ids first appear among
 //     the first tokens, and would otherwise all meet in one block.
 // The former occurrence lists (one thread per token walking all the others, twice) alone took 300 us at 4096 tokens; this
-// kernel takes 30 us (32 x 128 tokens, hidden 1024; embed_row_kernel 25, the table update 136 of the step's 200).
+// kernel takes 30 us (32 x 128 tokens, hidden 1024; the table update 136 of the step's
+// 200).  Three blocks per SM: four spill, 200 -> 207 us there although 280 tokens take 148 instead of 150.
 constexpr int TYPE_CHUNKS = 64;
 constexpr int TAB_COLS = 512;                                 // columns a word-table block works on
 constexpr int WARP_MAX = 16;                                  // tokens of one id that a single warp adds up
