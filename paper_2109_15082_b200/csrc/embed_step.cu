@@ -462,24 +462,26 @@ struct EmbedScratch {
   float* type_partial;
   size_t bytes;
 };
+// What one call leaves for the next (the quantized table) comes first and whatever depends on the number of tokens last: calls of
+// any size find the table at the same place.
 EmbedScratch carve(const mrem_embed_desc& d, long long max_tokens, void* base) {
   Carve A(base);
   EmbedScratch s;
-  const size_t es = d.act_dtype == MREM_BF16 ? 2 : 4;
-  const size_t MH = (size_t)max_tokens * d.hidden;
-  s.y_t = A.take(MH * es); s.y_s = A.take(MH * es); s.dE = A.take(MH * es); s.dy = A.take(MH * es); s.dsum = A.take(MH * es);
-  s.mean = (float*)A.take(4 * max_tokens); s.rstd = (float*)A.take(4 * max_tokens);
-  s.col_plane = (long long)COL_CHUNKS * d.hidden;
-  s.col_scratch = (float*)A.take(sizeof(float) * 3 * s.col_plane);
-  s.col_counters = (int*)A.take(sizeof(int) * (d.hidden / 32 + 2));
-  s.loss_partial = (float*)A.take(sizeof(float) * RED_BLOCKS);
   s.codes = (int8_t*)A.take((size_t)d.vocab * d.hidden);
   s.rowsum = (int32_t*)A.take(sizeof(int32_t) * d.vocab);
   s.scale = (float*)A.take(sizeof(float) * d.vocab);
   s.optim_sc = (OptimScalars*)A.take(sizeof(OptimScalars));
+  s.col_plane = (long long)COL_CHUNKS * d.hidden;
+  s.col_scratch = (float*)A.take(sizeof(float) * 3 * s.col_plane);
+  s.col_counters = (int*)A.take(sizeof(int) * (d.hidden / 32 + 2));
+  s.loss_partial = (float*)A.take(sizeof(float) * RED_BLOCKS);
   s.mark_bytes = sizeof(unsigned) * (3 * (size_t)d.vocab + 1 + d.n_types);
   s.marks = (unsigned*)A.take(s.mark_bytes);
   s.type_partial = (float*)A.take(sizeof(float) * (size_t)TYPE_CHUNKS * d.n_types * d.hidden);
+  const size_t es = d.act_dtype == MREM_BF16 ? 2 : 4;
+  const size_t MH = (size_t)max_tokens * d.hidden;
+  s.y_t = A.take(MH * es); s.y_s = A.take(MH * es); s.dE = A.take(MH * es); s.dy = A.take(MH * es); s.dsum = A.take(MH * es);
+  s.mean = (float*)A.take(4 * max_tokens); s.rstd = (float*)A.take(4 * max_tokens);
   s.bytes = (A.off + 255) & ~size_t(255);
   return s;
 }

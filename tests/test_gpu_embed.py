@@ -136,6 +136,26 @@ def test_embedding_rows_at_the_edges_of_their_warps(act_dtype, H):
         assert rel(e.g[k].cpu().numpy(), r["grads"][k]) < 2e-2, k
 
 
+# a shorter batch and another sequence length than the largest the workspace is for, then the largest again; without and
+# with rows wider than the one-kernel path takes
+@pytest.mark.parametrize("act_dtype,H", [("bf16", 128), ("bf16", 1040), ("f32", 64)])
+def test_embedding_steps_of_changing_size_share_one_quantized_table(act_dtype, H):
+    """Only the first call re-quantizes the table; every later one has to find the codes that the call before left, whatever
+    the two calls' token counts.  Tolerances as in the first test."""
+    e, desc, teacher, student, step, ids, tt = _problem(act_dtype, 4, H=H, batch=5, seq=40)
+    fwd_tol = 1e-3 if act_dtype == "bf16" else 1e-4
+    for t, (batch, seq) in enumerate([(5, 40), (2, 24), (1, 7), (5, 40)]):
+        tables, row_step = {k: v.cpu().numpy() for k, v in e.s.items()}, e.word_step.cpu().numpy()
+        i, ty = np.ascontiguousarray(ids[:batch, :seq]), np.ascontiguousarray(tt[:batch, :seq])
+        r = O.embed_loss_backward(desc, teacher, tables, row_step, 4, i, ty)
+        loss = float(e.step(torch.from_numpy(i).to(e.device), torch.from_numpy(ty).to(e.device), B.make_optim(step=t + 1, lr=1e-3))[0])
+        assert int(e.status[0]) == 0 and abs(loss - r["loss"]) <= 2e-2 * r["loss"], (t, loss, r["loss"])
+        for out, k in zip(e.outputs(batch, seq), ("e_t", "e_s")):
+            assert rel(out.float().cpu().numpy(), r[k]) < fwd_tol, (t, k)
+        for k in ("pos", "type", "ln_g", "ln_b"):
+            assert rel(e.g[k].cpu().numpy(), r["grads"][k]) < 2e-2, (t, k)
+
+
 def test_embedding_step_rejects_and_reports_bad_input():
     e, desc, teacher, student, step, ids, tt = _problem("bf16", 4, V=64, H=32, P=16, batch=2, seq=8)
     d_ids, d_tt = torch.from_numpy(ids).to(e.device), torch.from_numpy(tt).to(e.device)
