@@ -165,8 +165,8 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
     const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p),
                  magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
     const float lim_p = range_limit(s_p, p.p_hi);
-    // the row's largest probability is 1 / sum, rounded as stored: one test per warp tells whether anything clips
-    const bool clips = !__all_sync(0xffffffffu, __bfloat162float(__float2bfloat16_rn(st.y)) <= lim_p);
+    // one test per warp tells whether anything can be clipped
+    const bool clips = !__all_sync(0xffffffffu, probability_bound(st.x, st.y) <= lim_p);
     // this thread's probabilities, two chunks of 32; the loops over them stay rolled, the chunks rotate through the registers
     // (the kernel's code is executed once per CTA: with everything unrolled it was 130 KB, and a third of the stalls were
     //  instruction fetches)

@@ -36,6 +36,14 @@ __device__ __forceinline__ float range_limit(float step, float hi) {
   return lim;
 }
 
+// No stored probability of a row is above this (m = RN(alpha log2(e) max), inv = 1 / sum, both as the forward pass left them).
+// The largest one is not 2^0 inv: its exponent fma(max, alpha log2(e), -m) is the rounding error of m, up to 2^-24 |m|, and where
+// that is positive the probability can be stored one bf16 spacing above the stored inv.  The last factor covers the two
+// approximate exponentials and the roundings of the products.  Only whether a tile tests its elements one by one depends on this.
+__device__ __forceinline__ float probability_bound(float m, float inv) {
+  return __bfloat162float(__float2bfloat16_rn(inv * exp2_approx(fabsf(m) * 5.9604645e-8f) * (1.f + 9.5367432e-7f)));
+}
+
 // Straight-through pass of one symmetric quantizer over 32 values of a row: x (bf16 pairs before quantization, replaced by the
 // masked gradient as bf16 pairs), g(j) = the incoming gradient of pair j.  Returns the sum of the step-size terms.
 template <class G>

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
     const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p),
                  magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
     const float lim_p = range_limit(s_p, p.p_hi);
-    const bool clips = !__all_sync(0xffffffffu, __bfloat162float(__float2bfloat16_rn(st.y)) <= lim_p);   // largest P of the row: 1 / sum
+    const bool clips = !__all_sync(0xffffffffu, probability_bound(st.x, st.y) <= lim_p);   // (see attention_bwd.cu)
     // ---- this thread's probabilities: chunks part, part + 4, part + 8 of 32 keys
     // (rolled loops, the chunks rotating through the registers: see attention_bwd.cu)
     uint32_t pw0[16], pw1[16], pw2[16];
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
         const float2 st = p.stat[at];
         v = make_float4(-st.x, st.y, -p.dot[at], 0.f);
       }
-      over = over || __bfloat162float(__float2bfloat16_rn(v.y)) > lim_p;   // the largest P of the query's row
+      over = over || !(probability_bound(v.x, v.y) <= lim_p);
       qstat[i] = v;
     }
   const bool clips = __syncthreads_or(over);

@@ -7,7 +7,7 @@ import torch
 from oracle import mrem_oracle as O
 from paper_2109_15082_b200 import binding as B
 from paper_2109_15082_b200 import synth
-from tests.gpu_util import Problem
+from tests.gpu_util import Problem, rel
 from tests.test_gpu_module import compare_grads
 
 pytestmark = pytest.mark.gpu
@@ -66,5 +66,61 @@ def test_reading_the_probabilities_leaves_the_backward_pass_alone(seq):
 
         a = gradient(False)
         assert a.any() and torch.equal(a, gradient(True))
+    finally:
+        p.close()
+
+
+def _rounded_up_case(a_bits, lo_len, hi_len):
+    """A step s, codes cq and ck, a number of keys n and a step s_p such that n equal scores alpha 64 cq ck have probabilities
+    1 / n that are stored one bf16 spacing ABOVE the stored 1 / sum, with the upper end of P's range between the two: the
+    kernels' exponent of the largest score is the rounding error r of alpha log2(e) score, so their sum is n 2^r."""
+    f32 = np.float32
+    p_hi, cq, ck = (255, 120, 121) if a_bits == 8 else (15, 5, 6)
+    r, s = -1.0, None
+    for t in np.sqrt(np.linspace(7e3, 1e4, 200) / (8 * cq * ck)).astype(f32):        # scores of 7,000 to 10,000
+        alpha2 = f32(f32(f32(0.125) * t) * t) * f32(1.4426950408889634)
+        score = f32(64 * cq * ck)
+        err = float(alpha2) * float(score) - float(f32(alpha2 * score))
+        if err > r:
+            r, s = err, t
+    for n in range(lo_len, hi_len + 1):
+        up, low = float(O.round_bf16(np.array(1.0 / n))), float(O.round_bf16(np.array(2.0 ** -r / n)))
+        middle = (low + up) / 2
+        if low < up and 1.0 / n > (1 + 2e-5) * middle and 2.0 ** -r / n < (1 - 2e-5) * middle:
+            return s, cq, ck, n, f32((low + 0.25 * (up - low)) / p_hi), up
+    raise AssertionError("no such case")
+
+
+# one kernel and two, 8- and 4-bit codes
+@pytest.mark.parametrize("seq,a_bits", [(64, 8), (128, 4), (264, 8), (384, 4)])
+def test_probabilities_stored_above_the_reciprocal_sum_are_clipped(seq, a_bits):
+    """Every probability is one bf16 spacing beyond its quantizer's range although the row's 1 / sum, as stored, is not.  All of
+    them are then clipped: no gradient reaches Q, K and their steps, and the value gradients see the highest code.  The step
+    gradient of P is a sum of d times the highest code, 2e-2 from the oracle's as everywhere; the value gradients differ from
+    the kernel-per-operation path's by a few bf16 roundings (2^-9 each), where one code more would be 1 / 255 or 1 / 15."""
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=2)
+    H = wl.hidden
+    s, cq, ck, n, s_p, stored = _rounded_up_case(a_bits, seq // 2, seq)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002, a_bits=a_bits)
+    try:
+        m = p.m
+        p.vl = np.array([n, n], np.int32)
+        p.vld = torch.from_numpy(p.vl).to(m.device)
+        p.student[0]["Wqkv"][:2 * H] = 0
+        p.student[0]["bqkv"][:H], p.student[0]["bqkv"][H:2 * H] = cq * s, ck * s
+        p.a[0, 1], p.a[0, 2], p.a[0, 4] = s, s, s_p
+        m.load_student(p.student)
+        m.set_steps(p.ws, p.a, p.off)
+        r = p.run_oracle()["grads"][0]
+        got = []
+        for fused in (True, False):
+            m.set_fused_attention_backward(fused)
+            got.append(p.run_gpu()["grads"][0])
+            P = m.activation(B.STUDENT, 0, B.ACT_P, (2, wl.n_heads, seq, seq)).float()
+            assert (P[..., :n] == stored).all() and not P[..., n:].any()
+        g, per_op = got
+        assert not g["bqkv"][:2 * H].any() and not g["Wqkv"][:2 * H].any() and g["a"][1] == 0 and g["a"][2] == 0
+        assert abs(g["a"][4] - r["a"][4]) <= 2e-2 * abs(r["a"][4])
+        assert rel(g["bqkv"][2 * H:], per_op["bqkv"][2 * H:]) < 2e-3 and rel(g["Wqkv"][2 * H:], per_op["Wqkv"][2 * H:]) < 2e-3
     finally:
         p.close()
