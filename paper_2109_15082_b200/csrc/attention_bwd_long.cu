@@ -37,12 +37,12 @@ struct LongParams {
   unsigned long long wait_ns;
 };
 
-// Adds `n` per-CTA sums (the same array in every CTA, filled before the call) over the CTAs of the cluster, in rank order, in
-// the first CTA; all threads of all CTAs call it.
+// Step-size partials of the CTAs of a head go to the cluster's first CTA.  A CTA may touch another one's shared memory once
+// that one is known to have started: every thread arrives on the cluster's barrier after its CTA's set-up and waits on it just
+// before the remote store (16 x 16 heads x 384 x 384: no difference in time).
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void store_remote(float* local, uint32_t rank, float v) {
   uint32_t addr;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(local)), "r"(rank));
@@ -83,10 +83,12 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  cluster_arrive();                                        // (see store_remote)
   pdl_wait();
   pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const int len = p.len[b], n_valid = (len + 31) / 32;
+  float share = 0.f;                                       // this CTA's step-size partials, one per lane of warp 1
 
   if (warp == 0) {
     if (lane == 0) {
@@ -267,15 +269,16 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
     asm volatile("bar.sync 1, 512;" ::: "memory");
     if (threadIdx.x == 32) { tma_store_4d(&maps.out, sD, 0, q0, head, b); tma_store_commit(); }
     if (warp == 1 && lane < 3) {
-      float t = 0.f;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) t += red_part[k][lane];
-      store_remote(&cta_part[cluster_rank()][lane], 0, t);
+      for (int k = 0; k < 16; ++k) share += red_part[k][lane];
     }
     if (threadIdx.x == 32) tma_store_wait_all();
   }
   __syncthreads();
-  cluster_sync();
+  cluster_wait();
+  if (warp == 1 && lane < 3) store_remote(&cta_part[cluster_rank()][lane], 0, share);
+  cluster_arrive();                                        // the shares are there; no CTA leaves before its own has been handed in
+  cluster_wait();
   if (qb == 0 && threadIdx.x < 3) {
     float t = 0.f;
     for (int k = 0; k < (int)gridDim.x; ++k) t += cta_part[k][threadIdx.x];
@@ -322,10 +325,12 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  cluster_arrive();                                        // (see store_remote)
   pdl_wait();
   pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const int len = p.len[b], n_q = (p.S + 63) / 64;
+  float share = 0.f;                                       // (as in the query kernel)
   const bool active = k0 < len;                            // a block of padded keys has zero gradients
   const float s_p = *p.s_p, lim_p = range_limit(s_p, p.p_hi);
   bool over = false;
@@ -484,15 +489,16 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
       tma_store_commit();
     }
     if (warp == 1 && lane < 2) {
-      float t = 0.f;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) t += red_part[k][lane];
-      store_remote(&cta_part[cluster_rank()][lane], 0, t);
+      for (int k = 0; k < 8; ++k) share += red_part[k][lane];
     }
     if (threadIdx.x == 32) tma_store_wait_all();
   }
   __syncthreads();
-  cluster_sync();
+  cluster_wait();
+  if (warp == 1 && lane < 2) store_remote(&cta_part[cluster_rank()][lane], 0, share);
+  cluster_arrive();
+  cluster_wait();
   if (kb == 0 && threadIdx.x < 2) {
     float t = 0.f;
     for (int k = 0; k < (int)gridDim.x; ++k) t += cta_part[k][threadIdx.x];
