@@ -45,16 +45,17 @@ __device__ __forceinline__ float probability_bound(float m, float inv) {
 }
 
 // Straight-through pass of one symmetric quantizer over 32 values of a row: x (bf16 pairs before quantization, replaced by the
-// masked gradient as bf16 pairs), g(j) = the incoming gradient of pair j.  Returns the sum of the step-size terms.
+// masked gradient as bf16 pairs), g(j) = the incoming gradient of pair j.  Returns the sum of the step-size terms.  A NaN is
+// outside every range (its code is the lowest): the test for clipped values keeps it (max.NaN).
 template <class G>
 __device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi, float lim) {
   const float2 r2 = both(__frcp_rn(step)), ns2 = both(-step), magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
   __nv_bfloat162 mx = __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[0]));
 #pragma unroll
-  for (int j = 1; j < 16; ++j) mx = __hmax2(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[j])));
+  for (int j = 1; j < 16; ++j) mx = __hmax2_nan(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[j])));
   const float2 m = __bfloat1622float2(mx);
   float2 ds = both(0.f);
-  if (__all_sync(0xffffffffu, fmaxf(m.x, m.y) <= lim)) {       // nothing clipped in the whole warp
+  if (__all_sync(0xffffffffu, m.x <= lim && m.y <= lim)) {       // nothing clipped in the whole warp
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const float2 xv = unpack2(x[j]), gv = g(j);

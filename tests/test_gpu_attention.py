@@ -144,3 +144,28 @@ def test_step_gradients_of_sequences_that_are_mostly_padding(seq, lens):
             assert np.array_equal(p.run_gpu()["grads"][0]["a"], first[0]["a"])
     finally:
         p.close()
+
+
+# the quantized site the value belongs to, one kernel and two
+@pytest.mark.parametrize("seq", [72, 200])
+@pytest.mark.parametrize("site", ["q", "k", "v"])
+def test_a_value_that_is_not_a_number_takes_no_gradient(seq, site):
+    """Eq. 1's comparisons are false for a NaN: its code is the lowest one and the straight-through mask stops its gradient, in
+    the fused kernels as in the kernel-per-operation path; the step gradients of the others stay numbers."""
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=2)
+    p = Problem(wl, step_shrink=1.5, student_noise=0.002)            # (nothing else is clipped)
+    try:
+        m, at = p.m, 70 + wl.hidden * "qkv".index(site)
+        p.student[0]["bqkv"][at] = np.nan
+        m.load_student(p.student)
+        m.set_steps(p.ws, p.a, p.off)
+        got = []
+        for fused in (True, False):
+            m.set_fused_attention_backward(fused)
+            got.append(p.run_gpu()["grads"][0])
+        g, per_op = got
+        assert np.isfinite(g["a"]).all() and g["bqkv"][at] == 0 and per_op["bqkv"][at] == 0
+        assert np.abs(g["a"] - per_op["a"]).max() <= 2e-2 * np.abs(per_op["a"]).max()
+        assert rel(g["bqkv"], per_op["bqkv"]) < 2e-2 and rel(g["Wqkv"], per_op["Wqkv"]) < 2e-2
+    finally:
+        p.close()
