@@ -176,9 +176,8 @@ __device__ __forceinline__ void gelu_bwd_vec(const float* u, float* d, float s, 
         const bool in0 = zc.x == z.x, in1 = zc.y == z.y;
         uint32_t b0, b1;
         ds2 = fma2(dv, add2(rne_magic2(zc, b0, b1), make_float2(in0 ? -z.x : 0.f, in1 ? -z.y : 0.f)), ds2);
-        const float2 pass = make_float2(in0 ? dv.x : 0.f, in1 ? dv.y : 0.f);
-        dofs2 = add2(dofs2, fma2(pass, splat(-1.f), dv));
-        dv = pass;
+        dofs2 = add2(dofs2, make_float2(in0 ? 0.f : dv.x, in1 ? 0.f : dv.y));      // (not d - pass: inf - inf)
+        dv = make_float2(in0 ? dv.x : 0.f, in1 ? dv.y : 0.f);
       }
       dv = mul2(dv, gelu_grad_from_parts2(x, tail, ex));
       d[j] = dv.x; d[j + 1] = dv.y;

@@ -967,3 +967,27 @@ def test_closed_form_weight_scales_match_the_oracle(case):
         assert np.isfinite(g2["loss"]) and g2["loss"] != g["loss"]
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("act_dtype", ["bf16", "f32"])
+def test_offset_gradient_takes_no_part_of_unclipped_values_whatever_their_gradient(act_dtype):
+    """The offset gradient is the sum over the CLIPPED values of the GELU site (Sec. 3.1.1): with a range that clips none it is
+    exactly zero, also where the loss gradient is not finite (reported through the status word) and nothing else is a number."""
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=40, batch=2, act_dtype=act_dtype)
+    p = Problem(wl, step_shrink=1.5, student_noise=0.002)
+    try:
+        m = p.m
+        p.teacher[0]["ln2_g"][:] = 3e38
+        m.load_teacher(p.teacher)
+        p.off[0, 7] -= 0.05
+        m.set_steps(p.ws, p.a, p.off)
+        m.quantize_weights()
+        m.forward_teacher(p.xd, p.vld, wl.batch, wl.seq)
+        m.forward_student(p.xd, p.vld, wl.batch, wl.seq)
+        m.recon_loss()
+        m.backward()
+        assert float(m.grad(0, B.GRAD_OFFSET + B.Q_G, (1,))[0]) == 0.0
+        assert not torch.isfinite(m.grad(0, B.B1, (wl.ffn,))).all()
+        assert m.poll_status() == -8
+    finally:
+        p.close()
