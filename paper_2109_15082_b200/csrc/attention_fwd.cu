@@ -308,10 +308,13 @@ template <int TPR, bool QUANT>
 int launch_tpr(const CUtensorMap& map, const AttnParams& p, cudaStream_t st) {
   const int n_box = (p.S + 127) / 128, n_kb = (p.S + 63) / 64;
   const int smem = 1024 + 16384 * (n_box + (n_kb > 1 + n_box ? n_kb : 1 + n_box));
-  static int smem_set = 0;
-  if (smem > smem_set) {
-    if (cudaFuncSetAttribute(attention_fwd_kernel<TPR, QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GEMM_ERR_CUDA;
-    smem_set = smem;
+  // the limit for the longest sequence of this variant, whatever this one needs: threads that get here together set the same one
+  constexpr int MAX_BOX = TPR == 4 ? 3 : TPR;
+  static bool attr_set = false;
+  if (!attr_set) {
+    if (cudaFuncSetAttribute(attention_fwd_kernel<TPR, QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + 16384 * 3 * MAX_BOX) != cudaSuccess)
+      return GEMM_ERR_CUDA;
+    attr_set = true;
   }
   if (launch_k(attention_fwd_kernel<TPR, QUANT>, dim3((p.S + 127) / 128, p.h, p.B), 32 + 128 * TPR, smem, st, map, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;

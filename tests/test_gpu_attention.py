@@ -1,5 +1,9 @@
 """The fused attention kernels at the edges of their tiles: sequence lengths around 128, 256 and 384 (where threads per row,
 shared-memory layout and the number of kernels change), valid lengths of one key and around multiples of 16, 32 and 128."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -169,3 +173,48 @@ def test_a_value_that_is_not_a_number_takes_no_gradient(seq, site):
         assert rel(g["bqkv"], per_op["bqkv"]) < 2e-2 and rel(g["Wqkv"], per_op["Wqkv"]) < 2e-2
     finally:
         p.close()
+
+
+def test_contexts_of_different_lengths_make_their_first_pass_together():
+    """Contexts are independent: threads whose sequences take the same variants of the kernels with different amounts of shared
+    memory (and other variants) start at the same moment in a fresh process; every pass equals the same one made alone."""
+    code = """
+import threading
+import torch
+from tests.gpu_util import Problem
+from paper_2109_15082_b200 import synth
+lengths = (256, 136, 384, 264, 200, 328)
+ps, outs, errs = [], {}, []
+for seq in lengths:
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        p = Problem(synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=2))
+        ps.append((seq, p, st))
+torch.cuda.synchronize()
+gate = threading.Barrier(len(ps))
+def run(seq, p, st, key, wait):
+    try:
+        if wait:
+            gate.wait()
+        with torch.cuda.stream(st):
+            p.m.quantize_weights()
+            t = p.m.forward_teacher(p.xd, p.vld, 2, seq).clone()
+            s = p.m.forward_student(p.xd, p.vld, 2, seq).clone()
+        st.synchronize()
+        outs[key, seq] = (t, s)
+    except Exception as e:
+        errs.append((seq, repr(e)))
+threads = [threading.Thread(target=run, args=(*x, "together", True)) for x in ps]
+for t in threads: t.start()
+for t in threads: t.join()
+assert not errs, errs
+for x in ps: run(*x, "alone", False)
+assert not errs, errs
+for seq, p, st in ps:
+    assert all(torch.equal(a, b) for a, b in zip(outs["together", seq], outs["alone", seq])), seq
+    assert p.m.poll_status() == 0
+    p.close()
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
