@@ -276,13 +276,23 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// The encoder is a driver call: it fails in a thread that has made no runtime call yet (and so has no current context).  The
+// current device's context is then made current, as the first runtime call would, and the call repeated.
+template <typename... Args>
+CUresult encode_tiled(Args... args) {
+  const EncodeTiledFn fn = encode_fn();
+  if (!fn) return CUDA_ERROR_NOT_FOUND;
+  CUresult r = fn(args...);
+  int device = 0;
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&device) == cudaSuccess && cudaSetDevice(device) == cudaSuccess) r = fn(args...);
+  return r;
+}
+
 }  // namespace
 
 // Tensor map of one operand: 4-D (contiguous index, strided index, batch0, batch1).
 int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, int mn_extent, int K, int nb0, int nb1,
              int tile_mn, int block_k, int* chunked) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return GEMM_ERR_CUDA;
   if (chunked) *chunked = 0;
   if (chunked && op.mn_contig && elem_bytes == 2 && mn_extent % 64 == 0 && tile_mn % 64 == 0) {
     // (64 contiguous, k rows, chunk of 64, batch0, batch1): one box = every 64-wide piece of the tile, piece after piece
@@ -295,7 +305,7 @@ int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, in
     cuuint64_t strides[4] = {s1, 128, s3, s4};
     cuuint32_t box[5] = {64, (cuuint32_t)block_k, (cuuint32_t)(tile_mn / 64), 1, 1};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(op.ptr), dims, strides, box, estr,
+    CUresult r = encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(op.ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return GEMM_ERR_CUDA;
@@ -322,7 +332,7 @@ int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, in
   box[2] = box[3] = 1;
   cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUtensorMapDataType dt = elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8;
-  CUresult r = fn(map, dt, 4, const_cast<void*>(op.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  CUresult r = encode_tiled(map, dt, 4, const_cast<void*>(op.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? GEMM_OK : GEMM_ERR_CUDA;
 }
@@ -423,8 +433,7 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
     cuuint64_t dims[4] = {(cuuint64_t)g.N, (cuuint64_t)g.M, (cuuint64_t)g.nb0, (cuuint64_t)g.nb1};
     cuuint64_t strides[3] = {s1, s2, s3};
     cuuint32_t box[4] = {32, 32, 1, 1}, estr[4] = {1, 1, 1, 1};
-    EncodeTiledFn fn = encode_fn();
-    if (fn && fn(&mc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, epi.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    if (encode_tiled(&mc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, epi.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                  CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
       p.c_tma = 1;
   }

@@ -5,6 +5,8 @@ Tolerances: forward outputs 1e-3 relative L2 against the oracle in storage-emula
 Integer codes reaching an interior quantizer may differ in a small fraction of positions,
 because the float operations before it round differently on the two sides; the weight codes,
 which depend only on bound inputs, must match bit for bit."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -989,5 +991,31 @@ def test_offset_gradient_takes_no_part_of_unclipped_values_whatever_their_gradie
         assert float(m.grad(0, B.GRAD_OFFSET + B.Q_G, (1,))[0]) == 0.0
         assert not torch.isfinite(m.grad(0, B.B1, (wl.ffn,))).all()
         assert m.poll_status() == -8
+    finally:
+        p.close()
+
+
+def test_a_pass_may_be_the_first_cuda_call_of_its_thread():
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=40, batch=2)
+    p = Problem(wl)
+    try:
+        p.m.quantize_weights()
+        run = lambda: (p.m.forward_teacher(p.xd, p.vld, wl.batch, wl.seq), p.m.forward_student(p.xd, p.vld, wl.batch, wl.seq))
+        ref = [t.clone() for t in run()]
+        p.m.t_out.zero_(), p.m.s_out.zero_()
+        torch.cuda.synchronize()
+        errors = []
+
+        def body():
+            try:
+                run()
+            except B.MremError as e:
+                errors.append(e)
+
+        t = threading.Thread(target=body)
+        t.start()
+        t.join()
+        assert not errors, errors
+        assert torch.equal(p.m.t_out[:ref[0].numel()].view_as(ref[0]), ref[0]) and torch.equal(p.m.s_out[:ref[1].numel()].view_as(ref[1]), ref[1])
     finally:
         p.close()
