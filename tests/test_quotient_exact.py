@@ -63,10 +63,14 @@ def test_quotient_on_float32_numerators_is_within_one_ulp_and_almost_always_exac
     assert (diff != 0).mean() < 1e-5
 
 
+HALF_WINDOW = f32(2.0 ** -15)
+
+
 def _code_fast(n, s, lo, hi, exact_quotient):
     """numpy emulation, instruction by instruction, of the kernels' code path: first product kept inside
     [lo - 1, hi + 1], residual by FMA, correction, clip, nearest integer by adding and subtracting 1.5 * 2^23, and (unless
-    the quotient is known to be exact) a second look by IEEE division for values within 2^-10 of a half-integer."""
+    the quotient is known to be exact) a second look by IEEE division for values further than 1/2 - 2^-15 from that integer
+    (one ulp of a quotient of at most 255 is 2^-16)."""
     magic = f32(12582912.0)
     r = (f32(1.0) / s).astype(np.float32)
     with np.errstate(over="ignore", invalid="ignore"):
@@ -78,7 +82,7 @@ def _code_fast(n, s, lo, hi, exact_quotient):
     q = (t - magic).astype(np.float32)
     low_byte = t.view(np.uint32) & np.uint32(0xFF)
     if not exact_quotient:
-        again = np.abs(np.abs(zc - q) - f32(0.5)) < f32(2.0 ** -10)
+        again = np.abs(zc - q) > f32(0.5) - HALF_WINDOW
         with np.errstate(over="ignore"):
             zd = np.clip((n / s).astype(np.float32), f32(lo), f32(hi))
         t2 = (zd + magic).astype(np.float32)
