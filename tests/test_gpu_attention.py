@@ -175,6 +175,17 @@ def test_a_value_that_is_not_a_number_takes_no_gradient(seq, site):
         p.close()
 
 
+# longer than the fused kernels take; more heads than there are slots for their partial sums
+@pytest.mark.parametrize("seq,batch", [(392, 2), (16, 600)])
+def test_sizes_beyond_the_fused_backward_kernels(seq, batch):
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=batch, len_lo=seq // 4, len_hi=seq)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002)
+    try:
+        compare_grads(p.run_gpu()["grads"], p.run_oracle()["grads"], 2e-2, check_offset=True)
+    finally:
+        p.close()
+
+
 def test_contexts_of_different_lengths_make_their_first_pass_together():
     """Contexts are independent: threads whose sequences take the same variants of the kernels with different amounts of shared
     memory (and other variants) start at the same moment in a fresh process; every pass equals the same one made alone."""

@@ -3,8 +3,9 @@
 At hidden 1024 / FFN 4096 (BERT-large) and hidden 768 / FFN 3072 (BERT-base) with 4096 tokens the kernels take
 the paths the small module tests never reach: 128 x 256 tiles with several tiles per persistent CTA, the grouped
 weight-gradient launch walking 384 tiles of four problems, input-gradient products over MN-major operands,
-column reductions in their multi-chunk form, the 512-thread row kernels, the single-kernel attention backward
-at 16 heads, and (sequence length 384) the kernel-per-operation attention backward.  One layer of the full
+column reductions in their multi-chunk form, the widest row kernels, the single-kernel attention backward
+at 16 heads, and (sequence length 384) the two-kernel attention backward and, switched to it, the
+kernel-per-operation one.  One layer of the full
 width costs the float64 oracle a few seconds, so every gradient group is compared here: weights, biases,
 LayerNorm parameters, per-row weight steps, activation steps and the GELU-site offset, at the stated 2e-2
 relative L2, with clipping present (steps shrunk to 0.8 of their initial value, or the mean|w| rule of the
@@ -46,7 +47,7 @@ FULL_WIDTH = {
     # two BERT-large layers on a quarter batch: the loss gradient enters at both outputs, layer 1 hands its input
     # gradient to layer 0 through the LayerNorm backward that applies the straight-through pass
     "large_w4a8_2layers_8x128": (_wl("large6_w4a8", n_layers=2, batch=8), dict(step_shrink=0.8, student_noise=0.002)),
-    # sequence length 384, 2-bit half-integer grid with mean|w| steps: attention backward on the kernel-per-operation path
+    # sequence length 384, 2-bit half-integer grid with mean|w| steps: attention backward in two kernels
     "large_w2a8_4x384": (_wl("large6_w2a8_s384", n_layers=1, batch=4), dict(step_shrink=0.8, student_noise=0.002)),
     # BERT-base layer (hidden 768, 12 heads, FFN 3072), full batch, W4A8 and the 2-bit grid
     "base_w4a8_32x128": (_wl("base3_w4a8", n_layers=1), dict(step_shrink=0.8, student_noise=0.002)),
@@ -56,9 +57,18 @@ FULL_WIDTH = {
 
 @pytest.mark.parametrize("case", list(FULL_WIDTH))
 def test_every_gradient_at_full_width(case):
+    _every_gradient(case)
+
+
+def test_every_gradient_of_384_tokens_on_the_kernel_per_operation_attention_path():
+    _every_gradient("large_w2a8_4x384", fused_attention=False)
+
+
+def _every_gradient(case, fused_attention=True):
     wl, kw = FULL_WIDTH[case]
     p = Problem(wl, **kw)
     try:
+        p.m.set_fused_attention_backward(fused_attention)
         g = p.run_gpu()
         r = p.run_oracle()
         clipped = sum(int((np.abs(c["qx"]["z"]) > c["qx"]["hi"]).sum()) + int(((c["qG"]["z"] > c["qG"]["hi"]) | (c["qG"]["z"] < 0)).sum())
@@ -153,13 +163,17 @@ def _stage_report(name, got, ref, floor):
 
 @pytest.mark.parametrize("name", ["large6_w4a8", "base3_w4a8"])
 def test_teacher_layer_stage_by_stage_at_full_width(name):
+    teacher_layer_stage_by_stage(_wl(name, n_layers=1))
+
+
+def teacher_layer_stage_by_stage(wl):
     """Every tensor the full-precision pass stores, against the oracle's arithmetic for that one stage applied to
     what the GPU itself stored before it.  Taken stage by stage nothing accumulates: the two sides see identical
     inputs, so they can differ only where the exact value sat within the arithmetic's own error of a bf16 rounding
     boundary, and then by one spacing.  (Over a whole layer such flips feed the next sums and, through the
     LayerNorm statistics of rows with outlier channels, whole rows; the whole-layer figure is printed beside a
     float32 CPU replica's.)"""
-    wl = _wl(name, n_layers=1)
+    name = wl.name
     p = Problem(wl)
     try:
         m, H, F_, h = p.m, wl.hidden, wl.ffn, wl.n_heads

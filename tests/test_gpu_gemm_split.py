@@ -5,6 +5,10 @@ import torch
 
 from oracle import mrem_oracle as O
 from paper_2109_15082_b200 import binding as B
+from paper_2109_15082_b200 import synth
+from tests.gpu_util import Problem, compare_grads, rel
+from tests.test_gpu_full_width import teacher_layer_stage_by_stage
+from tests.test_gpu_module import rem_step_of_one_product
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -37,3 +41,50 @@ def test_shared_products_are_exact(M, N, blocks, ragged):
     B.mrem_gemm_i8(torch.from_numpy(a.astype(np.int8)).to(DEV), 0, torch.from_numpy(b.astype(np.int8)).to(DEV), M, N, K, acc, 0, status, stream)
     assert np.array_equal(acc.cpu().numpy().astype(np.int64), O.int_matmul(a, b))
     assert int(status[0]) == 0
+
+
+# The cost model splits these products.  At 3 x 40 tokens and BERT-large widths: all four of the full-precision pass (bias; bias
+# and residual; bias and GELU), FFN2 of the quantized pass, all input gradients.  At 3 x 72: output projection and FFN2, FFN2, all
+# input gradients but FFN2's.  At hidden and FFN 2048, 40 or 120 tokens: all of the quantized pass but QKV.
+
+def test_shared_products_of_the_full_precision_pass_stage_by_stage():
+    """Bias, bias + residual, bias + GELU: every stored tensor against the oracle's arithmetic for that stage."""
+    teacher_layer_stage_by_stage(synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, seq=40, batch=3, len_lo=10, len_hi=40))
+
+
+@pytest.mark.parametrize("seq", [40, 72])
+def test_gradients_through_shared_products(seq):
+    wl = synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, seq=seq, batch=3, len_lo=10, len_hi=seq)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002)
+    try:
+        g, r = p.run_gpu(), p.run_oracle()
+        assert rel(g["f_s"], r["f_s"]) < 1e-3 and abs(g["loss"] - r["loss"]) <= 2e-2 * r["loss"]
+        compare_grads(g["grads"], r["grads"], 2e-2, check_offset=True)
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("hidden,ffn", [(1024, 4096), (2048, 2048)])
+def test_a_sequence_alone_and_in_a_batch_give_the_same_bits(hidden, ffn):
+    """The quantized pass multiplies whole numbers and treats rows independently: a sequence whose products are shared between
+    thread blocks has the outputs, bit for bit, that it has among 32, whose products are not."""
+    wl = synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, hidden=hidden, n_heads=hidden // 64, ffn=ffn, seq=40, batch=32, len_lo=10,
+                      len_hi=40)
+    p = Problem(wl, student_noise=0.002)
+    try:
+        m = p.m
+        m.quantize_weights()
+        many = m.forward_student(p.xd, p.vld, 32, 40).clone()
+        for i in (0, 31):
+            one = m.forward_student(p.xd[i:i + 1].contiguous(), p.vld[i:i + 1].clone(), 1, 40)
+            assert torch.equal(one[:, 0], many[:, i]), i
+        three = m.forward_student(p.xd[5:8].contiguous(), p.vld[5:8].clone(), 3, 40)
+        assert torch.equal(three, many[:, 5:8])
+    finally:
+        p.close()
+
+
+# W2 with its offset as a column bias and without one (scale only), and the output projection
+@pytest.mark.parametrize("name,asym", [("W2", 3), ("W2", 1), ("Wo", 3)])
+def test_per_product_step_on_shared_products(name, asym):
+    rem_step_of_one_product(synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, seq=72, batch=3, len_lo=10, len_hi=72), name, asym)

@@ -161,13 +161,16 @@ def test_rem_step_of_one_product_matches_the_oracle(name, base, asym, a_bits):
     count (120 rows: one partial tile); then one real step: the updated matrix, steps and offset against the
     oracle's AdamW fed with those gradients, the re-quantized codes bit-exact against Eq. 1 on the updated
     values, and every other parameter untouched."""
-    wl = _wl(base, n_layers=2, hidden=128, n_heads=2, ffn=256, seq=40, batch=3, len_lo=10, len_hi=40)
+    rem_step_of_one_product(_wl(base, n_layers=2, hidden=128, n_heads=2, ffn=256, seq=40, batch=3, len_lo=10, len_hi=40), name, asym, a_bits)
+
+
+def rem_step_of_one_product(wl, name, asym, a_bits=None):
     p = Problem(wl, step_shrink=0.8, student_noise=0.002, asym=asym, a_bits=a_bits)
     try:
-        m, layer = p.m, 1
+        m, layer = p.m, wl.n_layers - 1
         pid, k = REM_MATRICES[name]
         site = O.REM_SITE[name]
-        rows, cols = 120, m.shapes[pid][1]
+        rows, cols = wl.batch * wl.seq, m.shapes[pid][1]
         a_np = synth.normal(5, "rem_a" + name, (rows, cols), 1.0) + (0.4 if name == "W2" else 0.0)
         a_dev = m.to_device(a_np)
         a = a_dev.float().cpu().numpy()                             # the stored bytes, widened
