@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
   const float2 ns_new = splat(-s_new), r_new = splat(__frcp_rn(s_new));
   const Adam2 ad = {splat(o.beta1), splat(__fsub_rn(1.f, o.beta1)), splat(o.beta2), splat(__fsub_rn(1.f, o.beta2)),
                     splat(o.rsqrt_bc2), splat(o.eps), splat(-o.lr_bc1), splat(__fsub_rn(1.f, __fmul_rn(o.lr, o.weight_decay)))};
+  const float vanishes = __fmul_rd(0.5f * s_new, 1.401298464e-45f);    // s 2^-150 in whole units of 2^-149 (GRID 1)
   float2 sum2 = splat(0.f);                                    // codes are whole numbers: exact in any order
   auto update = [&](int c, float4 wv, float4 d, float4 mm, float4 vv) {
     float2 wa = make_float2(wv.x, wv.y), wb = make_float2(wv.z, wv.w);
@@ -187,8 +188,9 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
       }
     } else {
       // 2 clamp(floor(w / s), -2, 1) + 1: a quotient of floats rounds to 1 or more exactly when w >= s, and to less than -1
-      // exactly when -w > s (the neighbours of s are further than half an ulp of 1 away from it, relatively)
-      auto level = [&](float x) { return x < 0.f ? (-x > s_new ? -3.f : -1.f) : (x >= s_new ? 3.f : 1.f); };
+      // exactly when -w > s (the neighbours of s are further than half an ulp of 1 away from it, relatively); it underflows to
+      // -0, whose level is that of 0, when -w <= s 2^-150.  A NaN takes the lowest level.
+      auto level = [&](float x) { return x >= -vanishes ? (x >= s_new ? 3.f : 1.f) : (-x <= s_new ? -1.f : -3.f); };
       fa = make_float2(level(wa.x), level(wa.y)); fb = make_float2(level(wb.x), level(wb.y));
       const float2 ta = add2(fa, splat(ROUND_MAGIC)), tb = add2(fb, splat(ROUND_MAGIC));
       b0 = __float_as_uint(ta.x); b1 = __float_as_uint(ta.y); b2 = __float_as_uint(tb.x); b3 = __float_as_uint(tb.y);

@@ -73,3 +73,36 @@ def test_fused_update_at_the_edges_of_its_row_variants(grid, ffn):
         finally:
             p.close()
             q.close()
+
+
+def test_half_integer_codes_of_the_update_are_those_of_the_quantizer():
+    """A learning rate of zero leaves the weights as they are, so the update has to leave the codes that the quantizer made of
+    them (by the division of Eq. 1): around the levels' ends, where the quotient underflows, and for values that are no numbers."""
+    wl = synth.shrink(synth.workloads()["base3_w2a8"], n_layers=1, hidden=64, n_heads=1, ffn=128, seq=24, batch=2, len_lo=5, len_hi=24)
+    p = Problem(wl)
+    try:
+        m, f32 = p.m, np.float32
+        w, s = p.student[0]["W1"], np.asarray(p.ws[0]["W1"], f32).reshape(-1)
+        s[:] = np.exp2(np.linspace(-12, 12, s.size)).astype(f32) * np.linspace(1, 2, s.size, endpoint=False).astype(f32)
+        edges = [0.0, 1e-45, 1e-44, 1e-42, 1e-38, np.inf]
+        for r, step in enumerate(s):
+            near = [np.nextafter(step, f32(0)), step, np.nextafter(step, f32(np.inf)), 2 * step]
+            tie = [f32(k) * f32(1e-45) for k in (np.floor(step / 2) + np.arange(-1, 3)) if k > 0]
+            row = np.array(edges + near + tie, f32)
+            row = np.concatenate([row, -row, [f32(np.nan)]])
+            w[r, :row.size] = row
+        m.load_student(p.student)
+        m.set_steps(p.ws, p.a, p.off)
+        m.quantize_weights()
+        before = [x.clone() for x in m.weight_codes(0, B.W1)]
+        m.forward_teacher(p.xd, p.vld, wl.batch, wl.seq)
+        m.forward_student(p.xd, p.vld, wl.batch, wl.seq)
+        m.recon_loss()
+        m.backward()
+        m.step(B.make_optim(lr=0.0, step=1, weight_decay=0.0))
+        assert np.array_equal(m.get_steps()[0][0]["W1"].reshape(-1), s)
+        after = m.weight_codes(0, B.W1)
+        assert set(after[0].unique().tolist()) == {-3, -1, 1, 3}
+        assert torch.equal(after[0], before[0]) and torch.equal(after[1], before[1])
+    finally:
+        p.close()
