@@ -276,13 +276,14 @@ int32_t mrem_selftest_wait_limit(mrem_ctx* ctx);
  * time of a step captured this way is the sum of its kernels' run times).  Takes effect at the next call or capture. */
 int32_t mrem_set_two_streams(mrem_ctx* ctx, int32_t on);
 
-/* Per context (default on): where the shapes allow it (bf16 storage, head size 64, seq <= 128, seq % 8 == 0)
- * the backward of the attention block (Sec. 3.1: the gradients of Q, K, V through the quantized scores,
- * softmax and context products, with the straight-through masks of the Q, K, V, P quantizers) runs as one
- * kernel; off (0) selects the kernel-per-operation path that covers every shape.  Both compute the same
- * quantities; they differ in where intermediates are rounded to the storage type.  Do not change it
- * between a student forward pass and its backward pass (the forward pass writes the codes of the attention
- * probabilities only for the kernel-per-operation path), nor between the capture and the replay of a graph. */
+/* Per context (default on): where the shapes allow it (bf16 storage, head size 64, seq <= 384, seq % 8 == 0,
+ * batch * heads <= 1184) the backward of the attention block (Sec. 3.1: the gradients of Q, K, V through the
+ * quantized scores, softmax and context products, with the straight-through masks of the context, Q, K, V, P
+ * quantizers) runs fused: as one kernel up to 128 tokens, as two above; off (0) selects the
+ * kernel-per-operation path that covers every shape.  Both compute the same quantities; they differ in where
+ * intermediates are rounded to the storage type.  Takes effect at the next student forward pass (which writes the
+ * attention probabilities and their codes only for the kernel-per-operation path; its backward pass follows it);
+ * a captured graph keeps the form it was captured with. */
 int32_t mrem_set_fused_attention_backward(mrem_ctx* ctx, int32_t on);
 
 /* Reads the device status word (blocks on the stream): MREM_OK, MREM_ERR_TIMEOUT or MREM_ERR_NONFINITE in
@@ -353,8 +354,8 @@ int32_t mrem_gemm(int32_t dtype, const void* d_a, int32_t a_mn, int64_t lda, int
  *     e_hat = LayerNorm(Q(word)[ids] + pos + type)                           (student tables),
  * Q = Eq. 1 with e_bits on the student's latent word table, one learnable step per row; position and
  * token-type tables and the LayerNorm are not quantized.  c = 1 / (batch * seq * hidden) with loss_mean.
- * Straight-through backward (a row gathered by several tokens gets the sum of their gradients, added in
- * token order); AdamW on word (with its row steps, kept >= 1e-8; the table is re-quantized in the same
+ * Straight-through backward (a row gathered by several tokens gets the sum of their gradients, added in a
+ * fixed order: token order, above 16 tokens in eight runs of it); AdamW on word (with its row steps, kept >= 1e-8; the table is re-quantized in the same
  * pass), pos, type (decayed like weight matrices) and the LayerNorm parameters (not decayed).
  * Stateless: every tensor is the caller's; nothing is allocated. */
 typedef struct {

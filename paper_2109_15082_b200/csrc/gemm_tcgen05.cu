@@ -348,6 +348,9 @@ namespace {
 // the tiles are few and the inner dimension is long.  Alone / shared, us: 216 x 768 x 3072 17.0 / 9.5 (int8 codes 10.4 / 7.4),
 // 216 x 768 x 2304 13.5 / 8.6, 512 x 768 x 3072 17.3 / 11.8, 1024 x 1024 x 4096 22.9 / 17.1, 128 x 1024 x 1024 7.8 / 6.9,
 // 216 x 768 x 768 6.7 / 6.3; on the other side of the line 512 x 1024 x 1024 8.2 / 9.2, 1024 x 1024 x 1024 8.5 / 8.8.
+// No more tiles than all clusters can hold at once: cudaOccupancyMaxActiveClusters gives 74 clusters of two and 33 of four for
+// every variant on an idle chip; the limits, 72 and 32, lie below that (no product of a 768 or 1024 wide layer has one of the
+// few tile counts between).
 int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count, bool can_split, int* splits) {
   const int m_tiles = (M + BLOCK_M - 1) / BLOCK_M;
   int best = 64;
@@ -360,9 +363,9 @@ int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count, bool can
     const double step_us = bn == 64 ? 0.32 : (bn == 128 ? 0.43 : 0.50);
     const double epi_us = bn == 64 ? 0.5 : (bn == 128 ? 1.0 : 2.0);
     const double cost = (double)waves * (k_blocks * step_us + epi_us);
-    if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; *splits = 1; }
     for (int s = 2; s <= 4 && can_split && bn <= 128; s *= 2) {
-      if (tiles * s > (s == 2 ? sm_count - 4 : sm_count - 20) || k_blocks < 4 * s) continue;      // all clusters at once
+      if (tiles * s > (s == 2 ? sm_count - 4 : sm_count - 20) || k_blocks < 4 * s) continue;
       const double exchange_us = 1.5 + 0.012 * (double)(tiles * s);
       const double split_cost = (double)((k_blocks + s - 1) / s) * step_us + epi_us / s + exchange_us;
       if (split_cost < best_cost - 1e-9) { best_cost = split_cost; best = bn; *splits = s; }

@@ -56,7 +56,7 @@ void launch_layernorm_fwd(const void* y, const float* gamma, const float* beta, 
                           void* out, float* mean, float* rstd, const float* step, int qmax, int8_t* q8, void* qt,
                           int dt, cudaStream_t st);
 
-// The bias of a product whose left operand carries an offset beta: beff[i] = b[i] + beta * wscale[i] * rowsum[i] (b null: 0).
+// The bias of a product whose left operand carries an offset beta: beff[i] = b[i] + beta * wscale[i] * rowsum[i].
 struct EffectiveBias { const float *b, *wscale; const int32_t* rowsum; float* beff; int n; };
 // g = stored(gelu(u)); codes of g (asymmetric when offset != null) as int8/uint8 and storage-type numbers.  eb (may be null,
 // needs an offset): the effective bias of the product that reads the codes, on the way.

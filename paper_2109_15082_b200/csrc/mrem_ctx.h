@@ -125,7 +125,7 @@ struct mrem_ctx {
   struct { const float *wp = nullptr, *bp = nullptr, *wc = nullptr, *bc = nullptr; int n_classes = 0; float* logit_loss = nullptr; float* logits = nullptr; } head;
   float loss_share = 1.f;            // this context's share of the whole batch (data parallel: local / global sequences)
   bool use_side_stream = true;       // run the teacher pass and the weight-gradient / update work on the second stream
-  bool fused_attention_bwd = true;   // use the single-kernel attention backward where it applies
+  bool fused_attention_bwd = true;   // use the fused attention backward (one kernel or two) where it applies
   bool codes_fresh = false;          // the weight codes match the current latent weights and steps
   mrem::Tracer tracer;               bool trace_on = false;
   void *h2d_xt, *h2d_xs; int32_t* h2d_len; float* d_loss_e2e;   // inputs and loss of the host-buffer step (fixed: graph inputs)

@@ -212,7 +212,7 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
     launch_quantize_act3(s.qkv, c->dt, M, H, 3 * H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], rx.lo, rx.hi, s.qkv_qt,
                          3 * H, c->stream);
     if (attention_fwd_supported(S, hd, c->dt)) {
-      // (the single-kernel attention backward forms the probabilities again from the codes of Q and K and the row
+      // (the fused attention backward forms the probabilities again from the codes of Q and K and the row
       //  statistics: they and their codes are written out only for the kernel-per-operation backward)
       s.p_kept = !(c->fused_attention_bwd && attention_bwd_supported(S, hd, c->dt, B * h));
       const AttentionStats stats{s.p_alpha, s.p_len, s.p_stat};
