@@ -5,25 +5,37 @@
 //   loss     c * || e_hat - e ||^2,  straight-through backward, AdamW on the student's tables, the word
 //            table's row steps and the LayerNorm parameters; the update re-quantizes the word table.
 // The word table is treated as a weight matrix with `vocab` output rows: its quantizer, straight-through
-// mask and fused AdamW + re-quantization are the kernels of the encoder matrices; LayerNorm, loss and
-// column reductions likewise.  New here: everything per token (both gathers, both LayerNorms, the loss, its
+// mask and fused AdamW + re-quantization are the kernels of the encoder matrices; of rows wider than the kernel
+// below takes, LayerNorm and loss likewise.  New here: everything per token (both gathers, both LayerNorms, the loss, its
 // gradient through the LayerNorm) in one kernel, and everything that adds up the token gradients (rows of the
 // word table, sums over the batch for the position and token-type tables) in a second one, with fixed
 // summation orders.  Nothing is allocated: the caller brings every tensor and one workspace.
 #include <cmath>
 
 #include "../../include/mrem.h"
-#include "optim.cuh"
+#include "row_update.cuh"
 #include "vec.cuh"
 
 namespace mrem {
 
 namespace {
 
-__device__ __forceinline__ void note_token(unsigned* row_first, int* row_last, int* row_count, int id, int t) {
-  atomicMin(row_first + id, (unsigned)t);
-  atomicMax(row_last + id, t);
-  atomicAdd(row_count + id, 1);                                     // (starts at -1)
+// The first and the last token of every id and their number (atomicMin / atomicMax of an index, atomicAdd of 1: no dependence on
+// scheduling); they say which table rows were gathered at all, who adds up a row's gradients, and how far to look.  A launch of
+// its own, so that the rows nobody gathered can be updated beside the token kernels.  One block more than the tokens need prepares
+// the optimizer's scalars.
+__global__ void __launch_bounds__(256) embed_mark_kernel(const int* __restrict__ ids, int M, int vocab, unsigned* __restrict__ row_first,
+                                                         int* __restrict__ row_last, int* __restrict__ row_count, const OptimArgs optim) {
+  pdl_wait();
+  pdl_trigger();
+  const int t = (int)blockIdx.x * 256 + (int)threadIdx.x;
+  if (t < M) {
+    const int id = min(max(ids[t], 0), vocab - 1);
+    atomicMin(row_first + id, (unsigned)t);
+    atomicMax(row_last + id, t);
+    atomicAdd(row_count + id, 1);                                   // (starts at -1)
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && optim.out) optim_prepare(optim);
 }
 
 // y[t, :] = row(ids[t]) + pos[t % S, :] + type[type_ids[t], :], rounded as stored; one block of 128 threads per token.
@@ -33,8 +45,7 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
                                                         const float* __restrict__ scale, const float* __restrict__ pos,
                                                         const float* __restrict__ type, const int* __restrict__ ids,
                                                         const int* __restrict__ type_ids, int S, int H, int vocab, int n_types,
-                                                        T* __restrict__ y, unsigned* row_first, int* row_last,
-                                                        int* row_count, int* __restrict__ status) {
+                                                        T* __restrict__ y, int* __restrict__ status) {
   pdl_wait();
   pdl_trigger();
   const long long t = blockIdx.x;
@@ -44,7 +55,6 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
     id = min(max(id, 0), vocab - 1);
     tt = min(max(tt, 0), n_types - 1);
   }
-  if (threadIdx.x == 0 && row_first) note_token(row_first, row_last, row_count, id, (int)t);
   const int s = (int)(t % S);
   const float sc = codes ? scale[id] : 0.f;
   for (int c = threadIdx.x; c < H; c += blockDim.x) {
@@ -59,10 +69,8 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
 // and without six of their seven launches.  Latency bounds it: with one vector per thread a token is one round of loads and three block sums
 // (both modules' means together, both variances, the two sums of the backward), and eight blocks share an SM.
 // (One warp per token with the whole row in its 128 registers: 22 % of the warps active, 29 us; the step of 30522 x 1024, 32 x 128
-// tokens 204 -> 200 us, of 30522 x 768, 5 x 56 tokens 154 -> 150.)  The first and the last token of every id and their number are noted (atomicMin /
-// atomicMax of an index, atomicAdd of 1: no dependence on scheduling); they say later which table rows were gathered at
-// all, who adds up a row's gradients, and how far to look.  One block more than the tokens need prepares the optimizer's
-// scalars beside them.
+// tokens 204 -> 200 us, of 30522 x 768, 5 x 56 tokens 154 -> 150.)  The blocks beyond row_blocks update idle rows of the word table,
+// a warp each: 25 us without them, 30 with 1,900 rows (57 MB, 8.5 us of the table's own update).
 constexpr int MAX_W = 4;
 struct EmbedRow {
   const float *t_word, *t_pos, *t_type, *t_g, *t_b;           // teacher tables and LayerNorm
@@ -71,10 +79,10 @@ struct EmbedRow {
   const int *ids, *type_ids;
   int S, H, vocab, n_types; long long M;
   float eps, c;                                               // c: loss scale
-  int* status; unsigned* row_first; int *row_last, *row_count; unsigned* ticket;   // marks and ticket start as 0xffffffff
+  int* status; unsigned* ticket;                              // (the ticket starts as 0xffffffff)
   float *mean, *rstd, *loss_partial, *loss;
-  int* col_counters; int n_col_counters;
-  int row_blocks; OptimArgs optim;
+  int row_blocks;
+  IdleRows idle;
 };
 
 template <int V>
@@ -114,12 +122,10 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
   __shared__ float2 part[3][W * TPB];                         // one set per sum: the next token's first is behind this one's last
   __shared__ int last;
   const int wid = threadIdx.x >> 5, H = p.H, c = (int)(threadIdx.x % (32 * W)) * V;
-  if ((int)blockIdx.x == p.row_blocks) {
-    if (threadIdx.x == 0) optim_prepare(p.optim);
+  if ((int)blockIdx.x >= p.row_blocks) {
+    update_idle_rows<2>(p.idle, ((int)blockIdx.x - p.row_blocks) * W * TPB + wid, ((int)gridDim.x - p.row_blocks) * W * TPB);
     return;
   }
-  if (blockIdx.x == 0)                                        // tickets of the column reduction that follows
-    for (int i = threadIdx.x; i < p.n_col_counters; i += blockDim.x) p.col_counters[i] = 0;
   float err = 0.f;
   for (long long t0 = (long long)blockIdx.x * TPB; t0 < p.M; t0 += (long long)p.row_blocks * TPB) {
     const long long t = t0 + wid / W;
@@ -130,7 +136,6 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
       id = min(max(id, 0), p.vocab - 1);
       tt = min(max(tt, 0), p.n_types - 1);
     }
-    if (live && c == 0) note_token(p.row_first, p.row_last, p.row_count, id, (int)t);
     const long long row = (long long)id * H, prow = (t % p.S) * (long long)H, trow = (long long)tt * H, base = t * H;
     float et[V], y[V];                                        // teacher row, student row, as stored before the LayerNorm
 #pragma unroll
@@ -237,24 +242,30 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 //   max_pos blocks: one position each, two half sums over the batch (even and odd sequences), then that row's update.
 //   TYPE_CHUNKS blocks per token type: one chunk of tokens each; the last chunk to finish adds the chunks in index order
 //     and updates the row.
-//   one block: update of the LayerNorm's parameters (their gradients come from the launch before).
-//   the rest, one warp per token and group of TAB_COLS columns: word table.  The warp of the FIRST token with an id adds the gradients of all tokens with
+//   LN_CHUNKS blocks: the LayerNorm's parameters, the same way.
+//   one warp per token and group of TAB_COLS columns: word table.  The warp of the FIRST token with an id adds the gradients of all tokens with
 //     it in token order: it compares 128 ids at a time up to the last one and keeps four rows' loads in flight.  A row
 //     gathered by more than WARP_MAX tokens is left to the whole block, its warps taking consecutive eighths of the tokens and
 //     the eight sums being added in warp order.  Warp w of block i has token w * blocks + i: frequent ids first appear among
 //     the first tokens, and would otherwise all meet in one block.
-// The former occurrence lists (one thread per token walking all the others, twice) alone took 300 us at 4096 tokens; this
-// kernel takes 30 us (32 x 128 tokens, hidden 1024; the table update 136 of the step's
-// 200).  Three blocks per SM: four spill, 200 -> 207 us there although 280 tokens take 148 instead of 150.
+//   The blocks beyond update idle rows of the word table, a warp each: memory that the sums leave idle.
+// The sums are chains of dependent loads.  The longest were the last chunks' totals (a column per thread, eight chunks at a time; now
+// four columns and sixteen chunks) and the walk over the ids (the next 128 are on their way now): step 217 -> 192 us at 32 x 128
+// tokens, 136 -> 125 at 5 x 56.  Three blocks: four spill, 200 -> 207 us there although 280 tokens take 148 instead of 150.
 constexpr int TYPE_CHUNKS = 64;
+constexpr int LN_CHUNKS = 48;
 constexpr int TAB_COLS = 512;                                 // columns a word-table block works on
 constexpr int WARP_MAX = 16;                                  // tokens of one id that a single warp adds up
 struct EmbedTables {
-  const int *ids, *type_ids; const unsigned* row_first; const int *row_last, *row_count; unsigned* type_ticket;
+  const int *ids, *type_ids; const unsigned* row_first; const int *row_last, *row_count; unsigned* type_ticket;      // (n_types + 1 tickets)
   int B, S, H, vocab, n_types, max_pos, M;
-  float *g_word, *g_pos, *g_type, *type_partial;
+  const float *mean, *rstd;
+  float *g_word, *g_pos, *g_type, *type_partial, *ln_partial;
   const OptimScalars* sc;                                     // null: gradients only
   AdamEntry pos, type, ln_g, ln_b;
+  bool vec;                                                   // these tensors start on 16-byte boundaries
+  int sum_blocks;                                             // blocks of the sums; those beyond take idle rows
+  IdleRows idle;
 };
 
 __device__ __forceinline__ void adam_at(const AdamEntry& e, const OptimScalars& o, long long i, float g) {
@@ -262,6 +273,37 @@ __device__ __forceinline__ void adam_at(const AdamEntry& e, const OptimScalars& 
   e.p[i] = adam_one(e.p[i], g, m, v, o, e.wd, e.min_value);
   e.m[i] = m;
   e.v[i] = v;
+}
+
+// the same of four consecutive elements from i on (16-byte aligned)
+__device__ __forceinline__ void adam4_at(const AdamEntry& e, const OptimScalars& o, long long i, float4 g) {
+  float4 p = *reinterpret_cast<const float4*>(e.p + i), m = *reinterpret_cast<const float4*>(e.m + i), v = *reinterpret_cast<const float4*>(e.v + i);
+  p.x = adam_one(p.x, g.x, m.x, v.x, o, e.wd, e.min_value);
+  p.y = adam_one(p.y, g.y, m.y, v.y, o, e.wd, e.min_value);
+  p.z = adam_one(p.z, g.z, m.z, v.z, o, e.wd, e.min_value);
+  p.w = adam_one(p.w, g.w, m.w, v.w, o, e.wd, e.min_value);
+  *reinterpret_cast<float4*>(e.p + i) = p;
+  *reinterpret_cast<float4*>(e.m + i) = m;
+  *reinterpret_cast<float4*>(e.v + i) = v;
+}
+// Gradients and tensors of the caller: 16-byte accesses where they allow them (`vec`).
+__device__ __forceinline__ void store4(float* p, float4 g, bool vec) {
+  if (vec) { *reinterpret_cast<float4*>(p) = g; return; }
+  p[0] = g.x; p[1] = g.y; p[2] = g.z; p[3] = g.w;
+}
+__device__ __forceinline__ void update4(const AdamEntry& e, const OptimScalars& o, long long i, float4 g, bool vec) {
+  if (vec) { adam4_at(e, o, i, g); return; }
+  adam_at(e, o, i, g.x); adam_at(e, o, i + 1, g.y); adam_at(e, o, i + 2, g.z); adam_at(e, o, i + 3, g.w);
+}
+// Sums over `n` chunks of part[ch * stride + c .. + 4), in chunk order, sixteen chunks' loads in flight.
+__device__ __forceinline__ float4 sum_chunks4(const float* part, int n, long long stride, int c) {
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+  for (int ch = 0; ch < n; ++ch) {
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(part + ch * stride + c));
+    acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
+  }
+  return acc;
 }
 
 // acc += the rows dy[t, c0 ..] of the tokens t in [b0, b1) whose (clamped) id is `id`, in token order, by one warp.
@@ -274,10 +316,17 @@ __device__ __forceinline__ void add_rows_of_id(const EmbedTables& p, const T* __
   for (int i = 0; i < NV; ++i)
 #pragma unroll
     for (int j = 0; j < V; ++j) acc[i][j] = 0.f;
+  int next[4];                                                // ids of the next 128 tokens, on their way while these are compared
+  auto fetch = [&](int b) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) next[k] = b + 32 * k + lane < b1 ? p.ids[b + 32 * k + lane] : -1;
+  };
+  fetch(b0);
   for (int b = b0; b < b1; b += 128) {
     int mine[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) mine[k] = b + 32 * k + lane < b1 ? min(max(p.ids[b + 32 * k + lane], 0), p.vocab - 1) : -1;
+    for (int k = 0; k < 4; ++k) mine[k] = b + 32 * k + lane < b1 ? min(max(next[k], 0), p.vocab - 1) : -1;
+    fetch(b + 128);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       unsigned hits = __ballot_sync(0xffffffffu, mine[k] == id);
@@ -316,9 +365,14 @@ __device__ __forceinline__ void add_rows_of_id(const EmbedTables& p, const T* __
 }
 
 template <typename T, int V>
-__global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_constant__ EmbedTables p, const T* __restrict__ dy) {
+__global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_constant__ EmbedTables p, const T* __restrict__ dy, const T* __restrict__ dsum,
+                                                              const T* __restrict__ y_s) {
   pdl_wait();
   pdl_trigger();
+  if ((int)blockIdx.x >= p.sum_blocks) {
+    update_idle_rows<2>(p.idle, ((int)blockIdx.x - p.sum_blocks) * 8 + (int)(threadIdx.x >> 5), ((int)gridDim.x - p.sum_blocks) * 8);
+    return;
+  }
   __shared__ float red[8][TAB_COLS];
   __shared__ int flag, group[8];
   constexpr int NV = TAB_COLS / (32 * V);                     // vectors per lane in a pass
@@ -368,10 +422,10 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
         for (int j = 0; j < V; ++j) red[j][tx] += acc[j];
       }
       __syncthreads();
-      for (int i = threadIdx.x; i < 128 * V && c0 + i < H; i += 256) {
-        const float g = red[i % V][i / V];
-        dst[c0 + i] = g;
-        if (is_pos && p.sc) adam_at(p.pos, o, (long long)s * H + c0 + i, g);
+      for (int i = 4 * threadIdx.x; i < 128 * V && c0 + i < H; i += 1024) {
+        const float4 g = make_float4(red[i % V][i / V], red[i % V + 1][i / V], red[i % V + 2][i / V], red[i % V + 3][i / V]);
+        store4(dst + c0 + i, g, p.vec || !is_pos);
+        if (is_pos && p.sc) update4(p.pos, o, (long long)s * H + c0 + i, g, p.vec);
       }
       __syncthreads();
     }
@@ -382,26 +436,67 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
     __syncthreads();
     if (!flag) return;
     __threadfence();
-    for (int c = threadIdx.x; c < H; c += 256) {
-      float acc = 0.f;
-#pragma unroll 8
-      for (int ch = 0; ch < TYPE_CHUNKS; ++ch) acc += __ldcg(p.type_partial + ((long long)ch * p.n_types + k) * H + c);
-      p.g_type[(long long)k * H + c] = acc;
-      if (p.sc) adam_at(p.type, o, (long long)k * H + c, acc);
+    for (int c = 4 * threadIdx.x; c < H; c += 1024) {
+      const float4 acc = sum_chunks4(p.type_partial + (long long)k * H, TYPE_CHUNKS, (long long)p.n_types * H, c);
+      store4(p.g_type + (long long)k * H + c, acc, p.vec);
+      if (p.sc) update4(p.type, o, (long long)k * H + c, acc, p.vec);
     }
     return;
   }
   blk -= n_sum;
-  if (blk == 0) {
-    if (p.sc)
-      for (int c = threadIdx.x; c < H; c += 256) {
-        adam_at(p.ln_g, o, c, p.ln_g.g[c]);
-        adam_at(p.ln_b, o, c, p.ln_b.g[c]);
+  if (blk < LN_CHUNKS) {
+    // gradients of the LayerNorm's gain and bias: sums over the tokens of d * (y - mean) * rstd and of d
+    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7, per = (p.M + LN_CHUNKS - 1) / LN_CHUNKS, t0 = blk * per, t1 = min(p.M, t0 + per);
+    for (int c0 = 0; c0 < H; c0 += 128 * V) {
+      const int c = c0 + tx * V;
+      float ab[V], ag[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) ab[j] = ag[j] = 0.f;
+      if (c < H) {
+#pragma unroll 4
+        for (int t = t0 + ty; t < t1; t += 2) {
+          const float mu = p.mean[t], rs = p.rstd[t];
+          float d[V], y[V];
+          load_vec<T, V>(dsum + (long long)t * H + c, d);
+          load_vec<T, V>(y_s + (long long)t * H + c, y);
+#pragma unroll
+          for (int j = 0; j < V; ++j) { ab[j] += d[j]; ag[j] += d[j] * ((y[j] - mu) * rs); }
+        }
       }
+      for (int k = 0; k < 2; ++k) {
+        float* dst = p.ln_partial + ((long long)blk * 2 + k) * H;
+        if (ty == 1) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) red[j][tx] = k ? ag[j] : ab[j];
+        }
+        __syncthreads();
+        if (ty == 0) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) red[j][tx] += k ? ag[j] : ab[j];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 128 * V && c0 + i < H; i += 256) dst[c0 + i] = red[i % V][i / V];
+        __syncthreads();
+      }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + p.n_types, 1u) + 2u == (unsigned)LN_CHUNKS;
+    __syncthreads();
+    if (!flag) return;
+    __threadfence();
+    for (int c = 4 * threadIdx.x; c < 2 * H; c += 1024) {      // (H is a multiple of 16: no group of four crosses the two)
+      const float4 acc = sum_chunks4(p.ln_partial, LN_CHUNKS, 2ll * H, c);
+      const AdamEntry& e = c < H ? p.ln_b : p.ln_g;
+      const int i = c < H ? c : c - H;
+      store4(e.g + i, acc, p.vec);
+      if (p.sc) update4(e, o, i, acc, p.vec);
+    }
     return;
   }
-  const int nb = (p.M + 7) / 8, c0 = ((blk - 1) / nb) * TAB_COLS;
-  blk = (blk - 1) % nb;
+  blk -= LN_CHUNKS;
+  const int nb = (p.M + 7) / 8, c0 = (blk / nb) * TAB_COLS;
+  blk = blk % nb;
   const int tok = wid * nb + blk;
   int mine = -1, count = 0;                                   // id whose row this warp's token is the first to gather
   if (tok < p.M) {
@@ -453,12 +548,10 @@ struct Carve {                         // the workspace, cut the same way by the
 };
 struct EmbedScratch {
   void *y_t, *y_s, *dE, *dy, *dsum;
-  float *mean, *rstd, *col_scratch, *loss_partial;
-  long long col_plane;
-  int* col_counters;
+  float *mean, *rstd, *ln_partial, *loss_partial;
   int8_t* codes; int32_t* rowsum; float* scale;
   OptimScalars* optim_sc;
-  unsigned* marks; size_t mark_bytes;      // first and last token of every id and their number, then the loss and token-type tickets
+  unsigned* marks; size_t mark_bytes;      // first and last token of every id and their number, then the tickets of the loss, the token types and the LayerNorm
   float* type_partial;
   size_t bytes;
 };
@@ -471,11 +564,9 @@ EmbedScratch carve(const mrem_embed_desc& d, long long max_tokens, void* base) {
   s.rowsum = (int32_t*)A.take(sizeof(int32_t) * d.vocab);
   s.scale = (float*)A.take(sizeof(float) * d.vocab);
   s.optim_sc = (OptimScalars*)A.take(sizeof(OptimScalars));
-  s.col_plane = (long long)COL_CHUNKS * d.hidden;
-  s.col_scratch = (float*)A.take(sizeof(float) * 3 * s.col_plane);
-  s.col_counters = (int*)A.take(sizeof(int) * (d.hidden / 32 + 2));
+  s.ln_partial = (float*)A.take(sizeof(float) * 2 * LN_CHUNKS * d.hidden);
   s.loss_partial = (float*)A.take(sizeof(float) * RED_BLOCKS);
-  s.mark_bytes = sizeof(unsigned) * (3 * (size_t)d.vocab + 1 + d.n_types);
+  s.mark_bytes = sizeof(unsigned) * (3 * (size_t)d.vocab + 2 + d.n_types);
   s.marks = (unsigned*)A.take(s.mark_bytes);
   s.type_partial = (float*)A.take(sizeof(float) * (size_t)TYPE_CHUNKS * d.n_types * d.hidden);
   const size_t es = d.act_dtype == MREM_BF16 ? 2 : 4;
@@ -548,6 +639,22 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   void* dsum = s.dsum;                                     // the gradient the LayerNorm sees
   OptimArgs oa{};
   if (o) oa = OptimArgs{s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay};
+  launch_k(embed_mark_kernel, (unsigned)((M + 255) / 256 + (o ? 1 : 0)), 256, 0, st, d_ids, (int)M, V, row_first, row_last, row_count, oa);
+  // Update of the word table: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one pass (the
+  // small tensors are updated by the launch that adds up their gradients, the other embedding tables decayed like weight matrices,
+  // LayerNorm not).  The rows that no token gathered need nothing of this step but the marks.  The two launches before the last take
+  // as many of them as memory can serve beside their own chains of loads; the last one, which is bound by memory, the rest: its
+  // blocks keep more bytes in flight.  30522 x 1024 with 32 x 128 tokens 199 -> 192 us, 30522 x 768 with 5 x 56 tokens 150 -> 125.
+  // (No idle rows beside the sums of many tokens: 197 and 125; seven eighths of the table beside the sums: 204 and 128; idle blocks
+  // spread evenly among those of the sums: 196 and 126.)
+  const RowUpdate table{x->word, x->g_word, x->m_word, x->v_word, x->word_step, x->m_word_step, x->v_word_step, nullptr,
+                        s.codes, s.rowsum, s.scale, nullptr, V, H};
+  int idle_at = o ? 0 : V;                                   // the next idle row to hand out
+  auto take_idle = [&](long long n) {
+    const int first = idle_at;
+    idle_at = (int)(n < 0 ? first : (first + n < V ? first + n : V));
+    return IdleRows{table, s.optim_sc, row_first, d->e_bits, first, idle_at};
+  };
   const int row_warps = (H + 32 * (dt == 1 ? 8 : 4) - 1) / (32 * (dt == 1 ? 8 : 4));
   if (row_warps <= MAX_W && aligned) {
     // one vector per thread: everything per token in one kernel
@@ -555,10 +662,11 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
     const long long want = (M + tpb - 1) / tpb;
     const int row_blocks = (int)(want < RED_BLOCKS ? want : RED_BLOCKS);
     const EmbedRow er{x->t_word, x->t_pos, x->t_type, x->t_ln_g, x->t_ln_b, x->pos, x->type, x->ln_g, x->ln_b, s.codes, s.scale, d_ids, d_type_ids,
-                      (int)seq, H, V, (int)d->n_types, M, d->ln_eps, cc, d_status, row_first, row_last, row_count, loss_ticket,
-                      s.mean, s.rstd, s.loss_partial, d_loss, s.col_counters, H / 32 + 2, row_blocks, oa};
-    const unsigned grid = (unsigned)(row_blocks + (o ? 1 : 0));
-    Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)), 0, st);
+                      (int)seq, H, V, (int)d->n_types, M, d->ln_eps, cc, d_status, loss_ticket,
+                      s.mean, s.rstd, s.loss_partial, d_loss, row_blocks, take_idle(M / 3 + 550000 / H)};
+    const int idle_warps = row_warps * tpb;
+    const unsigned grid = (unsigned)(row_blocks + (er.idle.end - er.idle.first + idle_warps - 1) / idle_warps);
+    Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)) + 29.0 * H * (er.idle.end - er.idle.first), 0, st);
 #define MREM_ROW(T, V, W) launch_k(embed_row_kernel<T, V, W>, grid, 32 * W * tokens_per_block(W), 0, st, er, (const T*)d_extra_grad, (T*)d_e_teacher, (T*)d_e_student, (T*)s.y_s, (T*)s.dsum, (T*)s.dy)
 #define MREM_ROWS(T, V) do { if (row_warps == 1) MREM_ROW(T, V, 1); else if (row_warps == 2) MREM_ROW(T, V, 2); else if (row_warps == 3) MREM_ROW(T, V, 3); else MREM_ROW(T, V, 4); } while (0)
     if (dt == 1) MREM_ROWS(bf16, 8); else MREM_ROWS(float, 4);
@@ -567,8 +675,8 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   } else {
     // wide rows: both embedding sums, the two LayerNorms, the loss and the LayerNorm backward as kernels of their own
 #define MREM_EMB(T) do { \
-    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, x->t_word, (const int8_t*)nullptr, (const float*)nullptr, x->t_pos, x->t_type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_t, (unsigned*)nullptr, (int*)nullptr, (int*)nullptr, d_status); \
-    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, (const float*)x->word, (const int8_t*)s.codes, (const float*)s.scale, (const float*)x->pos, (const float*)x->type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_s, row_first, row_last, row_count, d_status); } while (0)
+    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, x->t_word, (const int8_t*)nullptr, (const float*)nullptr, x->t_pos, x->t_type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_t, d_status); \
+    launch_k(embed_sum_kernel<T>, (unsigned)M, 128, 0, st, (const float*)x->word, (const int8_t*)s.codes, (const float*)s.scale, (const float*)x->pos, (const float*)x->type, d_ids, d_type_ids, (int)seq, H, V, (int)d->n_types, (T*)s.y_s, d_status); } while (0)
     if (dt == 1) MREM_EMB(bf16); else MREM_EMB(float);
 #undef MREM_EMB
     launch_layernorm_fwd(s.y_t, x->t_ln_g, x->t_ln_b, d->ln_eps, M, H, d_e_teacher, nullptr, nullptr, nullptr, 0, nullptr, nullptr, dt, st);
@@ -577,35 +685,36 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
     launch_loss_finalize(s.loss_partial, 1, cc, d_loss, nullptr, st);
     // (with a gradient arriving from the layers the embedding feeds, the LayerNorm sees the sum of the two)
     launch_layernorm_bwd(s.dE, d_extra_grad, s.y_s, s.mean, s.rstd, x->ln_g, M, H, s.dy, d_extra_grad ? s.dsum : nullptr, dt, st);
-    if (cudaMemsetAsync(s.col_counters, 0, sizeof(int) * (H / 32 + 2), st) != cudaSuccess) return MREM_ERR_CUDA;
     if (!d_extra_grad) dsum = s.dE;
-    if (o) launch_optim_prepare(s.optim_sc, x->d_step_counter, o->step, o->lr, o->decay_total_steps, o->beta1, o->beta2, o->eps, o->weight_decay, st);
   }
-  launch_col_reduce(dsum, H, s.y_s, s.mean, s.rstd, nullptr, 0, M, H, x->g_ln_b, x->g_ln_g, nullptr, s.col_scratch, s.col_plane,
-                    s.col_counters, dt, st);
   // word, position and token-type tables: sums of the token gradients.  Rows of the word table that no token gathered are
   // cleared by the update (row_first says which they are), without one here.
   if (!o && cudaMemsetAsync(x->g_word, 0, sizeof(float) * (size_t)V * H, st) != cudaSuccess) return MREM_ERR_CUDA;
+  const int n_sum = (int)(d->max_pos + (long long)TYPE_CHUNKS * d->n_types + LN_CHUNKS + ((M + 7) / 8) * ((H + TAB_COLS - 1) / TAB_COLS));
+  bool vec = true;
+  const float* const small[] = {x->pos, x->type, x->ln_g, x->ln_b, x->g_pos, x->g_type, x->g_ln_g, x->g_ln_b};
+  for (const float* q : small) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+  if (o) {
+    const float* const moments[] = {x->m_pos, x->v_pos, x->m_type, x->v_type, x->m_ln_g, x->v_ln_g, x->m_ln_b, x->v_ln_b};
+    for (const float* q : moments) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+  }
   const EmbedTables tb{d_ids, d_type_ids, row_first, row_last, row_count, type_ticket, (int)batch, (int)seq, H, V, (int)d->n_types,
-                       (int)d->max_pos, (int)M, x->g_word, x->g_pos, x->g_type, s.type_partial, o ? s.optim_sc : nullptr,
+                       (int)d->max_pos, (int)M, s.mean, s.rstd, x->g_word, x->g_pos, x->g_type, s.type_partial, s.ln_partial, o ? s.optim_sc : nullptr,
                        {x->pos, x->g_pos, x->m_pos, x->v_pos, 0, 1.f, -INFINITY}, {x->type, x->g_type, x->m_type, x->v_type, 0, 1.f, -INFINITY},
-                       {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, 0, 0.f, -INFINITY}, {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, 0, 0.f, -INFINITY}};
-  const unsigned tgrid = (unsigned)(d->max_pos + (long long)TYPE_CHUNKS * d->n_types + 1 + ((M + 7) / 8) * ((H + TAB_COLS - 1) / TAB_COLS));
+                       {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, 0, 0.f, -INFINITY}, {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, 0, 0.f, -INFINITY},
+                       vec, n_sum, take_idle(M / 3 + 3400000 / H)};
+  const unsigned tgrid = (unsigned)(n_sum + (tb.idle.end - tb.idle.first + 7) / 8);
   {
-    Scope sc("embed_tables", (double)M * H * 3.0 * (dt == 1 ? 2.0 : 4.0), 0, st);
-    if (dt == 1) launch_k(embed_tables_kernel<bf16, 8>, tgrid, 256, 0, st, tb, (const bf16*)s.dy);
-    else launch_k(embed_tables_kernel<float, 4>, tgrid, 256, 0, st, tb, (const float*)s.dy);
+    Scope sc("embed_tables", (double)M * H * 5.0 * (dt == 1 ? 2.0 : 4.0) + 29.0 * H * (tb.idle.end - tb.idle.first), 0, st);
+    if (dt == 1) launch_k(embed_tables_kernel<bf16, 8>, tgrid, 256, 0, st, tb, (const bf16*)s.dy, (const bf16*)dsum, (const bf16*)s.y_s);
+    else launch_k(embed_tables_kernel<float, 4>, tgrid, 256, 0, st, tb, (const float*)s.dy, (const float*)dsum, (const float*)s.y_s);
   }
   if (!o) {
     // gradients only: the word table's straight-through mask and its row-step gradients, left in g_word / g_word_step
     launch_ste_weight(x->word, x->word_step, 1, d->e_bits, 0, x->g_word, V, H, x->g_word_step, st);
     return cudaGetLastError() == cudaSuccess ? MREM_OK : MREM_ERR_CUDA;
   }
-  // update of the word table: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one
-  // pass (the small tensors, the other embedding tables decayed like weight matrices, LayerNorm not, are updated above)
-  const RowUpdate table{x->word, x->g_word, x->m_word, x->v_word, x->word_step, x->m_word_step, x->v_word_step, nullptr,
-                        s.codes, s.rowsum, s.scale, nullptr, V, H};
-  launch_fused_weight_update(&table, 1, s.optim_sc, d->e_bits, 0, 1, 1, dt, st, row_first);
+  launch_table_update(take_idle(V), TokenRows{d_ids, row_first, (int)M}, dt, st);
   return cudaGetLastError() == cudaSuccess ? MREM_OK : MREM_ERR_CUDA;
 }
 

@@ -200,8 +200,7 @@ void launch_adamw_table(const AdamEntry* d_table, int n_entries, long long total
 
 // Fused per-row update of weight matrices and their per-row steps: step gradient (or ds_in when the
 // gradients were already masked), AdamW on step and weights, re-quantization (codes, row sums,
-// scale, dequantized row).  row_used (may be null): one word per row, 0xffffffff where no gradient arrived; such a row's
-// g is taken as zero without being read, and written as zero (grid 0 and one matrix only).
+// scale, dequantized row).
 struct RowUpdate {
   float *w, *g, *m, *v;                // latent weights, their gradient, moments: rows x cols
   float *steps, *m_s, *v_s;            // one step per row, its moments
@@ -212,7 +211,11 @@ struct RowUpdate {
 constexpr int MAX_ROW_UPDATES = 4;
 // `n` matrices (at most MAX_ROW_UPDATES) in one launch.
 void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
-                                int dt, cudaStream_t st, const unsigned* row_used = nullptr);
+                                int dt, cudaStream_t st);
+// The same of a table (grid 0, no dequantized rows) whose rows `tokens` gathered, and of the idle rows of a range in the same launch.
+struct TokenRows { const int* ids; const unsigned* row_first; int n; };      // n tokens; the first one with an id, per row
+struct IdleRows;                                                             // row_update.cuh
+void launch_table_update(const IdleRows& idle, const TokenRows& tokens, int dt, cudaStream_t st);
 
 // ---- step-size initialisation
 // Per-row max|w| or mean|w| -> steps (per row, or one value when !per_row: two passes).

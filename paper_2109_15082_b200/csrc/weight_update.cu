@@ -10,7 +10,7 @@
 // (rows up to 4096 wide; longer rows are re-read).  Traffic per weight: read w, g, m, v
 // (16 B), write w, m, v (12 B), codes (1 B) and the dequantized value (2 or 4 B); the separate
 // passes it replaces move about twice that.
-#include "optim.cuh"
+#include "row_update.cuh"
 
 namespace mrem {
 
@@ -50,20 +50,13 @@ __device__ __forceinline__ float2 step_grad2(float2 acc, float2 w, float2 d, flo
   const float2 inside = make_float2(in0 ? -z.x : 0.f, in1 ? -z.y : 0.f);
   return fma2(d, add2(level, inside), acc);
 }
-struct Adam2 { float2 b1, ob1, b2, ob2, rsq, eps, neg_lr, decay; };
-__device__ __forceinline__ float2 adam2(float2 p, float2 g, float2& m, float2& v, const Adam2& a) {      // adam_one of both
-  m = fma2(a.b1, m, mul2(a.ob1, g));
-  v = fma2(a.b2, v, mul2(mul2(a.ob2, g), g));
-  const float2 denom = fma2(make_float2(sqrt_approx(v.x), sqrt_approx(v.y)), a.rsq, a.eps), num = mul2(a.neg_lr, m);
-  return add2(mul2(p, a.decay), make_float2(__fdividef(num.x, denom.x), __fdividef(num.y, denom.y)));
-}
-
 struct UpdateParams {
   RowUpdate mat[MAX_ROW_UPDATES];
   int row_end[MAX_ROW_UPDATES];        // running row count: matrix i owns the blocks [row_end[i - 1], row_end[i])
   int n, bits, train_w, train_s;
   const OptimScalars* sc;
-  const unsigned* row_used;
+  TokenRows tokens;
+  IdleRows idle;
 };
 
 // One block of NT threads per row, NV float4 vectors of w, g, m and v per thread in registers; rows wider than the widest
@@ -79,8 +72,9 @@ struct UpdateParams {
 #define UPD_VARIANTS(X) X(0, 96, 2, 10) X(1, 64, 4, 10) X(2, 128, 4, 5) X(3, 192, 4, 3) X(4, 256, 4, 2)
 constexpr int UPD_WIDEST = 4;
 // GRID (the weight grid, 0: Eq. 1's integers, 1: half-integer 2-bit levels) is a template parameter: the per-weight code
-// then holds one of the two rules, not both under predicates.  SPARSE: row_used says which rows got a gradient at all (an
-// embedding table, one matrix per launch: its pointers stay at fixed places of the parameters, 235 -> 204 us for the step).
+// then holds one of the two rules, not both under predicates.  SPARSE: an embedding table, one matrix per launch (its pointers
+// stay at fixed places of the parameters, 235 -> 204 us for the step).  Block b updates the row that token b gathered, if it is the
+// first to gather it; the blocks beyond the tokens have an idle row each: g is not read, and is cleared here instead of by a pass before.
 template <typename T, int NV, int NT, int BLOCKS, int GRID, bool SPARSE>
 __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const __grid_constant__ UpdateParams P) {
   pdl_wait();
@@ -90,13 +84,19 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
   __shared__ float ds_sh[NW];
   __shared__ int sum_sh[NW];
   int mi = 0;
+  int block_row = (int)blockIdx.x;
+  bool no_grad = false;
+  if (SPARSE) {
+    no_grad = block_row >= P.tokens.n;
+    const int id = no_grad ? P.idle.first + block_row - P.tokens.n : min(max(P.tokens.ids[block_row], 0), P.mat[0].rows - 1);
+    if (P.tokens.row_first[id] != (no_grad ? 0xffffffffu : (unsigned)block_row)) return;
+    block_row = id;
+  }
   if (!SPARSE)
     while (mi + 1 < P.n && (int)blockIdx.x >= P.row_end[mi]) ++mi;
   const RowUpdate& M = P.mat[mi];
-  const int row = (int)blockIdx.x - (mi ? P.row_end[mi - 1] : 0), t = threadIdx.x;
+  const int row = block_row - (mi ? P.row_end[mi - 1] : 0), t = threadIdx.x;
   const int train_w = P.train_w, train_s = P.train_s;
-  // a row marked 0xffffffff got no gradient: g is not read, and is cleared here instead of by a pass before this one
-  const bool no_grad = SPARSE && P.row_used[row] == 0xffffffffu;
   const long long base = (long long)row * M.cols;
   const int nvec = M.cols / 4;                                 // cols is a multiple of 16
   const bool cached = !WIDE || nvec <= NV * NT;
@@ -157,8 +157,7 @@ __global__ void __launch_bounds__(NT, BLOCKS) fused_weight_update_kernel(const _
   const float sc_new = GRID == 0 ? s_new : 0.5f * s_new;
   // 3 + 4. weights, then their new codes
   const float2 ns_new = splat(-s_new), r_new = splat(__frcp_rn(s_new));
-  const Adam2 ad = {splat(o.beta1), splat(__fsub_rn(1.f, o.beta1)), splat(o.beta2), splat(__fsub_rn(1.f, o.beta2)),
-                    splat(o.rsqrt_bc2), splat(o.eps), splat(-o.lr_bc1), splat(__fsub_rn(1.f, __fmul_rn(o.lr, o.weight_decay)))};
+  const Adam2 ad = make_adam2(o);
   const float vanishes = __fmul_rd(0.5f * s_new, 1.401298464e-45f);    // s 2^-150 in whole units of 2^-149 (GRID 1)
   float2 sum2 = splat(0.f);                                    // codes are whole numbers: exact in any order
   auto update = [&](int c, float4 wv, float4 d, float4 mm, float4 vv) {
@@ -233,7 +232,8 @@ template <typename T, int NV, int NT, int BLOCKS>
 void launch_rows(const UpdateParams& p, int grid, cudaStream_t st) {
   const int rows = p.row_end[p.n - 1];
   if (grid != 0) launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 1, false>, rows, NT, 0, st, p);
-  else if (p.row_used) launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 0, true>, rows, NT, 0, st, p);
+  else if (p.tokens.ids)
+    launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 0, true>, p.tokens.n + p.idle.end - p.idle.first, NT, 0, st, p);
   else launch_k(fused_weight_update_kernel<T, NV, NT, BLOCKS, 0, false>, rows, NT, 0, st, p);
 }
 template <typename T>
@@ -252,12 +252,12 @@ int variant_of(int cols) {
 }  // namespace
 
 void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
-                                int dt, cudaStream_t st, const unsigned* row_used) {
+                                int dt, cudaStream_t st) {
   unsigned done = 0;
   for (int i = 0; i < n; ++i) {
     if (done >> i & 1u) continue;
     UpdateParams p = {};
-    p.bits = bits; p.train_w = train_w; p.train_s = train_s; p.sc = sc; p.row_used = row_used;
+    p.bits = bits; p.train_w = train_w; p.train_s = train_s; p.sc = sc;
     const int variant = variant_of(mats[i].cols);
     double bytes = 0;
     int rows = 0;
@@ -271,6 +271,16 @@ void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars
     Scope scope("fused_weight_update", bytes, 0, st);
     if (dt == 1) launch_variant<bf16>(variant, p, grid, st); else launch_variant<float>(variant, p, grid, st);
   }
+}
+
+void launch_table_update(const IdleRows& idle, const TokenRows& tokens, int dt, cudaStream_t st) {
+  UpdateParams p = {};
+  p.bits = idle.bits; p.train_w = p.train_s = 1; p.sc = idle.sc; p.tokens = tokens; p.idle = idle;
+  p.mat[0] = idle.m;
+  p.row_end[0] = idle.m.rows;
+  p.n = 1;
+  Scope scope("fused_weight_update", (double)(idle.end - idle.first) * idle.m.cols * 29.0, 0, st);
+  if (dt == 1) launch_variant<bf16>(variant_of(idle.m.cols), p, 0, st); else launch_variant<float>(variant_of(idle.m.cols), p, 0, st);
 }
 
 }  // namespace mrem

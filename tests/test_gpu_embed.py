@@ -156,6 +156,44 @@ def test_embedding_steps_of_changing_size_share_one_quantized_table(act_dtype, H
             assert rel(e.g[k].cpu().numpy(), r["grads"][k]) < 2e-2, (t, k)
 
 
+# tables smaller than what the first launch of a step takes of them, ending inside the second, reaching into the last; widths of each
+# form of the row update; rows wider than the one-kernel path takes
+@pytest.mark.parametrize("V,H,batch,seq", [(1, 16, 1, 3), (300, 768, 2, 9), (631, 128, 3, 37), (2500, 1024, 5, 40), (900, 1040, 2, 11), (6000, 256, 1, 8)])
+def test_every_row_of_the_table_is_updated_once_whoever_gathered_it(V, H, batch, seq):
+    """Two updates with different tokens: rows gathered in both, one or neither.  Weights and moments against AdamW in float64 with
+    the gradient the call left (zero for a row nobody gathered); afterwards the codes that the updates left give the outputs,
+    bit for bit, of a table quantized anew.  Tolerances as in the first test; the moments carry the rounding of 1 - beta, taken
+    from beta in float32: at most 2^-25 / 1e-3 = 3e-5 of the second one."""
+    e, desc, teacher, student, step, ids, tt = _problem("bf16", 4, V=V, H=H, batch=batch, seq=seq)
+    d_tt = torch.from_numpy(tt).to(e.device)
+    opt = dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.01)
+    w, m, v = student["word"].astype(np.float64), np.zeros((V, H)), np.zeros((V, H))
+    for t in (1, 2):
+        i = ((ids + (t - 1) * (V // 3)) % V).astype(np.int32)
+        e.g["word"].fill_(float("nan"))
+        e.step(torch.from_numpy(i).to(e.device), d_tt, B.make_optim(step=t, **opt))
+        g, before = e.g["word"].cpu().numpy(), (step if t == 1 else before_step)
+        used = np.zeros(V, bool)
+        used[i.reshape(-1)] = True
+        assert not g[~used].any() and np.abs(g[used]).max(1).min() > 0
+        q = O.sym_qmax(4)                                                # the mask is applied inside the update
+        z = (w.astype(np.float32) / before[:, None].astype(np.float32)) if t == 1 else (after / before[:, None])
+        w, m, v = O.adamw_update(w, np.where(np.abs(z) <= q, g, 0.0), m, v, t, opt["lr"], 0.9, 0.999, 1e-8, 0.01)
+        after, before_step = e.s["word"].cpu().numpy(), e.word_step.cpu().numpy()
+        assert np.allclose(after, w, rtol=1e-5, atol=2e-3 * opt["lr"])
+        assert np.allclose(e.m["word"].cpu().numpy(), m, rtol=1e-5, atol=1e-12) and np.allclose(e.v["word"].cpu().numpy(), v, rtol=4e-5, atol=1e-20)
+    assert int(e.status[0]) == 0
+    for first in range(0, V, batch * seq):                               # every row through the quantized table
+        i = torch.from_numpy(((first + np.arange(batch * seq)) % V).astype(np.int32).reshape(batch, seq)).to(e.device)
+        outs = []
+        for fresh in (False, True):
+            e.dirty = fresh
+            e.step(i, d_tt, None)
+            outs.append(e.outputs(batch, seq)[1].clone())
+        assert torch.equal(outs[0], outs[1]), first
+        e.dirty = False
+
+
 def test_embedding_step_rejects_and_reports_bad_input():
     e, desc, teacher, student, step, ids, tt = _problem("bf16", 4, V=64, H=32, P=16, batch=2, seq=8)
     d_ids, d_tt = torch.from_numpy(ids).to(e.device), torch.from_numpy(tt).to(e.device)
