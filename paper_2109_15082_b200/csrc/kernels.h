@@ -148,14 +148,19 @@ void launch_layernorm_bwd(const void* dout, const void* dout2, const void* y, co
                           const float* gamma, long long rows, int cols, void* dy, void* dsum, int dt,
                           cudaStream_t st);
 
-// The same with the incoming gradient assembled on the fly from a straight-through mask and a skip connection:
-//   dv = dout (or 0 when null) + 1[lo <= x / *step <= hi] * dxhat + add;  dsum = dv;  dy = LayerNorm backward of dv.
-// part_s gets RED_BLOCKS partial sums of the quantizer's step-size gradient.  Returns false (nothing launched)
-// when the row does not fit the register-cached vector path; the caller then runs the separate kernels.
-bool layernorm_bwd_ste_supported(int cols, int dt);      // the row width fits (16-byte aligned tensors assumed)
-bool launch_layernorm_bwd_ste(const void* dout, const void* x, const void* dxhat, const void* add, const float* step,
-                              int lo, int hi, const void* y, const float* mean, const float* rstd, const float* gamma,
-                              long long rows, int cols, void* dy, void* dsum, float* part_s, int dt, cudaStream_t st);
+// The same together with the sums over the rows that its neighbours' parameters need: the incoming gradient is dout alone (x null) or
+// assembled on the fly from a straight-through mask and a skip connection,
+//   dv = dout (or 0 when null) + 1[lo <= x / *step <= hi] * dxhat + add,     dy = LayerNorm backward of dv;
+// col_part gets several parts of the sums over the rows of dv, of dv * (y - mean) * rstd and of dy (launch_col_finish adds them),
+// part_s (with x) RED_BLOCKS partial sums of the quantizer's step-size gradient.  Returns the number of parts, or 0 (nothing
+// launched) when the row does not fit the vector path; the caller then runs the separate kernels.
+constexpr int LN_PARTS = 592;                             // at most: four groups per SM
+bool layernorm_bwd_cols_supported(int cols, int dt);      // the row width fits (16-byte aligned tensors assumed)
+size_t layernorm_bwd_cols_floats(long long rows, int cols, int dt);      // floats of col_part, up to that many rows
+int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat, const void* add, const float* step, int lo, int hi,
+                              const void* y, const float* mean, const float* rstd, const float* gamma, long long rows, int cols,
+                              void* dy, float* part_s, float* col_part, int dt, cudaStream_t st);
+void launch_col_finish(const float* col_part, int n, int cols, float* out0, float* out1, float* out2, cudaStream_t st);
 
 // Column sums over rows: out0[c] = sum_r a[r,c]; with y/mean/rstd also out1[c] = sum_r a[r,c]*(y[r,c]-mean[r])*rstd[r];
 // with a2 also out2[c] = sum_r a2[r,c].  One kernel: per-chunk partials in `scratch` (three planes of

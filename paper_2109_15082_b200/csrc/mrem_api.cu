@@ -1,5 +1,6 @@
 // C-ABI of libmrem: context, workspace layout, parameter binding, initialisation, state.
 // The step itself (forward, loss, backward, update) lives in mrem_step.cu.
+#include <algorithm>
 #include <cstring>
 
 #include "mrem_ctx.h"
@@ -107,14 +108,16 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->x_mix = A.take(M * H * es);
   c->dF = A.take((size_t)L * M * H * es);
   c->d_y2 = A.take(M * H * es); c->d_ghat = A.take(M * F * es); c->d_u = A.take(M * F * es);
-  c->d_ahat = A.take(M * H * es); c->d_a = A.take(M * H * es); c->d_y1 = A.take(M * H * es);
+  // (d_sum and d_a hold the incoming gradients of the LayerNorms, or the partial sums of their columns)
+  const size_t ln = std::max<size_t>(M * H * es, layernorm_bwd_cols_floats(M, H, d.act_dtype == MREM_BF16 ? 1 : 0) * sizeof(float));
+  c->d_ahat = A.take(M * H * es); c->d_a = A.take(ln); c->d_y1 = A.take(M * H * es);
   c->d_ctxhat = A.take(M * H * es); c->d_ctx = A.take(M * H * es);
   c->d_phat = A.take(PS * es); c->d_s = A.take(PS * es);
   c->d_qkvhat = A.take(M * 3 * H * es); c->d_qkv = A.take(M * 3 * H * es);
-  c->d_xhat = A.take(M * H * es); c->d_sum = A.take(M * H * es);
+  c->d_xhat = A.take(M * H * es); c->d_sum = A.take(ln);
   c->carry[0] = A.take(M * H * es); c->carry[1] = A.take(M * H * es);
-  c->alt_d_y2 = A.take(M * H * es); c->alt_d_sum = A.take(M * H * es); c->alt_d_u = A.take(M * F * es);
-  c->alt_d_a = A.take(M * H * es); c->alt_d_y1 = A.take(M * H * es); c->alt_d_qkv = A.take(M * 3 * H * es);
+  c->alt_d_y2 = A.take(M * H * es); c->alt_d_sum = A.take(ln); c->alt_d_u = A.take(M * F * es);
+  c->alt_d_a = A.take(ln); c->alt_d_y1 = A.take(M * H * es); c->alt_d_qkv = A.take(M * 3 * H * es);
 
   c->stash.resize(L); c->wq.assign(L, std::vector<WeightBuf>(N_WMAT)); c->grad.resize(L);
   for (int l = 0; l < L; ++l) {

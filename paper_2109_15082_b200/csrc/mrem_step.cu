@@ -316,7 +316,7 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
                               {c->alt_d_y2, c->alt_d_sum, c->alt_d_u, c->alt_d_a, c->alt_d_y1, c->alt_d_qkv}};
   const void* carry = nullptr;
   // the straight-through passes that feed a LayerNorm's backward run inside it where the row fits its registers
-  const bool fuse_ln = layernorm_bwd_ste_supported(H, c->dt);
+  const bool fuse_ln = layernorm_bwd_cols_supported(H, c->dt);
   struct { const void* x; const void* add; const float* step; float* part; } pending = {nullptr, nullptr, nullptr, nullptr};
   for (int l = d.n_layers - 1; l >= 0; --l) {
     const LayerBind& b = c->bind[l];
@@ -334,11 +334,14 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
     // second LayerNorm: total gradient at the layer output = loss term + what the next layer sent back
     // (with `pending` the layer above left its input gradient unmasked: the straight-through pass of its input
     //  quantizer and its skip connection are applied while this LayerNorm's backward reads them)
+    // LayerNorm parameter gradients and the bias gradient of FFN2 (y2 = G_hat W2_hat^T + b2 + a) ride along as partial sums;
+    // what adds those up feeds only the update and the weight-gradient epilogue: side stream
     bool sent_back = carry != nullptr;
+    int col_blocks = 0;
     if (pending.x) {
-      const bool fused = launch_layernorm_bwd_ste(dF, pending.x, c->d_xhat, pending.add, pending.step, rx.lo, rx.hi, s.y2, s.mean2, s.rstd2,
-                                                  b.student[MREM_LN2_G], M, H, q.d_y2, q.d_sum, pending.part, c->dt, st);
-      if (!fused) {
+      col_blocks = launch_layernorm_bwd_cols(dF, pending.x, c->d_xhat, pending.add, pending.step, rx.lo, rx.hi, s.y2, s.mean2, s.rstd2,
+                                             b.student[MREM_LN2_G], M, H, q.d_y2, pending.part, (float*)q.d_sum, c->dt, st);
+      if (!col_blocks) {
         launch_ste_act(pending.x, H, c->d_xhat, H, pending.add, H, c->carry[0], H, M, H, pending.step, nullptr, rx.lo, rx.hi,
                        pending.part, nullptr, c->dt, st);
         launch_layernorm_bwd(dF, c->carry[0], s.y2, s.mean2, s.rstd2, b.student[MREM_LN2_G], M, H, q.d_y2, q.d_sum, c->dt, st);
@@ -346,13 +349,18 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
       sent_back = true;
       pending.x = nullptr;
     } else {
-      launch_layernorm_bwd(dF, carry, s.y2, s.mean2, s.rstd2, b.student[MREM_LN2_G], M, H, q.d_y2, carry ? q.d_sum : nullptr, c->dt, st);
+      if (!carry)
+        col_blocks = launch_layernorm_bwd_cols(dF, nullptr, nullptr, nullptr, nullptr, 0, 0, s.y2, s.mean2, s.rstd2, b.student[MREM_LN2_G], M, H,
+                                               q.d_y2, nullptr, (float*)q.d_sum, c->dt, st);
+      if (!col_blocks)
+        launch_layernorm_bwd(dF, carry, s.y2, s.mean2, s.rstd2, b.student[MREM_LN2_G], M, H, q.d_y2, carry ? q.d_sum : nullptr, c->dt, st);
     }
-    // LayerNorm parameter gradients and the bias gradient of FFN2 (y2 = G_hat W2_hat^T + b2 + a) in one pass
-    // (column sums feed only the update and the weight-gradient epilogue: side stream)
     fork();
-    launch_col_reduce(sent_back ? q.d_sum : dF, H, s.y2, s.mean2, s.rstd2, q.d_y2, H, M, H, g.p[MREM_LN2_B], g.p[MREM_LN2_G],
-                      g.p[MREM_B2], c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
+    if (col_blocks)
+      launch_col_finish((float*)q.d_sum, col_blocks, H, g.p[MREM_LN2_B], g.p[MREM_LN2_G], g.p[MREM_B2], side);
+    else
+      launch_col_reduce(sent_back ? q.d_sum : dF, H, s.y2, s.mean2, s.rstd2, q.d_y2, H, M, H, g.p[MREM_LN2_B], g.p[MREM_LN2_G],
+                        g.p[MREM_B2], c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
     r.gemm(view(q.d_y2, H), weights(w[W_2].what, F, 1), (int)M, F, H, 1, 1, Epi(c->d_ghat, ok, F).e);
     {
       Epi e(g.p[MREM_W2], OUT_F32, F);
@@ -374,16 +382,20 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
     r.gemm(view(q.d_u, F), weights(w[W_1].what, H, 1), (int)M, H, F, 1, 1, Epi(c->d_ahat, ok, H).e);
     rw.defer(view(q.d_u, F, 1), view(s.a_qt, H, 1), F, H, (int)M, Epi(g.p[MREM_W1], OUT_F32, H).alpha(1.f, b.a_steps[S_A]).e);
     // straight-through pass of the FFN1 input quantizer + skip connection -> d_a, and the first LayerNorm's backward
-    if (!(fuse_ln && launch_layernorm_bwd_ste(nullptr, s.a, c->d_ahat, q.d_y2, b.a_steps[S_A], rx.lo, rx.hi, s.y1, s.mean1, s.rstd1,
-                                              b.student[MREM_LN1_G], M, H, q.d_y1, q.d_a, part + S_A * RED_BLOCKS, c->dt, st))) {
+    col_blocks = launch_layernorm_bwd_cols(nullptr, s.a, c->d_ahat, q.d_y2, b.a_steps[S_A], rx.lo, rx.hi, s.y1, s.mean1, s.rstd1,
+                                           b.student[MREM_LN1_G], M, H, q.d_y1, part + S_A * RED_BLOCKS, (float*)q.d_a, c->dt, st);
+    if (!col_blocks) {
       launch_ste_act(s.a, H, c->d_ahat, H, q.d_y2, H, q.d_a, H, M, H, b.a_steps[S_A], nullptr, rx.lo, rx.hi,
                      part + S_A * RED_BLOCKS, nullptr, c->dt, st);
       launch_layernorm_bwd(q.d_a, nullptr, s.y1, s.mean1, s.rstd1, b.student[MREM_LN1_G], M, H, q.d_y1, nullptr, c->dt, st);
     }
     // attention output projection:  y1 = ctx_hat Wo_hat^T + bo + x  (its bias gradient rides along)
     fork();
-    launch_col_reduce(q.d_a, H, s.y1, s.mean1, s.rstd1, q.d_y1, H, M, H, g.p[MREM_LN1_B], g.p[MREM_LN1_G], g.p[MREM_BO],
-                      c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
+    if (col_blocks)
+      launch_col_finish((float*)q.d_a, col_blocks, H, g.p[MREM_LN1_B], g.p[MREM_LN1_G], g.p[MREM_BO], side);
+    else
+      launch_col_reduce(q.d_a, H, s.y1, s.mean1, s.rstd1, q.d_y1, H, M, H, g.p[MREM_LN1_B], g.p[MREM_LN1_G], g.p[MREM_BO],
+                        c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
     // Up to 2048 tokens the feed-forward half's weight-gradient products go now: their update (two thirds of the layer's
     // weights) runs under the attention half, and the last layer leaves less of it for the end (3 x 72 tokens: step 506 -> 501
     // us, 8 x 256: 1038 -> 1020).  With more tokens the products take longer than the updates, and one launch for all four

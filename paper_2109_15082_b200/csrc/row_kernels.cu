@@ -214,84 +214,179 @@ __global__ void __launch_bounds__(128) ln_bwd_kernel(const T* __restrict__ dout,
   }
 }
 
-// ------------------------------------------------------------------ LayerNorm backward fed by a straight-through mask
-// The gradient that enters the LayerNorm is assembled on the fly:
+// ------------------------------------------------------------------ LayerNorm backward with its column sums
+// The gradient that enters the LayerNorm, with STE assembled on the fly:
 //   dv = dout (when given) + 1[lo <= x / step <= hi] * dxhat + add,
-// i.e. the straight-through pass of the activation quantizer that saw x (Sec. 3.1.1) followed by the skip
-// connection, which the separate kernels write to memory and read back.  dv goes to dsum (the column
-// reductions read it) and, rounded as stored, into the LayerNorm backward.  The quantizer's step-size
-// gradient leaves as one partial sum per block (fixed order; slots beyond the grid are zeroed).
-// Rows up to 32 * V * MAXNV wide, one warp per row, warps stride over the rows.
-template <typename T, int V>
-__global__ void __launch_bounds__(128, 7) ln_bwd_ste_kernel(const T* __restrict__ dout, const T* __restrict__ x,
-                                                         const T* __restrict__ dxhat, const T* __restrict__ add,
-                                                         const float* __restrict__ step, float lo, float hi,
-                                                         const T* __restrict__ y, const float* __restrict__ mean,
-                                                         const float* __restrict__ rstd, const float* __restrict__ gamma,
-                                                         long long rows, int cols, T* __restrict__ dy,
-                                                         T* __restrict__ dsum, float* __restrict__ part_s, int n_slots) {
+// i.e. the straight-through pass of the activation quantizer that saw x (Sec. 3.1.1) followed by the skip connection; without it
+// dv = dout.  dv, rounded as stored, goes into the LayerNorm backward; the quantizer's step-size gradient leaves as one partial sum
+// per block (fixed order; slots beyond the grid are zeroed).
+// The gradients of the LayerNorm's bias and gain and of the bias of the product before it are sums over the rows of dv, of
+// dv * (y - mean) * rstd and of dy: a thread keeps one vector of columns and adds its rows in row order, and every group of the W
+// warps that share a row leaves 3 * cols partial sums; col_finish_kernel adds the groups' in index order.
+// No more than 128 threads a block and no shared memory to speak of, so that blocks fit beside a product of the other stream (with
+// 256 threads and the groups added up in shared memory they did not).  Two rows in flight per group.
+// One warp per row with the row in its registers, dv written out, and a launch that read dv, y and dy again for the sums: the steps
+// of 32 x 128 tokens, hidden 1024, 3512 us (now 3465), of 16 x 384 5911 (5828), of 8 x 256, hidden 768, 995 (984), of 3 x 72 461
+// (456).
+__host__ __device__ constexpr int ln_groups(int W) { return W >= 3 ? 1 : 4 / W; }
+constexpr int LN_ROWS = 2;                                     // rows a group has in flight
+template <typename T, int V, int W, bool STE>
+__global__ void __launch_bounds__(32 * W * ln_groups(W), 4)
+ln_bwd_cols_kernel(const T* __restrict__ dout, const T* __restrict__ x, const T* __restrict__ dxhat, const T* __restrict__ add,
+                   const float* __restrict__ step, float lo, float hi, const T* __restrict__ y, const float* __restrict__ mean,
+                   const float* __restrict__ rstd, const float* __restrict__ gamma, long long rows, int cols, T* __restrict__ dy,
+                   float* __restrict__ part_s, int n_slots, float* __restrict__ col_part) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float sh[4];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const float s = *step, r_s = __frcp_rn(s);
+  constexpr int G = ln_groups(W), R = LN_ROWS, NW = W * G, RW = RawWords<T, V>::N;
+  __shared__ float2 sums[2][NW][R];
+  __shared__ float sh[NW];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = wid / W, tc = (int)threadIdx.x - grp * 32 * W, c = tc * V;
+  const bool on = c < cols;
+  const float s = STE ? *step : 1.f, r_s = __frcp_rn(s);
+  float a0[V], a1[V], a2[V], gm[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j) a0[j] = a1[j] = a2[j] = gm[j] = 0.f;
+  if (on) load_cols<V>(gamma + c, gm);
   float ds = 0.f;
-  for (long long row = blockIdx.x * 4ll + wid; row < rows; row += gridDim.x * 4ll) {
-    const float mu = mean[row], rs = rstd[row];
-    const long long base = row * cols;
-    float d[MAXNV][V], xn[MAXNV][V];
-    float s1 = 0.f, s2 = 0.f;
+  int flip = 0;
+  for (long long r0 = (long long)blockIdx.x * (G * R); r0 < rows; r0 += (long long)gridDim.x * (G * R), flip ^= 1) {
+    uint32_t wo[R][RW], wx[R][RW], wd[R][RW], wa[R][RW], wy[R][RW];
+    float mu[R], rs[R];
+    bool live[R];
 #pragma unroll
-    for (int i = 0; i < MAXNV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < cols) {
-        float xv[V], e[V];
-        load_vec<T, V>(x + base + c, xv);
-        load_vec<T, V>(dxhat + base + c, d[i]);
-        load_vec<T, V>(add + base + c, e);
+    for (int k = 0; k < R; ++k) {                              // all loads first
+      const long long r = r0 + k * G + grp, i = r * cols + c;
+      live[k] = r < rows;
+      mu[k] = rs[k] = 0.f;
+      if (live[k]) { mu[k] = mean[r]; rs[k] = rstd[r]; }
+      live[k] = live[k] && on;
+      if (!live[k]) continue;
+      if (STE) {
+        load_raw<T, V>(x + i, wx[k]);
+        load_raw<T, V>(dxhat + i, wd[k]);
+        load_raw<T, V>(add + i, wa[k]);
+      }
+      if (!STE || dout) load_raw<T, V>(dout + i, wo[k]);
+      load_raw<T, V>(y + i, wy[k]);
+    }
+    float d[R][V], xn[R][V];
+    float2 t[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      t[k] = make_float2(0.f, 0.f);
+      if (!live[k]) continue;
+      if (STE) {
+        float e[V];
+        widen_raw<T, V>(wx[k], e);
+        widen_raw<T, V>(wd[k], d[k]);
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-          const float z = quotient(xv[j], s, r_s);
+          const float z = quotient(e[j], s, r_s);
           const bool in = z >= lo && z <= hi;
-          ds += d[i][j] * (rne_magic(fminf(fmaxf(z, lo), hi)) - (in ? z : 0.f));
-          d[i][j] = (in ? d[i][j] : 0.f) + e[j];
+          ds += d[k][j] * (rne_magic(fminf(fmaxf(z, lo), hi)) - (in ? z : 0.f));
+          d[k][j] = in ? d[k][j] : 0.f;
         }
+        widen_raw<T, V>(wa[k], e);
+#pragma unroll
+        for (int j = 0; j < V; ++j) d[k][j] += e[j];
         if (dout) {
-          load_vec<T, V>(dout + base + c, e);
+          widen_raw<T, V>(wo[k], e);
 #pragma unroll
-          for (int j = 0; j < V; ++j) d[i][j] += e[j];
+          for (int j = 0; j < V; ++j) d[k][j] += e[j];
         }
-        store_vec<T, V>(dsum + base + c, d[i]);
-        load_vec<T, V>(y + base + c, xn[i]);
-        float gm[V];
-        load_cols<V>(gamma + c, gm);
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          xn[i][j] = (xn[i][j] - mu) * rs;
-          d[i][j] = stored<T>(d[i][j]) * gm[j];
-          s1 += d[i][j];
-          s2 += d[i][j] * xn[i][j];
-        }
+        for (int j = 0; j < V; ++j) d[k][j] = stored<T>(d[k][j]);
+      } else {
+        widen_raw<T, V>(wo[k], d[k]);
+      }
+      widen_raw<T, V>(wy[k], xn[k]);
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        xn[k][j] -= mu[k];
+        a0[j] += d[k][j];
+        a1[j] += d[k][j] * xn[k][j] * rs[k];
+        xn[k][j] *= rs[k];
+        d[k][j] *= gm[j];
+        t[k].x += d[k][j];
+        t[k].y += d[k][j] * xn[k][j];
       }
     }
-    s1 = warp_sum(s1) / (float)cols;
-    s2 = warp_sum(s2) / (float)cols;
 #pragma unroll
-    for (int i = 0; i < MAXNV; ++i) {
-      const int c = (lane + 32 * i) * V;
-      if (c < cols) {
+    for (int k = 0; k < R; ++k) {
+      t[k].x = warp_sum(t[k].x);
+      t[k].y = warp_sum(t[k].y);
+      if (W > 1 && lane == 0) sums[flip][wid][k] = t[k];
+    }
+    if constexpr (W > 1) {
+      __syncthreads();                                         // (the other set is behind the next iteration's barrier)
 #pragma unroll
-        for (int j = 0; j < V; ++j) d[i][j] = rs * (d[i][j] - s1 - xn[i][j] * s2);
-        store_vec<T, V>(dy + base + c, d[i]);
+      for (int k = 0; k < R; ++k) {
+        t[k] = sums[flip][grp * W][k];
+#pragma unroll
+        for (int w = 1; w < W; ++w) { t[k].x += sums[flip][grp * W + w][k].x; t[k].y += sums[flip][grp * W + w][k].y; }
       }
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      if (!live[k]) continue;
+      const float s1 = t[k].x / (float)cols, s2 = t[k].y / (float)cols;
+#pragma unroll
+      for (int j = 0; j < V; ++j) d[k][j] = rs[k] * (d[k][j] - s1 - xn[k][j] * s2);
+      store_vec<T, V>(dy + (r0 + k * G + grp) * cols + c, d[k]);
+#pragma unroll
+      for (int j = 0; j < V; ++j) a2[j] += stored<T>(d[k][j]);
     }
   }
-  ds = warp_sum(ds);
-  if (lane == 0) sh[wid] = ds;
+  if (on) {
+    float* dst = col_part + ((long long)blockIdx.x * G + grp) * 3 * cols + c;
+#pragma unroll
+    for (int j = 0; j < V; j += 4) {
+      *reinterpret_cast<float4*>(dst + j) = make_float4(a0[j], a0[j + 1], a0[j + 2], a0[j + 3]);
+      *reinterpret_cast<float4*>(dst + cols + j) = make_float4(a1[j], a1[j + 1], a1[j + 2], a1[j + 3]);
+      *reinterpret_cast<float4*>(dst + 2 * cols + j) = make_float4(a2[j], a2[j + 1], a2[j + 2], a2[j + 3]);
+    }
+  }
+  if (STE) {
+    ds = warp_sum(ds);
+    if (lane == 0) sh[wid] = ds;
+    __syncthreads();
+  }
+  if (STE) {
+    if (threadIdx.x == 0) {
+      float v = sh[0];
+#pragma unroll
+      for (int w = 1; w < NW; ++w) v += sh[w];
+      part_s[blockIdx.x] = v;
+    }
+    if (blockIdx.x == 0)
+      for (int i = gridDim.x + threadIdx.x; i < n_slots; i += blockDim.x) part_s[i] = 0.f;
+  }
+}
+
+// out_k[c] = sum over n parts of part[i][k][c], in index order within 32 runs of them and the runs in order; 32 columns a block.
+__global__ void __launch_bounds__(256) col_finish_kernel(const float* __restrict__ part, int n, int cols, float* __restrict__ out0,
+                                                         float* __restrict__ out1, float* __restrict__ out2) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ __align__(16) float4 red[32][8];
+  const int run = threadIdx.x >> 3, k4 = threadIdx.x & 7, width = 3 * cols;
+  const int i = ((int)blockIdx.x * 8 + k4) * 4, per = (n + 31) / 32, k0 = run * per, k1 = min(n, k0 + per);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (i < width) {
+#pragma unroll 10
+    for (int k = k0; k < k1; ++k) {
+      const float4 e = *reinterpret_cast<const float4*>(part + (long long)k * width + i);
+      v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w;
+    }
+  }
+  red[run][k4] = v;
   __syncthreads();
-  if (threadIdx.x == 0) part_s[blockIdx.x] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
-  if (blockIdx.x == 0)
-    for (int i = gridDim.x + threadIdx.x; i < n_slots; i += blockDim.x) part_s[i] = 0.f;
+  if (run != 0 || i >= width) return;
+#pragma unroll
+  for (int w = 1; w < 32; ++w) { const float4 e = red[w][k4]; v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w; }
+  const int pl = i / cols, col = i - pl * cols;                // (cols is a multiple of 4)
+  *reinterpret_cast<float4*>((pl == 0 ? out0 : (pl == 1 ? out1 : out2)) + col) = v;
 }
 
 // ------------------------------------------------------------------ column sums over rows
@@ -590,30 +685,42 @@ void launch_layernorm_bwd(const void* dout, const void* dout2, const void* y, co
   });
 }
 
-bool layernorm_bwd_ste_supported(int cols, int dt) {
+// Warps that share a row of the kernel with column sums; 0: rows it does not take.
+static int ln_cols_warps(int cols, int dt) {
   const int V = dt == 1 ? 8 : 4;
-  return cols % V == 0 && cols <= 32 * V * MAXNV;
+  return cols % V == 0 && cols <= 32 * V * MAXNV ? (cols + 32 * V - 1) / (32 * V) : 0;
+}
+bool layernorm_bwd_cols_supported(int cols, int dt) { return ln_cols_warps(cols, dt) > 0; }
+// groups: two rows each while there are fewer rows than that takes
+static int ln_cols_grid(long long rows, int W) {
+  const int per = ln_groups(W) * LN_ROWS;
+  const long long want = (rows + per - 1) / per, limit = LN_PARTS / ln_groups(W);
+  return (int)(want < limit ? want : limit);
+}
+size_t layernorm_bwd_cols_floats(long long rows, int cols, int dt) {
+  const int W = ln_cols_warps(cols, dt);
+  return W == 0 ? 0 : (size_t)ln_cols_grid(rows, W) * ln_groups(W) * 3 * cols;
 }
 
-bool launch_layernorm_bwd_ste(const void* dout, const void* x, const void* dxhat, const void* add, const float* step,
-                              int lo, int hi, const void* y, const float* mean, const float* rstd, const float* gamma,
-                              long long rows, int cols, void* dy, void* dsum, float* part_s, int dt, cudaStream_t st) {
-  if (rows <= 0) return false;
-  bool done = false;
-  MREM_DT(dt, T, {
-    constexpr int V = 16 / (int)sizeof(T);
-    const bool v = cols % V == 0 && cols <= 32 * V * MAXNV && al16(dout) && al16(x) && al16(dxhat) && al16(add) && al16(y) &&
-                   al16(dy) && al16(dsum) && al16(gamma);
-    if (v) {
-      Scope sc("layernorm_bwd_ste", (double)rows * cols * (dt == 1 ? 2.0 : 4.0) * (6 + (dout ? 1 : 0)), 0, st);
-      const long long want = (rows + 3) / 4;
-      const int grid = (int)(want < RED_BLOCKS ? want : RED_BLOCKS);
-      launch_k(ln_bwd_ste_kernel<T, V>, grid, 128, 0, st, (const T*)dout, (const T*)x, (const T*)dxhat, (const T*)add, step,
-               (float)lo, (float)hi, (const T*)y, mean, rstd, gamma, rows, cols, (T*)dy, (T*)dsum, part_s, RED_BLOCKS);
-      done = true;
-    }
-  });
-  return done;
+int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat, const void* add, const float* step, int lo, int hi,
+                              const void* y, const float* mean, const float* rstd, const float* gamma, long long rows, int cols,
+                              void* dy, float* part_s, float* col_part, int dt, cudaStream_t st) {
+  const int W = ln_cols_warps(cols, dt);
+  if (rows <= 0 || W == 0 || !(al16(dout) && al16(x) && al16(dxhat) && al16(add) && al16(y) && al16(dy) && al16(gamma))) return 0;
+  Scope sc(x ? "layernorm_bwd_ste" : "layernorm_bwd", (double)rows * cols * (dt == 1 ? 2.0 : 4.0) * (x ? (dout ? 6 : 5) : 3), 0, st);
+  const int grid = ln_cols_grid(rows, W);
+#define MREM_LN(T, V, W, STE) launch_k(ln_bwd_cols_kernel<T, V, W, STE>, grid, 32 * W * ln_groups(W), 0, st, (const T*)dout, (const T*)x, (const T*)dxhat, (const T*)add, step, (float)lo, (float)hi, (const T*)y, mean, rstd, gamma, rows, cols, (T*)dy, part_s, RED_BLOCKS, col_part)
+#define MREM_LNS(T, V, STE) do { if (W == 1) MREM_LN(T, V, 1, STE); else if (W == 2) MREM_LN(T, V, 2, STE); else if (W == 3) MREM_LN(T, V, 3, STE); else MREM_LN(T, V, 4, STE); } while (0)
+  if (dt == 1) { if (x) MREM_LNS(bf16, 8, true); else MREM_LNS(bf16, 8, false); }
+  else { if (x) MREM_LNS(float, 4, true); else MREM_LNS(float, 4, false); }
+#undef MREM_LNS
+#undef MREM_LN
+  return grid * ln_groups(W);
+}
+
+void launch_col_finish(const float* col_part, int n, int cols, float* out0, float* out1, float* out2, cudaStream_t st) {
+  Scope sc("col_reduce", (double)n * cols * 12.0, 0, st);
+  launch_k(col_finish_kernel, (3 * cols + 31) / 32, 256, 0, st, col_part, n, cols, out0, out1, out2);
 }
 
 void launch_col_reduce(const void* a, long long ld_a, const void* y, const float* mean, const float* rstd,
