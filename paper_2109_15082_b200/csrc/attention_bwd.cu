@@ -41,6 +41,7 @@ struct AttnBwdParams {
   float q_hi;                // code range -q_hi .. q_hi of the symmetric Q / K / V / context sites
   float p_hi;                // upper end of the code range of the P site (probabilities are not negative)
   float *part_q, *part_k, *part_v, *part_p, *part_c;   // [red_slots] each: one partial per CTA, the rest zeroed
+  float* col_part;           // [B, 3, H] column sums of dQ, dK, dV
   int red_slots;
   int* status;
   unsigned long long wait_ns;  // limit of each wait on an mbarrier
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
   __shared__ uint32_t tmem_slot;
   __shared__ float red_dot[2][128];
   __shared__ float red_part[8][5];
+  __shared__ __align__(8) float red_col[3][8 * 64];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int head = blockIdx.x, b = blockIdx.y;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -279,7 +281,11 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
       if (threadIdx.x == 32) {
         tma_store_4d(&maps.out, g == 1 ? sD : sV, 0, 0, (g == 0 ? 2 * p.h : (g == 1 ? 0 : p.h)) + head, b);
         tma_store_commit();
-        if (g == 0) {
+      }
+      tile_col_sums<8>(tile, p.S, warp - 1, lane, red_col[g]);
+      if (g == 0) {
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (threadIdx.x == 32) {
           tma_store_wait_read<0>();                        // dV has left the tile: K before quantization
           mbar_expect_tx(bar(B_RK), 16384u);
           tma_load_4d(sV, &maps.raw, bar(B_RK), 0, 0, p.h + head, b);
@@ -301,6 +307,10 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
       for (int k = 0; k < 8; ++k) t += red_part[k][lane];
       float* dst = lane == 0 ? p.part_p : (lane == 1 ? p.part_q : (lane == 2 ? p.part_k : (lane == 3 ? p.part_v : p.part_c)));
       dst[b * p.h + head] = t;
+    }
+    if (const int i = (int)threadIdx.x - 32; i < 192) {      // V, Q, K as above
+      const int g = i >> 6, plane = g == 0 ? 2 : g - 1;
+      p.col_part[((long long)b * 3 + plane) * p.H + head * HD + (i & 63)] = add_col_sums<8>(red_col[g], i & 63);
     }
     if (head == 0 && b == 0)             // the slots no CTA owns
       for (int i = p.B * p.h + (int)threadIdx.x - 32; i < p.red_slots; i += 256) {
@@ -331,6 +341,7 @@ int launch_attention_bwd(const AttentionBwd& a, cudaStream_t st) {
   p.q_hi = (float)a.q_hi; p.p_hi = (float)a.p_hi;
   p.part_q = a.part_q; p.part_k = a.part_k; p.part_v = a.part_v; p.part_p = a.part_p; p.part_c = a.part_c;
   p.red_slots = RED_BLOCKS;
+  p.col_part = a.col_part;
   p.status = a.status;
   p.wait_ns = g_wait_limit_ns;
   // tensor maps over [tokens, 3H] and [tokens, H] tensors: (64 of a head, S rows, head slots, B)

@@ -97,6 +97,7 @@ struct AttentionBwd {
   void* dqkv;                             // [B*S, 3H] out
   void* dctx_masked; float* dot;          // scratch above 128 tokens: [B*S, H] and [B, h, S]
   float *part_q, *part_k, *part_v, *part_p, *part_c;
+  float* col_part;                        // up to 128 tokens: [B, 3, H] out, column sums of dqkv per sequence
   int* status;
 };
 bool attention_bwd_supported(int S, int head_dim, int dt, int batch_heads);

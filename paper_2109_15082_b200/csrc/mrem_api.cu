@@ -105,11 +105,12 @@ static void layout(mrem_ctx* c, char* base, size_t* total) {
   c->t_y2 = A.take(M * H * es);
   c->scores = (float*)A.take(PS * sizeof(float));
   c->att_dot = (float*)A.take(sizeof(float) * d.max_batch * d.n_heads * d.max_seq);
+  for (float*& cols : c->att_cols) cols = (float*)A.take(sizeof(float) * 3 * H * d.max_batch);
   c->x_mix = A.take(M * H * es);
   c->dF = A.take((size_t)L * M * H * es);
-  c->d_y2 = A.take(M * H * es); c->d_ghat = A.take(M * F * es); c->d_u = A.take(M * F * es);
   // (d_sum and d_a hold the incoming gradients of the LayerNorms, or the partial sums of their columns)
   const size_t ln = std::max<size_t>(M * H * es, layernorm_bwd_cols_floats(M, H, d.act_dtype == MREM_BF16 ? 1 : 0) * sizeof(float));
+  c->d_y2 = A.take(M * H * es); c->d_ghat = A.take(M * F * es); c->d_u = A.take(M * F * es);
   c->d_ahat = A.take(M * H * es); c->d_a = A.take(ln); c->d_y1 = A.take(M * H * es);
   c->d_ctxhat = A.take(M * H * es); c->d_ctx = A.take(M * H * es);
   c->d_phat = A.take(PS * es); c->d_s = A.take(PS * es);

@@ -89,6 +89,7 @@ struct mrem_ctx {
   // shared scratch
   void *t_qkv, *t_P, *t_ctx, *t_y1, *t_a, *t_g, *t_y2;   // teacher activations
   float* scores;
+  float* att_cols[2];                                   // column sums of dqkv per sequence, alternate layers
   float* att_dot;                                       // [B, h, S] row sums of the attention backward
   void* x_mix;                                          // Eq. 4 input of the student
   void* dF;                                             // [L, M, H] loss gradients

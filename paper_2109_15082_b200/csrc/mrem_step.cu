@@ -412,7 +412,8 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
       const AttentionBwd ab{s.qkv_qt, s.qkv, s.ctx, c->d_ctxhat, B, S, h, H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], b.a_steps[S_P],
                             b.a_steps[S_C], s.p_alpha, s.p_len, s.p_stat, rx.hi, rp.hi, q.d_qkv, c->d_ctx, c->att_dot,
                             part + S_Q * RED_BLOCKS,
-                            part + S_K * RED_BLOCKS, part + S_V * RED_BLOCKS, part + S_P * RED_BLOCKS, part + S_C * RED_BLOCKS, c->status};
+                            part + S_K * RED_BLOCKS, part + S_V * RED_BLOCKS, part + S_P * RED_BLOCKS, part + S_C * RED_BLOCKS,
+                            c->att_cols[l & 1], c->status};
       r.note(launch_attention_bwd(ab, st), "attention backward launch failed");
     } else {
       launch_ste_act(s.ctx, H, c->d_ctxhat, H, nullptr, 0, c->d_ctx, H, M, H, b.a_steps[S_C], nullptr, rx.lo, rx.hi,
@@ -432,7 +433,10 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
     }
     // QKV projection:  qkv = X_hat Wqkv_hat^T + bqkv
     fork();
-    launch_col_reduce(q.d_qkv, 3 * H, nullptr, nullptr, nullptr, nullptr, 0, M, 3 * H, g.p[MREM_BQKV], nullptr, nullptr, c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
+    if (!s.p_kept && S <= 128)                        // (above, the attention kernels are faster without the sums)
+      launch_col_finish(c->att_cols[l & 1], B, H, g.p[MREM_BQKV], g.p[MREM_BQKV] + H, g.p[MREM_BQKV] + 2 * H, side);
+    else
+      launch_col_reduce(q.d_qkv, 3 * H, nullptr, nullptr, nullptr, nullptr, 0, M, 3 * H, g.p[MREM_BQKV], nullptr, nullptr, c->col_scratch, c->col_plane, c->col_counters, c->dt, side);
     r.gemm(view(q.d_qkv, 3 * H), weights(w[W_QKV].what, H, 1), (int)M, H, 3 * H, 1, 1, Epi(c->d_xhat, ok, H).e);
     rw.defer(view(q.d_qkv, 3 * H, 1), view(s.x_qt, H, 1), 3 * H, H, (int)M, Epi(g.p[MREM_WQKV], OUT_F32, H).alpha(1.f, b.a_steps[S_X]).e);
     rw.flush_deferred();                              // the weight-gradient products that are left
