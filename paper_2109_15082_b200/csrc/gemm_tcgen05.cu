@@ -70,10 +70,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   tc_fence_after();
   // A B operand that the preceding kernel does not write (weights): the producer fetches the B tiles of its first
   // stages now, while that kernel is still finishing; the matching A tiles follow after the wait.
-  int prefetched = 0;
-  if (threadIdx.x == 0 && p.b_static && (int)blockIdx.x < p.num_tiles) {
+  const int prefetched = p.b_static && (int)blockIdx.x < p.num_tiles ? (p.k_blocks < p.num_stages ? p.k_blocks : p.num_stages) : 0;
+  if (threadIdx.x == 0 && prefetched > 0) {
     const TileCoord t = decode_tile(p, blockIdx.x);
-    prefetched = p.k_blocks < p.num_stages ? p.k_blocks : p.num_stages;
     for (int kb = 0; kb < prefetched; ++kb) {
       const uint32_t bar = smem_u32(&full_bar[kb]);
       const uint32_t sb = tiles_base + kb * p.stage_bytes + A_STAGE_BYTES;
@@ -93,19 +92,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   volatile int* vabort = &abort_flag;
 
   if (warp == 0) {
-    // ---------------- TMA producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < p.num_tiles && ok; tile += gridDim.x) {
-        const TileCoord t = decode_tile(p, tile);
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!mbar_wait_or_abort(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, p.wait_ns)) {
-            if (!*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
-            ok = false;
-            break;
-          }
+    // ---------------- TMA producer: like the issuer, the whole warp walks the loop and one elected lane issues (see elect_one).  Its chain
+    // of instructions sets the pace of every tile below 256 columns: 0.287 us per block of the inner dimension whatever the
+    // width (0.21 in a copy that loads nothing); from the whole warp 0.276.  2048 x 768 x 3072 17.9 -> 17.3 us, 1500 x 1024 x 4096 22.7 ->
+    // 22.4, int8 2200 x 768 x 3072 11.8 -> 11.45.  (Looking at the next stage's barrier before this stage's loads: 0.265, but 256-wide tiles
+    // slower; step of 32 x 128 tokens, hidden 1024 3484 -> 3510 us.  The same in the issuer's loop: 1 % slower at every width.)
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < p.num_tiles && ok; tile += gridDim.x) {
+      const TileCoord t = decode_tile(p, tile);
+      for (int kb = 0; kb < p.k_blocks; ++kb) {
+        if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, p.wait_ns)) {
+          if (leader && !*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
+          ok = false;
+          break;
+        }
+        if (leader) {
           const uint32_t bar = smem_u32(&full_bar[stage]);
           const uint32_t sa = tiles_base + stage * p.stage_bytes, sb = sa + A_STAGE_BYTES;
           const bool b_done = tile == (int)blockIdx.x && kb < prefetched;     // fetched (and announced) before the wait
@@ -126,9 +130,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           } else {
             for (int j = 0; j < p.block_n / 64; ++j) tma_load_4d(sb + j * 8192, &map_b, bar, t.n0 + 64 * j, k0, t.b0, t.b1);
           }
-          if (++stage == p.num_stages) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == p.num_stages) { stage = 0; phase ^= 1u; }
       }
+    }
+    if (leader) {
       pdl_trigger();                     // the last tiles are on their way: the next kernel's launch hides behind their products
       if (!ok) {
         // let the copies already in flight land before the CTA may exit
@@ -138,6 +145,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer: the whole warp walks the loop, one elected lane issues (see elect_one)
     const bool leader = elect_one();

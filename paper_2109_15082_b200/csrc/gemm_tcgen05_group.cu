@@ -74,45 +74,50 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
   volatile int* vabort = &abort_flag;
 
   if (warp == 0) {
-    // ---------------- TMA producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        int local;
-        const int pi = find_problem(g, tile, local);
-        const TcParams& p = g.p[pi];
-        const CUtensorMap* map_a = &maps.a[pi];
-        const CUtensorMap* map_b = &maps.b[pi];
-        const TileCoord t = decode_tile(p, local);
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!mbar_wait_or_abort(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, g.p[0].wait_ns)) {
-            if (!*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
-            ok = false;
-            break;
-          }
+    // ---------------- TMA producer (see tc_gemm_kernel)
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      int local;
+      const int pi = find_problem(g, tile, local);
+      const TcParams& p = g.p[pi];
+      const CUtensorMap* map_a = &maps.a[pi];
+      const CUtensorMap* map_b = &maps.b[pi];
+      const TileCoord t = decode_tile(p, local);
+      const int k_blocks = p.k_blocks, a_mn = p.a_mn, b_mn = p.b_mn;
+      for (int kb = 0; kb < k_blocks; ++kb) {
+        if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, g.p[0].wait_ns)) {
+          if (leader && !*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
+          ok = false;
+          break;
+        }
+        if (leader) {
           const uint32_t bar = smem_u32(&full_bar[stage]);
           const uint32_t sa = tiles_base + stage * g.stage_bytes, sb = sa + A_STAGE_BYTES;
           mbar_expect_tx(bar, (uint32_t)g.stage_bytes);
           const int k0 = kb * p.block_k;
-          if (!p.a_mn) {
+          if (!a_mn) {
             tma_load_4d(sa, map_a, bar, k0, t.m0, t.b0, t.b1);
-          } else if (p.a_mn == 2) {
+          } else if (a_mn == 2) {
             tma_load_5d(sa, map_a, bar, 0, k0, t.m0 >> 6, t.b0, t.b1);
           } else {
             for (int j = 0; j < BLOCK_M / 64; ++j) tma_load_4d(sa + j * 8192, map_a, bar, t.m0 + 64 * j, k0, t.b0, t.b1);
           }
-          if (!p.b_mn) {
+          if (!b_mn) {
             tma_load_4d(sb, map_b, bar, k0, t.n0, t.b0, t.b1);
-          } else if (p.b_mn == 2) {
+          } else if (b_mn == 2) {
             tma_load_5d(sb, map_b, bar, 0, k0, t.n0 >> 6, t.b0, t.b1);
           } else {
             for (int j = 0; j < p.block_n / 64; ++j) tma_load_4d(sb + j * 8192, map_b, bar, t.n0 + 64 * j, k0, t.b0, t.b1);
           }
-          if (++stage == g.num_stages) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == g.num_stages) { stage = 0; phase ^= 1u; }
       }
+    }
+    if (leader) {
       pdl_trigger();                     // see tc_gemm_kernel
       if (!ok) {
         // let the copies already in flight land before the CTA may exit
@@ -122,6 +127,7 @@ tc_gemm_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_consta
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer: the whole warp walks the loop, one elected lane issues (see elect_one)
     const bool leader = elect_one();

@@ -77,9 +77,8 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     else if (p.b_mn == 2) tma_load_5d(sb, &map_b, bar, 0, k0, t.n0 >> 6, t.b0, t.b1);
     else for (int j = 0; j < p.block_n / 64; ++j) tma_load_4d(sb + j * 8192, &map_b, bar, t.n0 + 64 * j, k0, t.b0, t.b1);
   };
-  int prefetched = 0;                    // see tc_gemm_kernel
-  if (threadIdx.x == 0 && p.b_static) {
-    prefetched = min(kb1 - kb0, p.num_stages);
+  const int prefetched = p.b_static ? min(kb1 - kb0, p.num_stages) : 0;      // see tc_gemm_kernel
+  if (threadIdx.x == 0) {
     for (int i = 0; i < prefetched; ++i) {
       mbar_expect_tx(smem_u32(&full_bar[i]), (uint32_t)p.stage_bytes);
       load_b(kb0 + i, i);
@@ -104,16 +103,17 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   bool got = true;
 
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait_or_abort(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, p.wait_ns)) {
-          if (!*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
-          ok = false;
-          break;
-        }
+    const bool leader = elect_one();     // see tc_gemm_kernel
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase ^ 1u, vabort, p.wait_ns)) {
+        if (leader && !*vabort) fail(p, DEV_TIMEOUT_MMA, vabort);
+        ok = false;
+        break;
+      }
+      if (leader) {
         const uint32_t bar = smem_u32(&full_bar[stage]), sa = tiles_base + stage * p.stage_bytes;
         const bool b_done = kb - kb0 < prefetched;
         if (!b_done) mbar_expect_tx(bar, (uint32_t)p.stage_bytes);
@@ -122,8 +122,11 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         else if (p.a_mn == 2) tma_load_5d(sa, &map_a, bar, 0, k0, t.m0 >> 6, t.b0, t.b1);
         else for (int j = 0; j < BLOCK_M / 64; ++j) tma_load_4d(sa + j * 8192, &map_a, bar, t.m0 + 64 * j, k0, t.b0, t.b1);
         if (!b_done) load_b(kb, stage);
-        if (++stage == p.num_stages) { stage = 0; phase ^= 1u; }
       }
+      __syncwarp();
+      if (++stage == p.num_stages) { stage = 0; phase ^= 1u; }
+    }
+    if (leader) {
       pdl_trigger();
       if (!ok) {
         // let the copies already in flight land before the CTA may exit
