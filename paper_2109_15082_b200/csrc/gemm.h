@@ -10,9 +10,10 @@ namespace mrem {
 enum GemmRc : int { GEMM_OK = 0, GEMM_ERR_ARG = -1, GEMM_ERR_ALIGN = -2, GEMM_ERR_CUDA = -6 };
 
 // Tensor-core path (tcgen05).  kind 0: bf16 x bf16 -> fp32; kind 1: (u8|s8) x s8 -> int32 (exact).
-// block_n 0 picks the tile width.  Operands need 16-byte aligned bases and strides.
+// block_n 0 picks the tile width; `beside`: for a launch whose idle SMs another stream's kernels fill.  Operands need 16-byte aligned
+// bases and strides.
 int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B, const GemmShape& g,
-            const Epilogue& epi, int block_n, int* d_status, int sm_count, cudaStream_t stream);
+            const Epilogue& epi, int block_n, int* d_status, int sm_count, cudaStream_t stream, bool beside = false);
 
 // Verification aid: one block that lets a bounded wait run out (limit_ns) and reports DEV_TIMEOUT_TMA in *d_status.
 cudaError_t launch_wait_probe(int* d_status, unsigned long long limit_ns, cudaStream_t stream);
@@ -22,7 +23,7 @@ cudaError_t launch_wait_probe(int* d_status, unsigned long long limit_ns, cudaSt
 constexpr int MAX_GEMM_GROUP = 4;
 struct GemmGroupItem { OperandDesc A, B; GemmShape g; Epilogue epi; };
 bool tc_gemm_group_eligible(const GemmGroupItem* items, int n);
-int tc_gemm_group(const GemmGroupItem* items, int n, int* d_status, int sm_count, cudaStream_t stream);
+int tc_gemm_group(const GemmGroupItem* items, int n, int* d_status, int sm_count, cudaStream_t stream, bool beside = false);
 
 // 4-D TMA tensor map (128-byte swizzle) of an operand: (contiguous index, strided index, batch0, batch1).
 // K-major operands get boxes of block_k x tile_mn elements, MN-major ones 64 x block_k.

@@ -363,6 +363,8 @@ __device__ __forceinline__ bool direct_epilogue_ok(const Epilogue& e) {
 
 }  // namespace tc
 
+// gemm_tcgen05.cu: the tile width for n products in one launch.
+int tc_pick_block_n(const int* M, const int* N, const int* k_blocks, int n, int batches, int sm_count, bool wide_out, bool beside);
 // gemm_tcgen05_split.cu: several CTAs per tile; tc_gemm prepares everything and decides.
 bool tc_gemm_split_eligible(int kind, const GemmShape& g, const Epilogue& e);
 int tc_gemm_split_launch(int kind, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const tc::TcParams& params, int splits,

@@ -347,19 +347,14 @@ int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, in
 
 namespace {
 
-// Tile width by a cost model fitted to event timings on the encoder shapes: a persistent CTA works through
-// `waves` tiles one after the other, a tile costs k_blocks main-loop steps plus an epilogue share that is
-// not hidden.  A step of a narrow tile is cheaper, but far from proportionally (the A tile is re-fetched
-// for every column block and the shared-memory traffic per flop grows), so wide tiles win unless they
-// leave most SMs idle.
 // `splits` > 1: that many CTAs share each tile's inner dimension (tc_gemm_split_kernel), worth the exchange of partial sums where
 // the tiles are few and the inner dimension is long.  Alone / shared, us: 216 x 768 x 3072 17.0 / 9.5 (int8 codes 10.4 / 7.4),
 // 216 x 768 x 2304 13.5 / 8.6, 512 x 768 x 3072 17.3 / 11.8, 1024 x 1024 x 4096 22.9 / 17.1, 128 x 1024 x 1024 7.8 / 6.9,
 // 216 x 768 x 768 6.7 / 6.3; on the other side of the line 512 x 1024 x 1024 8.2 / 9.2, 1024 x 1024 x 1024 8.5 / 8.8.
 // No more tiles than all clusters can hold at once: cudaOccupancyMaxActiveClusters gives 74 clusters of two and 33 of four for
 // every variant on an idle chip; the limits, 72 and 32, lie below that (no product of a 768 or 1024 wide layer has one of the
-// few tile counts between).
-int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count, bool can_split, int* splits) {
+// few tile counts between).  Returns the tile width of the shared form (at most 128), or 0 with *splits = 1.
+int pick_split(int M, int N, int k_blocks, int batches, int sm_count, int* splits) {
   const int m_tiles = (M + BLOCK_M - 1) / BLOCK_M;
   int best = 64;
   double best_cost = 1e30;
@@ -372,29 +367,66 @@ int pick_block_n(int M, int N, int k_blocks, int batches, int sm_count, bool can
     const double epi_us = bn == 64 ? 0.5 : (bn == 128 ? 1.0 : 2.0);
     const double cost = (double)waves * (k_blocks * step_us + epi_us);
     if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; *splits = 1; }
-    for (int s = 2; s <= 4 && can_split && bn <= 128; s *= 2) {
+    for (int s = 2; s <= 4 && bn <= 128; s *= 2) {
       if (tiles * s > (s == 2 ? sm_count - 4 : sm_count - 20) || k_blocks < 4 * s) continue;
       const double exchange_us = 1.5 + 0.012 * (double)(tiles * s);
       const double split_cost = (double)((k_blocks + s - 1) / s) * step_us + epi_us / s + exchange_us;
       if (split_cost < best_cost - 1e-9) { best_cost = split_cost; best = bn; *splits = s; }
     }
   }
-  return best;
+  return *splits > 1 ? best : 0;
 }
 
 }  // namespace
 
+// Tile width by a cost model fitted to event timings (us): a persistent CTA works through `waves` tiles one after the other; a block of
+// the inner dimension takes nearly the same time at any width (the producer's pace), a tile's epilogue is hidden by the next tile's
+// main loop if that is longer, and the last one's, with launch, set-up and pipeline fill, is not.  So the widest tile that leaves no wave
+// nearly empty wins: 192 columns where 256 do.  Widths 256 / 192 alone, us: 6144 x 1024 x 4096 46 / 44, 6144 x 1024 x 1024
+// 14.8 / 13.8, 4096 x 768 x 3072 19.1 / 18.0, 4096 x 768 x 768 8.2 / 7.7, 2048 x 3072 x 768 12.4 / 11.7, int8 2200 x 2304 x 768
+// 8.6 / 8.0; on the other side 4096 x 4096 x 1024 27 / 30, 4096 x 1024 x 4096 25 / 41.  Forward of both modules, one after the other, 32 x
+// 128 tokens, hidden 768: 602 -> 577 us; 11 x 200 tokens with gradients 387 -> 376.  But those SMs are not idle when another stream's
+// kernels run `beside` the launch, and 192 columns take more SM time in all (step of 16 x 384 tokens, hidden 1024: 5850 -> 5974
+// us; 32 x 128, hidden 768: 1198 -> 1202): then not.  fp32 outputs (`wide_out`) take longer to store.
+int tc_pick_block_n(const int* M, const int* N, const int* k_blocks, int n, int batches, int sm_count, bool wide_out, bool beside) {
+  static const struct { int bn; double step, tile, fixed, fixed_f32; } widths[] = {
+      {64, 0.29, 0.8, 2.8, 3.5}, {128, 0.30, 1.5, 3.4, 4.4}, {192, 0.31, 2.2, 3.7, 5.3}, {256, 0.345, 2.8, 4.3, 6.4}};
+  int best = 64;
+  double best_cost = 1e30;
+  for (const auto& w : widths) {
+    if ((wide_out && w.bn == 64) || (beside && w.bn == 192)) continue;       // (groups: measured from 128 on)
+    int widest = 0, kb = 0;
+    long long tiles = 0;
+    for (int i = 0; i < n; ++i) {
+      tiles += (long long)((M[i] + BLOCK_M - 1) / BLOCK_M) * ((N[i] + w.bn - 1) / w.bn) * batches;
+      widest = N[i] > widest ? N[i] : widest;
+      kb = k_blocks[i] > kb ? k_blocks[i] : kb;
+    }
+    if (w.bn > 64 && w.bn / 2 >= widest && best_cost < 1e30) break;
+    const long long waves = (tiles + sm_count - 1) / sm_count;
+    const double loop = kb * w.step, hidden = loop > w.tile ? loop : w.tile;
+    const double cost = loop + (double)(waves - 1) * hidden + (wide_out ? w.fixed_f32 : w.fixed);
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = w.bn; }
+  }
+  return best;
+}
+
 int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B, const GemmShape& g,
-            const Epilogue& epi, int block_n, int* d_status, int sm_count, cudaStream_t stream) {
+            const Epilogue& epi, int block_n, int* d_status, int sm_count, cudaStream_t stream, bool beside) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.nb0 <= 0 || g.nb1 <= 0) return GEMM_ERR_ARG;
   const int es = kind == 0 ? 2 : 1;
   if (kind == 1 && (A.mn_contig || B.mn_contig)) return GEMM_ERR_ARG;
   TcParams p;
   p.M = g.M; p.N = g.N; p.K = g.K; p.nb0 = g.nb0; p.nb1 = g.nb1;
   int splits = 1;
-  p.block_n = block_n > 0 ? block_n : pick_block_n(g.M, g.N, (g.K + 128 / es - 1) / (128 / es), g.nb0 * g.nb1, sm_count,
-                                                   tc_gemm_split_eligible(kind, g, epi), &splits);
-  if (p.block_n != 64 && p.block_n != 128 && p.block_n != 256) return GEMM_ERR_ARG;
+  p.block_n = block_n;
+  if (block_n <= 0) {
+    const int kb = (g.K + 128 / es - 1) / (128 / es), batches = g.nb0 * g.nb1;
+    p.block_n = tc_gemm_split_eligible(kind, g, epi) ? pick_split(g.M, g.N, kb, batches, sm_count, &splits) : 0;
+    if (p.block_n == 0) p.block_n = tc_pick_block_n(&g.M, &g.N, &kb, 1, batches, sm_count, false, beside);
+  } else if (block_n != 64 && block_n != 128 && block_n != 256) {
+    return GEMM_ERR_ARG;
+  }
   p.block_k = 128 / es;
   p.m_tiles = (g.M + BLOCK_M - 1) / BLOCK_M;
   p.n_tiles = (g.N + p.block_n - 1) / p.block_n;

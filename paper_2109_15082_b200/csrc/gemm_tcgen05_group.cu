@@ -4,8 +4,10 @@
 // of a kernel of its own.  The tiles of all problems form one list that the CTAs walk round-robin with
 // the pipeline of tc_gemm_kernel: warp 0 streams operand tiles by TMA into a ring of shared-memory
 // stages, warp 1 issues tcgen05.mma into one of two TMEM accumulators, warps 2..9 drain the other one.
-// Every problem brings its own tensor maps, shape, operand layouts and epilogue; the tile width (256)
-// and therefore the stage layout are common.  All waits on mbarriers are bounded in time.
+// Every problem brings its own tensor maps, shape, operand layouts and epilogue; the tile width
+// and therefore the stage layout are common.  Widths 256 / 192 / 128 for the four gradients of a layer, us: hidden 1024, 4096 tokens 84
+// / 94 / 127; hidden 768, 4096 tokens 51 / 49 / 63, 2200 tokens 30.5 / 27.9 / 37; hidden 512, 1000 tokens 12.2 / 10.6 / 14.7; hidden 128,
+// 128 tokens 7.1 / 5.9 / 5.0.  All waits on mbarriers are bounded in time.
 #include <cuda.h>
 
 #include <cstdio>
@@ -237,12 +239,15 @@ bool tc_gemm_group_eligible(const GemmGroupItem* items, int n) {
   return true;
 }
 
-int tc_gemm_group(const GemmGroupItem* items, int n, int* d_status, int sm_count, cudaStream_t stream) {
+int tc_gemm_group(const GemmGroupItem* items, int n, int* d_status, int sm_count, cudaStream_t stream, bool beside) {
   if (!tc_gemm_group_eligible(items, n)) return GEMM_ERR_ARG;
   GroupParams gp;
   GroupMaps maps;
   gp.n = n;
-  const int block_n = 256, block_k = 64;
+  const int block_k = 64;
+  int rows[MAX_GEMM_GROUP], cols[MAX_GEMM_GROUP], blocks[MAX_GEMM_GROUP];
+  for (int i = 0; i < n; ++i) { rows[i] = items[i].g.M; cols[i] = items[i].g.N; blocks[i] = (items[i].g.K + block_k - 1) / block_k; }
+  const int block_n = tc_pick_block_n(rows, cols, blocks, n, 1, sm_count, true, beside);
   gp.stage_bytes = A_STAGE_BYTES + block_n * 128;
   gp.num_stages = SINGLE_CTA_SMEM_BUDGET / gp.stage_bytes;
   int tiles = 0;

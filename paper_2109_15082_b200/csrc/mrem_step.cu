@@ -46,6 +46,7 @@ struct Runner {
   mrem_ctx* c;
   int rc = MREM_OK;
   cudaStream_t st;
+  bool beside = false;               // the other stream has work at the same time
   explicit Runner(mrem_ctx* ctx) : c(ctx), st(ctx->stream) {}
   Runner(mrem_ctx* ctx, cudaStream_t stream) : c(ctx), st(stream) {}
   int okind() const { return c->dt == 1 ? OUT_BF16 : OUT_F32; }
@@ -61,7 +62,7 @@ struct Runner {
   void gemm(const View& A, const View& B, int M, int N, int K, int nb0, int nb1, const Epilogue& e) {
     OperandDesc a{A.p, A.ld, A.sb0, A.sb1, A.mn, 0}, b{B.p, B.ld, B.sb0, B.sb1, B.mn, B.is_static};
     GemmShape g{M, N, K, nb0, nb1};
-    if (c->dt == 1) note(tc_gemm(0, 0, a, b, g, e, 0, c->status, c->sm_count, st), "bf16 GEMM launch failed");
+    if (c->dt == 1) note(tc_gemm(0, 0, a, b, g, e, 0, c->status, c->sm_count, st, beside), "bf16 GEMM launch failed");
     else note(simt_gemm_f32(a, b, g, e, st), "f32 GEMM launch failed");
   }
   // weight-gradient products (bf16 in, fp32 out) of one layer: collected, then launched as one grouped kernel
@@ -75,10 +76,10 @@ struct Runner {
   void flush_deferred() {
     if (deferred.empty()) return;
     if ((int)deferred.size() <= MAX_GEMM_GROUP && tc_gemm_group_eligible(deferred.data(), (int)deferred.size())) {
-      note(tc_gemm_group(deferred.data(), (int)deferred.size(), c->status, c->sm_count, st), "grouped weight-gradient GEMM launch failed");
+      note(tc_gemm_group(deferred.data(), (int)deferred.size(), c->status, c->sm_count, st, beside), "grouped weight-gradient GEMM launch failed");
     } else {
       for (const GemmGroupItem& it : deferred)
-        note(tc_gemm(0, 0, it.A, it.B, it.g, it.epi, 0, c->status, c->sm_count, st), "bf16 GEMM launch failed");
+        note(tc_gemm(0, 0, it.A, it.B, it.g, it.epi, 0, c->status, c->sm_count, st, beside), "bf16 GEMM launch failed");
     }
     deferred.clear();
   }
@@ -86,7 +87,7 @@ struct Runner {
   void gemm_i8(const int8_t* A, int a_unsigned, const int8_t* B, int M, int N, int K, const Epilogue& e) {
     OperandDesc a{A, K, 0, 0, 0, 0}, b{B, K, 0, 0, 0, 1};      // B: weight codes, written by the last update
     GemmShape g{M, N, K, 1, 1};
-    note(tc_gemm(1, a_unsigned, a, b, g, e, 0, c->status, c->sm_count, st), "int8 GEMM launch failed");
+    note(tc_gemm(1, a_unsigned, a, b, g, e, 0, c->status, c->sm_count, st, beside), "int8 GEMM launch failed");
   }
 };
 
@@ -128,6 +129,7 @@ int float_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S, 
   const long long M = (long long)B * S;
   cudaStream_t st = (!student_params && !init_steps && c->teacher_stream) ? c->teacher_stream : c->stream;
   Runner r(c, st);
+  r.beside = c->teacher_stream != nullptr;
   const int ok = r.okind();
   const void* cur = x;
   for (int l = 0; l < d.n_layers; ++l) {
@@ -193,6 +195,7 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
   const int H = d.hidden, F = d.ffn, h = d.n_heads, hd = H / h;
   const long long M = (long long)B * S;
   Runner r(c);
+  r.beside = c->teacher_stream != nullptr;
   const int ok = r.okind();
   const void* cur = x;
   for (int l = 0; l < d.n_layers; ++l) {
@@ -291,6 +294,7 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
   const bool two_streams = c->use_side_stream && c->side_stream && !c->trace_on;
   cudaStream_t side = two_streams ? c->side_stream : c->stream;
   Runner rw(c, side);                            // weight-gradient products
+  r.beside = rw.beside = two_streams && o;
   bool sync_failed = false;
   auto fork = [&]() {                            // side stream: wait for what the main stream has enqueued so far
     if (two_streams && (cudaEventRecord(c->ev_fork, c->stream) != cudaSuccess || cudaStreamWaitEvent(side, c->ev_fork, 0) != cudaSuccess))
@@ -681,6 +685,7 @@ int32_t mrem_rem_step(mrem_ctx* c, int32_t layer, int32_t tensor_id, const void*
   const bool two_streams = c->use_side_stream && c->side_stream && !c->trace_on;
   cudaStream_t side = two_streams ? c->side_stream : st;
   Runner rs(c, side);
+  r.beside = rs.beside = two_streams;
   bool sync_failed = false;
   auto after = [&](cudaEvent_t ev, cudaStream_t waits, cudaStream_t done) {      // `waits` goes on when `done` has got here
     if (two_streams && (cudaEventRecord(ev, done) != cudaSuccess || cudaStreamWaitEvent(waits, ev, 0) != cudaSuccess)) sync_failed = true;

@@ -184,6 +184,29 @@ def test_gemm_float_layouts(dtype, a_mn, b_mn, M, N, K, nb):
     assert rel < 2e-6, rel
 
 
+# sizes whose tiles are 192 columns wide (two rounds of tiles where 256 columns take two as well): whole tiles, one of 32 columns
+# at the end, rows of the output on no 32-byte boundary; a ragged last block of the inner dimension
+@pytest.mark.parametrize("N", [2304, 2336, 2250])
+def test_gemm_exact_on_tiles_of_192_columns(N):
+    M, K = 2200, 264
+    rng = np.random.default_rng(N)
+    a, b = rng.integers(-127, 128, (M, 2 * K)), rng.integers(-127, 128, (N, 2 * K))
+    ref = O.int_matmul(a[:, :K], b[:, :K])                     # |sum| < 2^24: exact in fp32
+    st = _status()
+    for a_mn, b_mn in ((0, 0), (0, 1), (1, 1)):
+        if b_mn and N % 8:
+            continue                                           # the strides of an operand are multiples of 16 bytes
+        ad = torch.from_numpy(_layout(a[None, :, :K], a_mn)).to(DEV).to(torch.bfloat16).contiguous()
+        bd = torch.from_numpy(_layout(b[None, :, :K], b_mn)).to(DEV).to(torch.bfloat16).contiguous()
+        out = torch.full((M, N), 0.5, device=DEV)
+        B.mrem_gemm(B.BF16, ad, a_mn, M if a_mn else K, 0, bd, b_mn, N if b_mn else K, 0, M, N, K, 1, 1.0, out, N, 0, 0, st, _stream())
+        assert np.array_equal(out.cpu().numpy().astype(np.int64), ref), (a_mn, b_mn)
+    acc = torch.full((M, N), -1, dtype=torch.int32, device=DEV)
+    B.mrem_gemm_i8(torch.from_numpy(a.astype(np.int8)).to(DEV), 0, torch.from_numpy(b.astype(np.int8)).to(DEV), M, N, 2 * K, acc, 0, st, _stream())
+    assert np.array_equal(acc.cpu().numpy().astype(np.int64), O.int_matmul(a, b))
+    assert int(st[0]) == 0
+
+
 @pytest.mark.parametrize("shape", [(128, 64, 384, 2), (320, 576, 208, 1), (4096, 1024, 128, 1)])
 @pytest.mark.parametrize("a_mn,b_mn", [(0, 0), (0, 1), (1, 0), (1, 1)])
 def test_gemm_bf16_on_integer_codes_is_exact(a_mn, b_mn, shape):
