@@ -364,29 +364,34 @@ ln_bwd_cols_kernel(const T* __restrict__ dout, const T* __restrict__ x, const T*
   }
 }
 
-// out_k[c] = sum over n parts of part[i][k][c], in index order within 32 runs of them and the runs in order; 32 columns a block.
+// out_k[c] = sum over n parts of part[i][k][c], in index order within 32 runs of them and the runs in order; 32 columns a block.  Added
+// in 64 bits, so that the sums are as exact as the parts: in 32 bits these two chains (19 and 32 long at 592 parts) were most of the error.
 __global__ void __launch_bounds__(256) col_finish_kernel(const float* __restrict__ part, int n, int cols, float* __restrict__ out0,
                                                          float* __restrict__ out1, float* __restrict__ out2) {
   pdl_wait();
   pdl_trigger();
-  __shared__ __align__(16) float4 red[32][8];
+  __shared__ double red[32][33];
   const int run = threadIdx.x >> 3, k4 = threadIdx.x & 7, width = 3 * cols;
   const int i = ((int)blockIdx.x * 8 + k4) * 4, per = (n + 31) / 32, k0 = run * per, k1 = min(n, k0 + per);
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  double v[4] = {0., 0., 0., 0.};
   if (i < width) {
-#pragma unroll 10
-    for (int k = k0; k < k1; ++k) {
+#pragma unroll 5
+    for (int k = k0; k < k1; k += 2) {                        // (pairs in 32 bits: half the conversions)
       const float4 e = *reinterpret_cast<const float4*>(part + (long long)k * width + i);
-      v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w;
+      const float4 f = k + 1 < k1 ? *reinterpret_cast<const float4*>(part + (long long)(k + 1) * width + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[0] += e.x + f.x; v[1] += e.y + f.y; v[2] += e.z + f.z; v[3] += e.w + f.w;
     }
   }
-  red[run][k4] = v;
-  __syncthreads();
-  if (run != 0 || i >= width) return;
 #pragma unroll
-  for (int w = 1; w < 32; ++w) { const float4 e = red[w][k4]; v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w; }
-  const int pl = i / cols, col = i - pl * cols;                // (cols is a multiple of 4)
-  *reinterpret_cast<float4*>((pl == 0 ? out0 : (pl == 1 ? out1 : out2)) + col) = v;
+  for (int j = 0; j < 4; ++j) red[run][4 * k4 + j] = v[j];
+  __syncthreads();
+  const int c = (int)threadIdx.x, o = (int)blockIdx.x * 32 + c;
+  if (c >= 32 || o >= width) return;
+  double t = red[0][c];
+#pragma unroll
+  for (int w = 1; w < 32; ++w) t += red[w][c];
+  const int pl = o / cols;
+  (pl == 0 ? out0 : (pl == 1 ? out1 : out2))[o - pl * cols] = (float)t;
 }
 
 // ------------------------------------------------------------------ column sums over rows
