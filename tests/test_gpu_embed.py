@@ -32,6 +32,21 @@ def _problem(act_dtype, e_bits, V=500, H=128, P=48, batch=5, seq=40, seed=3):
     return e, desc, teacher, student, step, ids.astype(np.int32), tt
 
 
+# a few rows a chunk, chunks without rows; many rows a chunk
+@pytest.mark.parametrize("H,batch,seq", [(128, 7, 33), (528, 1, 20), (256, 32, 128)])
+def test_layernorm_sums_of_the_embedding_are_close_to_those_of_64_bits(H, batch, seq):
+    """The bias gradient is the sum over the tokens of 2 c (student - teacher).  A rounding of the result is 0.4 2^-24 of it in the
+    2-norm, each level of 32-bit additions adds as much in quadrature: about six (chains of few rows, of twelve chunks, and
+    the ends), 1.0 2^-24 (1.0 seen; 1.8 where the chunks are one chain)."""
+    e, _, _, _, _, ids, tt = _problem("f32", 4, H=H, P=128, batch=batch, seq=seq)
+    e.step(torch.from_numpy(ids).to(e.device), torch.from_numpy(tt).to(e.device), None)
+    e_t, e_s = e.outputs(batch, seq)
+    c2 = 2 * (torch.ones((), device=e.device) / torch.full((), float(batch * seq * H), device=e.device))
+    d = (c2 * (e_s - e_t)).view(-1, H).double()
+    assert rel(e.g["ln_b"].cpu().numpy(), d.sum(0).cpu().numpy()) < 1.3 * 2.0 ** -24
+    assert int(e.status[0]) == 0
+
+
 # the last case has the sizes of BERT-large's embedding layers and of the benchmark batch (32 x 128 tokens)
 @pytest.mark.parametrize("act_dtype,e_bits,sizes", [("bf16", 4, {}), ("bf16", 2, {}), ("f32", 8, {}),
                                                     ("bf16", 4, dict(V=30522, H=1024, P=512, batch=32, seq=128))])
