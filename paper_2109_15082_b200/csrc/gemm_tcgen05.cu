@@ -387,7 +387,11 @@ int pick_split(int M, int N, int k_blocks, int batches, int sm_count, int* split
 // 8.6 / 8.0; on the other side 4096 x 4096 x 1024 27 / 30, 4096 x 1024 x 4096 25 / 41.  Forward of both modules, one after the other, 32 x
 // 128 tokens, hidden 768: 602 -> 577 us; 11 x 200 tokens with gradients 387 -> 376.  But those SMs are not idle when another stream's
 // kernels run `beside` the launch, and 192 columns take more SM time in all (step of 16 x 384 tokens, hidden 1024: 5850 -> 5974
-// us; 32 x 128, hidden 768: 1198 -> 1202): then not.  fp32 outputs (`wide_out`) take longer to store.
+// us; 32 x 128, hidden 768: 1198 -> 1202): then not.  That holds for a step's teacher pass, its backward pass with the update under it and
+// the per-product step, whichever streams they are issued to.  Not for the student's pass, whose int8 products are half as long (without
+// 192 columns 8 x 256, hidden 768 976 -> 981 us, 16 x 384 and 32 x 128 within 0.1 %), nor for gradients alone, which leave little
+// to the other stream (32 x 128, hidden 768 441 -> 448 us, 11 x 200 377 -> 383, hidden 1024 within 0.5 %).  `wide_out`: a group's fp32
+// outputs, which take longer to store (single products' are costed as bf16).
 int tc_pick_block_n(const int* M, const int* N, const int* k_blocks, int n, int batches, int sm_count, bool wide_out, bool beside) {
   static const struct { int bn; double step, tile, fixed, fixed_f32; } widths[] = {
       {64, 0.29, 0.8, 2.8, 3.5}, {128, 0.30, 1.5, 3.4, 4.4}, {192, 0.31, 2.2, 3.7, 5.3}, {256, 0.345, 2.8, 4.3, 6.4}};
@@ -500,9 +504,10 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
   }
   const int grid = p.num_tiles < sm_count ? p.num_tiles : sm_count;
   Scope sc([&] {
-    char buf[40];
-    snprintf(buf, sizeof(buf), "%s %dx%dx%d%s%s b%d", kind == 0 ? "gemm_bf16" : "gemm_i8", g.M, g.N, g.K,
-             A.mn_contig ? "T" : "N", B.mn_contig ? "N" : "T", g.nb0 * g.nb1);
+    char buf[40];                          // (shape, operand layouts, batches, tile width, thread blocks per tile)
+    int len = snprintf(buf, sizeof(buf), "%s %dx%dx%d%s%s b%d w%d", kind == 0 ? "gemm_bf16" : "gemm_i8", g.M, g.N, g.K,
+                       A.mn_contig ? "T" : "N", B.mn_contig ? "N" : "T", g.nb0 * g.nb1, p.block_n);
+    if (splits > 1 && len < (int)sizeof(buf)) snprintf(buf + len, sizeof(buf) - len, "/%d", splits);
     return std::string(buf);
   }, 2.0 * g.M * g.N * (double)g.K * g.nb0 * g.nb1, 1, stream, 0);
   if (splits > 1) return tc_gemm_split_launch(kind, ma, mb, mc, p, splits, stream);

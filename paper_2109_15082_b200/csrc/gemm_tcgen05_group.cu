@@ -291,7 +291,7 @@ int tc_gemm_group(const GemmGroupItem* items, int n, int* d_status, int sm_count
   const int grid = tiles < sm_count ? tiles : sm_count;
   Scope sc([&] {
     char buf[48];
-    snprintf(buf, sizeof(buf), "gemm_bf16 group of %d, %d tiles", n, tiles);
+    snprintf(buf, sizeof(buf), "gemm_bf16 group of %d, %d tiles w%d", n, tiles, block_n);
     return std::string(buf);
   }, flops, 1, stream, 0);
   if (launch_k(tc_gemm_group_kernel, grid, GEMM_THREADS, smem, stream, maps, gp) != cudaSuccess) return GEMM_ERR_CUDA;

@@ -121,7 +121,8 @@ struct mrem_ctx {
   cudaStream_t side_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_layer[2] = {nullptr, nullptr};   // side stream done with the gradient buffers of a layer parity
-  cudaStream_t teacher_stream = nullptr;   // set for the duration of a step that runs the teacher pass beside the student's
+  cudaStream_t teacher_stream = nullptr;   // set while a step enqueues the teacher pass beside the student's
+  bool teacher_beside = false;             // set while a step enqueues the teacher pass: the student's fills the SMs that its products leave idle
   // classification head of the model's last module (null: none): the output-logit term of the loss
   struct { const float *wp = nullptr, *bp = nullptr, *wc = nullptr, *bc = nullptr; int n_classes = 0; float* logit_loss = nullptr; float* logits = nullptr; } head;
   float loss_share = 1.f;            // this context's share of the whole batch (data parallel: local / global sequences)

@@ -23,15 +23,19 @@ int enqueue_step(mrem_ctx* c, const void* xt, const void* xs, float lambda, cons
   // teacher's runs on the side stream beside the student's (its tensor-core products under the student's quantizer
   // kernels).  BERT-base, 3 layers, 32 x 128, lambda 0.5: one after the other 1276 us, side by side 1208.  Only with the fused
   // attention kernel, whose path shares no scratch between the passes.
-  const bool beside = c->use_side_stream && c->side_stream && !c->trace_on && c->d.n_heads > 0 &&
-                      attention_fwd_supported(seq, c->d.hidden / c->d.n_heads, c->dt);
+  const bool pair = c->d.n_heads > 0 && attention_fwd_supported(seq, c->d.hidden / c->d.n_heads, c->dt);
+  const bool beside = pair && c->use_side_stream && c->side_stream && !c->trace_on;
+  c->teacher_beside = pair;      // (also on one stream, and while kernels are traced one by one: the step's kernels stay the same)
   if (rc == MREM_OK && beside) {
-    if (cudaEventRecord(c->ev_fork, c->stream) != cudaSuccess || cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0) != cudaSuccess)
+    if (cudaEventRecord(c->ev_fork, c->stream) != cudaSuccess || cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0) != cudaSuccess) {
+      c->teacher_beside = false;
       return fail(c, MREM_ERR_CUDA, "step: stream fork failed");
+    }
     c->teacher_stream = c->side_stream;
   }
   if (rc == MREM_OK) rc = mrem_module_forward(c, MREM_TEACHER, xt, nullptr, 0.f, len, batch, seq, t_out);
   c->teacher_stream = nullptr;
+  c->teacher_beside = false;
   if (rc == MREM_OK) rc = mrem_module_forward(c, MREM_STUDENT, xs, xt, lambda, len, batch, seq, s_out);
   if (beside && (cudaEventRecord(c->ev_join, c->side_stream) != cudaSuccess || cudaStreamWaitEvent(c->stream, c->ev_join, 0) != cudaSuccess))
     return fail(c, MREM_ERR_CUDA, "step: stream join failed");

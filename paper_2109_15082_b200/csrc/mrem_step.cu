@@ -46,7 +46,7 @@ struct Runner {
   mrem_ctx* c;
   int rc = MREM_OK;
   cudaStream_t st;
-  bool beside = false;               // the other stream has work at the same time
+  bool beside = false;               // the SMs its products leave idle are filled from the other stream (see tc_pick_block_n)
   explicit Runner(mrem_ctx* ctx) : c(ctx), st(ctx->stream) {}
   Runner(mrem_ctx* ctx, cudaStream_t stream) : c(ctx), st(stream) {}
   int okind() const { return c->dt == 1 ? OUT_BF16 : OUT_F32; }
@@ -129,7 +129,7 @@ int float_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S, 
   const long long M = (long long)B * S;
   cudaStream_t st = (!student_params && !init_steps && c->teacher_stream) ? c->teacher_stream : c->stream;
   Runner r(c, st);
-  r.beside = c->teacher_stream != nullptr;
+  r.beside = c->teacher_beside;
   const int ok = r.okind();
   const void* cur = x;
   for (int l = 0; l < d.n_layers; ++l) {
@@ -194,8 +194,7 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
   const mrem_module_desc& d = c->d;
   const int H = d.hidden, F = d.ffn, h = d.n_heads, hd = H / h;
   const long long M = (long long)B * S;
-  Runner r(c);
-  r.beside = c->teacher_stream != nullptr;
+  Runner r(c);                                   // (nothing here runs `beside` another stream: see tc_pick_block_n)
   const int ok = r.okind();
   const void* cur = x;
   for (int l = 0; l < d.n_layers; ++l) {
@@ -294,7 +293,7 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
   const bool two_streams = c->use_side_stream && c->side_stream && !c->trace_on;
   cudaStream_t side = two_streams ? c->side_stream : c->stream;
   Runner rw(c, side);                            // weight-gradient products
-  r.beside = rw.beside = two_streams && o;
+  r.beside = rw.beside = o != nullptr;
   bool sync_failed = false;
   auto fork = [&]() {                            // side stream: wait for what the main stream has enqueued so far
     if (two_streams && (cudaEventRecord(c->ev_fork, c->stream) != cudaSuccess || cudaStreamWaitEvent(side, c->ev_fork, 0) != cudaSuccess))
@@ -685,7 +684,7 @@ int32_t mrem_rem_step(mrem_ctx* c, int32_t layer, int32_t tensor_id, const void*
   const bool two_streams = c->use_side_stream && c->side_stream && !c->trace_on;
   cudaStream_t side = two_streams ? c->side_stream : st;
   Runner rs(c, side);
-  r.beside = rs.beside = two_streams;
+  r.beside = rs.beside = true;
   bool sync_failed = false;
   auto after = [&](cudaEvent_t ev, cudaStream_t waits, cudaStream_t done) {      // `waits` goes on when `done` has got here
     if (two_streams && (cudaEventRecord(ev, done) != cudaSuccess || cudaStreamWaitEvent(waits, ev, 0) != cudaSuccess)) sync_failed = true;

@@ -17,6 +17,16 @@ def rel(got, ref):
     return float(np.linalg.norm(got - ref) / max(np.linalg.norm(ref), 1e-300))
 
 
+def traced(m, fn):
+    """{name: launches} of the kernels that fn launches on the module's context; a product's name says its tiles' width."""
+    B.mrem_trace_enable(m.ctx, 1)
+    try:
+        fn()
+        return {e["name"]: e["launches"] for e in B.mrem_trace_read(m.ctx, 128) if e["name"] != "(empty kernel)"}
+    finally:
+        B.mrem_trace_enable(m.ctx, 0)
+
+
 class Problem:
     """A module pair on the GPU and its twin in the oracle, from identical bytes."""
 

@@ -14,7 +14,7 @@ import torch
 from oracle import mrem_oracle as O
 from paper_2109_15082_b200 import binding as B
 from paper_2109_15082_b200 import synth
-from tests.gpu_util import Problem, compare_grads, rel
+from tests.gpu_util import Problem, compare_grads, rel, traced
 from tests.torch_storage_ref import teacher_layer_torch
 
 pytestmark = pytest.mark.gpu
@@ -379,6 +379,36 @@ def test_graph_replay_and_host_step_equal_eager():
         assert losses == results[0][0]
         assert np.array_equal(w1, results[0][1])
     assert results[0][0][2] != results[0][0][0]
+
+
+def test_a_traced_step_launches_the_step_s_products():
+    """12 x 128 tokens, hidden 768, on 148 SMs: alone, the teacher's QKV product is one round of 144 tiles of 192 columns; in a step,
+    whose student pass fills idle SMs, of 108 tiles of 256.  A step that is traced, or issued to one stream, launches what the step on
+    two streams does, and a call by itself chooses for itself again, also after a step that failed."""
+    wl = _wl("base3_w4a8", n_layers=1, seq=128, batch=12, len_lo=128)
+    p = Problem(wl)
+    try:
+        m = p.m
+        x, vl = p.xd.cpu().pin_memory(), torch.from_numpy(p.vl).pin_memory()
+        opt = B.make_optim(lr=1e-4, step=1)
+        step = lambda lam=0.0: B.mrem_recon_step_host(m.ctx, x, x, vl, wl.batch, wl.seq, lam, opt)
+        alone = lambda: traced(m, lambda: m.forward_teacher(p.xd, p.vld, wl.batch, wl.seq))
+        qkv = "gemm_bf16 1536x2304x768NT b1 w%d"
+        first = alone()
+        assert first[qkv % 192] == 1 and qkv % 256 not in first, first
+        m.quantize_weights()
+        in_step = traced(m, step)
+        assert in_step[qkv % 256] == 1 and qkv % 192 not in in_step, in_step
+        assert in_step["gemm_i8 1536x2304x768NT b1 w192"] == 1, in_step
+        B.mrem_set_two_streams(m.ctx, 0)
+        assert traced(m, step) == in_step
+        B.mrem_set_two_streams(m.ctx, 1)
+        with pytest.raises(B.MremError):
+            step(2.0)
+        assert alone() == first
+        assert m.poll_status() == 0
+    finally:
+        p.close()
 
 
 @pytest.mark.parametrize("lam", [0.35, 1.0])
