@@ -147,6 +147,12 @@ def compare_grads(gpu, ora, tol, skip_small=1e-12, check_offset=True, scalar_tol
     return worst
 
 
+def loss_gradients_apart(gpu, ora):
+    """Relative L2 distance of the loss gradients, in which all gradients are linear: differences of two outputs stored in bf16,
+    a few times as large as the outputs' spacing."""
+    return max(rel(gpu["f_s"][l] - gpu["f_t"][l], ora["f_s"][l] - ora["f_t"][l]) for l in range(len(ora["f_s"])))
+
+
 def code_flip_rate(codes_gpu, codes_ref):
     return float((np.asarray(codes_gpu) != np.asarray(codes_ref)).mean())
 

@@ -18,7 +18,7 @@ import torch
 from oracle import mrem_oracle as O
 from paper_2109_15082_b200 import binding as B
 from paper_2109_15082_b200 import synth
-from tests.gpu_util import Problem, bf16_closeness, bf16_step, compare_grads, rel
+from tests.gpu_util import Problem, bf16_closeness, bf16_step, compare_grads, loss_gradients_apart, rel, traced
 from tests.torch_storage_ref import bf16_numbers_apart, teacher_layer_torch
 
 pytestmark = pytest.mark.gpu
@@ -99,6 +99,44 @@ def _every_gradient(case, fused_attention=True):
         # to 5 %, each against max(|reference|, 5 % of the layer's largest); every tensor-valued gradient stays at 2 %
         worst = compare_grads(g["grads"], r["grads"], GRAD_TOL, check_offset=True, deep_scalar_floor=0.05, deep_group_tol=0.05)
         print(case, "loss", g["loss"], r["loss"], "clipped activations", clipped, "clipped weights", w_clipped, "worst gradient", worst)
+    finally:
+        p.close()
+
+
+# the tiles' widths of the two groups, feed-forward and attention, on 148 SMs; every width has an N that is no multiple of it
+@pytest.mark.parametrize("hidden,ffn,batch,seq,widths", [(320, 640, 3, 40, {"w128"}), (576, 2240, 3, 72, {"w192", "w128"}),
+                                                         (768, 3040, 9, 128, {"w256", "w128"})])
+def test_grouped_weight_gradients_on_tiles_of_every_width(hidden, ffn, batch, seq, widths):
+    wl = _wl("base3_w4a8", n_layers=1, hidden=hidden, n_heads=hidden // 64, ffn=ffn, seq=seq, batch=batch, len_lo=seq // 3, len_hi=seq)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002)
+    try:
+        got, r = p.run_gpu(), p.run_oracle()
+        names = traced(p.m, p.run_gpu)
+        assert {n.split()[-1] for n in names if n.startswith("gemm_bf16 group")} == widths, names
+        apart = loss_gradients_apart(got, r)
+        assert apart < 5e-2, apart
+        for k in O.WEIGHTS:
+            assert rel(got["grads"][0][k], r["grads"][0][k]) < GRAD_TOL + apart, (k, rel(got["grads"][0][k], r["grads"][0][k]), apart)
+    finally:
+        p.close()
+
+
+# 192 columns: scale and bias (QKV, FFN1 at 2200 tokens), scale, bias and residual (output projection, FFN2 at 3200 and 4096)
+@pytest.mark.parametrize("batch,seq,wide", [(11, 200, {"2304x768", "3072x768"}), (25, 128, {"768x768", "768x3072"}), (32, 128, {"768x768", "768x3072"})])
+def test_a_sequence_in_a_batch_on_tiles_of_192_columns_has_the_bits_it_has_alone(batch, seq, wide):
+    """The quantized pass multiplies whole numbers and treats rows independently (see tests/test_gpu_gemm_split.py)."""
+    wl = _wl("base3_w4a8", n_layers=1, batch=batch, seq=seq, len_lo=seq // 3, len_hi=seq)
+    p = Problem(wl, student_noise=0.002)
+    try:
+        m = p.m
+        m.quantize_weights()
+        names = traced(m, lambda: m.forward_student(p.xd, p.vld, batch, seq))
+        at_192 = {n.split()[1].split("x", 1)[1].rstrip("NT") for n in names if n.startswith("gemm_i8") and n.endswith("w192")}
+        assert wide <= at_192, names
+        many = m.forward_student(p.xd, p.vld, batch, seq).clone()
+        for i in (0, batch // 2, batch - 1):
+            assert torch.equal(m.forward_student(p.xd[i:i + 1].contiguous(), p.vld[i:i + 1].clone(), 1, seq)[:, 0], many[:, i]), i
+        assert m.poll_status() == 0
     finally:
         p.close()
 
