@@ -653,6 +653,8 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   // LayerNorm not).  The rows that no token gathered need nothing of this step but the marks.  The two launches before the last take
   // as many of them as memory can serve beside their own chains of loads; the last one, which is bound by memory, the rest: its
   // blocks keep more bytes in flight.  30522 x 1024 with 32 x 128 tokens 199 -> 192 us, 30522 x 768 with 5 x 56 tokens 150 -> 125.
+  // Their shares, a number of rows that grows with the tokens, whose chains last that long, and a constant number of bytes (16 and 99 MB at
+  // 29 bytes a weight) for what a launch waits at its ends, were fitted at these two sizes.
   // (No idle rows beside the sums of many tokens: 197 and 125; seven eighths of the table beside the sums: 204 and 128; idle blocks
   // spread evenly among those of the sums: 196 and 126.)
   const RowUpdate table{x->word, x->g_word, x->m_word, x->v_word, x->word_step, x->m_word_step, x->v_word_step, nullptr,

@@ -351,6 +351,10 @@ namespace {
 // the tiles are few and the inner dimension is long.  Alone / shared, us: 216 x 768 x 3072 17.0 / 9.5 (int8 codes 10.4 / 7.4),
 // 216 x 768 x 2304 13.5 / 8.6, 512 x 768 x 3072 17.3 / 11.8, 1024 x 1024 x 4096 22.9 / 17.1, 128 x 1024 x 1024 7.8 / 6.9,
 // 216 x 768 x 768 6.7 / 6.3; on the other side of the line 512 x 1024 x 1024 8.2 / 9.2, 1024 x 1024 x 1024 8.5 / 8.8.
+// The figures of both sides below are of the loops before the loads were issued from a whole warp.  Judged by tc_pick_block_n's newer ones
+// the sharing would end earlier at 1.1 % of the products of 128 to 1024 wide layers (fewer than 2400 tokens): there it is still the better one,
+// alone (best width) / shared: 1160 x 512 x 1536 10.1 / 9.7, 1664 x 512 x 2048 12.5 / 11.1, 1280 x 768 x 2304 13.7 / 11.6, 768 x 256 x 768
+// 6.55 / 6.3, int8 256 x 512 x 1536 6.9 / 6.1, 896 x 768 x 3072 10.7 / 9.5, 1152 x 1024 x 4096 13.0 / 10.9.
 // No more tiles than all clusters can hold at once: cudaOccupancyMaxActiveClusters gives 74 clusters of two and 33 of four for
 // every variant on an idle chip; the limits, 72 and 32, lie below that (no product of a 768 or 1024 wide layer has one of the
 // few tile counts between).  Returns the tile width of the shared form (at most 128), or 0 with *splits = 1.

@@ -163,8 +163,8 @@ int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat
                               void* dy, float* part_s, float* col_part, int dt, cudaStream_t st);
 void launch_col_finish(const float* col_part, int n, int cols, float* out0, float* out1, float* out2, cudaStream_t st);
 
-// Column sums over rows: out0[c] = sum_r a[r,c]; with y/mean/rstd also out1[c] = sum_r a[r,c]*(y[r,c]-mean[r])*rstd[r];
-// with a2 also out2[c] = sum_r a2[r,c].  One kernel: per-chunk partials in `scratch` (three planes of
+// Column sums over rows: out0[c] = sum_r a[r,c]; with y/mean/rstd and a2, which come together, also
+// out1[c] = sum_r a[r,c]*(y[r,c]-mean[r])*rstd[r] and out2[c] = sum_r a2[r,c].  One kernel: per-chunk partials in `scratch` (three planes of
 // `plane_floats` floats each, plane_floats >= cols; the launcher takes as many row chunks as a plane holds),
 // summed in a fixed order by the last block of each column group.  `counters` (>= cols/32 + 1 ints) must be
 // zero before the first launch; the kernel leaves them zero.

@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(128) ln_bwd_kernel(const T* __restrict__ dout,
 // No more than 128 threads a block and no shared memory to speak of, so that blocks fit beside a product of the other stream (with
 // 256 threads and the groups added up in shared memory they did not).  Two rows in flight per group.
 // One warp per row with the row in its registers, dv written out, and a launch that read dv, y and dy again for the sums: the steps
-// of 32 x 128 tokens, hidden 1024, 3512 us (now 3465), of 16 x 384 5911 (5828), of 8 x 256, hidden 768, 995 (984), of 3 x 72 461
-// (456).
+// of 32 x 128 tokens, hidden 1024, 3512 us (now 3465), of 8 x 256, hidden 768, 995 (984), of 3 x 72 461 (456); 16 x 384, hidden 1024 within
+// the 0.8 % by which two runs differ.
 __host__ __device__ constexpr int ln_groups(int W) { return W >= 3 ? 1 : 4 / W; }
 constexpr int LN_ROWS = 2;                                     // rows a group has in flight
 template <typename T, int V, int W, bool STE>
@@ -395,16 +395,17 @@ __global__ void __launch_bounds__(256) col_finish_kernel(const float* __restrict
 }
 
 // ------------------------------------------------------------------ column sums over rows
-// out0[c] = sum_r a[r,c];  out1[c] = sum_r a[r,c] * (y[r,c] - mean[r]) * rstd[r] (when y);  out2[c] = sum_r a2[r,c]
-// (when a2).  A block of 8 x 32 threads owns 8*V columns (one 128-byte line per row for 16-byte vectors) of
-// one chunk of rows (gridDim.y chunks): a thread keeps NB rows' loads in flight (as many as the registers hold for one,
-// two or three tensors: latency bounds this kernel) and adds them in row
+// out0[c] = sum_r a[r,c];  with y and a2 also out1[c] = sum_r a[r,c] * (y[r,c] - mean[r]) * rstd[r] and out2[c] = sum_r a2[r,c].
+// A block of 8 x 32 threads owns 8*V columns (one 128-byte line per row for 16-byte vectors) of
+// one chunk of rows (gridDim.y chunks): a thread keeps NB rows' loads in flight (as many as the registers hold for one
+// or three tensors: latency bounds this kernel) and adds them in row
 // order, the block adds its 32 row groups in index order; the last block to finish a column group (ticket
 // counter) adds the chunks' partials in index order, so the result does not depend on scheduling.
 // Four rows at a time whatever the tensors, and eight chunks at a time in the last block: 11 x 200 tokens, hidden 768, gradients 394 -> 391 us;
-// 32 x 128, hidden 1024, six layers 3559 -> 3540; the embedding step of the same tokens 201.3 -> 200.4.
+// 32 x 128, hidden 1024, six layers 3559 -> 3540 (both before the sums of three tensors joined the LayerNorm backward, which leaves
+// this kernel those of rows too wide for it and those of one tensor).
 constexpr int COLRED_CT = 8, COLRED_RT = 32;
-template <typename T, int V, bool HAS_Y, bool HAS_A2, int NB>
+template <typename T, int V, bool ALL, int NB>
 __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict__ a, long long ld_a,
                                                             const T* __restrict__ y, const float* __restrict__ mean,
                                                             const float* __restrict__ rstd, const T* __restrict__ a2,
@@ -415,8 +416,7 @@ __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict_
   pdl_wait();
   pdl_trigger();
   constexpr int BC = COLRED_CT * V;                        // columns per block
-  static_assert(HAS_Y || !HAS_A2, "the planes are counted");
-  constexpr int PLANES = HAS_A2 ? 3 : (HAS_Y ? 2 : 1);
+  constexpr int PLANES = ALL ? 3 : 1;
   __shared__ float sh[PLANES][COLRED_RT][BC + 1];
   __shared__ int is_last;
   const int tx = threadIdx.x % COLRED_CT, ty = threadIdx.x / COLRED_CT;
@@ -430,15 +430,18 @@ __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict_
   if (c < cols) {
     constexpr int RW = RawWords<T, V>::N;
     for (long long rb = r0 + ty; rb < r1; rb += NB * COLRED_RT) {
-      uint32_t v[NB][RW], w[HAS_Y ? NB : 1][RW], u[HAS_A2 ? NB : 1][RW];
+      uint32_t v[NB][RW], w[ALL ? NB : 1][RW], u[ALL ? NB : 1][RW];
       float mu[NB], rs[NB];
 #pragma unroll
       for (int k = 0; k < NB; ++k) {                      // all loads of NB rows first (raw words: few registers)
         const long long r = rb + COLRED_RT * k;
         if (r < r1) {
           load_raw<T, V>(a + r * ld_a + c, v[k]);
-          if (HAS_Y) { load_raw<T, V>(y + r * cols + c, w[k]); mu[k] = mean[r]; rs[k] = rstd[r]; }
-          if (HAS_A2) load_raw<T, V>(a2 + r * ld_a2 + c, u[k]);
+          if (ALL) {
+            load_raw<T, V>(y + r * cols + c, w[k]);
+            mu[k] = mean[r]; rs[k] = rstd[r];
+            load_raw<T, V>(a2 + r * ld_a2 + c, u[k]);
+          }
         }
       }
 #pragma unroll
@@ -448,12 +451,10 @@ __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict_
           widen_raw<T, V>(v[k], fv);
 #pragma unroll
           for (int j = 0; j < V; ++j) a0[j] += fv[j];
-          if (HAS_Y) {
+          if (ALL) {
             widen_raw<T, V>(w[k], fw);
 #pragma unroll
             for (int j = 0; j < V; ++j) a1[j] += fv[j] * (fw[j] - mu[k]) * rs[k];
-          }
-          if (HAS_A2) {
             widen_raw<T, V>(u[k], fw);
 #pragma unroll
             for (int j = 0; j < V; ++j) a2s[j] += fw[j];
@@ -465,8 +466,7 @@ __global__ void __launch_bounds__(256, 2) col_reduce_kernel(const T* __restrict_
 #pragma unroll
   for (int j = 0; j < V; ++j) {
     sh[0][ty][tx * V + j] = a0[j];
-    if constexpr (HAS_Y) sh[1][ty][tx * V + j] = a1[j];
-    if constexpr (HAS_A2) sh[2][ty][tx * V + j] = a2s[j];
+    if constexpr (ALL) { sh[1][ty][tx * V + j] = a1[j]; sh[2][ty][tx * V + j] = a2s[j]; }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < PLANES * BC; i += 256) {
@@ -731,8 +731,8 @@ void launch_col_finish(const float* col_part, int n, int cols, float* out0, floa
 void launch_col_reduce(const void* a, long long ld_a, const void* y, const float* mean, const float* rstd,
                        const void* a2, long long ld_a2, long long rows, int cols, float* out0, float* out1,
                        float* out2, float* scratch, long long plane_floats, int* counters, int dt, cudaStream_t st) {
-  Scope sc("col_reduce", (double)rows * cols * (dt == 1 ? 2.0 : 4.0) * (1 + (y ? 1 : 0) + (a2 ? 1 : 0)), 0, st);
-  // (a2 never comes without y)
+  Scope sc("col_reduce", (double)rows * cols * (dt == 1 ? 2.0 : 4.0) * (y ? 3 : 1), 0, st);
+  // (y and a2 come together)
   // as many row chunks as one plane of the scratch holds, up to two blocks per SM (one wave) and 128 rows per chunk
 #define MREM_COLRED(T, V) do { const int col_blocks = (cols + COLRED_CT * V - 1) / (COLRED_CT * V); \
     long long chunks = plane_floats / cols; \
@@ -740,10 +740,9 @@ void launch_col_reduce(const void* a, long long ld_a, const void* y, const float
     if (chunks > (rows + 4 * COLRED_RT - 1) / (4 * COLRED_RT)) chunks = (rows + 4 * COLRED_RT - 1) / (4 * COLRED_RT); \
     if (chunks < 1) chunks = 1; \
     dim3 grid(col_blocks, (unsigned)chunks); \
-    if (y && a2) MREM_COLRED_K(T, V, true, true, 4); \
-    else if (y) MREM_COLRED_K(T, V, true, false, 6); \
-    else MREM_COLRED_K(T, V, false, false, 12); } while (0)
-#define MREM_COLRED_K(T, V, Y, A2, NB) launch_k(col_reduce_kernel<T, V, Y, A2, NB>, grid, 256, 0, st, (const T*)a, ld_a, (const T*)y, mean, rstd, (const T*)a2, ld_a2, rows, cols, out0, out1, out2, scratch, plane_floats, counters)
+    if (y) MREM_COLRED_K(T, V, true, 4); \
+    else MREM_COLRED_K(T, V, false, 12); } while (0)
+#define MREM_COLRED_K(T, V, ALL, NB) launch_k(col_reduce_kernel<T, V, ALL, NB>, grid, 256, 0, st, (const T*)a, ld_a, (const T*)y, mean, rstd, (const T*)a2, ld_a2, rows, cols, out0, out1, out2, scratch, plane_floats, counters)
   const bool vec_ok = cols % 8 == 0 && ld_a % 8 == 0 && ld_a2 % 8 == 0 && al16(a) && al16(y) && al16(a2);
   if (dt == 1) { if (vec_ok) MREM_COLRED(bf16, 8); else MREM_COLRED(bf16, 1); }
   else { if (vec_ok) MREM_COLRED(float, 4); else MREM_COLRED(float, 1); }

@@ -65,7 +65,8 @@ struct UpdateParams {
 // with one float4 per thread, the two block sums, the step's own update behind a barrier and the scalars cost each thread as
 // much as its four weights.  So: few threads per row, every thread forms the row's new step itself, and the arithmetic runs
 // on pairs.  Measured: a layer of 1024 x 4096 shapes 87 -> 74 us (floor 59), its three 1024-wide matrices 56 -> 47 us in one
-// launch; 30522 x 1024 table 165 -> 136 us (7.1 TB/s), 30522 x 768 128 -> 116 us.
+// launch; a whole table in one launch, 30522 x 1024 165 -> 136 us (7.1 TB/s), 30522 x 768 128 -> 116 us (today the launches before take
+// part of its rows: embed_step.cu).
 // Variants (X(index, NT, NV, blocks per SM)), by the widest row they hold: 16 weights a thread keep the most bytes in flight
 // (1024 wide: 64 x 4 vectors 136 us, 128 x 2 144 us, 256 x 1 152 us for that table), but 64 x 3 for 768 wide rows, with
 // the same ten blocks on an SM, does not (128 us; 96 x 2 at 62 registers 116 us).
@@ -279,6 +280,7 @@ void launch_table_update(const IdleRows& idle, const TokenRows& tokens, int dt, 
   p.mat[0] = idle.m;
   p.row_end[0] = idle.m.rows;
   p.n = 1;
+  // (bytes: the rows without a gradient only; how many have one the host does not know)
   Scope scope("fused_weight_update", (double)(idle.end - idle.first) * idle.m.cols * 29.0, 0, st);
   if (dt == 1) launch_variant<bf16>(variant_of(idle.m.cols), p, 0, st); else launch_variant<float>(variant_of(idle.m.cols), p, 0, st);
 }
