@@ -155,7 +155,7 @@ void launch_layernorm_bwd(const void* dout, const void* dout2, const void* y, co
 // col_part gets several parts of the sums over the rows of dv, of dv * (y - mean) * rstd and of dy (launch_col_finish adds them),
 // part_s (with x) RED_BLOCKS partial sums of the quantizer's step-size gradient.  Returns the number of parts, or 0 (nothing
 // launched) when the row does not fit the vector path; the caller then runs the separate kernels.
-constexpr int LN_PARTS = 592;                             // at most: four groups per SM
+constexpr int LN_PARTS = 592;                             // at most, of rows from 512 columns on: four groups per SM
 bool layernorm_bwd_cols_supported(int cols, int dt);      // the row width fits (16-byte aligned tensors assumed)
 size_t layernorm_bwd_cols_floats(long long rows, int cols, int dt);      // floats of col_part, up to that many rows
 int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat, const void* add, const float* step, int lo, int hi,

@@ -696,15 +696,19 @@ static int ln_cols_warps(int cols, int dt) {
   return cols % V == 0 && cols <= 32 * V * MAXNV ? (cols + 32 * V - 1) / (32 * V) : 0;
 }
 bool layernorm_bwd_cols_supported(int cols, int dt) { return ln_cols_warps(cols, dt) > 0; }
-// groups: two rows each while there are fewer rows than that takes
-static int ln_cols_grid(long long rows, int W) {
+// groups: two rows each while there are fewer rows than that takes.  Narrow rows have more groups, as many as the bytes of LN_PARTS partial
+// sums 512 wide: with LN_PARTS a few warps per SM walked ten rows each, and a step of 48 x 128 tokens took 489 us at hidden 128 (now 459;
+// 463 with the sums in a launch of their own) and 606 at hidden 256 (582; 593), but 612 with four times LN_PARTS.
+static int ln_cols_grid(long long rows, int cols, int W) {
   const int per = ln_groups(W) * LN_ROWS;
-  const long long want = (rows + per - 1) / per, limit = LN_PARTS / ln_groups(W);
+  int parts = LN_PARTS * 512 / cols;
+  parts = parts < LN_PARTS ? LN_PARTS : (parts > 4 * LN_PARTS ? 4 * LN_PARTS : parts);
+  const long long want = (rows + per - 1) / per, limit = parts / ln_groups(W);
   return (int)(want < limit ? want : limit);
 }
 size_t layernorm_bwd_cols_floats(long long rows, int cols, int dt) {
   const int W = ln_cols_warps(cols, dt);
-  return W == 0 ? 0 : (size_t)ln_cols_grid(rows, W) * ln_groups(W) * 3 * cols;
+  return W == 0 ? 0 : (size_t)ln_cols_grid(rows, cols, W) * ln_groups(W) * 3 * cols;
 }
 
 int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat, const void* add, const float* step, int lo, int hi,
@@ -713,7 +717,7 @@ int launch_layernorm_bwd_cols(const void* dout, const void* x, const void* dxhat
   const int W = ln_cols_warps(cols, dt);
   if (rows <= 0 || W == 0 || !(al16(dout) && al16(x) && al16(dxhat) && al16(add) && al16(y) && al16(dy) && al16(gamma))) return 0;
   Scope sc(x ? "layernorm_bwd_ste" : "layernorm_bwd", (double)rows * cols * (dt == 1 ? 2.0 : 4.0) * (x ? (dout ? 6 : 5) : 3), 0, st);
-  const int grid = ln_cols_grid(rows, W);
+  const int grid = ln_cols_grid(rows, cols, W);
 #define MREM_LN(T, V, W, STE) launch_k(ln_bwd_cols_kernel<T, V, W, STE>, grid, 32 * W * ln_groups(W), 0, st, (const T*)dout, (const T*)x, (const T*)dxhat, (const T*)add, step, (float)lo, (float)hi, (const T*)y, mean, rstd, gamma, rows, cols, (T*)dy, part_s, RED_BLOCKS, col_part)
 #define MREM_LNS(T, V, STE) do { if (W == 1) MREM_LN(T, V, 1, STE); else if (W == 2) MREM_LN(T, V, 2, STE); else if (W == 3) MREM_LN(T, V, 3, STE); else MREM_LN(T, V, 4, STE); } while (0)
   if (dt == 1) { if (x) MREM_LNS(bf16, 8, true); else MREM_LNS(bf16, 8, false); }
