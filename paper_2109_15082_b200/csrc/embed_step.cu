@@ -242,7 +242,7 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 //   max_pos blocks: one position each, two half sums over the batch (even and odd sequences), then that row's update.
 //   TYPE_CHUNKS blocks per token type: one chunk of tokens each; the last chunk to finish adds the chunks in index order
 //     and updates the row.
-//   LN_CHUNKS blocks: the LayerNorm's parameters, the same way.
+//   ln_chunks blocks: the LayerNorm's parameters, the same way.
 //   one warp per token and group of TAB_COLS columns: word table.  The warp of the FIRST token with an id adds the gradients of all tokens with
 //     it in token order: it compares 128 ids at a time up to the last one and keeps four rows' loads in flight.  A row
 //     gathered by more than WARP_MAX tokens is left to the whole block, its warps taking consecutive eighths of the tokens and
@@ -253,8 +253,11 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 // four columns and sixteen chunks) and the walk over the ids (the next 128 are on their way now): step 217 -> 192 us at 32 x 128
 // tokens, 136 -> 125 at 5 x 56.  Three blocks: four spill, 200 -> 207 us there although 280 tokens take 148 instead of 150.
 constexpr int TYPE_CHUNKS = 64;
-constexpr int LN_CHUNKS = 48;
-static_assert(TYPE_CHUNKS % 4 == 0 && LN_CHUNKS % 4 == 0, "see sum_chunks4");
+// Chunks of the LayerNorm's sums: above 4096 tokens twice as many, or their chains are the longest of the launch (table 1000 x 512, 48 x 128
+// tokens 67.0 -> 65.6 us; 30522 x 768, 5 x 56 tokens 125 with 48, 130 with 96).
+constexpr int LN_CHUNKS_MAX = 96;
+inline int ln_chunks(long long tokens) { return tokens <= 4096 ? LN_CHUNKS_MAX / 2 : LN_CHUNKS_MAX; }
+static_assert(TYPE_CHUNKS % 4 == 0 && LN_CHUNKS_MAX % 8 == 0, "see sum_chunks4");
 constexpr int TAB_COLS = 512;                                 // columns a word-table block works on
 constexpr int WARP_MAX = 16;                                  // tokens of one id that a single warp adds up
 struct EmbedTables {
@@ -265,7 +268,7 @@ struct EmbedTables {
   const OptimScalars* sc;                                     // null: gradients only
   AdamEntry pos, type, ln_g, ln_b;
   bool vec;                                                   // these tensors start on 16-byte boundaries
-  int sum_blocks;                                             // blocks of the sums; those beyond take idle rows
+  int ln_chunks, sum_blocks;                                  // blocks of the sums; those beyond take idle rows
   IdleRows idle;
 };
 
@@ -452,9 +455,9 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
     return;
   }
   blk -= n_sum;
-  if (blk < LN_CHUNKS) {
+  if (blk < p.ln_chunks) {
     // gradients of the LayerNorm's gain and bias: sums over the tokens of d * (y - mean) * rstd and of d
-    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7, per = (p.M + LN_CHUNKS - 1) / LN_CHUNKS, t0 = blk * per, t1 = min(p.M, t0 + per);
+    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7, per = (p.M + p.ln_chunks - 1) / p.ln_chunks, t0 = blk * per, t1 = min(p.M, t0 + per);
     for (int c0 = 0; c0 < H; c0 += 128 * V) {
       const int c = c0 + tx * V;
       float ab[V], ag[V];
@@ -489,12 +492,12 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + p.n_types, 1u) + 2u == (unsigned)LN_CHUNKS;
+    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + p.n_types, 1u) + 2u == (unsigned)p.ln_chunks;
     __syncthreads();
     if (!flag) return;
     __threadfence();
     for (int c = 4 * threadIdx.x; c < 2 * H; c += 1024) {      // (H is a multiple of 16: no group of four crosses the two)
-      const float4 acc = sum_chunks4(p.ln_partial, LN_CHUNKS, 2ll * H, c);
+      const float4 acc = sum_chunks4(p.ln_partial, p.ln_chunks, 2ll * H, c);
       const AdamEntry& e = c < H ? p.ln_b : p.ln_g;
       const int i = c < H ? c : c - H;
       store4(e.g + i, acc, p.vec);
@@ -502,7 +505,7 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
     }
     return;
   }
-  blk -= LN_CHUNKS;
+  blk -= p.ln_chunks;
   const int nb = (p.M + 7) / 8, c0 = (blk / nb) * TAB_COLS;
   blk = blk % nb;
   const int tok = wid * nb + blk;
@@ -572,7 +575,7 @@ EmbedScratch carve(const mrem_embed_desc& d, long long max_tokens, void* base) {
   s.rowsum = (int32_t*)A.take(sizeof(int32_t) * d.vocab);
   s.scale = (float*)A.take(sizeof(float) * d.vocab);
   s.optim_sc = (OptimScalars*)A.take(sizeof(OptimScalars));
-  s.ln_partial = (float*)A.take(sizeof(float) * 2 * LN_CHUNKS * d.hidden);
+  s.ln_partial = (float*)A.take(sizeof(float) * 2 * LN_CHUNKS_MAX * d.hidden);
   s.loss_partial = (float*)A.take(sizeof(float) * RED_BLOCKS);
   s.mark_bytes = sizeof(unsigned) * (3 * (size_t)d.vocab + 2 + d.n_types);
   s.marks = (unsigned*)A.take(s.mark_bytes);
@@ -700,7 +703,7 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   // word, position and token-type tables: sums of the token gradients.  Rows of the word table that no token gathered are
   // cleared by the update (row_first says which they are), without one here.
   if (!o && cudaMemsetAsync(x->g_word, 0, sizeof(float) * (size_t)V * H, st) != cudaSuccess) return MREM_ERR_CUDA;
-  const int n_sum = (int)(d->max_pos + (long long)TYPE_CHUNKS * d->n_types + LN_CHUNKS + ((M + 7) / 8) * ((H + TAB_COLS - 1) / TAB_COLS));
+  const int n_sum = (int)(d->max_pos + (long long)TYPE_CHUNKS * d->n_types + ln_chunks(M) + ((M + 7) / 8) * ((H + TAB_COLS - 1) / TAB_COLS));
   bool vec = true;
   const float* const small[] = {x->pos, x->type, x->ln_g, x->ln_b, x->g_pos, x->g_type, x->g_ln_g, x->g_ln_b};
   for (const float* q : small) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
@@ -712,7 +715,7 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
                        (int)d->max_pos, (int)M, s.mean, s.rstd, x->g_word, x->g_pos, x->g_type, s.type_partial, s.ln_partial, o ? s.optim_sc : nullptr,
                        {x->pos, x->g_pos, x->m_pos, x->v_pos, 0, 1.f, -INFINITY}, {x->type, x->g_type, x->m_type, x->v_type, 0, 1.f, -INFINITY},
                        {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, 0, 0.f, -INFINITY}, {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, 0, 0.f, -INFINITY},
-                       vec, n_sum, take_idle(M / 3 + 3400000 / H)};
+                       vec, ln_chunks(M), n_sum, take_idle(M / 3 + 3400000 / H)};
   const unsigned tgrid = (unsigned)(n_sum + (tb.idle.end - tb.idle.first + 7) / 8);
   {
     Scope sc("embed_tables", (double)M * H * 5.0 * (dt == 1 ? 2.0 : 4.0) + 29.0 * H * (tb.idle.end - tb.idle.first), 0, st);

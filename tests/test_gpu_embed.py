@@ -32,8 +32,8 @@ def _problem(act_dtype, e_bits, V=500, H=128, P=48, batch=5, seq=40, seed=3):
     return e, desc, teacher, student, step, ids.astype(np.int32), tt
 
 
-# a few rows a chunk, chunks without rows; many rows a chunk
-@pytest.mark.parametrize("H,batch,seq", [(128, 7, 33), (528, 1, 20), (256, 32, 128)])
+# a few rows a chunk, chunks without rows; many rows a chunk, the most with 48 chunks and the fewest with 96
+@pytest.mark.parametrize("H,batch,seq", [(128, 7, 33), (528, 1, 20), (256, 32, 128), (128, 41, 100)])
 def test_layernorm_sums_of_the_embedding_are_close_to_those_of_64_bits(H, batch, seq):
     """The bias gradient is the sum over the tokens of 2 c (student - teacher).  A rounding of the result is 0.4 2^-24 of it in the
     2-norm, each level of 32-bit additions adds as much in quadrature: about six (chains of few rows, of twelve chunks, and
