@@ -517,21 +517,25 @@ def main():
             B.mrem_set_two_streams(m.ctx, 1)
             B.mrem_graph_capture_step(m.ctx, xbuf, xbuf, 0.0, lenbuf, wl.batch, wl.seq, m.t_out, m.s_out, m.loss, opt)
 
-        # ---- per-kernel timing (CUDA events around every launch of a few eager steps).  The step as a whole: its separate calls,
-        #      which nothing runs beside, choose other tile widths
-        n_trace = 3
-        hb = [calib[idx[t].long()].cpu().pin_memory() for t in range(min(4, total))]
-        hl = [lens_steps[t].cpu().pin_memory() for t in range(min(4, total))]
-        m.quantize_weights()
+        # ---- per-kernel timing (CUDA events around every launch of a few eager steps)
         B.mrem_trace_enable(m.ctx, 1)
+        n_trace = 3
         for t in range(n_trace):
-            B.mrem_recon_step_host(m.ctx, hb[t % len(hb)], hb[t % len(hb)], hl[t % len(hl)], wl.batch, wl.seq, 0.0, opt)
+            stage(t)
+            m.quantize_weights()
+            m.forward_teacher(xbuf, lenbuf, wl.batch, wl.seq)
+            m.forward_student(xbuf, lenbuf, wl.batch, wl.seq)
+            m.recon_loss()
+            m.backward()
+            m.step(opt)
         trace = B.mrem_trace_read(m.ctx, 128)
         B.mrem_trace_enable(m.ctx, 0)
 
         # ---- end to end: host buffers in, loss out, every step
         e2e = None
         if not args.no_e2e:
+            hb = [calib[idx[t].long()].cpu().pin_memory() for t in range(min(4, total))]
+            hl = [lens_steps[t].cpu().pin_memory() for t in range(min(4, total))]
             ke = max(3, min(K, 50))
             for t in range(2):
                 B.mrem_recon_step_host(m.ctx, hb[t % len(hb)], hb[t % len(hb)], hl[t % len(hl)], wl.batch, wl.seq, 0.0, opt)
