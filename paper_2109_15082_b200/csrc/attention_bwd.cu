@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(ATB_THREADS, 2) attention_bwd_kernel(const __g
       for (int i = p.B * p.h + (int)threadIdx.x - 32; i < p.red_slots; i += 256) {
         p.part_p[i] = 0.f; p.part_q[i] = 0.f; p.part_k[i] = 0.f; p.part_v[i] = 0.f; p.part_c[i] = 0.f;
       }
-    if (threadIdx.x == 32) tma_store_wait_all();
+    if (threadIdx.x == 32) tma_store_wait_read<0>();
   }
   __syncthreads();
   if (warp == 0) {

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
           tc_mma<0>(tmem + TMEM_DQ, smem_desc(sX + (ks >> 2) * 16384 + (ks & 3) * 32, 16u, 1024u), smem_desc(sK + ks * 2048, 8192u, 1024u),
                     f32 | (1u << 16) | ((uint32_t)(HD >> 3) << 17), (uint32_t)(ks != 0));
       tc_commit(bar(B_O));
-      tma_store_wait_all();
+      tma_store_wait_read<0>();
     }
   } else {
     const int quad = warp & 3, part = (warp - 1) >> 2;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) attention_bwd_q_kernel(const __g
 #pragma unroll
       for (int k = 0; k < 16; ++k) share += red_part[k][lane];
     }
-    if (threadIdx.x == 32) tma_store_wait_all();
+    if (threadIdx.x == 32) tma_store_wait_read<0>();
   }
   __syncthreads();
   cluster_wait();
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
 #pragma unroll
       for (int k = 0; k < 8; ++k) share += red_part[k][lane];
     }
-    if (threadIdx.x == 32) tma_store_wait_all();
+    if (threadIdx.x == 32) tma_store_wait_read<0>();
   }
   __syncthreads();
   cluster_wait();

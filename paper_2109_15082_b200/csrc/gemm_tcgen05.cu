@@ -242,7 +242,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
-    if (boxed && lane == 0) tma_store_wait_all();          // the boxes are read and written out before the CTA ends
+    if (boxed && lane == 0) tma_store_wait_read<0>();      // the boxes are read before the CTA ends
   }
 
   tc_fence_before();

@@ -218,7 +218,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
       }
       finish_chunk<KIND, OUT, OUT == OUT_I32 ? 0 : MODE>(e, acc, res, alpha, rb, cv + 32 * c, row_off + col_begin + 32 * c, row_ok, sx, col_begin + 32 * c);
     }
-    if (p.c_tma && lane == 0) tma_store_wait_all();
+    if (p.c_tma && lane == 0) tma_store_wait_read<0>();
     __syncwarp();
   }
   tc_fence_before();
