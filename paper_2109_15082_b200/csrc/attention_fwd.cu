@@ -6,74 +6,45 @@
 // codes is exact in fp32), fetched by TMA with 128-byte swizzle.  Outputs: the probabilities
 // (and their codes) for the backward pass, the context rows, and for the student the codes of
 // the context (int8 for the next int8 product, bf16 for the backward).
-// Head size 64, sequence length up to 384.  All waits are time-bounded.
+// Head size 64, up to 128 tokens here (above: attention_fwd_long.cu).  All waits are time-bounded.
 //
 // What bounds it: one CTA is a serial chain (tiles by TMA, product, softmax, product, rows out) and the softmax arithmetic
-// fills the issue slots only when several CTAs, or several threads per row, share an SM.  So P takes the place of Q and K
-// in shared memory and the context that of the scores in TMEM, and the rest is a matter of TPR, the threads per query row:
-//   S <= 128:  TPR 1, 48 KB and 128 TMEM columns: four CTAs per SM, no barrier inside the softmax (was two CTAs of two
-//              threads per row: 512 CTAs were two rounds on 148 SMs and are one now);
-//   S <= 256:  TPR 2, two CTAs per SM;   S <= 384:  TPR 4, one CTA per SM (384 score columns), 16 warps instead of 8.
+// fills the issue slots only when several CTAs share an SM.  So P takes the place of Q and K in shared memory and the context that of
+// the scores in TMEM, and with a thread per row, 48 KB and 128 TMEM columns four CTAs fit (two CTAs of two threads per row: 512
+// CTAs were two rounds on 148 SMs and are one now).
 // Keys beyond the valid length cost nothing: their chunks are neither multiplied nor exponentiated.  Instruction fetch counts too: everything runs
-// once or a few times per CTA, so the loops over chunks stay rolled (67 KB of code became 35).
-// 32 x 16 heads x 128 x 128: 20.6 -> 15 us (mean of teacher and student pass); 16 x 16 x 384 x 384: 98 -> 55 us.
-#include "gemm.h"
-#include "kernels.h"
-#include "tc_ptx.cuh"
+// once or a few times per CTA, so the loops over chunks stay rolled.
+// 32 x 16 heads x 128 x 128: 20.6 -> 15 us (mean of teacher and student pass).  Since then maximum and sum in one pass over the scores and the
+// context out by tiled stores instead of a row per lane: 32 x 12 heads 20.8 -> 15.1 us (student), 16.0 -> 14.1 (teacher); scalars of the context
+// fetched behind the last product cost a step of 4 x 32 tokens 2 us.
+#include "attention_fwd.cuh"
 
 namespace mrem {
 
+using namespace attf;
+
 namespace {
 
-constexpr int HD = 64;
-
-struct AttnParams {
-  int S, h, B, H;
-  int tmem_cols;             // allocation (power of two >= S, at least 64)
-  float alpha_const;         // score scale = alpha_const * (*a_p0) * (*a_p1)
-  const float *a_p0, *a_p1;
-  const float *c_p0, *c_p1;  // context scale = (*c_p0) * (*c_p1); null = 1
-  const int* valid_len;
-  const float* p_step;       // quantizer of the probabilities (student), null = none
-  float p_lo, p_hi;
-  const float* c_step;       // symmetric quantizer of the context (student), null = none
-  float c_qmax;
-  bf16 *P, *P_qt;            // [B, h, S, S]
-  bf16* ctx;                 // [B*S, H]
-  int8_t* ctx_q8;            // [B*S, H]
-  bf16* ctx_qt;              // [B*S, H]
-  AttentionStats stats;      // for the backward pass (null members: none)
-  int* status;
-  unsigned long long wait_ns;  // limit of each wait on an mbarrier
-};
-
-__device__ __forceinline__ void store16(void* p, const uint32_t* w) {
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// TPR threads per query row; QUANT: the student pass (quantizers of the probabilities and of the context).
-// Warp 0: TMA and MMA issue; warps 1 .. 4 TPR: softmax and epilogue, TPR warps per TMEM lane quadrant.
-template <int TPR, bool QUANT>
-__global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(const __grid_constant__ CUtensorMap map_qkv,
-                                                                                const __grid_constant__ AttnParams p) {
+// QUANT: the student pass (quantizers of the probabilities and of the context).
+// Warp 0: TMA and MMA issue; warps 1 .. 4: softmax and epilogue, a thread per query row.
+template <bool QUANT>
+__global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_constant__ CtxMaps out,
+                                                               const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_qk, bar_v, bar_s, bar_p, bar_o;
   __shared__ uint32_t tmem_slot;
-  __shared__ float red[2][TPR][128];                         // [max | sum][part][row]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qb = blockIdx.x, head = blockIdx.y, b = blockIdx.z;
-  const int q0 = qb * 128;
+  const int head = blockIdx.y, b = blockIdx.z;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int n_box = (p.S + 127) / 128;                       // 128-row TMA boxes of keys / values
   // P takes the place of Q and K once the scores are in TMEM
-  const uint32_t sV = base, sP = sV + n_box * 16384, sQ = sP, sK = sQ + 16384;
+  const uint32_t sV = base, sP = sV + 16384, sQ = sP, sK = sQ + 16384;
   uint8_t* gP = smem_raw + (sP - smem_u32(smem_raw));        // generic pointer to the P operand tile
 
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar_qk), 1);
     mbar_init(smem_u32(&bar_v), 1);
     mbar_init(smem_u32(&bar_s), 1);
-    mbar_init(smem_u32(&bar_p), 128 * TPR);
+    mbar_init(smem_u32(&bar_p), 128);
     mbar_init(smem_u32(&bar_o), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -96,27 +67,21 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
   if (warp == 0) {
     if (lane == 0) {
       // ---- loads: Q block, the valid keys, the valid values (slots of the qkv tensor: head, h + head, 2h + head)
-      const int boxes = (len + 127) / 128, n16 = (len + 15) & ~15;
-      mbar_expect_tx(smem_u32(&bar_qk), 16384u * (uint32_t)(1 + boxes));
-      tma_load_4d(sQ, &map_qkv, smem_u32(&bar_qk), 0, q0, head, b);
-#pragma unroll 1
-      for (int i = 0; i < boxes; ++i) tma_load_4d(sK + i * 16384, &map_qkv, smem_u32(&bar_qk), 0, i * 128, p.h + head, b);
-      mbar_expect_tx(smem_u32(&bar_v), 16384u * (uint32_t)boxes);
-#pragma unroll 1
-      for (int i = 0; i < boxes; ++i) tma_load_4d(sV + i * 16384, &map_qkv, smem_u32(&bar_v), 0, i * 128, 2 * p.h + head, b);
+      mbar_expect_tx(smem_u32(&bar_qk), 2u * 16384u);
+      tma_load_4d(sQ, &map_qkv, smem_u32(&bar_qk), 0, 0, head, b);
+      tma_load_4d(sK, &map_qkv, smem_u32(&bar_qk), 0, 0, p.h + head, b);
+      mbar_expect_tx(smem_u32(&bar_v), 16384u);
+      tma_load_4d(sV, &map_qkv, smem_u32(&bar_v), 0, 0, 2 * p.h + head, b);
+      const int n16 = (len + 15) & ~15;
       bool ok = mbar_wait(smem_u32(&bar_qk), 0, p.wait_ns);
       if (!ok) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_TMA);
       tc_fence_after();
-      // ---- scores: [128 x n16] = Q [128 x 64] * K^T, in pieces of at most 256 keys
+      // ---- scores: [128 x n16] = Q [128 x 64] * K^T
       if (ok) {
-        for (int n0 = 0; n0 < n16; n0 += 256) {
-          const int n = min(256, n16 - n0);
-          const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (8u << 24);
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n16 >> 3) << 17) | (8u << 24);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            tc_mma<0>(tmem + (uint32_t)n0, smem_desc(sQ + k * 32, 16u, 1024u), smem_desc(sK + n0 * 128 + k * 32, 16u, 1024u),
-                      idesc, (uint32_t)(k != 0));
-        }
+        for (int k = 0; k < 4; ++k)
+          tc_mma<0>(tmem, smem_desc(sQ + k * 32, 16u, 1024u), smem_desc(sK + k * 32, 16u, 1024u), idesc, (uint32_t)(k != 0));
       }
       tc_commit(smem_u32(&bar_s));
       // ---- context: [128 x 64] = P [128 x keys] * V [keys x 64]  (V is the MN-major operand), over the scores
@@ -134,106 +99,49 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
       tc_commit(smem_u32(&bar_o));
     }
   } else {
-    const int quad = warp & 3, part = (warp - 1) >> 2;
+    const int quad = warp & 3;
     const int r = quad * 32 + lane;                      // row inside the block
-    const int q = q0 + r;
-    const bool row_ok = q < p.S;
+    const bool row_ok = r < p.S;
     float alpha = p.alpha_const;
     if (p.a_p0) alpha *= *p.a_p0;
     if (p.a_p1) alpha *= *p.a_p1;
     const float ps = QUANT ? *p.p_step : 1.f, r_ps = __frcp_rn(ps);
+    // (every scalar here: a load behind the last product would be waited for)
+    float calpha = 1.f;
+    if (p.c_p0) calpha *= *p.c_p0;
+    if (p.c_p1) calpha *= *p.c_p1;
+    const float cs = QUANT ? *p.c_step : 1.f;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
     const int n_valid = (len + 31) / 32;                 // 32-key chunks that hold a valid key: the others are zeros
     const bool got = mbar_wait(smem_u32(&bar_s), 0, p.wait_ns);
     if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
     tc_fence_after();
-    // scores in units of log2(e): exp(alpha * a - max) = 2^(alpha2 * a - max2); alpha > 0, so the maximum
-    // can be taken over the raw accumulators
     const float alpha2 = alpha * 1.4426950408889634f;
     float mx = -INFINITY;
-#pragma unroll 1
-    for (int c = part; c < n_valid; c += TPR) {
-      uint32_t a[32];
-      tmem_ld32(trow + (uint32_t)(c * 32), a);
-      if (c * 32 + 32 <= len) {                          // all 32 keys valid (warp-uniform)
-        float m4[4] = {mx, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-        for (int j = 0; j < 32; ++j) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(a[j]));
-        mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c * 32 + j < len) mx = fmaxf(mx, __uint_as_float(a[j]));
-      }
-    }
-    if constexpr (TPR > 1) {
-      red[0][part][r] = mx;
-      asm volatile("bar.sync 1, %0;" ::"n"(128 * TPR) : "memory");
-#pragma unroll
-      for (int k = 0; k < TPR; ++k) mx = fmaxf(mx, red[0][k][r]);
-    }
-    const float mx2 = alpha2 * mx;
-    const float2 alpha22 = make_float2(alpha2, alpha2), nmx2 = make_float2(-mx2, -mx2);
     float2 sums[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
-    for (int c = part; c < n_valid; c += TPR) {
+    for (int c = 0; c < n_valid; ++c) {
       uint32_t a[32];
       tmem_ld32(trow + (uint32_t)(c * 32), a);
-      const int ncol = len - c * 32;                     // (>= 32: all keys valid)
-#pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        const float2 t = fma2(make_float2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])), alpha22, nmx2);
-        float2 e = make_float2(exp2_approx(t.x), exp2_approx(t.y));
-        if (ncol < 32) { e.x = j < ncol ? e.x : 0.f; e.y = j + 1 < ncol ? e.y : 0.f; }
-        sums[(j >> 1) & 1] = add2(sums[(j >> 1) & 1], e);
-      }
+      join_chunk(a, len - c * 32, alpha2, mx, sums);
     }
-    float sum = (sums[0].x + sums[0].y) + (sums[1].x + sums[1].y);
-    if constexpr (TPR > 1) {
-      red[1][part][r] = sum;
-      asm volatile("bar.sync 1, %0;" ::"n"(128 * TPR) : "memory");
-      sum = red[1][0][r];
-#pragma unroll
-      for (int k = 1; k < TPR; ++k) sum += red[1][k][r];
-    }
+    const float mx2 = __fmul_rn(alpha2, mx);
+    const float sum = (sums[0].x + sums[0].y) + (sums[1].x + sums[1].y);
     const float inv_sum = __frcp_rn(sum);
-    if (p.stats.row && part == 0) {
-      if (row_ok) p.stats.row[((long long)b * p.h + head) * p.S + q] = make_float2(mx2, inv_sum);
-      if (r == 0 && qb == 0 && head == 0) { p.stats.len[b] = len; if (b == 0) *p.stats.alpha = alpha; }
+    if (p.stats.row) {
+      if (row_ok) p.stats.row[((long long)b * p.h + head) * p.S + r] = make_float2(mx2, inv_sum);
+      if (r == 0 && head == 0) { p.stats.len[b] = len; if (b == 0) *p.stats.alpha = alpha; }
     }
-    const float2 inv2 = make_float2(inv_sum, inv_sum), r2 = make_float2(r_ps, r_ps), ns2 = make_float2(-ps, -ps);
-    const float2 magic2 = make_float2(ROUND_MAGIC, ROUND_MAGIC), nmagic2 = make_float2(-ROUND_MAGIC, -ROUND_MAGIC);
-    const long long prow = (((long long)b * p.h + head) * p.S + q) * p.S;
+    const RowScale k{splat(alpha2), splat(-mx2), make_float2(inv_sum, inv_sum), splat(r_ps), splat(-ps), p.p_hi};
+    const long long prow = (((long long)b * p.h + head) * p.S + r) * p.S;
     const int n_store = p.P ? (p.S + 31) / 32 : n_valid;
 #pragma unroll 1
-    for (int c = part; c < n_store; c += TPR) {
+    for (int c = 0; c < n_store; ++c) {
       uint32_t pw[16], cw[16];                            // 32 probabilities / codes packed as bf16 pairs
       if (c < n_valid) {
         uint32_t a[32];
         tmem_ld32(trow + (uint32_t)(c * 32), a);
-        const int ncol = len - c * 32;
-#pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          // (the exponentials are formed a second time: cheaper than keeping them in TMEM)
-          const float2 t = fma2(make_float2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])), alpha22, nmx2);
-          float2 v = mul2(make_float2(exp2_approx(t.x), exp2_approx(t.y)), inv2);
-          if (ncol < 32) { v.x = j < ncol ? v.x : 0.f; v.y = j + 1 < ncol ? v.y : 0.f; }
-          const __nv_bfloat162 pb = __floats2bfloat162_rn(v.x, v.y);
-          pw[j >> 1] = *reinterpret_cast<const uint32_t*>(&pb);
-          if constexpr (QUANT) {
-            // the quotient of a bf16 value is the IEEE division of Eq. 1 (see quotient()); probabilities are not negative,
-            // so only the upper bound of the code range can clip
-            const float2 f = make_float2(__uint_as_float(pw[j >> 1] << 16), __uint_as_float(pw[j >> 1] & 0xffff0000u));
-            const float2 z0 = mul2(f, r2);
-            float2 z = fma2(fma2(z0, ns2, f), r2, z0);
-            z = make_float2(fminf(z.x, p.p_hi), fminf(z.y, p.p_hi));
-            const float2 k = add2(add2(z, magic2), nmagic2);
-            const __nv_bfloat162 cb = __floats2bfloat162_rn(k.x, k.y);
-            cw[j >> 1] = *reinterpret_cast<const uint32_t*>(&cb);
-          } else {
-            cw[j >> 1] = pw[j >> 1];
-          }
-        }
+        probabilities32<QUANT>(a, len - c * 32, k, pw, cw);
         // operand tile: block of 64 keys, row r, 16-byte chunk index XOR (r & 7)  (128-byte swizzle)
         uint8_t* rowp = gP + (c >> 1) * 16384 + r * 128;
 #pragma unroll
@@ -259,40 +167,18 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
     const bool got2 = mbar_wait(smem_u32(&bar_o), 0, p.wait_ns);
     if (!__all_sync(0xffffffffu, got2) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
     tc_fence_after();
-    float calpha = 1.f;
-    if (p.c_p0) calpha *= *p.c_p0;
-    if (p.c_p1) calpha *= *p.c_p1;
-    const float cs = QUANT ? *p.c_step : 1.f, r_cs = __frcp_rn(cs);
-    const long long crow = ((long long)b * p.S + q) * p.H + head * HD;
+    if (p.ctx) {                                         // (all products have run: the tiles of P and V are free)
 #pragma unroll 1
-    for (int hh = part; hh < 2; hh += TPR) {
-      uint32_t a[32];
-      tmem_ld32(trow + (uint32_t)(hh * 32), a);
-      uint32_t w[16], cq[16], c8[8];
-#pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        const __nv_bfloat162 vb = __floats2bfloat162_rn(calpha * __uint_as_float(a[j]), calpha * __uint_as_float(a[j + 1]));
-        w[j >> 1] = *reinterpret_cast<const uint32_t*>(&vb);
-        if constexpr (QUANT) {
-          const float2 f = __bfloat1622float2(vb);
-          uint32_t b0, b1;                                 // rounding words: low byte = the 8-bit code
-          const float i0 = rne_magic(fminf(fmaxf(quotient(f.x, cs, r_cs), -p.c_qmax), p.c_qmax), b0);
-          const float i1 = rne_magic(fminf(fmaxf(quotient(f.y, cs, r_cs), -p.c_qmax), p.c_qmax), b1);
-          const __nv_bfloat162 cb = __floats2bfloat162_rn(i0, i1);
-          cq[j >> 1] = *reinterpret_cast<const uint32_t*>(&cb);
-          const uint32_t two = __byte_perm(b0, b1, 0x0040) & 0xffffu;
-          if ((j & 2) == 0) c8[j >> 2] = two; else c8[j >> 2] |= two << 16;
-        }
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t a[32];
+        tmem_ld32(trow + (uint32_t)(hh * 32), a);
+        context32<QUANT>(p, a, calpha, cs, r, hh, gP, gP + 16384, gP - 16384);
       }
-      if (row_ok && p.ctx) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) store16(p.ctx + crow + hh * 32 + t * 8, w + 4 * t);
-        if constexpr (QUANT) {
-#pragma unroll
-          for (int t = 0; t < 4; ++t) store16(p.ctx_qt + crow + hh * 32 + t * 8, cq + 4 * t);
-          store16(p.ctx_q8 + crow + hh * 32, c8);
-          store16(p.ctx_q8 + crow + hh * 32 + 16, c8 + 4);
-        }
+      fence_async_shared();
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (threadIdx.x == 32) {
+        store_context<QUANT>(out, sP, sP + 16384, sV, 0, head, b);
+        tma_store_wait_read<0>();
       }
     }
     tc_fence_before();
@@ -304,19 +190,15 @@ __global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(
   }
 }
 
-template <int TPR, bool QUANT>
-int launch_tpr(const CUtensorMap& map, const AttnParams& p, cudaStream_t st) {
-  const int n_box = (p.S + 127) / 128, n_kb = (p.S + 63) / 64;
-  const int smem = 1024 + 16384 * (n_box + (n_kb > 1 + n_box ? n_kb : 1 + n_box));
-  // the limit for the longest sequence of this variant, whatever this one needs: threads that get here together set the same one
-  constexpr int MAX_BOX = TPR == 4 ? 3 : TPR;
+template <bool QUANT>
+int launch_short(const CUtensorMap& map, const CtxMaps& out, const AttnParams& p, cudaStream_t st) {
+  constexpr int smem = 1024 + 16384 * 3;
   static bool attr_set = false;
   if (!attr_set) {
-    if (cudaFuncSetAttribute(attention_fwd_kernel<TPR, QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + 16384 * 3 * MAX_BOX) != cudaSuccess)
-      return GEMM_ERR_CUDA;
+    if (cudaFuncSetAttribute(attention_fwd_kernel<QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GEMM_ERR_CUDA;
     attr_set = true;
   }
-  if (launch_k(attention_fwd_kernel<TPR, QUANT>, dim3((p.S + 127) / 128, p.h, p.B), 32 + 128 * TPR, smem, st, map, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  if (launch_k(attention_fwd_kernel<QUANT>, dim3(1, p.h, p.B), 160, smem, st, map, out, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }
 
@@ -336,20 +218,23 @@ int launch_attention_fwd(const void* qkv, int B, int S, int h, int H, const int*
   p.tmem_cols = cols;
   p.alpha_const = alpha_const; p.a_p0 = a_p0; p.a_p1 = a_p1; p.c_p0 = c_p0; p.c_p1 = c_p1;
   p.valid_len = valid_len;
+  p.order = 0;
   p.p_step = p_step; p.p_lo = (float)p_lo; p.p_hi = (float)p_hi;
   p.c_step = c_step; p.c_qmax = (float)c_qmax;
   p.P = (bf16*)P; p.P_qt = (bf16*)P_qt; p.ctx = (bf16*)ctx; p.ctx_q8 = ctx_q8; p.ctx_qt = (bf16*)ctx_qt;
   p.stats = stats ? *stats : AttentionStats{nullptr, nullptr, nullptr};
   p.status = status;
   p.wait_ns = g_wait_limit_ns;
+  Scope sc("attention_fwd_tcgen05", 4.0 * B * h * (double)S * S * HD, 1, st);
+  if (S > 128) return launch_attention_fwd_long(p, qkv, st);
   // one map over the [tokens, 3H] tensor: (64 of a head, S rows, 3h head slots, B)
   OperandDesc op{qkv, 3LL * H, HD, (long long)S * 3 * H, 0};
   CUtensorMap map;
-  const int rc = make_operand_map(&map, op, 2, S, HD, 3 * h, B, 128, HD);
+  int rc = make_operand_map(&map, op, 2, S, HD, 3 * h, B, 128, HD);
+  CtxMaps out;
+  if (rc == GEMM_OK) rc = make_ctx_maps(&out, p, map);
   if (rc != GEMM_OK) return rc;
-  Scope sc("attention_fwd_tcgen05", 4.0 * B * h * (double)S * S * HD, 1, st);
-  if (p_step) return S <= 128 ? launch_tpr<1, true>(map, p, st) : (S <= 256 ? launch_tpr<2, true>(map, p, st) : launch_tpr<4, true>(map, p, st));
-  return S <= 128 ? launch_tpr<1, false>(map, p, st) : (S <= 256 ? launch_tpr<2, false>(map, p, st) : launch_tpr<4, false>(map, p, st));
+  return p_step ? launch_short<true>(map, out, p, st) : launch_short<false>(map, out, p, st);
 }
 
 }  // namespace mrem

@@ -298,7 +298,7 @@ CUresult encode_tiled(Args... args) {
 
 }  // namespace
 
-// Tensor map of one operand: 4-D (contiguous index, strided index, batch0, batch1).
+// Tensor map of one operand: 4-D (contiguous index, strided index, batch0, batch1).  128-byte swizzle; rows of 64 bytes have a 64-byte one.
 int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, int mn_extent, int K, int nb0, int nb1,
              int tile_mn, int block_k, int* chunked) {
   if (chunked) *chunked = 0;
@@ -341,7 +341,7 @@ int make_operand_map(CUtensorMap* map, const OperandDesc& op, int elem_bytes, in
   cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUtensorMapDataType dt = elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8;
   CUresult r = encode_tiled(map, dt, 4, const_cast<void*>(op.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  box[0] * elem_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? GEMM_OK : GEMM_ERR_CUDA;
 }
 

@@ -74,6 +74,26 @@ def test_reading_the_probabilities_leaves_the_backward_pass_alone(seq):
         p.close()
 
 
+# more blocks than run at once: they take the sequences longest first (equal lengths, one key, whole chunks and one more among them)
+@pytest.mark.parametrize("seq,batch", [(136, 12), (320, 8), (136, 32)])
+def test_sequences_of_a_large_batch_are_those_of_a_small_one(seq, batch):
+    """The quantized pass treats sequences independently (whole numbers, and row sums in the same order): bit for bit the outputs
+    of the same sequences two at a time, which are too few blocks to be ordered."""
+    wl = synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, seq=seq, batch=batch, len_lo=1, len_hi=seq)
+    p = Problem(wl, step_shrink=0.8, student_noise=0.002)
+    try:
+        m = p.m
+        lens = np.array(([seq, 1, 64, 65, seq, 128, 129, seq - 1, 64, 33, 32, 97] * 3)[:batch], np.int32)
+        vld = torch.from_numpy(lens).to(m.device)
+        m.quantize_weights()
+        many = m.forward_student(p.xd, vld, batch, seq).clone()
+        for i in range(0, batch, 6):
+            two = m.forward_student(p.xd[i:i + 2].contiguous(), vld[i:i + 2].clone(), 2, seq)
+            assert torch.equal(two, many[:, i:i + 2]), i
+    finally:
+        p.close()
+
+
 def _rounded_up_case(a_bits, lo_len, hi_len):
     """A step s, codes cq and ck, a number of keys n and a step s_p such that n equal scores alpha 64 cq ck have probabilities
     1 / n that are stored one bf16 spacing ABOVE the stored 1 / sum, with the upper end of P's range between the two: the
