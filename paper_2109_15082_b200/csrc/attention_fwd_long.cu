@@ -56,8 +56,9 @@ __global__ void __launch_bounds__(LONG_THREADS, 2) attention_fwd_long_kernel(con
   pdl_wait();
   pdl_trigger();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
-  const int b = p.order ? longest_first(p.valid_len, p.B, (int)blockIdx.z) : (int)blockIdx.z;
-  int len = p.valid_len ? p.valid_len[b] : p.S;
+  const Sequence sq = p.order ? longest_first(p.valid_len, p.B, (int)blockIdx.z) : Sequence{(int)blockIdx.z, p.valid_len ? p.valid_len[blockIdx.z] : p.S};
+  const int b = sq.b;
+  int len = sq.len;
   len = len < 1 ? 1 : (len > p.S ? p.S : len);
   const int n = (len + 63) / 64;                             // chunks with a valid key
 

@@ -203,16 +203,18 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// The sequence of rank z when the n <= 32 sequences of a batch are ordered by length, longest first (whole warps; `len` as the
-// caller gave it).  Blocks of long sequences that start last would run alone at the end of a launch.
-__device__ __forceinline__ int longest_first(const int* len, int n, int z) {
-  const int lane = (int)(threadIdx.x & 31), mine = lane < n ? len[lane] : (int)0x80000000;
+// The sequence of rank z when the n <= 32 sequences of a batch are ordered by length, longest first, and its length (whole warps;
+// `lens` as the caller gave it).  Blocks of long sequences that start last would run alone at the end of a launch.
+struct Sequence { int b, len; };
+__device__ __forceinline__ Sequence longest_first(const int* lens, int n, int z) {
+  const int lane = (int)(threadIdx.x & 31), mine = lane < n ? lens[lane] : (int)0x80000000;
   int rank = 0;
   for (int k = 0; k < n; ++k) {
     const int other = __shfl_sync(0xffffffffu, mine, k);
     rank += other > mine || (other == mine && k < lane);
   }
-  return __ffs(__ballot_sync(0xffffffffu, rank == z)) - 1;      // (lanes beyond n have rank n)
+  const int b = __ffs(__ballot_sync(0xffffffffu, rank == z)) - 1;      // (lanes beyond n have rank n)
+  return Sequence{b, __shfl_sync(0xffffffffu, mine, b)};
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle.  lbo/sbo in bytes.
