@@ -36,6 +36,11 @@ __device__ __forceinline__ float range_limit(float step, float hi) {
   return lim;
 }
 
+// What the straight-through pass of a site needs besides its step.  The two take a dependent chain of some 200 clocks to form, so they are
+// formed while the first tiles are on their way, and wait in shared memory (a copy per warp: no barrier).
+struct SiteTerms { float lim, r; };
+__device__ __forceinline__ SiteTerms site_terms(float step, float hi) { return SiteTerms{range_limit(step, hi), __frcp_rn(step)}; }
+
 // No stored probability of a row is above this (m = RN(alpha log2(e) max), inv = 1 / sum, both as the forward pass left them).
 // The largest one is not 2^0 inv: its exponent fma(max, alpha log2(e), -m) is the rounding error of m, up to 2^-24 |m|, and where
 // that is positive the probability can be stored one bf16 spacing above the stored inv.  The last factor covers the two
@@ -44,20 +49,21 @@ __device__ __forceinline__ float probability_bound(float m, float inv) {
   return __bfloat162float(__float2bfloat16_rn(inv * exp2_approx(fabsf(m) * 5.9604645e-8f) * (1.f + 9.5367432e-7f)));
 }
 
-// Straight-through pass of one symmetric quantizer over 32 values of a row: x (bf16 pairs before quantization, replaced by the
+// Straight-through pass of one symmetric quantizer over 2 NP values of a row: x (bf16 pairs before quantization, replaced by the
 // masked gradient as bf16 pairs), g(j) = the incoming gradient of pair j.  Returns the sum of the step-size terms.  A NaN is
 // outside every range (its code is the lowest): the test for clipped values keeps it (max.NaN).
-template <class G>
-__device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi, float lim) {
-  const float2 r2 = both(__frcp_rn(step)), ns2 = both(-step), magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
+template <int NP, class G>
+__device__ __forceinline__ float ste_pairs(uint32_t* x, G&& g, float step, float hi, SiteTerms site) {
+  const float lim = site.lim;
+  const float2 r2 = both(site.r), ns2 = both(-step), magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
   __nv_bfloat162 mx = __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[0]));
 #pragma unroll
-  for (int j = 1; j < 16; ++j) mx = __hmax2_nan(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[j])));
+  for (int j = 1; j < NP; ++j) mx = __hmax2_nan(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[j])));
   const float2 m = __bfloat1622float2(mx);
   float2 ds = both(0.f);
   if (__all_sync(0xffffffffu, m.x <= lim && m.y <= lim)) {       // nothing clipped in the whole warp
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NP; ++j) {
       const float2 xv = unpack2(x[j]), gv = g(j);
       const float2 z0 = mul2(xv, r2), z = fma2(fma2(z0, ns2, xv), r2, z0);
       const float2 q = add2(add2(z, magic2), nmagic2);
@@ -66,7 +72,7 @@ __device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi,
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NP; ++j) {
       const float2 xv = unpack2(x[j]);
       float2 gv = g(j);
       const float2 z0 = mul2(xv, r2), z = fma2(fma2(z0, ns2, xv), r2, z0);
@@ -80,15 +86,22 @@ __device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi,
   return ds.x + ds.y;
 }
 
-// 32 columns (64 bytes) of a row of a 128-byte-swizzled tile of 128 rows x 128 bytes
-__device__ __forceinline__ void tile_load(const uint8_t* tile, int r, int half, uint32_t* w) {
+template <class G>
+__device__ __forceinline__ float ste32(uint32_t* x, G&& g, float step, float hi, SiteTerms site) { return ste_pairs<16>(x, g, step, hi, site); }
+
+// Piece `part` of a row of a 128-byte-swizzled tile of 128 rows x 128 bytes: 8 NW columns (16 NW bytes)
+template <int NW>
+__device__ __forceinline__ void piece_load(const uint8_t* tile, int r, int part, uint32_t* w) {
 #pragma unroll
-  for (int t = 0; t < 4; ++t) ld16(tile + r * 128 + (((half * 4 + t) ^ (r & 7)) * 16), w + 4 * t);
+  for (int t = 0; t < NW; ++t) ld16(tile + r * 128 + (((part * NW + t) ^ (r & 7)) * 16), w + 4 * t);
 }
-__device__ __forceinline__ void tile_store(uint8_t* tile, int r, int half, const uint32_t* w) {
+template <int NW>
+__device__ __forceinline__ void piece_store(uint8_t* tile, int r, int part, const uint32_t* w) {
 #pragma unroll
-  for (int t = 0; t < 4; ++t) st16(tile + r * 128 + (((half * 4 + t) ^ (r & 7)) * 16), w + 4 * t);
+  for (int t = 0; t < NW; ++t) st16(tile + r * 128 + (((part * NW + t) ^ (r & 7)) * 16), w + 4 * t);
 }
+__device__ __forceinline__ void tile_load(const uint8_t* tile, int r, int half, uint32_t* w) { piece_load<4>(tile, r, half, w); }
+__device__ __forceinline__ void tile_store(uint8_t* tile, int r, int half, const uint32_t* w) { piece_store<4>(tile, r, half, w); }
 
 // Sums over the first `rows` rows of such a tile of bf16 values, for the bias gradient of the product that made Q, K and V: a warp
 // of NW takes 128 / NW rows and a lane two columns (a row per load, all banks), its sums go to red[warp][64].  The tile is read as

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(Q_THREADS, 2) attention_bwd_q_kernel(const __g
   __shared__ uint32_t tmem_slot;
   __shared__ float red_dot[2][128];
   __shared__ float red_part[8][3];
+  __shared__ SiteTerms sites[8][3];                        // per warp: Q, context, P (attention_bwd.cuh)
   __shared__ float cta_part[3][3];                         // [cluster rank][site]
   constexpr int TMEM_S = 0, TMEM_DP = 64, TMEM_DQ = 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -180,20 +181,21 @@ __global__ void __launch_bounds__(Q_THREADS, 2) attention_bwd_q_kernel(const __g
     bool got = true;
     auto wait = [&](int i, int round) { got = got && mbar_wait(bar(i), (uint32_t)(round & 1), p.wait_ns); __syncwarp(); };
     auto signal = [&](int i) { __syncwarp(); if (lane == 0) mbar_arrive(bar(i)); };
+    if (lane < 3) sites[warp - 1][lane] = site_terms(lane == 0 ? s_q : (lane == 1 ? s_c : s_p), lane == 2 ? p.p_hi : p.q_hi);
     wait(B_CTX, 0);
     float ds_c, ds_q;
     {                                                      // STE of the context's quantizer, 32 columns per thread, in place
       uint32_t d[16], x[16];
       tile_load(gD, r, half, d);
       tile_load(gX, r, half, x);
-      ds_c = ste32(x, [&](int j) { return unpack2(d[j]); }, s_c, p.q_hi, range_limit(s_c, p.q_hi));
+      ds_c = ste32(x, [&](int j) { return unpack2(d[j]); }, s_c, p.q_hi, sites[warp - 1][1]);
       tile_store(gD, r, half, x);
     }
     fence_async_shared();
     signal(B_STE);
-    const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p),
+    const float2 alpha22 = both(alpha2), nmx2 = both(-st.x), inv2 = both(st.y), sv2 = both(s_v), r2 = both(sites[warp - 1][2].r), ns2 = both(-s_p),
                  magic2 = both(ROUND_MAGIC), nmagic2 = both(-ROUND_MAGIC), m1 = both(-1.f);
-    const float lim_p = range_limit(s_p, p.p_hi);
+    const float lim_p = sites[warp - 1][2].lim;
     const bool clips = !__all_sync(0xffffffffu, probability_bound(st.x, st.y) <= lim_p);   // (see attention_bwd.cu)
     // this thread's 32 probabilities of step s, as the forward pass formed them, and dP beside them; the accumulators go back
     // as soon as the warp has read them
@@ -278,7 +280,7 @@ __global__ void __launch_bounds__(Q_THREADS, 2) attention_bwd_q_kernel(const __g
       tmem_ld32(trow + TMEM_DQ, a);
       tile_load(gR, r, half, x);
       const float2 sc2 = both(p.inv_sqrt_d * s_k);
-      ds_q = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, s_q, p.q_hi, range_limit(s_q, p.q_hi));
+      ds_q = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, s_q, p.q_hi, sites[warp - 1][0]);
       tile_store(gR, r, half, x);
       if (!row_ok) ds_q = 0.f;
     }
@@ -328,6 +330,7 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
   __shared__ __align__(8) uint64_t bars[N_BARS];
   __shared__ uint32_t tmem_slot;
   __shared__ float red_part[8][2];
+  __shared__ SiteTerms sites[8][2];                        // per warp: V, K (attention_bwd.cuh)
   __shared__ float cta_part[3][2];
   constexpr int TMEM_S = 0, TMEM_DP = 64, TMEM_DV = 128, TMEM_DK = 192;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -447,6 +450,8 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
       const uint32_t keep = key < len ? 0xffffffffu : 0u;
       const float2 alpha22 = both(alpha2), sv2 = both(s_v), r2 = both(__frcp_rn(s_p)), ns2 = both(-s_p), magic2 = both(ROUND_MAGIC),
                    nmagic2 = both(-ROUND_MAGIC);
+      if (lane < 2) sites[warp - 1][lane] = site_terms(lane == 0 ? s_v : s_k, p.q_hi);
+      __syncwarp();
       bool got = true;
 #pragma unroll 1
       for (int c = 0; c < n_q; ++c) {
@@ -502,7 +507,7 @@ __global__ void __launch_bounds__(KV_THREADS, 2) attention_bwd_kv_kernel(const _
         tmem_ld32(trow + (uint32_t)((g == 0 ? TMEM_DV : TMEM_DK) + half * 32), a);
         tile_load(tile, r, half, x);
         const float2 sc2 = both(g == 0 ? s_p : p.inv_sqrt_d * s_q);
-        float ds = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, step, p.q_hi, range_limit(step, p.q_hi));
+        float ds = ste32(x, [&](int j) { return mul2(acc2(a, j), sc2); }, step, p.q_hi, sites[warp - 1][g]);
         tile_store(tile, r, half, x);
         ds = key < p.S ? ds : 0.f;
         if (g == 0) ds_v = ds; else ds_k = ds;

@@ -26,13 +26,16 @@ using namespace attf;
 namespace {
 
 // QUANT: the student pass (quantizers of the probabilities and of the context).
-// Warp 0: TMA and MMA issue; warps 1 .. 4: softmax and epilogue, a thread per query row.
-template <bool QUANT>
-__global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_constant__ CtxMaps out,
+// Warp 0: TMA and MMA issue; warps 1 .. 4 TPR: softmax and epilogue, TPR threads per query row: one, and four CTAs per SM, or four, and one, where
+// every CTA has an SM to itself: each thread then has one chunk of 32 keys and 16 columns of the context
+// (figures: attention_bwd.cu).
+template <int TPR, bool QUANT>
+__global__ void __launch_bounds__(32 + 128 * TPR, 4 / TPR) attention_fwd_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_constant__ CtxMaps out,
                                                                const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_qk, bar_v, bar_s, bar_p, bar_o;
   __shared__ uint32_t tmem_slot;
+  __shared__ float2 red[TPR][128];                           // [part][row]: maximum, sum
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int head = blockIdx.y, b = blockIdx.z;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -44,7 +47,7 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
     mbar_init(smem_u32(&bar_qk), 1);
     mbar_init(smem_u32(&bar_v), 1);
     mbar_init(smem_u32(&bar_s), 1);
-    mbar_init(smem_u32(&bar_p), 128);
+    mbar_init(smem_u32(&bar_p), 128 * TPR);
     mbar_init(smem_u32(&bar_o), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -99,7 +102,7 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
       tc_commit(smem_u32(&bar_o));
     }
   } else {
-    const int quad = warp & 3;
+    const int quad = warp & 3, part = (warp - 1) >> 2;
     const int r = quad * 32 + lane;                      // row inside the block
     const bool row_ok = r < p.S;
     float alpha = p.alpha_const;
@@ -117,18 +120,24 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
     if (!__all_sync(0xffffffffu, got) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
     tc_fence_after();
     const float alpha2 = alpha * 1.4426950408889634f;
-    float mx = -INFINITY;
-    float2 sums[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    RowPart row{-INFINITY, 0.f};
 #pragma unroll 1
-    for (int c = 0; c < n_valid; ++c) {
+    for (int c = part; c < n_valid; c += TPR) {
       uint32_t a[32];
       tmem_ld32(trow + (uint32_t)(c * 32), a);
-      join_chunk(a, len - c * 32, alpha2, mx, sums);
+      join(row, chunk_part(a, len - c * 32, alpha2), alpha2);
     }
-    const float mx2 = __fmul_rn(alpha2, mx);
-    const float sum = (sums[0].x + sums[0].y) + (sums[1].x + sums[1].y);
+    if constexpr (TPR > 1) {                             // (TPR * 32 >= S: a chunk per thread)
+      red[part][r] = make_float2(row.max, row.sum);
+      asm volatile("bar.sync 1, %0;" ::"n"(128 * TPR) : "memory");
+      row = RowPart{-INFINITY, 0.f};
+#pragma unroll
+      for (int k = 0; k < TPR; ++k)
+        if (k < n_valid) join(row, RowPart{red[k][r].x, red[k][r].y}, alpha2);
+    }
+    const float mx2 = __fmul_rn(alpha2, row.max), sum = row.sum;
     const float inv_sum = __frcp_rn(sum);
-    if (p.stats.row) {
+    if (p.stats.row && part == 0) {
       if (row_ok) p.stats.row[((long long)b * p.h + head) * p.S + r] = make_float2(mx2, inv_sum);
       if (r == 0 && head == 0) { p.stats.len[b] = len; if (b == 0) *p.stats.alpha = alpha; }
     }
@@ -136,7 +145,7 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
     const long long prow = (((long long)b * p.h + head) * p.S + r) * p.S;
     const int n_store = p.P ? (p.S + 31) / 32 : n_valid;
 #pragma unroll 1
-    for (int c = 0; c < n_store; ++c) {
+    for (int c = part; c < n_store; c += TPR) {
       uint32_t pw[16], cw[16];                            // 32 probabilities / codes packed as bf16 pairs
       if (c < n_valid) {
         uint32_t a[32];
@@ -168,14 +177,20 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
     if (!__all_sync(0xffffffffu, got2) && lane == 0) atomicCAS(p.status, 0, (int)DEV_TIMEOUT_MMA);
     tc_fence_after();
     if (p.ctx) {                                         // (all products have run: the tiles of P and V are free)
+      if constexpr (TPR == 1) {
 #pragma unroll 1
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t a[32];
-        tmem_ld32(trow + (uint32_t)(hh * 32), a);
-        context32<QUANT>(p, a, calpha, cs, r, hh, gP, gP + 16384, gP - 16384);
+        for (int hh = 0; hh < 2; ++hh) {
+          uint32_t a[32];
+          tmem_ld32(trow + (uint32_t)(hh * 32), a);
+          context_piece<QUANT, 32>(p, a, calpha, cs, r, hh, gP, gP + 16384, gP - 16384);
+        }
+      } else {
+        uint32_t a[16];
+        tmem_ld16(trow + (uint32_t)(part * 16), a);
+        context_piece<QUANT, 16>(p, a, calpha, cs, r, part, gP, gP + 16384, gP - 16384);
       }
       fence_async_shared();
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(128 * TPR) : "memory");
       if (threadIdx.x == 32) {
         store_context<QUANT>(out, sP, sP + 16384, sV, 0, head, b);
         tma_store_wait_read<0>();
@@ -190,15 +205,15 @@ __global__ void __launch_bounds__(160, 4) attention_fwd_kernel(const __grid_cons
   }
 }
 
-template <bool QUANT>
+template <int TPR, bool QUANT>
 int launch_short(const CUtensorMap& map, const CtxMaps& out, const AttnParams& p, cudaStream_t st) {
   constexpr int smem = 1024 + 16384 * 3;
   static bool attr_set = false;
   if (!attr_set) {
-    if (cudaFuncSetAttribute(attention_fwd_kernel<QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GEMM_ERR_CUDA;
+    if (cudaFuncSetAttribute(attention_fwd_kernel<TPR, QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GEMM_ERR_CUDA;
     attr_set = true;
   }
-  if (launch_k(attention_fwd_kernel<QUANT>, dim3(1, p.h, p.B), 160, smem, st, map, out, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  if (launch_k(attention_fwd_kernel<TPR, QUANT>, dim3(1, p.h, p.B), 32 + 128 * TPR, smem, st, map, out, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }
 
@@ -234,7 +249,8 @@ int launch_attention_fwd(const void* qkv, int B, int S, int h, int H, const int*
   CtxMaps out;
   if (rc == GEMM_OK) rc = make_ctx_maps(&out, p, map);
   if (rc != GEMM_OK) return rc;
-  return p_step ? launch_short<true>(map, out, p, st) : launch_short<false>(map, out, p, st);
+  if (B * h <= 148) return p_step ? launch_short<4, true>(map, out, p, st) : launch_short<4, false>(map, out, p, st);     // a CTA per SM
+  return p_step ? launch_short<1, true>(map, out, p, st) : launch_short<1, false>(map, out, p, st);
 }
 
 }  // namespace mrem

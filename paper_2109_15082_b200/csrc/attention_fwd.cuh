@@ -40,31 +40,37 @@ __device__ __forceinline__ float max3(float a, float b, float c) {   // NaNs as 
   return d;
 }
 
-// The row's maximum and sum of exponentials so far, joined by 32 scores (accumulators a, the first ncol >= 1 of them valid).  In units of
-// log2(e): exp(alpha * a - max) = 2^(alpha2 * a - max2); alpha > 0, so the maximum can be taken over the raw accumulators.  max2 is
-// rounded (not a part of an fma): an exponential formed with it again later is the same number.
-__device__ __forceinline__ void join_chunk(uint32_t* a, int ncol, float alpha2, float& mx, float2 (&sums)[2]) {
+// A row's softmax is put together from chunks of 32 scores: maximum of a chunk, sum of its exponentials with that maximum, then the
+// chunks in order.  However many threads share a row, a sequence has the same sums bit for bit.
+// In units of log2(e): exp(alpha * a - max) = 2^(alpha2 * a - max2); alpha > 0, so the maximum can be taken over the raw accumulators.
+// max2 is rounded (not a part of an fma): an exponential formed with it again later is the same number.
+struct RowPart { float max, sum; };
+// of 32 scores (accumulators a, the first ncol >= 1 of them valid)
+__device__ __forceinline__ RowPart chunk_part(uint32_t* a, int ncol, float alpha2) {
   if (ncol < 32) {                                       // (warp-uniform, a row's last chunk only: nothing below tests the keys)
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (j >= ncol) a[j] = 0xff800000u;                 // -inf
   }
-  float m4[4] = {mx, __uint_as_float(a[0]), __uint_as_float(a[1]), __uint_as_float(a[2])};
+  float m4[4] = {__uint_as_float(a[0]), __uint_as_float(a[1]), __uint_as_float(a[2]), __uint_as_float(a[3])};
 #pragma unroll
-  for (int j = 3; j < 31; j += 2) m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], __uint_as_float(a[j]), __uint_as_float(a[j + 1]));
-  const float m = fmaxf(max3(m4[0], m4[1], m4[2]), fmaxf(m4[3], __uint_as_float(a[31]))), m2 = __fmul_rn(alpha2, m);
-  if (__any_sync(0xffffffffu, m != mx)) {
-    const float f = m == mx ? 1.f : exp2_approx(__fmul_rn(alpha2, mx) - m2);
-    sums[0] = mul2(sums[0], splat(f));
-    sums[1] = mul2(sums[1], splat(f));
-  }
-  mx = m;
-  const float2 nmx2 = splat(m == -INFINITY ? 0.f : -m2); // (nothing but -inf so far: adds zeros)
+  for (int j = 4; j < 32; j += 2) m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], __uint_as_float(a[j]), __uint_as_float(a[j + 1]));
+  const float m = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]);
+  const float2 nmx2 = splat(m == -INFINITY ? 0.f : -__fmul_rn(alpha2, m));             // (nothing but -inf: a sum of zeros)
+  float2 sums[2] = {splat(0.f), splat(0.f)};
 #pragma unroll
   for (int j = 0; j < 32; j += 2) {
     const float2 t = fma2(make_float2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])), splat(alpha2), nmx2);
     sums[(j >> 1) & 1] = add2(sums[(j >> 1) & 1], make_float2(exp2_approx(t.x), exp2_approx(t.y)));
   }
+  return RowPart{m, (sums[0].x + sums[0].y) + (sums[1].x + sums[1].y)};
+}
+// row += part (a row starts as {-inf, 0})
+__device__ __forceinline__ void join(RowPart& row, const RowPart& part, float alpha2) {
+  const float m = fmaxf(row.max, part.max), m2 = __fmul_rn(alpha2, m);
+  const float f = row.max == m ? 1.f : exp2_approx(__fmul_rn(alpha2, row.max) - m2);
+  const float g = part.max == m ? 1.f : exp2_approx(__fmul_rn(alpha2, part.max) - m2);
+  row = RowPart{m, __fmaf_rn(part.sum, g, __fmul_rn(row.sum, f))};
 }
 
 // 32 scores of a row (accumulators a, the first ncol of them valid) -> their probabilities as bf16 pairs (pw) and what the second
@@ -104,17 +110,17 @@ __device__ __forceinline__ void probabilities32(const uint32_t* a, int ncol, con
   }
 }
 
-// 32 columns of a context row (accumulators a) into operand-like tiles of 128 rows that leave by tiled stores: bf16 values, and with a
+// Piece `part` of a context row, N columns (accumulators a), into operand-like tiles of 128 rows that leave by tiled stores: bf16 values, and with a
 // quantizer their codes as bf16 numbers and as bytes.  (Stored from registers, a row per lane, every instruction touched 32 lines:
 // 2.3 us of a CTA's 15 at 16 x 16 x 384 x 384.)
 struct CtxMaps { CUtensorMap ctx, qt, q8; };
-template <bool QUANT>
-__device__ __forceinline__ void context32(const AttnParams& p, const uint32_t* a, float calpha, float cs, int r, int half, uint8_t* t_ctx, uint8_t* t_qt,
-                                          uint8_t* t_q8) {
-  uint32_t w[16], cq[16], c8[8];
+template <bool QUANT, int N>
+__device__ __forceinline__ void context_piece(const AttnParams& p, const uint32_t* a, float calpha, float cs, int r, int part, uint8_t* t_ctx, uint8_t* t_qt,
+                                              uint8_t* t_q8) {
+  uint32_t w[N / 2], cq[N / 2], c8[N / 4];
   const float r_cs = __frcp_rn(cs);
 #pragma unroll
-  for (int j = 0; j < 32; j += 2) {
+  for (int j = 0; j < N; j += 2) {
     const __nv_bfloat162 vb = __floats2bfloat162_rn(calpha * __uint_as_float(a[j]), calpha * __uint_as_float(a[j + 1]));
     w[j >> 1] = *reinterpret_cast<const uint32_t*>(&vb);
     if constexpr (QUANT) {
@@ -130,14 +136,14 @@ __device__ __forceinline__ void context32(const AttnParams& p, const uint32_t* a
   }
   // 128-byte swizzle: 16-byte piece index XOR (row & 7); rows of 64 bytes, 64-byte swizzle: XOR (row / 2 & 3)
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int at = r * 128 + ((half * 4 + t) ^ (r & 7)) * 16;
+  for (int t = 0; t < N / 8; ++t) {
+    const int at = r * 128 + ((part * (N / 8) + t) ^ (r & 7)) * 16;
     store16(t_ctx + at, w + 4 * t);
     if constexpr (QUANT) store16(t_qt + at, cq + 4 * t);
   }
   if constexpr (QUANT) {
 #pragma unroll
-    for (int t = 0; t < 2; ++t) store16(t_q8 + r * 64 + ((half * 2 + t) ^ ((r >> 1) & 3)) * 16, c8 + 4 * t);
+    for (int t = 0; t < N / 16; ++t) store16(t_q8 + r * 64 + ((part * (N / 16) + t) ^ ((r >> 1) & 3)) * 16, c8 + 4 * t);
   }
 }
 // one thread, once every row is written and fenced: 128 rows from q0 on of (head, b); rows beyond the sequence are clipped

@@ -141,26 +141,21 @@ __global__ void __launch_bounds__(LONG_THREADS, 2) attention_fwd_long_kernel(con
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_F0 + (s & 1)));
     };
-    // scores in units of log2(e): exp(alpha * a - max) = 2^(alpha2 * a - max2); alpha > 0, so the maximum
-    // can be taken over the raw accumulators
     const float alpha2 = alpha * 1.4426950408889634f;
-    float mx = -INFINITY;
-    float2 sums[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    RowPart row{-INFINITY, 0.f};
 #pragma unroll 1
     for (int c = 0; c < n; ++c) {
       uint32_t a[32];
       fetch(c, a);
       const int ncol = len - c * 64 - half * 32;             // (>= 32: all keys valid)
-      if (ncol <= 0) continue;
-      join_chunk(a, ncol, alpha2, mx, sums);
+      if (ncol > 0) join(row, chunk_part(a, ncol, alpha2), alpha2);
     }
-    red[half][r] = make_float2(mx, (sums[0].x + sums[0].y) + (sums[1].x + sums[1].y));
+    red[half][r] = make_float2(row.max, row.sum);
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    const float2 h0 = red[0][r], h1 = red[1][r];
-    mx = fmaxf(h0.x, h1.x);
-    const float mx2 = __fmul_rn(alpha2, mx);               // (rounded, as each half subtracted it: not a part of an fma)
-    // (the second half of a row has no valid key when the sequence is shorter than that: nothing to add)
-    const float sum = h0.y * exp2_approx(__fmul_rn(alpha2, h0.x) - mx2) + (len > 32 ? h1.y * exp2_approx(__fmul_rn(alpha2, h1.x) - mx2) : 0.f);
+    row = RowPart{red[0][r].x, red[0][r].y};
+    // (a sequence of up to 32 tokens has no key in the second half of its chunk)
+    if (len > 32) join(row, RowPart{red[1][r].x, red[1][r].y}, alpha2);
+    const float mx2 = __fmul_rn(alpha2, row.max), sum = row.sum;
     const float inv_sum = __frcp_rn(sum);
     if (p.stats.row && half == 0) {
       if (row_ok) p.stats.row[((long long)b * p.h + head) * p.S + q] = make_float2(mx2, inv_sum);
@@ -211,7 +206,7 @@ __global__ void __launch_bounds__(LONG_THREADS, 2) attention_fwd_long_kernel(con
     uint32_t a[32];
     tmem_ld32(trow + (uint32_t)(TMEM_O + half * 32), a);
     if (p.ctx) {
-      context32<QUANT>(p, a, calpha, cs, r, half, gP - 16384, gP, gP + 16384);
+      context_piece<QUANT, 32>(p, a, calpha, cs, r, half, gP - 16384, gP, gP + 16384);
       fence_async_shared();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (threadIdx.x == 32) {

@@ -74,16 +74,17 @@ def test_reading_the_probabilities_leaves_the_backward_pass_alone(seq):
         p.close()
 
 
-# more blocks than run at once: they take the sequences longest first (equal lengths, one key, whole chunks and one more among them)
-@pytest.mark.parametrize("seq,batch", [(136, 12), (320, 8), (136, 32)])
+# above 128 tokens more blocks than run at once: they take the sequences longest first (equal lengths, one key, whole chunks and
+# one more among them); up to 128 tokens more blocks than SMs: a thread per row instead of four
+@pytest.mark.parametrize("seq,batch", [(136, 12), (320, 8), (136, 32), (8, 32), (72, 12), (104, 12), (128, 18)])
 def test_sequences_of_a_large_batch_are_those_of_a_small_one(seq, batch):
     """The quantized pass treats sequences independently (whole numbers, and row sums in the same order): bit for bit the outputs
-    of the same sequences two at a time, which are too few blocks to be ordered."""
+    of the same sequences two at a time, which are few blocks."""
     wl = synth.shrink(synth.workloads()["large6_w4a8"], n_layers=1, seq=seq, batch=batch, len_lo=1, len_hi=seq)
     p = Problem(wl, step_shrink=0.8, student_noise=0.002)
     try:
         m = p.m
-        lens = np.array(([seq, 1, 64, 65, seq, 128, 129, seq - 1, 64, 33, 32, 97] * 3)[:batch], np.int32)
+        lens = np.array(([seq, 1, 64, 65, seq, 128, 129, seq - 1, 64, 33, 32, 97] * 3)[:batch], np.int32).clip(1, seq)
         vld = torch.from_numpy(lens).to(m.device)
         m.quantize_weights()
         many = m.forward_student(p.xd, vld, batch, seq).clone()
@@ -94,19 +95,20 @@ def test_sequences_of_a_large_batch_are_those_of_a_small_one(seq, batch):
         p.close()
 
 
-# step-size partials: a slot per block, and one more block than there are slots (the blocks of a head share one)
-@pytest.mark.parametrize("batch", [295, 297])
-def test_step_gradients_of_more_blocks_than_partial_sums(batch):
-    """Against the kernel-per-operation path: the weight gradient by a few bf16 roundings of dS and dQKV (2^-9 each, averaged over
-    40,000 rows: 1e-2 leaves a factor of two for each), the step gradients as everywhere within 2e-2 of the largest."""
-    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=136, batch=batch, len_lo=1, len_hi=136)
+# above 128 tokens a slot of step-size partials per block, and one more block than there are slots (the blocks of a head share one);
+# up to 128 tokens as many blocks as SMs (four threads per row), and more (two)
+@pytest.mark.parametrize("seq,batch", [(136, 295), (136, 297), (40, 74), (40, 75), (128, 75)])
+def test_gradients_on_both_sides_of_the_number_of_blocks(seq, batch):
+    """Against the kernel-per-operation path: the weight and bias gradients by a few bf16 roundings of dS and dQKV (2^-9 each, averaged
+    over thousands of rows: 1e-2 leaves a factor of two for each), the step gradients as everywhere within 2e-2 of the largest."""
+    wl = synth.shrink(synth.workloads()["base3_w4a8"], n_layers=1, hidden=128, n_heads=2, ffn=256, seq=seq, batch=batch, len_lo=1, len_hi=seq)
     p = Problem(wl, step_shrink=0.8, student_noise=0.002)
     try:
         got = []
         for fused in (True, False):
             p.m.set_fused_attention_backward(fused)
             got.append(p.run_gpu()["grads"][0])
-        assert rel(got[0]["Wqkv"], got[1]["Wqkv"]) < 1e-2
+        assert rel(got[0]["Wqkv"], got[1]["Wqkv"]) < 1e-2 and rel(got[0]["bqkv"], got[1]["bqkv"]) < 1e-2
         a, b = got[0]["a"], got[1]["a"]
         assert np.isfinite(a).all() and np.abs(a - b).max() < 2e-2 * np.abs(b).max(), (a, b)
     finally:
