@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(128) embed_sum_kernel(const float* __restrict_
 // and without six of their seven launches.  Latency bounds it: with one vector per thread a token is one round of loads and three block sums
 // (both modules' means together, both variances, the two sums of the backward), and eight blocks share an SM.
 // (One warp per token with the whole row in its 128 registers: 22 % of the warps active, 29 us; the step of 30522 x 1024, 32 x 128
-// tokens 204 -> 200 us, of 30522 x 768, 5 x 56 tokens 154 -> 150.)  The blocks beyond row_blocks update idle rows of the word table,
-// a warp each: 25 us without them, 30 with 1,900 rows (57 MB, 8.5 us of the table's own update).
+// tokens 204 -> 200 us, of 30522 x 768, 5 x 56 tokens 154 -> 150.)
+// (Rows of the table updated by blocks behind those of the tokens gained less than the same rows beside the sums.)
 constexpr int MAX_W = 4;
 struct EmbedRow {
   const float *t_word, *t_pos, *t_type, *t_g, *t_b;           // teacher tables and LayerNorm
@@ -82,7 +82,6 @@ struct EmbedRow {
   int* status; unsigned* ticket;                              // (the ticket starts as 0xffffffff)
   float *mean, *rstd, *loss_partial, *loss;
   int row_blocks;
-  IdleRows idle;
 };
 
 template <int V>
@@ -122,15 +121,18 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
   __shared__ float2 part[3][W * TPB];                         // one set per sum: the next token's first is behind this one's last
   __shared__ int last;
   const int wid = threadIdx.x >> 5, H = p.H, c = (int)(threadIdx.x % (32 * W)) * V;
-  if ((int)blockIdx.x >= p.row_blocks) {
-    update_idle_rows<2>(p.idle, ((int)blockIdx.x - p.row_blocks) * W * TPB + wid, ((int)gridDim.x - p.row_blocks) * W * TPB);
-    return;
-  }
   float err = 0.f;
+  int next_id = 0, next_tt = 0;                               // (a token's ids are fetched one token ahead of its rows)
+  auto fetch = [&](long long t) {
+    next_id = t < p.M ? p.ids[t] : 0;
+    next_tt = t < p.M && p.type_ids ? p.type_ids[t] : 0;
+  };
+  fetch((long long)blockIdx.x * TPB + wid / W);
   for (long long t0 = (long long)blockIdx.x * TPB; t0 < p.M; t0 += (long long)p.row_blocks * TPB) {
     const long long t = t0 + wid / W;
     const bool live = t < p.M, on = live && c < H;
-    int id = live ? p.ids[t] : 0, tt = live && p.type_ids ? p.type_ids[t] : 0;
+    int id = next_id, tt = next_tt;
+    fetch(t + (long long)p.row_blocks * TPB);
     if (id < 0 || id >= p.vocab || tt < 0 || tt >= p.n_types) {   // recorded, then clamped: no out-of-range access
       if (c == 0) atomicCAS(p.status, 0, (int)DEV_BAD_INDEX);
       id = min(max(id, 0), p.vocab - 1);
@@ -239,6 +241,7 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 
 // Every sum over the token gradients dy in one launch (256 threads a block), and AdamW on the small tensors as their sums
 // become complete:
+//   (in the order ln_chunks, token types, word table, positions: the longest chains first)
 //   max_pos blocks: one position each, two half sums over the batch (even and odd sequences), then that row's update.
 //   TYPE_CHUNKS blocks per token type: one chunk of tokens each; the last chunk to finish adds the chunks in index order
 //     and updates the row.
@@ -248,10 +251,12 @@ embed_row_kernel(const __grid_constant__ EmbedRow p, const T* __restrict__ extra
 //     gathered by more than WARP_MAX tokens is left to the whole block, its warps taking consecutive eighths of the tokens and
 //     the eight sums being added in warp order.  Warp w of block i has token w * blocks + i: frequent ids first appear among
 //     the first tokens, and would otherwise all meet in one block.
-//   The blocks beyond update idle rows of the word table, a warp each: memory that the sums leave idle.
+//   Before all of these, up to two blocks per SM walk through idle rows of the word table, a warp per row, and do not wait for the token
+//     kernel: they stream through memory that its last tokens and the sums leave idle.
 // The sums are chains of dependent loads.  The longest were the last chunks' totals (a column per thread, eight chunks at a time; now
 // four columns and sixteen chunks) and the walk over the ids (the next 128 are on their way now): step 217 -> 192 us at 32 x 128
 // tokens, 136 -> 125 at 5 x 56.  Three blocks: four spill, 200 -> 207 us there although 280 tokens take 148 instead of 150.
+constexpr int IDLE_BLOCKS = 148;                              // one per SM
 constexpr int TYPE_CHUNKS = 64;
 // Chunks of the LayerNorm's sums: above 4096 tokens twice as many, or their chains are the longest of the launch (table 1000 x 512, 48 x 128
 // tokens 67.0 -> 65.6 us; 30522 x 768, 5 x 56 tokens 125 with 48, 130 with 96).
@@ -268,7 +273,7 @@ struct EmbedTables {
   const OptimScalars* sc;                                     // null: gradients only
   AdamEntry pos, type, ln_g, ln_b;
   bool vec;                                                   // these tensors start on 16-byte boundaries
-  int ln_chunks, sum_blocks;                                  // blocks of the sums; those beyond take idle rows
+  int ln_chunks, sum_blocks;                                  // blocks of the sums; those before take idle rows
   IdleRows idle;
 };
 
@@ -378,25 +383,78 @@ __device__ __forceinline__ void add_rows_of_id(const EmbedTables& p, const T* __
 template <typename T, int V>
 __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_constant__ EmbedTables p, const T* __restrict__ dy, const T* __restrict__ dsum,
                                                               const T* __restrict__ y_s) {
-  pdl_wait();
-  pdl_trigger();
-  if ((int)blockIdx.x >= p.sum_blocks) {
-    update_idle_rows<2>(p.idle, ((int)blockIdx.x - p.sum_blocks) * 8 + (int)(threadIdx.x >> 5), ((int)gridDim.x - p.sum_blocks) * 8);
+  const int idle_blocks = (int)gridDim.x - p.sum_blocks;
+  if ((int)blockIdx.x < idle_blocks) {
+    pdl_trigger();
+    update_idle_rows<2>(p.idle, (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), idle_blocks * 8);
     return;
   }
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][TAB_COLS];
   __shared__ int flag, group[8];
   constexpr int NV = TAB_COLS / (32 * V);                     // vectors per lane in a pass
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, H = p.H;
-  const int n_sum = p.max_pos + TYPE_CHUNKS * p.n_types;
   OptimScalars o{};
   if (p.sc) o = *p.sc;
-  int blk = (int)blockIdx.x;
-  if (blk < n_sum) {
+  int blk = (int)blockIdx.x - idle_blocks;
+  if (blk < p.ln_chunks) {
+    // gradients of the LayerNorm's gain and bias: sums over the tokens of d * (y - mean) * rstd and of d
+    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7, per = (p.M + p.ln_chunks - 1) / p.ln_chunks, t0 = blk * per, t1 = min(p.M, t0 + per);
+    for (int c0 = 0; c0 < H; c0 += 128 * V) {
+      const int c = c0 + tx * V;
+      float ab[V], ag[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) ab[j] = ag[j] = 0.f;
+      if (c < H) {
+#pragma unroll 4
+        for (int t = t0 + ty; t < t1; t += 2) {
+          const float mu = p.mean[t], rs = p.rstd[t];
+          float d[V], y[V];
+          load_vec<T, V>(dsum + (long long)t * H + c, d);
+          load_vec<T, V>(y_s + (long long)t * H + c, y);
+#pragma unroll
+          for (int j = 0; j < V; ++j) { ab[j] += d[j]; ag[j] += d[j] * ((y[j] - mu) * rs); }
+        }
+      }
+      for (int k = 0; k < 2; ++k) {
+        float* dst = p.ln_partial + ((long long)blk * 2 + k) * H;
+        if (ty == 1) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) red[j][tx] = k ? ag[j] : ab[j];
+        }
+        __syncthreads();
+        if (ty == 0) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) red[j][tx] += k ? ag[j] : ab[j];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 128 * V && c0 + i < H; i += 256) dst[c0 + i] = red[i % V][i / V];
+        __syncthreads();
+      }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + p.n_types, 1u) + 2u == (unsigned)p.ln_chunks;
+    __syncthreads();
+    if (!flag) return;
+    __threadfence();
+    for (int c = 4 * threadIdx.x; c < 2 * H; c += 1024) {      // (H is a multiple of 16: no group of four crosses the two)
+      const float4 acc = sum_chunks4(p.ln_partial, p.ln_chunks, 2ll * H, c);
+      const AdamEntry& e = c < H ? p.ln_b : p.ln_g;
+      const int i = c < H ? c : c - H;
+      store4(e.g + i, acc, p.vec);
+      if (p.sc) update4(e, o, i, acc, p.vec);
+    }
+    return;
+  }
+  blk -= p.ln_chunks;
+  const int n_type = TYPE_CHUNKS * p.n_types, nb = (p.M + 7) / 8, n_word = nb * ((p.H + TAB_COLS - 1) / TAB_COLS);
+  if (blk < n_type || blk >= n_type + n_word) {
     // sums over rows of dy: threads 0..127 take the even rows of the set, 128..255 the odd ones
     const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7;
-    const bool is_pos = blk < p.max_pos;
-    if (!is_pos) blk -= p.max_pos;
+    const bool is_pos = blk >= n_type;
+    if (is_pos) blk -= n_type + n_word;
     const int s = blk, k = blk / TYPE_CHUNKS, chunk = blk % TYPE_CHUNKS;
     const int per = (p.M + TYPE_CHUNKS - 1) / TYPE_CHUNKS, t0 = chunk * per, t1 = min(p.M, t0 + per);
     float* dst = is_pos ? p.g_pos + (long long)s * H : p.type_partial + ((long long)chunk * p.n_types + k) * H;
@@ -454,59 +512,8 @@ __global__ void __launch_bounds__(256, 3) embed_tables_kernel(const __grid_const
     }
     return;
   }
-  blk -= n_sum;
-  if (blk < p.ln_chunks) {
-    // gradients of the LayerNorm's gain and bias: sums over the tokens of d * (y - mean) * rstd and of d
-    const int tx = threadIdx.x & 127, ty = threadIdx.x >> 7, per = (p.M + p.ln_chunks - 1) / p.ln_chunks, t0 = blk * per, t1 = min(p.M, t0 + per);
-    for (int c0 = 0; c0 < H; c0 += 128 * V) {
-      const int c = c0 + tx * V;
-      float ab[V], ag[V];
-#pragma unroll
-      for (int j = 0; j < V; ++j) ab[j] = ag[j] = 0.f;
-      if (c < H) {
-#pragma unroll 4
-        for (int t = t0 + ty; t < t1; t += 2) {
-          const float mu = p.mean[t], rs = p.rstd[t];
-          float d[V], y[V];
-          load_vec<T, V>(dsum + (long long)t * H + c, d);
-          load_vec<T, V>(y_s + (long long)t * H + c, y);
-#pragma unroll
-          for (int j = 0; j < V; ++j) { ab[j] += d[j]; ag[j] += d[j] * ((y[j] - mu) * rs); }
-        }
-      }
-      for (int k = 0; k < 2; ++k) {
-        float* dst = p.ln_partial + ((long long)blk * 2 + k) * H;
-        if (ty == 1) {
-#pragma unroll
-          for (int j = 0; j < V; ++j) red[j][tx] = k ? ag[j] : ab[j];
-        }
-        __syncthreads();
-        if (ty == 0) {
-#pragma unroll
-          for (int j = 0; j < V; ++j) red[j][tx] += k ? ag[j] : ab[j];
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 128 * V && c0 + i < H; i += 256) dst[c0 + i] = red[i % V][i / V];
-        __syncthreads();
-      }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) flag = atomicAdd(p.type_ticket + p.n_types, 1u) + 2u == (unsigned)p.ln_chunks;
-    __syncthreads();
-    if (!flag) return;
-    __threadfence();
-    for (int c = 4 * threadIdx.x; c < 2 * H; c += 1024) {      // (H is a multiple of 16: no group of four crosses the two)
-      const float4 acc = sum_chunks4(p.ln_partial, p.ln_chunks, 2ll * H, c);
-      const AdamEntry& e = c < H ? p.ln_b : p.ln_g;
-      const int i = c < H ? c : c - H;
-      store4(e.g + i, acc, p.vec);
-      if (p.sc) update4(e, o, i, acc, p.vec);
-    }
-    return;
-  }
-  blk -= p.ln_chunks;
-  const int nb = (p.M + 7) / 8, c0 = (blk / nb) * TAB_COLS;
+  blk -= n_type;
+  const int c0 = (blk / nb) * TAB_COLS;
   blk = blk % nb;
   const int tok = wid * nb + blk;
   int mine = -1, count = 0;                                   // id whose row this warp's token is the first to gather
@@ -653,19 +660,20 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
   launch_k(embed_mark_kernel, (unsigned)((M + 255) / 256 + (o ? 1 : 0)), 256, 0, st, d_ids, (int)M, V, row_first, row_last, row_count, oa);
   // Update of the word table: mask + step gradient + AdamW on the steps and the table + Eq. 1 with the new values in one pass (the
   // small tensors are updated by the launch that adds up their gradients, the other embedding tables decayed like weight matrices,
-  // LayerNorm not).  The rows that no token gathered need nothing of this step but the marks.  The two launches before the last take
-  // as many of them as memory can serve beside their own chains of loads; the last one, which is bound by memory, the rest: its
-  // blocks keep more bytes in flight.  30522 x 1024 with 32 x 128 tokens 199 -> 192 us, 30522 x 768 with 5 x 56 tokens 150 -> 125.
-  // Their shares, a number of rows that grows with the tokens, whose chains last that long, and a constant number of bytes (16 and 99 MB at
-  // 29 bytes a weight) for what a launch waits at its ends, were fitted at these two sizes.
-  // (No idle rows beside the sums of many tokens: 197 and 125; seven eighths of the table beside the sums: 204 and 128; idle blocks
-  // spread evenly among those of the sums: 196 and 126.)
+  // LayerNorm not).  The rows that no token gathered need nothing of this step but the marks and the optimizer's scalars, which are complete
+  // before the token kernel lets its successors start.  So the launch of the sums begins with a few blocks that walk through such rows
+  // without waiting for the token kernel, and the last launch, whose blocks keep more bytes in flight, begins with the rest and does
+  // not wait for the sums.  30522 x 1024 with 32 x 128 tokens 194.5 -> 181.6 us, 30522 x 768 with 5 x 56 125.4 -> 119.2, with 48 x 128 170.7 ->
+  // 160.1, 21128 x 512 with 8 x 64 74.4 -> 68.1 (before: blocks behind those of the token kernel and of the sums, everything waiting).
+  // The share of the sums' launch, a number of rows that grows with the tokens, whose chains last that long, and 145 MB at 29 bytes a weight
+  // (half as many: 184.7, 121.3, 165.2, 71.3), and its blocks, one of three per SM or with few tokens two (two with many: 185.5, 166.4; one with
+  // few: 121.7, 74.0; as many as it takes: 186.6, 121.4, 166.5, 71.4), were fitted at these sizes.
   const RowUpdate table{x->word, x->g_word, x->m_word, x->v_word, x->word_step, x->m_word_step, x->v_word_step, nullptr,
                         s.codes, s.rowsum, s.scale, nullptr, V, H};
   int idle_at = o ? 0 : V;                                   // the next idle row to hand out
   auto take_idle = [&](long long n) {
     const int first = idle_at;
-    idle_at = (int)(n < 0 ? first : (first + n < V ? first + n : V));
+    idle_at = (int)(first + n < V ? first + n : V);
     return IdleRows{table, s.optim_sc, row_first, d->e_bits, first, idle_at};
   };
   const int row_warps = (H + 32 * (dt == 1 ? 8 : 4) - 1) / (32 * (dt == 1 ? 8 : 4));
@@ -676,11 +684,9 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
     const int row_blocks = (int)(want < RED_BLOCKS ? want : RED_BLOCKS);
     const EmbedRow er{x->t_word, x->t_pos, x->t_type, x->t_ln_g, x->t_ln_b, x->pos, x->type, x->ln_g, x->ln_b, s.codes, s.scale, d_ids, d_type_ids,
                       (int)seq, H, V, (int)d->n_types, M, d->ln_eps, cc, d_status, loss_ticket,
-                      s.mean, s.rstd, s.loss_partial, d_loss, row_blocks, take_idle(M / 3 + 550000 / H)};
-    const int idle_warps = row_warps * tpb;
-    const unsigned grid = (unsigned)(row_blocks + (er.idle.end - er.idle.first + idle_warps - 1) / idle_warps);
-    Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)) + 29.0 * H * (er.idle.end - er.idle.first), 0, st);
-#define MREM_ROW(T, V, W) launch_k(embed_row_kernel<T, V, W>, grid, 32 * W * tokens_per_block(W), 0, st, er, (const T*)d_extra_grad, (T*)d_e_teacher, (T*)d_e_student, (T*)s.y_s, (T*)s.dsum, (T*)s.dy)
+                      s.mean, s.rstd, s.loss_partial, d_loss, row_blocks};
+    Scope sc("embed_row", (double)M * H * (8.0 + 1.0 + (dt == 1 ? 2.0 : 4.0) * (d_extra_grad ? 6 : 5)), 0, st);
+#define MREM_ROW(T, V, W) launch_k(embed_row_kernel<T, V, W>, row_blocks, 32 * W * tokens_per_block(W), 0, st, er, (const T*)d_extra_grad, (T*)d_e_teacher, (T*)d_e_student, (T*)s.y_s, (T*)s.dsum, (T*)s.dy)
 #define MREM_ROWS(T, V) do { if (row_warps == 1) MREM_ROW(T, V, 1); else if (row_warps == 2) MREM_ROW(T, V, 2); else if (row_warps == 3) MREM_ROW(T, V, 3); else MREM_ROW(T, V, 4); } while (0)
     if (dt == 1) MREM_ROWS(bf16, 8); else MREM_ROWS(float, 4);
 #undef MREM_ROWS
@@ -715,8 +721,10 @@ int32_t mrem_embed_step(const mrem_embed_desc* d, const mrem_embed_tensors* x, v
                        (int)d->max_pos, (int)M, s.mean, s.rstd, x->g_word, x->g_pos, x->g_type, s.type_partial, s.ln_partial, o ? s.optim_sc : nullptr,
                        {x->pos, x->g_pos, x->m_pos, x->v_pos, 0, 1.f, -INFINITY}, {x->type, x->g_type, x->m_type, x->v_type, 0, 1.f, -INFINITY},
                        {x->ln_g, x->g_ln_g, x->m_ln_g, x->v_ln_g, 0, 0.f, -INFINITY}, {x->ln_b, x->g_ln_b, x->m_ln_b, x->v_ln_b, 0, 0.f, -INFINITY},
-                       vec, ln_chunks(M), n_sum, take_idle(M / 3 + 3400000 / H)};
-  const unsigned tgrid = (unsigned)(n_sum + (tb.idle.end - tb.idle.first + 7) / 8);
+                       vec, ln_chunks(M), n_sum, take_idle(M + 5000000 / H)};
+  const int idle_rows = tb.idle.end - tb.idle.first, idle_limit = M <= 1024 ? 2 * IDLE_BLOCKS : IDLE_BLOCKS,
+            idle_blocks = (idle_rows + 7) / 8 < idle_limit ? (idle_rows + 7) / 8 : idle_limit;
+  const unsigned tgrid = (unsigned)(n_sum + idle_blocks);
   {
     Scope sc("embed_tables", (double)M * H * 5.0 * (dt == 1 ? 2.0 : 4.0) + 29.0 * H * (tb.idle.end - tb.idle.first), 0, st);
     if (dt == 1) launch_k(embed_tables_kernel<bf16, 8>, tgrid, 256, 0, st, tb, (const bf16*)s.dy, (const bf16*)dsum, (const bf16*)s.y_s);

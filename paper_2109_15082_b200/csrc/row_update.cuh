@@ -17,10 +17,18 @@ __device__ __forceinline__ float2 adam2(float2 p, float2 g, float2& m, float2& v
   return add2(mul2(p, a.decay), make_float2(__fdividef(num.x, denom.x), __fdividef(num.y, denom.y)));
 }
 
+// A word that a launch before the one before wrote, read by a block that has not waited for the one before: the word is in memory, and the
+// acquire keeps this thread's later loads (of the step's scalars) from what its SM's L1 held before.
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // The rows in [first, end) of a table of which `used` says 0xffffffff: no token gathered them, so their gradient is zero (written
 // as such), their step gradient too, and nothing but the optimizer's scalars is needed to update them.  A warp updates a row by
-// itself, without a barrier and whatever its block does besides: blocks of these rows are the tail of launches that wait on
-// latency, not on memory, for as long as the table's traffic lasts.  The same arithmetic as the fused update's, integer grid.
+// itself, without a barrier and whatever its block does besides: blocks of these rows run beside those of launches that wait on
+// latency, not on memory, and may do so before the launch before their own has ended.  The same arithmetic as the fused update's, integer grid.
 struct IdleRows {
   RowUpdate m;
   const OptimScalars* sc;
@@ -32,11 +40,12 @@ template <int U>
 __device__ __forceinline__ void update_idle_rows(const IdleRows& r, int warp, int n_warps) {
   const int lane = threadIdx.x & 31, nvec = r.m.cols / 4;
   const float qmax = (float)((1 << (r.bits - 1)) - 1);
+  if (r.first < r.end) load_acquire(r.used + r.first);
   const OptimScalars o = *r.sc;
   const Adam2 ad = make_adam2(o);
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int row = r.first + warp; row < r.end; row += n_warps) {
-    if (r.used[row] != 0xffffffffu) continue;
+    if (__ldcg(r.used + row) != 0xffffffffu) continue;
     const long long base = (long long)row * r.m.cols;
     float4* w4 = reinterpret_cast<float4*>(r.m.w + base);
     float4* g4 = reinterpret_cast<float4*>(r.m.g + base);
