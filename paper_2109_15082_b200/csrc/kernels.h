@@ -217,7 +217,7 @@ struct RowUpdate {
 constexpr int MAX_ROW_UPDATES = 4;
 // `n` matrices (at most MAX_ROW_UPDATES) in one launch.
 void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
-                                int dt, cudaStream_t st);
+                                int dt, cudaStream_t st, bool twins = false);
 // The same of a table (grid 0, no dequantized rows) whose rows `tokens` gathered, and of the idle rows of a range in the same launch.
 struct TokenRows { const int* ids; const unsigned* row_first; int n; };      // n tokens; the first one with an id, per row
 struct IdleRows;                                                             // row_update.cuh

@@ -258,7 +258,7 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
 }
 
 // The fused update of `n` of one layer's matrices, from index k0 on, and their row steps (Algorithm 2: Update(w), Update(s)).
-void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st) {
+void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st, bool twins = false) {
   const mrem_module_desc& d = c->d;
   const int train_w = (d.trainable_mask & MREM_TRAIN_WEIGHTS) != 0, train_s = (d.trainable_mask & MREM_TRAIN_W_STEPS) != 0;
   LayerGrad& g = c->grad[l];
@@ -274,7 +274,7 @@ void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st) 
       mats[i] = RowUpdate{c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->bind[l].w_steps[k], g.m_ws[k], g.v_ws[k],
                           c->w_ste_done ? g.ws[k] : nullptr, w.codes, w.rowsum, w.scale, w.what, w.rows, w.cols};
   }
-  if (!closed_form_weights(d)) launch_fused_weight_update(mats, n, c->optim_sc, d.w_bits, d.w_grid, train_w, train_s, c->dt, st);
+  if (!closed_form_weights(d)) launch_fused_weight_update(mats, n, c->optim_sc, d.w_bits, d.w_grid, train_w, train_s, c->dt, st, twins);
 }
 
 // ------------------------------------------------------------------ backward
@@ -406,7 +406,7 @@ int student_backward(mrem_ctx* c, const mrem_optim* o) {
     // (The products that read these two matrices are behind the fork above.)
     if (halves) {
       rw.flush_deferred();
-      if (o) enqueue_matrix_updates(c, l, W_1, 2, side);
+      if (o) enqueue_matrix_updates(c, l, W_1, 2, side, true);
     }
     r.gemm(view(q.d_y1, H), weights(w[W_O].what, H, 1), (int)M, H, H, 1, 1, Epi(c->d_ctxhat, ok, H).e);
     rw.defer(view(q.d_y1, H, 1), view(s.ctx_qt, H, 1), H, H, (int)M, Epi(g.p[MREM_WO], OUT_F32, H).alpha(1.f, b.a_steps[S_C]).e);

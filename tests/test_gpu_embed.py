@@ -171,9 +171,10 @@ def test_embedding_steps_of_changing_size_share_one_quantized_table(act_dtype, H
             assert rel(e.g[k].cpu().numpy(), r["grads"][k]) < 2e-2, (t, k)
 
 
-# tables smaller than what the first launch of a step takes of them, ending inside the second, reaching into the last; widths of each
+# tables smaller than what the sums' launch of a step takes of them, reaching into the last; widths of each
 # form of the row update; rows wider than the one-kernel path takes
-@pytest.mark.parametrize("V,H,batch,seq", [(1, 16, 1, 3), (300, 768, 2, 9), (631, 128, 3, 37), (2500, 1024, 5, 40), (900, 1040, 2, 11), (6000, 256, 1, 8)])
+@pytest.mark.parametrize("V,H,batch,seq", [(1, 16, 1, 3), (300, 768, 2, 9), (631, 128, 3, 37), (2500, 1024, 5, 40), (900, 1040, 2, 11), (6000, 256, 1, 8),
+                                               (7000, 1024, 2, 9), (8000, 1024, 30, 40)])     # (rows left to the last launch)
 def test_every_row_of_the_table_is_updated_once_whoever_gathered_it(V, H, batch, seq):
     """Two updates with different tokens: rows gathered in both, one or neither.  Weights and moments against AdamW in float64 with
     the gradient the call left (zero for a row nobody gathered); afterwards the codes that the updates left give the outputs,
