@@ -155,9 +155,12 @@ struct StoreCtx {
   uint32_t box;               // shared address of the warp's box (1024-byte aligned)
   int row0, b0, b1;           // C row of lane 0, batch coordinates
   int lane;
+  const CUtensorMap* code_map = nullptr;       // the same for the codes (MODE & 32), whose box follows the last warp's
+  const float2* code_terms = nullptr;          // step and reciprocal of each column segment's quantizer, in shared memory
 };
+constexpr int CODE_BOX_OFFSET = EPI_WARPS * OUT_BOX_BYTES;
 
-// MODE >= 0: bit 0 column scale, bit 1 column bias, bit 2 residual, bit 3 GELU, known at compile time;
+// MODE >= 0: bit 0 column scale, bit 1 column bias, bit 2 residual, bit 3 GELU, bit 5 codes of the output, known at compile time;
 // MODE < 0: the same four read from the Epilogue at run time.
 template <int MODE> struct EpiFlags {
   bool scale, bias, res, act;
@@ -182,6 +185,7 @@ template <int KIND, int OUT, int MODE>
 __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* r, const uint32_t* res, float alpha, float rb,
                                              const float* cv, long long off, bool row_ok, const StoreCtx& sx, int n) {
   constexpr bool ROW_BIAS = MODE < 0 || (MODE & 16) != 0;      // (epilogue_mode: the bf16 variants have none)
+  constexpr bool CODES = MODE >= 0 && (MODE & 32) != 0;
   if (OUT == OUT_I32) {
     if (row_ok) {
       int* out = reinterpret_cast<int*>(e.out) + off;
@@ -234,7 +238,7 @@ __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* 
       o[j] = *reinterpret_cast<const uint32_t*>(&h);
     }
     if (sx.map) {
-      if (sx.lane == 0) tma_store_wait_read<0>();          // the box's previous store has read it
+      if (sx.lane == 0) tma_store_wait_read<CODES ? 1 : 0>();          // the box's previous store has read it
       __syncwarp();
       const uint32_t row_addr = sx.box + (uint32_t)sx.lane * 64u, sw = ((uint32_t)sx.lane >> 1) & 3u;
 #pragma unroll
@@ -244,6 +248,29 @@ __device__ __forceinline__ void finish_chunk(const Epilogue& e, const uint32_t* 
       if (sx.lane == 0) {
         tma_store_4d(sx.map, sx.box, n, sx.row0, sx.b0, sx.b1);
         tma_store_commit();
+      }
+      if constexpr (CODES) {                               // (always with tensor maps) the codes of what has just been stored
+        const float2 t = sx.code_terms[(n >= e.code_cols ? 1 : 0) + (n >= 2 * e.code_cols ? 1 : 0)];
+        const float2 neg_s = splat(-t.x), r2 = splat(t.y);
+        const float hi = e.code_max;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {                     // codes_f of bfloat16 numerators
+          const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&o[j])), z0 = clamp2(mul2(x, r2), -hi - 1.f, hi + 1.f);
+          const float2 z = clamp2(fma2(fma2(z0, neg_s, x), r2, z0), -hi, hi);
+          const float2 q = add2(add2(z, splat(ROUND_MAGIC)), splat(-ROUND_MAGIC));
+          const __nv_bfloat162 h = __floats2bfloat162_rn(q.x, q.y);
+          o[j] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        if (sx.lane == 0) tma_store_wait_read<1>();
+        __syncwarp();
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) sts128(row_addr + CODE_BOX_OFFSET + ((j ^ sw) << 4), o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+        fence_async_shared();
+        __syncwarp();
+        if (sx.lane == 0) {
+          tma_store_4d(sx.code_map, sx.box + CODE_BOX_OFFSET, n, sx.row0, sx.b0, sx.b1);
+          tma_store_commit();
+        }
       }
     } else if (row_ok) {
       bf16* out = reinterpret_cast<bf16*>(e.out) + off;
@@ -329,7 +356,7 @@ template <int KIND, int MODE>
 __device__ __forceinline__ void drain_dispatch(const Epilogue& e, uint32_t taddr, int nchunks, float alpha, float rb,
                                                const float* cv, long long off, bool row_ok, uint32_t* res0,
                                                const StoreCtx& sx, int n) {
-  if (MODE >= 16) {
+  if (MODE >= 0 && (MODE & 16)) {
     drain_chunks<KIND, OUT_F32, MODE>(e, taddr, nchunks, alpha, rb, cv, off, row_ok, res0, sx, n);
   } else if (MODE >= 0 || e.out_kind == OUT_BF16) {
     drain_chunks<KIND, OUT_BF16, MODE>(e, taddr, nchunks, alpha, rb, cv, off, row_ok, res0, sx, n);
@@ -346,10 +373,20 @@ __device__ __forceinline__ void drain_dispatch(const Epilogue& e, uint32_t taddr
 // everything else runs the variant that reads them at run time (-1).
 inline int epilogue_mode(int kind, const Epilogue& e) {
   const int mode = (e.col_scale ? 1 : 0) | (e.col_bias ? 2 : 0) | (e.residual ? 4 : 0) | (e.act == 1 ? 8 : 0);
+  if (e.codes) return kind == 1 && e.out_kind == OUT_BF16 && !e.row_bias && mode == 3 ? 35 : -2;      // (bit 5)
   if (e.out_kind == OUT_F32) return (kind == 0 && mode == 0) ? 16 : -1;
   if (e.out_kind != OUT_BF16 || e.row_bias) return -1;
   if (kind == 0) return (mode == 0 || mode == 2 || mode == 6 || mode == 10) ? mode : -1;
   return (mode == 1 || mode == 3 || mode == 7) ? mode : -1;
+}
+
+// Step and reciprocal of the quantizers of MODE & 32, one warp's copy.
+__device__ __forceinline__ void stage_code_terms(const Epilogue& e, float2* terms, int lane) {
+  if (lane < 3) {
+    const float s = *e.code_step[lane];
+    terms[lane] = make_float2(s, __frcp_rn(s));
+  }
+  __syncwarp();
 }
 
 // True when rows of out (and residual) start on 32-byte boundaries for every row, batch and 32-column chunk,
@@ -367,6 +404,6 @@ __device__ __forceinline__ bool direct_epilogue_ok(const Epilogue& e) {
 int tc_pick_block_n(const int* M, const int* N, const int* k_blocks, int n, int batches, int sm_count, bool wide_out, bool beside);
 // gemm_tcgen05_split.cu: several CTAs per tile; tc_gemm prepares everything and decides.
 bool tc_gemm_split_eligible(int kind, const GemmShape& g, const Epilogue& e);
-int tc_gemm_split_launch(int kind, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const tc::TcParams& params, int splits,
+int tc_gemm_split_launch(int kind, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const CUtensorMap& md, const tc::TcParams& params, int splits,
                          cudaStream_t stream);
 }  // namespace mrem

@@ -8,6 +8,10 @@
 // through a 2 KB shared-memory box per warp and tiled stores, anything else straight from
 // registers with 32-byte vector stores.  The epilogue of tile i overlaps the main loop of
 // tile i+1.
+// The student's QKV product also writes the codes of its stored output (MODE bit 5): a quantizer launch between it and the attention
+// read 25 MB and wrote 25 at 32 x 128 tokens, hidden 1024, and was 3.5 us of a small step's chain a layer.  Passes timed in turn: 32 x 128,
+// hidden 768, forward of both modules 556 -> 547 us; 8 x 256 936 -> 919; 11 x 200 with gradients 356 -> 353; 3 x 72 422.5 -> 419.6; 4 x 32, hidden 128
+// 82.4 -> 81.0; beside the teacher's pass with many tokens (32 x 128, two streams) unchanged.
 // Either operand may be stored k-contiguous ("K-major") or m/n-contiguous ("MN-major");
 // the second form serves the backward products (dX = dY * W_hat, dW = dY^T * X_hat) and
 // the attention products without any transposed copy.
@@ -33,7 +37,7 @@ namespace {
 template <int KIND, int MODE>
 __global__ void __launch_bounds__(GEMM_THREADS, 2)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_c, const __grid_constant__ TcParams p) {
+               const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_d, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];
   __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];
@@ -42,6 +46,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ __align__(16) float col_terms[EPI_WARPS][2 * COLVEC];
+  constexpr bool CODES = MODE >= 0 && (MODE & 32) != 0;
+  __shared__ float2 code_terms[CODES ? EPI_WARPS : 1][3];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -205,7 +211,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // bf16 rows leave through this warp's shared-memory box (behind the operand stages) and tiled stores
     const bool boxed = direct && p.c_tma;
     StoreCtx sx{boxed ? &map_c : nullptr, tiles_base + (uint32_t)(p.num_stages * p.stage_bytes) + (uint32_t)((warp - 2) * OUT_BOX_BYTES),
-                0, 0, 0, lane};
+                0, 0, 0, lane, &map_d, code_terms[CODES ? warp - 2 : 0]};
+    if constexpr (CODES) stage_code_terms(e, code_terms[warp - 2], lane);
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
@@ -432,6 +439,10 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
     const int kb = (g.K + 128 / es - 1) / (128 / es), batches = g.nb0 * g.nb1;
     p.block_n = tc_gemm_split_eligible(kind, g, epi) ? pick_split(g.M, g.N, kb, batches, sm_count, &splits) : 0;
     if (p.block_n == 0) p.block_n = tc_pick_block_n(&g.M, &g.N, &kb, 1, batches, sm_count, false, beside);
+    // With codes a tile of 256 columns has three stages only, and its long epilogue is hidden by the next tile's main loop or not at all: 192
+    // where there is no next tile.  Steps / passes with 256 and with 192: 8 x 256, hidden 768 (144 tiles) 929 and 919 us; 32 x 128, hidden 768
+    // (288 tiles) 547 and 554, hidden 1024 (384 tiles) the same.
+    if (epi.codes && p.block_n == 256 && (long long)((g.M + BLOCK_M - 1) / BLOCK_M) * ((g.N + 255) / 256) * batches <= sm_count) p.block_n = 192;
   } else if (block_n != 64 && block_n != 128 && block_n != 256) {
     return GEMM_ERR_ARG;
   }
@@ -441,7 +452,8 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
   p.k_blocks = (g.K + p.block_k - 1) / p.block_k;
   p.num_tiles = p.m_tiles * p.n_tiles * g.nb0 * g.nb1;
   p.stage_bytes = A_STAGE_BYTES + p.block_n * 128;
-  p.num_stages = SINGLE_CTA_SMEM_BUDGET / p.stage_bytes;
+  const int code_boxes = epi.codes ? EPI_WARPS * OUT_BOX_BYTES : 0;         // (a second box per epilogue warp: fewer stages)
+  p.num_stages = (SINGLE_CTA_SMEM_BUDGET - code_boxes) / p.stage_bytes;
   if (p.num_stages > MAX_STAGES) p.num_stages = MAX_STAGES;
   p.a_mn = A.mn_contig; p.b_mn = B.mn_contig;
   p.b_static = B.is_static;
@@ -474,7 +486,7 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
   if (a_chunked) p.a_mn = 2;
   if (b_chunked) p.b_mn = 2;
   // bf16 output whose rows and batches start on 16-byte boundaries: tiled stores of 32 x 32 boxes
-  CUtensorMap mc = ma;
+  CUtensorMap mc = ma, md = ma;
   p.c_tma = 0;
   if (epi.out_kind == OUT_BF16 && (reinterpret_cast<uintptr_t>(epi.out) & 15) == 0 && epi.ldc % 8 == 0 && epi.ldc >= g.N &&
       (g.nb0 == 1 || epi.c_b0 % 8 == 0) && (g.nb1 == 1 || epi.c_b1 % 8 == 0)) {
@@ -484,16 +496,24 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
     cuuint64_t dims[4] = {(cuuint64_t)g.N, (cuuint64_t)g.M, (cuuint64_t)g.nb0, (cuuint64_t)g.nb1};
     cuuint64_t strides[3] = {s1, s2, s3};
     cuuint32_t box[4] = {32, 32, 1, 1}, estr[4] = {1, 1, 1, 1};
-    if (encode_tiled(&mc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, epi.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
-      p.c_tma = 1;
+    auto out_map = [&](CUtensorMap* m, void* ptr) {
+      return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    if (out_map(&mc, epi.out)) p.c_tma = 1;
+    if (epi.codes && ((reinterpret_cast<uintptr_t>(epi.codes) & 15) || !p.c_tma || !out_map(&md, epi.codes))) return GEMM_ERR_ALIGN;
+  } else if (epi.codes) {
+    return GEMM_ERR_ALIGN;
   }
+  if (epi.codes && (g.N % 32 || epi.code_cols % 32 || epi.code_cols * 3 < g.N || epi.ldc % 16 || (reinterpret_cast<uintptr_t>(epi.out) & 31) ||
+                    (reinterpret_cast<uintptr_t>(epi.col_scale) & 15) || (reinterpret_cast<uintptr_t>(epi.col_bias) & 15)))
+    return GEMM_ERR_ALIGN;
 
-  const int smem = p.num_stages * p.stage_bytes + 1024 + EPI_WARPS * OUT_BOX_BYTES;
-  typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
+  const int smem = p.num_stages * p.stage_bytes + 1024 + EPI_WARPS * OUT_BOX_BYTES + code_boxes;
+  typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
   static const struct { int kind, mode; Kern fn; } variants[] = {
       {0, -1, tc_gemm_kernel<0, -1>}, {0, 0, tc_gemm_kernel<0, 0>}, {0, 2, tc_gemm_kernel<0, 2>}, {0, 6, tc_gemm_kernel<0, 6>},
-      {0, 10, tc_gemm_kernel<0, 10>}, {0, 16, tc_gemm_kernel<0, 16>}, {1, -1, tc_gemm_kernel<1, -1>}, {1, 1, tc_gemm_kernel<1, 1>}, {1, 3, tc_gemm_kernel<1, 3>}, {1, 7, tc_gemm_kernel<1, 7>}};
+      {0, 10, tc_gemm_kernel<0, 10>}, {0, 16, tc_gemm_kernel<0, 16>}, {1, -1, tc_gemm_kernel<1, -1>}, {1, 1, tc_gemm_kernel<1, 1>}, {1, 3, tc_gemm_kernel<1, 3>}, {1, 7, tc_gemm_kernel<1, 7>}, {1, 35, tc_gemm_kernel<1, 35>}};
   constexpr int n_variants = sizeof(variants) / sizeof(variants[0]);
   static bool attr_set[n_variants] = {};
   const int mode = epilogue_mode(kind, epi);
@@ -514,8 +534,8 @@ int tc_gemm(int kind, int a_unsigned, const OperandDesc& A, const OperandDesc& B
     if (splits > 1 && len < (int)sizeof(buf)) snprintf(buf + len, sizeof(buf) - len, "/%d", splits);
     return std::string(buf);
   }, 2.0 * g.M * g.N * (double)g.K * g.nb0 * g.nb1, 1, stream, 0);
-  if (splits > 1) return tc_gemm_split_launch(kind, ma, mb, mc, p, splits, stream);
-  if (launch_k(kern, grid, GEMM_THREADS, smem, stream, ma, mb, mc, p) != cudaSuccess) return GEMM_ERR_CUDA;
+  if (splits > 1) return tc_gemm_split_launch(kind, ma, mb, mc, md, p, splits, stream);
+  if (launch_k(kern, grid, GEMM_THREADS, smem, stream, ma, mb, mc, md, p) != cudaSuccess) return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }
 

@@ -35,7 +35,7 @@ __device__ __forceinline__ void st_own(uint32_t addr, uint32_t v) { asm volatile
 template <int KIND, int MODE>
 __global__ void __maxnreg__(128)
 tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                     const __grid_constant__ CUtensorMap map_c, const __grid_constant__ TcParams p, int splits) {
+                     const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_d, const __grid_constant__ TcParams p, int splits) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];
   __shared__ __align__(8) uint64_t empty_bar[MAX_STAGES];
@@ -44,6 +44,8 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   __shared__ int abort_flag;
   __shared__ __align__(16) float col_terms[EPI_WARPS][2 * COLVEC];
 
+  constexpr bool CODES = MODE >= 0 && (MODE & 32) != 0;
+  __shared__ float2 code_terms[CODES ? EPI_WARPS : 1][3];
   constexpr int OUT = MODE < 0 ? OUT_I32 : (MODE & 16 ? OUT_F32 : OUT_BF16);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -173,6 +175,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     if (owner == rank) {
       if (row_ok) rb = row_term(e, row);
       if (nfull > 0) stage_col_terms<MODE>(e, cv, alpha, col_begin, 32 * chunks, p.N, lane);
+      if constexpr (CODES) stage_code_terms(e, code_terms[warp - 2], lane);
     }
     got = mbar_wait_or_abort(smem_u32(&tfull_bar), 0u, vabort, p.wait_ns);
     got = __all_sync(0xffffffffu, got);
@@ -192,7 +195,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   cluster_wait();
   if (warp >= 2 && got && owner == rank) {
     StoreCtx sx{p.c_tma ? &map_c : nullptr, tiles_base + (uint32_t)(p.num_stages * p.stage_bytes) + (uint32_t)((warp - 2) * OUT_BOX_BYTES),
-                t.m0 + quad * 32, t.b0, t.b1, lane};
+                t.m0 + quad * 32, t.b0, t.b1, lane, &map_d, code_terms[CODES ? warp - 2 : 0]};
 #pragma unroll 1
     for (int c = 0; c < nfull; ++c) {
       uint32_t own[32], acc[32], res[16];
@@ -230,12 +233,12 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   }
 }
 
-typedef void (*SplitKern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams, int);
+typedef void (*SplitKern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams, int);
 const struct { int kind, mode; SplitKern fn; } kVariants[] = {
     {0, 0, tc_gemm_split_kernel<0, 0>}, {0, 2, tc_gemm_split_kernel<0, 2>}, {0, 6, tc_gemm_split_kernel<0, 6>},
-    {0, 10, tc_gemm_split_kernel<0, 10>}, {0, 16, tc_gemm_split_kernel<0, 16>}, {1, -1, tc_gemm_split_kernel<1, -1>}, {1, 1, tc_gemm_split_kernel<1, 1>}, {1, 3, tc_gemm_split_kernel<1, 3>}, {1, 7, tc_gemm_split_kernel<1, 7>}};
+    {0, 10, tc_gemm_split_kernel<0, 10>}, {0, 16, tc_gemm_split_kernel<0, 16>}, {1, -1, tc_gemm_split_kernel<1, -1>}, {1, 1, tc_gemm_split_kernel<1, 1>}, {1, 3, tc_gemm_split_kernel<1, 3>}, {1, 7, tc_gemm_split_kernel<1, 7>}, {1, 35, tc_gemm_split_kernel<1, 35>}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
-constexpr int SPLIT_STAGES = 6;
+constexpr int SPLIT_STAGES = 6;                          // one fewer where a second box per epilogue warp holds codes
 
 int variant_of(int kind, const Epilogue& e) {
   const int mode = epilogue_mode(kind, e);
@@ -244,7 +247,9 @@ int variant_of(int kind, const Epilogue& e) {
     if (kVariants[i].kind == kind && kVariants[i].mode == mode) return i;
   return -1;
 }
-int split_smem(int block_n) { return SPLIT_STAGES * (A_STAGE_BYTES + block_n * 128) + 1024 + EPI_WARPS * OUT_BOX_BYTES; }
+int split_smem(int block_n, bool codes) {
+  return (SPLIT_STAGES - codes) * (A_STAGE_BYTES + block_n * 128) + 1024 + EPI_WARPS * OUT_BOX_BYTES * (1 + codes);
+}
 
 }  // namespace
 
@@ -255,18 +260,19 @@ bool tc_gemm_split_eligible(int kind, const GemmShape& g, const Epilogue& e) {
          al(e.col_scale, 16) && al(e.col_bias, 16);
 }
 
-int tc_gemm_split_launch(int kind, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const TcParams& params, int splits,
+int tc_gemm_split_launch(int kind, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const CUtensorMap& md, const TcParams& params, int splits,
                          cudaStream_t stream) {
   const int vi = variant_of(kind, params.epi);
   if (vi < 0) return GEMM_ERR_ARG;
   TcParams p = params;
-  p.num_stages = SPLIT_STAGES;
+  const bool codes = p.epi.codes != nullptr;
+  p.num_stages = SPLIT_STAGES - codes;
   static bool attr_set[kNumVariants] = {};
   if (!attr_set[vi]) {
-    if (cudaFuncSetAttribute(kVariants[vi].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, split_smem(128)) != cudaSuccess) return GEMM_ERR_CUDA;
+    if (cudaFuncSetAttribute(kVariants[vi].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, split_smem(128, codes)) != cudaSuccess) return GEMM_ERR_CUDA;
     attr_set[vi] = true;
   }
-  if (launch_cluster(kVariants[vi].fn, p.num_tiles * splits, GEMM_THREADS, split_smem(p.block_n), stream, splits, ma, mb, mc, p, splits) != cudaSuccess)
+  if (launch_cluster(kVariants[vi].fn, p.num_tiles * splits, GEMM_THREADS, split_smem(p.block_n, codes), stream, splits, ma, mb, mc, md, p, splits) != cudaSuccess)
     return GEMM_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
 }

@@ -343,6 +343,12 @@ struct Epilogue {
   const float* col_bias;       // [N] or null
   const float* row_bias;       // [M] or null
   const float* row_scale;      // one value, or null: 1
+  // also the codes of Eq. 1 of the stored values, as bf16 numbers in the layout of `out` (null: none): one symmetric quantizer per
+  // code_cols columns (a multiple of 32), at most three
+  void* codes = nullptr;
+  const float* code_step[3] = {nullptr, nullptr, nullptr};
+  int code_cols = 0;
+  float code_max = 0.f;
 };
 __device__ __forceinline__ float row_term(const Epilogue& e, int row) {
   return e.row_bias ? (e.row_scale ? *e.row_scale : 1.f) * e.row_bias[row] : 0.f;

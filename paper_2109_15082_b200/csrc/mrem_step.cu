@@ -40,6 +40,11 @@ struct Epi {                       // shorthand builder of an Epilogue
   Epi& rowbias(const float* p, const float* scale) { e.row_bias = p; e.row_scale = scale; return *this; }
   Epi& residual(const void* p) { e.residual = p; return *this; }
   Epi& gelu() { e.act = 1; return *this; }
+  // the codes of three segments of `cols` columns beside the stored values
+  Epi& codes3(void* p, const float* s0, const float* s1, const float* s2, int cols, float hi) {
+    e.codes = p; e.code_step[0] = s0; e.code_step[1] = s1; e.code_step[2] = s2; e.code_cols = cols; e.code_max = hi;
+    return *this;
+  }
 };
 
 struct Runner {
@@ -209,10 +214,15 @@ int student_forward(mrem_ctx* c, const void* x, const int32_t* len, int B, int S
 
     // (layers above the first get the codes of their input from the LayerNorm that produced it)
     if (l == 0) launch_quantize_act(cur, c->dt, M, H, H, b.a_steps[S_X], nullptr, rx.lo, rx.hi, s.x_q8, H, s.x_qt, H, c->stream);
-    r.gemm_i8(s.x_q8, 0, w[W_QKV].codes, (int)M, 3 * H, H,
-              Epi(s.qkv, ok, 3 * H).alpha(1.f, b.a_steps[S_X]).colscale(w[W_QKV].scale).colbias(b.student[MREM_BQKV]).e);
-    launch_quantize_act3(s.qkv, c->dt, M, H, 3 * H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], rx.lo, rx.hi, s.qkv_qt,
-                         3 * H, c->stream);
+    Epi eq(s.qkv, ok, 3 * H);
+    eq.alpha(1.f, b.a_steps[S_X]).colscale(w[W_QKV].scale).colbias(b.student[MREM_BQKV]);
+    // the codes of Q, K and V from the product's epilogue, where its tiled stores apply
+    const bool qkv_codes = c->dt == 1 && H % 32 == 0;
+    if (qkv_codes) eq.codes3(s.qkv_qt, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], H, (float)rx.hi);
+    r.gemm_i8(s.x_q8, 0, w[W_QKV].codes, (int)M, 3 * H, H, eq.e);
+    if (!qkv_codes)
+      launch_quantize_act3(s.qkv, c->dt, M, H, 3 * H, b.a_steps[S_Q], b.a_steps[S_K], b.a_steps[S_V], rx.lo, rx.hi, s.qkv_qt,
+                           3 * H, c->stream);
     if (attention_fwd_supported(S, hd, c->dt)) {
       // (the fused attention backward forms the probabilities again from the codes of Q and K and the row
       //  statistics: they and their codes are written out only for the kernel-per-operation backward)
