@@ -21,12 +21,11 @@ namespace mrem {
 namespace {
 
 // Ternary rule: 256 threads per row, up to 4 float4 vectors per thread in registers (rows up to 4096 wide).  Refitted
-// scale: two vectors per thread and as many threads as that takes (rows up to 4096 wide; 96 threads for 768, 384 for
-// 3072: no idle lanes at the encoder's widths).  Wider rows are re-read by 256 threads.
+// scale: two to eight vectors per thread and as many warps as that takes (rows up to 4096 wide).  Wider rows are re-read by
+// 256 threads.
 constexpr int TW_THREADS = 256;
 constexpr int TW_MAXV = 4;
-constexpr int LAQ_V = 2;
-constexpr int LAQ_MAX_WARPS = 16;
+constexpr int LAQ_MAX_WARPS = 4;
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -237,95 +236,137 @@ __device__ __forceinline__ void laq_row(const float* w_row, int cols, int row, i
   }
 }
 
-// The rule on a row held in registers, LAQ_V vectors per thread (missing ones are zeros: their code is 0 and they add
-// nothing).  The rounds that only feed the two sums get them without float64 arithmetic per weight: w / 2^(e - 23), e = the
-// exponent of max|w|, is split once into two integers of 12 bits and a rest of at most 1/2,
-//   w = (4096 nh + nm + nl) 2^(e - 23),
-// so that sums of q nh and q nm over a thread's weights are exact in float32 (below 2^24 for codes of up to 4 bits) and, as
-// integers, over the block; the rest enters at 2^-39 of max|w|.  7 instructions per weight and round instead of 38, four
-// integer warp reductions instead of a float64 butterfly, one barrier instead of two.
-// BERT-base module of three layers: step 1801 -> 1693 us.
-struct LaqShared { int4 sums[2][LAQ_MAX_WARPS]; double d[32]; int i[64]; float f[32]; };
+// The rule on a row held in registers, V vectors of four per thread (missing ones are zeros: their code is 0 and they add
+// nothing), up to LAQ_MAX_WARPS warps a row.  Everything but the codes that go out is the same for w and |w|: <q, w> =
+// <|q|, |w|>, so the rounds work on |w| and need one bound.  The two sums of a round get neither float64 arithmetic nor
+// conversions per weight: with e = the exponent of max|w|, |w| in units of 2^(e - 31) is a whole number of 32 bits for every
+// weight of at least 2^(e - 8), and the others have code 0 while alpha >= 2^(e - 6); its four bytes, each kept beside those of the
+// three neighbouring weights, meet the four codes in byte dot products, and the sums are exact (a byte sum of a block is below
+// 2^23, two of them 8 bits apart below 2^31: codes of up to 4 bits).  Other rows, and more bits, take float64 sums.
+// Bound by instruction issue and latency: 5 instructions per weight and round and about 70 per warp for the sums, so a warp takes a
+// row of up to 1024 alone (no barrier) and three or four take wider ones.  A layer's four matrices, hidden 768, with the update: 145 us
+// with 8 weights a thread (3 warps for 768, 12 for 3072) and float32 sums of two 12-bit parts and a rest, now 107; the step of three
+// layers, 32 x 128 tokens, 1347 -> 1263 us (rows of 768 on three, two, one warp 1324, 1285, 1263).
+template <int V> struct LaqRow { float2 a[2 * V]; uint32_t limb[V][4], neg[V]; };   // |w|; bytes of four; ff where negative
+struct LaqShared { uint4 sums[2][LAQ_MAX_WARPS]; double d[32]; int i[64]; float f[32]; };
 
-template <typename T>
-__device__ __forceinline__ void laq_row_cached(const float4 (&wr)[LAQ_V], int cols, int row, int bits, int8_t* codes_row,
-                                               int32_t* rowsum, float* scale, T* what_row, LaqShared& sh) {
-  constexpr int NW = 4 * LAQ_V;
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {     // (0x8 in a nibble: the byte's sign, eight times)
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
+__device__ __forceinline__ double uint_as_double(uint32_t x) { return __hiloint2double(0x43300000, (int)x) - 4503599627370496.0; }
+
+template <int V>
+__device__ __forceinline__ void laq_take(LaqRow<V>& rw, int i, float4 w) {
+  rw.a[2 * i] = make_float2(fabsf(w.x), fabsf(w.y));
+  rw.a[2 * i + 1] = make_float2(fabsf(w.z), fabsf(w.w));
+  rw.neg[i] = prmt(prmt(__float_as_uint(w.x), __float_as_uint(w.y), 0x00fb), prmt(__float_as_uint(w.z), __float_as_uint(w.w), 0x00fb), 0x5410);
+}
+
+// The codes of four |w| by the division of Eq. 1, one per byte.  (A call: the few weights next to a rounding boundary, and rows
+// without byte sums; inlined at every vector it filled the instruction cache.)
+__device__ __noinline__ uint32_t laq_codes_exact(float4 a, float alpha, float qmax) {
+  return (uint32_t)laq_code(a.x, alpha, qmax) | ((uint32_t)laq_code(a.y, alpha, qmax) << 8) | ((uint32_t)laq_code(a.z, alpha, qmax) << 16) |
+         ((uint32_t)laq_code(a.w, alpha, qmax) << 24);
+}
+__device__ __forceinline__ double laq_dot(uint32_t q, float4 a) {
+  return (uint_as_double(q & 0xffu) * (double)a.x + uint_as_double((q >> 8) & 0xffu) * (double)a.y) +
+         (uint_as_double((q >> 16) & 0xffu) * (double)a.z + uint_as_double(q >> 24) * (double)a.w);
+}
+
+// Sums over the block of v.x, v.y, v.z (and v.w): every thread gets them.  `slot` alternates from call to call.
+template <bool W>
+__device__ __forceinline__ uint4 block_sum_u4(uint4 v, uint4* slot, int wid, int nw) {
+  v.x = __reduce_add_sync(0xffffffffu, v.x);
+  v.y = __reduce_add_sync(0xffffffffu, v.y);
+  v.z = __reduce_add_sync(0xffffffffu, v.z);
+  if (W) v.w = __reduce_add_sync(0xffffffffu, v.w);
+  if (nw == 1) return v;
+  if ((threadIdx.x & 31) == 0) slot[wid] = v;
+  __syncthreads();
+  v = slot[0];
+  for (int k = 1; k < nw; ++k) {
+    const uint4 e = slot[k];
+    v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w;
+  }
+  return v;
+}
+
+template <typename T, int V>
+__device__ __forceinline__ void laq_row_cached(LaqRow<V>& rw, int cols, int row, int bits, int8_t* codes_row, int32_t* rowsum,
+                                               float* scale, T* what_row, LaqShared& sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, nvec = cols / 4;
   const float qmax = (float)((1 << (bits - 1)) - 1);
-  float2 w[NW / 2];
-#pragma unroll
-  for (int i = 0; i < LAQ_V; ++i) { w[2 * i] = make_float2(wr[i].x, wr[i].y); w[2 * i + 1] = make_float2(wr[i].z, wr[i].w); }
   double s = 0.0;
   float mx = 0.f;
 #pragma unroll
-  for (int e = 0; e < NW / 2; ++e) {
-    s += (double)fabsf(w[e].x) + (double)fabsf(w[e].y);
-    mx = fmaxf(mx, fmaxf(fabsf(w[e].x), fabsf(w[e].y)));
+  for (int e = 0; e < 2 * V; ++e) {
+    s += (double)rw.a[e].x + (double)rw.a[e].y;
+    mx = fmaxf(mx, fmaxf(rw.a[e].x, rw.a[e].y));
   }
-  s = block_sum_d(s, sh.d);
-  mx = block_max(mx, sh.f);
+  s = warp_sum_d(s);
+  mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+  if (nw > 1) {
+    if (lane == 0) { sh.d[wid] = s; sh.f[wid] = mx; }
+    __syncthreads();
+    s = sh.d[0];
+    mx = sh.f[0];
+    for (int k = 1; k < nw; ++k) { s += sh.d[k]; mx = fmaxf(mx, sh.f[k]); }
+    __syncthreads();
+  }
   float alpha = (float)(fmin(3.0 * (s / (double)cols), (double)mx) / (double)qmax);
   const bool split = bits <= 4 && mx > 1e-30f && mx < 1e30f;
-  const int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
-  float2 nh[NW / 2], nm[NW / 2], nl[NW / 2];
-  double unit = 0.0;                                       // 2^(ex - 23)
-  if (split) {
-    const float inv_u = __uint_as_float((uint32_t)(127 + 11 - ex) << 23);
-    unit = (double)__uint_as_float((uint32_t)(127 - 23 + ex) << 23);
+  const int eb = (int)(__float_as_uint(mx) >> 23);         // e + 127
+  const float lowest = split ? fmaxf(1e-30f, __uint_as_float((uint32_t)(eb - 6) << 23)) : INFINITY;
+  const double unit = __hiloint2double((eb - 127 - 31 + 1023) << 20, 0);
 #pragma unroll
-    for (int e = 0; e < NW / 2; ++e) {
-      const float tx = w[e].x * inv_u, ty = w[e].y * inv_u;     // exact, below 2^12
-      nh[e] = make_float2(rne_magic(tx), rne_magic(ty));
-      const float ux = (tx - nh[e].x) * 4096.f, uy = (ty - nh[e].y) * 4096.f;
-      nm[e] = make_float2(rne_magic(ux), rne_magic(uy));
-      nl[e] = make_float2(ux - nm[e].x, uy - nm[e].y);
+  for (int i = 0; i < V; ++i) {
+    uint32_t x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t u = __float_as_uint((j & 1) ? rw.a[2 * i + (j >> 1)].y : rw.a[2 * i + (j >> 1)].x);
+      x[j] = __funnelshift_rc((u << 8) | 0x80000000u, 0u, (uint32_t)eb - (u >> 23));   // (32 places or more: 0)
     }
+    const uint32_t l0 = prmt(x[0], x[1], 0x5140), l1 = prmt(x[2], x[3], 0x5140), h0 = prmt(x[0], x[1], 0x7362), h1 = prmt(x[2], x[3], 0x7362);
+    rw.limb[i][0] = prmt(l0, l1, 0x5410);
+    rw.limb[i][1] = prmt(l0, l1, 0x7632);
+    rw.limb[i][2] = prmt(h0, h1, 0x5410);
+    rw.limb[i][3] = prmt(h0, h1, 0x7632);
   }
+  int it = 0;
   for (int r = 0; r + 1 < LAQ_ROUNDS; ++r) {
-    float next;
-    if (split && alpha > 1e-30f) {                         // 1 / alpha and the residual stay in the normal range
+    float next = 0.f;
+    if (alpha >= lowest) {
       const float r_alpha = __frcp_rn(alpha);
-      const float2 r2 = make_float2(r_alpha, r_alpha), na2 = make_float2(-alpha, -alpha), magic2 = make_float2(ROUND_MAGIC, ROUND_MAGIC),
-                   nmagic2 = make_float2(-ROUND_MAGIC, -ROUND_MAGIC);
-      float2 ah = make_float2(0.f, 0.f), am = ah, al = ah, aq = ah;
+      uint32_t b0 = 0u, b1 = 0u, b2 = 0u, b3 = 0u, qq = 0u;
 #pragma unroll
-      for (int e = 0; e < NW / 2; ++e) {                   // (quotient() and the rounding on pairs)
-        const float2 z0 = mul2(w[e], r2), z = fma2(fma2(z0, na2, w[e]), r2, z0);
-        const float2 q = add2(add2(make_float2(fminf(fmaxf(z.x, -qmax), qmax), fminf(fmaxf(z.y, -qmax), qmax)), magic2), nmagic2);
-        ah = fma2(q, nh[e], ah);
-        am = fma2(q, nm[e], am);
-        al = fma2(q, nl[e], al);
-        aq = fma2(q, q, aq);
+      for (int i = 0; i < V; ++i) {
+        const float2 z = quotient2(rw.a[2 * i], splat(-alpha), splat(r_alpha)), y = quotient2(rw.a[2 * i + 1], splat(-alpha), splat(r_alpha));
+        const float2 t = add2(make_float2(fminf(z.x, qmax), fminf(z.y, qmax)), splat(ROUND_MAGIC));
+        const float2 u = add2(make_float2(fminf(y.x, qmax), fminf(y.y, qmax)), splat(ROUND_MAGIC));
+        const uint32_t q = pack_low_bytes(__float_as_uint(t.x), __float_as_uint(t.y), __float_as_uint(u.x), __float_as_uint(u.y));
+        b0 = __dp4a(rw.limb[i][0], q, b0);
+        b1 = __dp4a(rw.limb[i][1], q, b1);
+        b2 = __dp4a(rw.limb[i][2], q, b2);
+        b3 = __dp4a(rw.limb[i][3], q, b3);
+        qq = __dp4a(q, q, qq);
       }
-      const int4 mine = make_int4(__reduce_add_sync(0xffffffffu, __float2int_rn(ah.x + ah.y)), __reduce_add_sync(0xffffffffu, __float2int_rn(am.x + am.y)),
-                                  __reduce_add_sync(0xffffffffu, __float2int_rn((al.x + al.y) * 65536.f)), __reduce_add_sync(0xffffffffu, __float2int_rn(aq.x + aq.y)));
-      if (lane == 0) sh.sums[r & 1][wid] = mine;
-      __syncthreads();
-      int4 t = make_int4(0, 0, 0, 0);
-      if (nw <= 4) {
-        for (int k = 0; k < nw; ++k) {
-          const int4 v = sh.sums[r & 1][k];
-          t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
-        }
-      } else {
-        if (lane < nw) t = sh.sums[r & 1][lane];
-        t = make_int4(__reduce_add_sync(0xffffffffu, t.x), __reduce_add_sync(0xffffffffu, t.y), __reduce_add_sync(0xffffffffu, t.z),
-                      __reduce_add_sync(0xffffffffu, t.w));
-      }
+      const uint4 t = block_sum_u4<false>(make_uint4(b0 + (b1 << 8), b2 + (b3 << 8), qq, 0u), sh.sums[it++ & 1], wid, nw);
       // <q, w> / <q, q>: float32 quotient and one correction from the float64 residual (2^-46 before the rounding to float32)
-      const double qw = fma((double)t.z, 1.52587890625e-05, fma((double)t.x, 4096.0, (double)t.y)) * unit;
-      const float rq = __frcp_rn((float)t.w), a0 = (float)qw * rq;
-      next = t.w > 0 ? (float)fma(fma(-(double)a0, (double)t.w, qw), (double)rq, (double)a0) : 0.f;
+      const double qw = fma(uint_as_double(t.y), 65536.0, uint_as_double(t.x)) * unit, n = uint_as_double(t.z);
+      const float rq = __frcp_rn((float)t.z), a0 = (float)qw * rq;
+      if (t.z) next = (float)fma(fma(-(double)a0, n, qw), (double)rq, (double)a0);
     } else {
       double qw = 0.0;
       int qq = 0;
       if (alpha > 0.f) {
 #pragma unroll
-        for (int e = 0; e < NW / 2; ++e) {
-          const int qx = laq_code(w[e].x, alpha, qmax), qy = laq_code(w[e].y, alpha, qmax);
-          qw += (double)qx * (double)w[e].x + (double)qy * (double)w[e].y;
-          qq += qx * qx + qy * qy;
+        for (int i = 0; i < V; ++i) {
+          const float4 a4 = make_float4(rw.a[2 * i].x, rw.a[2 * i].y, rw.a[2 * i + 1].x, rw.a[2 * i + 1].y);
+          const uint32_t q = laq_codes_exact(a4, alpha, qmax);
+          qw += laq_dot(q, a4);
+          qq += (int)__dp4a(q, q, 0u);
         }
       }
       block_sum_di(qw, qq, sh.d, sh.i);
@@ -334,87 +375,89 @@ __device__ __forceinline__ void laq_row_cached(const float4 (&wr)[LAQ_V], int co
     if (next == alpha) break;
     alpha = next;
   }
-  // last round: the codes of this alpha (by the division of Eq. 1) go out with the scale refitted to them (float64)
-  double qw = 0.0;
-  int qq = 0, sum = 0;
-  float q[NW];
-  const bool normal = alpha > 1e-30f && alpha < 1e30f;
+  // last round: the codes of this alpha (by the division of Eq. 1) go out with the scale refitted to them
+  const bool whole = alpha >= lowest;
   const float r_alpha = __frcp_rn(alpha);
+  double qw = 0.0;
+  uint32_t b0 = 0u, b1 = 0u, b2 = 0u, b3 = 0u, qq = 0u, code[V];
+  int sum = 0;
 #pragma unroll
-  for (int i = 0; i < LAQ_V; ++i) {
+  for (int i = 0; i < V; ++i) {
     const int c = threadIdx.x + i * blockDim.x;
-    uint32_t b[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = 4 * i + j;
-      const float we = (j & 1) ? w[e >> 1].y : w[e >> 1].x;
-      int k = 0;
-      q[e] = 0.f;
-      if (normal) {
-        q[e] = code_f<false>(we, alpha, r_alpha, -qmax, qmax, b[j]);
-        k = (int)(int8_t)(b[j] & 0xffu);
-      } else if (alpha > 0.f) {
-        k = laq_code(we, alpha, qmax);
-        q[e] = (float)k;
-        b[j] = (uint32_t)k;
-      }
-      qw += int_as_double(k) * (double)we;
-      qq += k * k;
-      sum += k;
+    const float4 a4 = make_float4(rw.a[2 * i].x, rw.a[2 * i].y, rw.a[2 * i + 1].x, rw.a[2 * i + 1].y);
+    uint32_t q = 0u, k[4];
+    bool again = !whole;
+    if (whole) {
+      const float2 z = quotient2(rw.a[2 * i], splat(-alpha), splat(r_alpha)), y = quotient2(rw.a[2 * i + 1], splat(-alpha), splat(r_alpha));
+      const float2 zc = make_float2(fminf(z.x, qmax), fminf(z.y, qmax)), yc = make_float2(fminf(y.x, qmax), fminf(y.y, qmax));
+      const float2 t = rne_magic2(zc, k[0], k[1]), u = rne_magic2(yc, k[2], k[3]);
+      again = fmaxf(fmaxf(fabsf(zc.x - t.x), fabsf(zc.y - t.y)), fmaxf(fabsf(yc.x - u.x), fabsf(yc.y - u.y))) > 0.5f - HALF_WINDOW;
+      q = pack_low_bytes(k[0], k[1], k[2], k[3]);
     }
-    if (c < nvec) *reinterpret_cast<uint32_t*>(codes_row + 4 * c) = pack_low_bytes(b[0], b[1], b[2], b[3]);
+    if (again) q = alpha > 0.f ? laq_codes_exact(a4, alpha, qmax) : 0u;
+    if (!whole) qw += laq_dot(q, a4);
+    b0 = __dp4a(rw.limb[i][0], q, b0);
+    b1 = __dp4a(rw.limb[i][1], q, b1);
+    b2 = __dp4a(rw.limb[i][2], q, b2);
+    b3 = __dp4a(rw.limb[i][3], q, b3);
+    qq = __dp4a(q, q, qq);
+    code[i] = (q & ~rw.neg[i]) | (((0x80808080u - q) ^ 0x80808080u) & rw.neg[i]);    // (no borrow: codes are at most 127)
+    sum = __dp4a((int)code[i], 0x01010101, sum);
+    if (c < nvec) *reinterpret_cast<uint32_t*>(codes_row + 4 * c) = code[i];
   }
-  qw = warp_sum_d(qw);
-  qq = __reduce_add_sync(0xffffffffu, qq);
-  sum = __reduce_add_sync(0xffffffffu, sum);
-  __syncthreads();
-  if (lane == 0) { sh.d[wid] = qw; sh.i[wid] = qq; sh.i[32 + wid] = sum; }
-  __syncthreads();
-  qw = warp_sum_d(lane < nw ? sh.d[lane] : 0.0);
-  qq = __reduce_add_sync(0xffffffffu, lane < nw ? sh.i[lane] : 0);
-  const float next = qq > 0 ? (float)(qw / (double)qq) : 0.f;
+  const uint4 t = block_sum_u4<true>(make_uint4(b0 + (b1 << 8), b2 + (b3 << 8), qq, (uint32_t)sum), sh.sums[it & 1], wid, nw);
+  if (whole) {
+    qw = fma(uint_as_double(t.y), 65536.0, uint_as_double(t.x)) * unit;
+  } else {
+    int none = 0;
+    block_sum_di(qw, none, sh.d, sh.i);
+  }
+  float next = t.z ? (float)(qw / uint_as_double(t.z)) : 0.f;
+  if (!(s == s)) next = (float)s;                          // a weight that is not a number has no byte sums, and no scale either
   if (what_row) {
 #pragma unroll
-    for (int i = 0; i < LAQ_V; ++i) {
+    for (int i = 0; i < V; ++i) {
       const int c = threadIdx.x + i * blockDim.x;
-      if (c < nvec) store4<T>(what_row + 4 * c, next * q[4 * i], next * q[4 * i + 1], next * q[4 * i + 2], next * q[4 * i + 3]);
+      const uint32_t u = code[i] ^ 0x80808080u;            // code + 128, then 2^23 + code + 128 as a float
+      auto value = [&](uint32_t sel) { return next * (__uint_as_float(prmt(u, 0x4b000000u, sel)) - 8388736.f); };
+      if (c < nvec) store4<T>(what_row + 4 * c, value(0x7650), value(0x7651), value(0x7652), value(0x7653));
     }
   }
-  if (wid == 0) {
-    sum = __reduce_add_sync(0xffffffffu, lane < nw ? sh.i[32 + lane] : 0);
-    if (lane == 0) {
-      rowsum[row] = sum;
-      scale[row] = next;
-    }
+  if (threadIdx.x == 0) {
+    rowsum[row] = (int)t.w;
+    scale[row] = next;
   }
 }
 
-// The two kernels of the refitted scale on rows held in registers; NT: upper bound of the block size.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) laq_quantize_kernel(const float* __restrict__ w, int cols, int bits,
-                                                                     int8_t* __restrict__ codes, int32_t* __restrict__ rowsum,
-                                                                     float* __restrict__ scale, T* __restrict__ what) {
+// Blocks of the two kernels below that an SM is to hold (registers: about 9 V and 35)
+constexpr int laq_blocks(int V) { return V == 8 ? 4 : (V == 6 ? 5 : (V == 4 ? 6 : 8)); }
+
+// The two kernels of the refitted scale on rows held in registers.
+template <typename T, int V>
+__global__ void __launch_bounds__(32 * LAQ_MAX_WARPS, laq_blocks(V)) laq_quantize_kernel(const float* __restrict__ w, int cols, int bits,
+                                                                                       int8_t* __restrict__ codes, int32_t* __restrict__ rowsum,
+                                                                                       float* __restrict__ scale, T* __restrict__ what) {
   pdl_wait();
   pdl_trigger();
   __shared__ LaqShared sh;
   const long long base = (long long)blockIdx.x * cols;
   const float4* w4 = reinterpret_cast<const float4*>(w + base);
-  float4 wr[LAQ_V];
+  LaqRow<V> rw;
 #pragma unroll
-  for (int i = 0; i < LAQ_V; ++i) {
+  for (int i = 0; i < V; ++i) {
     const int c = threadIdx.x + i * blockDim.x;
-    wr[i] = c < cols / 4 ? w4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+    laq_take(rw, i, c < cols / 4 ? w4[c] : make_float4(0.f, 0.f, 0.f, 0.f));
   }
-  laq_row_cached<T>(wr, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
+  laq_row_cached<T, V>(rw, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) laq_update_kernel(float* __restrict__ w, const float* __restrict__ g,
-                                                                   float* __restrict__ m, float* __restrict__ v,
-                                                                   const OptimScalars* __restrict__ sc, int cols, int train_w,
-                                                                   int bits, int8_t* __restrict__ codes,
-                                                                   int32_t* __restrict__ rowsum, float* __restrict__ scale,
-                                                                   T* __restrict__ what) {
+template <typename T, int V>
+__global__ void __launch_bounds__(32 * LAQ_MAX_WARPS, laq_blocks(V)) laq_update_kernel(float* __restrict__ w, const float* __restrict__ g,
+                                                                                     float* __restrict__ m, float* __restrict__ v,
+                                                                                     const OptimScalars* __restrict__ sc, int cols, int train_w,
+                                                                                     int bits, int8_t* __restrict__ codes,
+                                                                                     int32_t* __restrict__ rowsum, float* __restrict__ scale,
+                                                                                     T* __restrict__ what) {
   pdl_wait();
   pdl_trigger();
   __shared__ LaqShared sh;
@@ -425,21 +468,24 @@ __global__ void __launch_bounds__(NT, 1024 / NT) laq_update_kernel(float* __rest
   const float4* g4 = reinterpret_cast<const float4*>(g + base);
   float4* m4 = reinterpret_cast<float4*>(m + base);
   float4* v4 = reinterpret_cast<float4*>(v + base);
-  float4 wr[LAQ_V], gr[LAQ_V], mr[LAQ_V], vr[LAQ_V];
+  constexpr int N = V <= 4 ? 2 : V / 2;                    // vectors whose loads are in flight together
+  LaqRow<V> rw;
 #pragma unroll
-  for (int i = 0; i < LAQ_V; ++i) {                        // all loads in flight first
-    const int c = threadIdx.x + i * blockDim.x;
-    wr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (c < nvec) {
-      wr[i] = w4[c];
-      if (train_w) { gr[i] = g4[c]; mr[i] = m4[c]; vr[i] = v4[c]; }
-    }
-  }
-  if (train_w) {
+  for (int i0 = 0; i0 < V; i0 += N) {
+    float4 wr[N], gr[N], mr[N], vr[N];
 #pragma unroll
-    for (int i = 0; i < LAQ_V; ++i) {
-      const int c = threadIdx.x + i * blockDim.x;
+    for (int i = 0; i < N; ++i) {
+      const int c = threadIdx.x + (i0 + i) * blockDim.x;
+      wr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (c < nvec) {
+        wr[i] = w4[c];
+        if (train_w) { gr[i] = g4[c]; mr[i] = m4[c]; vr[i] = v4[c]; }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int c = threadIdx.x + (i0 + i) * blockDim.x;
+      if (train_w && c < nvec) {
         wr[i].x = adam_one(wr[i].x, gr[i].x, mr[i].x, vr[i].x, o, 1.f, -INFINITY);
         wr[i].y = adam_one(wr[i].y, gr[i].y, mr[i].y, vr[i].y, o, 1.f, -INFINITY);
         wr[i].z = adam_one(wr[i].z, gr[i].z, mr[i].z, vr[i].z, o, 1.f, -INFINITY);
@@ -448,15 +494,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) laq_update_kernel(float* __rest
         m4[c] = mr[i];
         v4[c] = vr[i];
       }
+      laq_take(rw, i0 + i, wr[i]);
     }
   }
-  laq_row_cached<T>(wr, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
+  laq_row_cached<T, V>(rw, cols, blockIdx.x, bits, codes + base, rowsum, scale, what ? what + base : nullptr, sh);
 }
 
-// Block size of the two kernels above, or 0 when the row does not fit.
-inline int laq_threads(int cols) {
-  const int warps = (cols / 4 + 32 * LAQ_V - 1) / (32 * LAQ_V);
-  return warps <= LAQ_MAX_WARPS ? 32 * warps : 0;
+// Vectors per thread (2, 4, 6 or 8) and warps of the two kernels above: the fewest instructions a round, the sums of a warp
+// counted as those of three vectors; 0 warps when the row does not fit.
+inline int laq_warps(int cols, int& V) {
+  const int n = (cols / 4 + 31) / 32;
+  int warps = 0;
+  for (int t = 2; t <= 8; t += 2) {
+    const int k = (n + t - 1) / t;
+    if (k <= LAQ_MAX_WARPS && (!warps || k * (t + 3) < warps * (V + 3))) { warps = k; V = t; }
+  }
+  return warps;
 }
 
 template <typename T, int RULE, int NT, int MAXV>
@@ -553,15 +606,20 @@ void launch_closed_form_quantize(const float* w, int rows, int cols, int rule, i
                                  float* scale, void* what, int dt, cudaStream_t st) {
   Scope sc("quantize_weight", (double)rows * cols * (5.0 + (what ? (dt == 1 ? 2.0 : 4.0) : 0.0)) + rows * 8.0, 0, st);
   auto go = [&](auto kernel, int nt, auto* out) { launch_k(kernel, rows, nt, 0, st, w, cols, bits, codes, rowsum, scale, out); };
-  const int nt = rule == 3 ? laq_threads(cols) : 0;
+  int V = 0;
+  const int warps = rule == 3 ? laq_warps(cols, V) : 0;
   if (dt == 1) {
-    if (nt > 128) go(laq_quantize_kernel<bf16, 512>, nt, (bf16*)what);
-    else if (nt) go(laq_quantize_kernel<bf16, 128>, nt, (bf16*)what);
+    if (warps && V == 2) go(laq_quantize_kernel<bf16, 2>, 32 * warps, (bf16*)what);
+    else if (warps && V == 4) go(laq_quantize_kernel<bf16, 4>, 32 * warps, (bf16*)what);
+    else if (warps && V == 6) go(laq_quantize_kernel<bf16, 6>, 32 * warps, (bf16*)what);
+    else if (warps) go(laq_quantize_kernel<bf16, 8>, 32 * warps, (bf16*)what);
     else if (rule == 3) go(closed_form_quantize_kernel<bf16, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
     else go(closed_form_quantize_kernel<bf16, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
   } else {
-    if (nt > 128) go(laq_quantize_kernel<float, 512>, nt, (float*)what);
-    else if (nt) go(laq_quantize_kernel<float, 128>, nt, (float*)what);
+    if (warps && V == 2) go(laq_quantize_kernel<float, 2>, 32 * warps, (float*)what);
+    else if (warps && V == 4) go(laq_quantize_kernel<float, 4>, 32 * warps, (float*)what);
+    else if (warps && V == 6) go(laq_quantize_kernel<float, 6>, 32 * warps, (float*)what);
+    else if (warps) go(laq_quantize_kernel<float, 8>, 32 * warps, (float*)what);
     else if (rule == 3) go(closed_form_quantize_kernel<float, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
     else go(closed_form_quantize_kernel<float, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
   }
@@ -574,15 +632,20 @@ void launch_closed_form_update(float* w, const float* g, float* m, float* v, con
   auto go = [&](auto kernel, int nt, auto* out) {
     launch_k(kernel, rows, nt, 0, st, w, g, m, v, sc, cols, train_w, bits, codes, rowsum, scale, out);
   };
-  const int nt = rule == 3 ? laq_threads(cols) : 0;
+  int V = 0;
+  const int warps = rule == 3 ? laq_warps(cols, V) : 0;
   if (dt == 1) {
-    if (nt > 128) go(laq_update_kernel<bf16, 512>, nt, (bf16*)what);
-    else if (nt) go(laq_update_kernel<bf16, 128>, nt, (bf16*)what);
+    if (warps && V == 2) go(laq_update_kernel<bf16, 2>, 32 * warps, (bf16*)what);
+    else if (warps && V == 4) go(laq_update_kernel<bf16, 4>, 32 * warps, (bf16*)what);
+    else if (warps && V == 6) go(laq_update_kernel<bf16, 6>, 32 * warps, (bf16*)what);
+    else if (warps) go(laq_update_kernel<bf16, 8>, 32 * warps, (bf16*)what);
     else if (rule == 3) go(closed_form_update_kernel<bf16, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
     else go(closed_form_update_kernel<bf16, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (bf16*)what);
   } else {
-    if (nt > 128) go(laq_update_kernel<float, 512>, nt, (float*)what);
-    else if (nt) go(laq_update_kernel<float, 128>, nt, (float*)what);
+    if (warps && V == 2) go(laq_update_kernel<float, 2>, 32 * warps, (float*)what);
+    else if (warps && V == 4) go(laq_update_kernel<float, 4>, 32 * warps, (float*)what);
+    else if (warps && V == 6) go(laq_update_kernel<float, 6>, 32 * warps, (float*)what);
+    else if (warps) go(laq_update_kernel<float, 8>, 32 * warps, (float*)what);
     else if (rule == 3) go(closed_form_update_kernel<float, 3, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
     else go(closed_form_update_kernel<float, 2, TW_THREADS, TW_MAXV>, TW_THREADS, (float*)what);
   }
