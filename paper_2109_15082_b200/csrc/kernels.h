@@ -18,14 +18,11 @@ void launch_quantize_weight(const float* w, int rows, int cols, const float* ste
 // Weight codes with a scale recomputed from the weights, one step-free rule per output row (Sec. 5.1 names one for
 // 2-bit and one for 4-bit weights).  rule 2: ternary, delta = 0.7 mean|w|, codes sign(w) 1[|w| > delta], scale =
 // mean of the kept |w|.  rule 3: codes in Omega(bits) and scale by alternating least squares (q = Pi(w / alpha),
-// alpha = <q, w> / <q, q>) from min(3 mean|w|, max|w|) / qmax.  The fused update is AdamW with the gradient of
+// alpha = <q, w> / <q, q>) from min(3 mean|w|, max|w|) / qmax.  The fused update (below) is AdamW with the gradient of
 // w_hat passed through unchanged, then the rule on the new weights.
 void launch_closed_form_quantize(const float* w, int rows, int cols, int rule, int bits, int8_t* codes, int32_t* rowsum,
                                  float* scale, void* what, int dt, cudaStream_t st);
 struct OptimScalars;
-void launch_closed_form_update(float* w, const float* g, float* m, float* v, const OptimScalars* sc, int rows, int cols,
-                               int train_w, int rule, int bits, int8_t* codes, int32_t* rowsum, float* scale, void* what,
-                               int dt, cudaStream_t st);
 
 // Activation quantizer over a 2-D view x[rows, cols] with row stride ld_x:
 // z = (x - offset) / step, q = rne(clip(z, lo, hi)).  Writes int8/uint8 codes (row stride
@@ -218,7 +215,9 @@ constexpr int MAX_ROW_UPDATES = 4;
 // `n` matrices (at most MAX_ROW_UPDATES) in one launch.
 void launch_fused_weight_update(const RowUpdate* mats, int n, const OptimScalars* sc, int bits, int grid, int train_w, int train_s,
                                 int dt, cudaStream_t st, bool twins = false);
-// The same of a table (grid 0, no dequantized rows) whose rows `tokens` gathered, and of the idle rows of a range in the same launch.
+// The update with a closed-form scale (rule 2 or 3 of launch_closed_form_quantize) of `n` matrices, one launch per row kernel they take.
+void launch_closed_form_update(const RowUpdate* mats, int n, const OptimScalars* sc, int train_w, int rule, int bits, int dt, cudaStream_t st);
+// The same as the fused update of a table (grid 0, no dequantized rows) whose rows `tokens` gathered, and of the idle rows of a range in the same launch.
 struct TokenRows { const int* ids; const unsigned* row_first; int n; };      // n tokens; the first one with an id, per row
 struct IdleRows;                                                             // row_update.cuh
 void launch_table_update(const IdleRows& idle, const TokenRows& tokens, int dt, cudaStream_t st);

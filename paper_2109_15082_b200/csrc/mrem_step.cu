@@ -277,14 +277,11 @@ void enqueue_matrix_updates(mrem_ctx* c, int l, int k0, int n, cudaStream_t st, 
   for (int i = 0; i < n; ++i) {
     const int k = k0 + i, pid = kMatParam[k];
     WeightBuf& w = c->wq[l][k];
-    if (closed_form_weights(d))
-      launch_closed_form_update(c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->optim_sc, w.rows, w.cols, train_w,
-                                d.w_grid, d.w_bits, w.codes, w.rowsum, w.scale, w.what, c->dt, st);
-    else
-      mats[i] = RowUpdate{c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->bind[l].w_steps[k], g.m_ws[k], g.v_ws[k],
-                          c->w_ste_done ? g.ws[k] : nullptr, w.codes, w.rowsum, w.scale, w.what, w.rows, w.cols};
+    mats[i] = RowUpdate{c->bind[l].student[pid], g.p[pid], g.m_p[pid], g.v_p[pid], c->bind[l].w_steps[k], g.m_ws[k], g.v_ws[k],
+                        c->w_ste_done ? g.ws[k] : nullptr, w.codes, w.rowsum, w.scale, w.what, w.rows, w.cols};
   }
-  if (!closed_form_weights(d)) launch_fused_weight_update(mats, n, c->optim_sc, d.w_bits, d.w_grid, train_w, train_s, c->dt, st, twins);
+  if (closed_form_weights(d)) launch_closed_form_update(mats, n, c->optim_sc, train_w, d.w_grid, d.w_bits, c->dt, st);
+  else launch_fused_weight_update(mats, n, c->optim_sc, d.w_bits, d.w_grid, train_w, train_s, c->dt, st, twins);
 }
 
 // ------------------------------------------------------------------ backward
