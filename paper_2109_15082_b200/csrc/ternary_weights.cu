@@ -270,6 +270,16 @@ __device__ __noinline__ uint32_t laq_codes_exact(float4 a, float alpha, float qm
   return (uint32_t)laq_code(a.x, alpha, qmax) | ((uint32_t)laq_code(a.y, alpha, qmax) << 8) | ((uint32_t)laq_code(a.z, alpha, qmax) << 16) |
          ((uint32_t)laq_code(a.w, alpha, qmax) << 24);
 }
+// The same without the division but where it decides (code_f); alpha in (1e-30, 1e30).
+__device__ __forceinline__ uint32_t laq_codes(float4 a, float alpha, float r_alpha, float qmax) {
+  const float2 z = quotient2(make_float2(a.x, a.y), splat(-alpha), splat(r_alpha)), y = quotient2(make_float2(a.z, a.w), splat(-alpha), splat(r_alpha));
+  const float2 zc = make_float2(fminf(z.x, qmax), fminf(z.y, qmax)), yc = make_float2(fminf(y.x, qmax), fminf(y.y, qmax));
+  uint32_t k[4];
+  const float2 t = rne_magic2(zc, k[0], k[1]), u = rne_magic2(yc, k[2], k[3]);
+  if (fmaxf(fmaxf(fabsf(zc.x - t.x), fabsf(zc.y - t.y)), fmaxf(fabsf(yc.x - u.x), fabsf(yc.y - u.y))) > 0.5f - HALF_WINDOW)
+    return laq_codes_exact(a, alpha, qmax);
+  return pack_low_bytes(k[0], k[1], k[2], k[3]);
+}
 __device__ __forceinline__ double laq_dot(uint32_t q, float4 a) {
   return (uint_as_double(q & 0xffu) * (double)a.x + uint_as_double((q >> 8) & 0xffu) * (double)a.y) +
          (uint_as_double((q >> 16) & 0xffu) * (double)a.z + uint_as_double(q >> 24) * (double)a.w);
@@ -361,10 +371,12 @@ __device__ __forceinline__ void laq_row_cached(LaqRow<V>& rw, int cols, int row,
       double qw = 0.0;
       int qq = 0;
       if (alpha > 0.f) {
+        const bool normal = alpha > 1e-30f && alpha < 1e30f;
+        const float r_alpha = __frcp_rn(alpha);
 #pragma unroll
         for (int i = 0; i < V; ++i) {
           const float4 a4 = make_float4(rw.a[2 * i].x, rw.a[2 * i].y, rw.a[2 * i + 1].x, rw.a[2 * i + 1].y);
-          const uint32_t q = laq_codes_exact(a4, alpha, qmax);
+          const uint32_t q = normal ? laq_codes(a4, alpha, r_alpha, qmax) : laq_codes_exact(a4, alpha, qmax);
           qw += laq_dot(q, a4);
           qq += (int)__dp4a(q, q, 0u);
         }
@@ -376,7 +388,7 @@ __device__ __forceinline__ void laq_row_cached(LaqRow<V>& rw, int cols, int row,
     alpha = next;
   }
   // last round: the codes of this alpha (by the division of Eq. 1) go out with the scale refitted to them
-  const bool whole = alpha >= lowest;
+  const bool whole = alpha >= lowest, normal = alpha > 1e-30f && alpha < 1e30f;
   const float r_alpha = __frcp_rn(alpha);
   double qw = 0.0;
   uint32_t b0 = 0u, b1 = 0u, b2 = 0u, b3 = 0u, qq = 0u, code[V];
@@ -385,16 +397,7 @@ __device__ __forceinline__ void laq_row_cached(LaqRow<V>& rw, int cols, int row,
   for (int i = 0; i < V; ++i) {
     const int c = threadIdx.x + i * blockDim.x;
     const float4 a4 = make_float4(rw.a[2 * i].x, rw.a[2 * i].y, rw.a[2 * i + 1].x, rw.a[2 * i + 1].y);
-    uint32_t q = 0u, k[4];
-    bool again = !whole;
-    if (whole) {
-      const float2 z = quotient2(rw.a[2 * i], splat(-alpha), splat(r_alpha)), y = quotient2(rw.a[2 * i + 1], splat(-alpha), splat(r_alpha));
-      const float2 zc = make_float2(fminf(z.x, qmax), fminf(z.y, qmax)), yc = make_float2(fminf(y.x, qmax), fminf(y.y, qmax));
-      const float2 t = rne_magic2(zc, k[0], k[1]), u = rne_magic2(yc, k[2], k[3]);
-      again = fmaxf(fmaxf(fabsf(zc.x - t.x), fabsf(zc.y - t.y)), fmaxf(fabsf(yc.x - u.x), fabsf(yc.y - u.y))) > 0.5f - HALF_WINDOW;
-      q = pack_low_bytes(k[0], k[1], k[2], k[3]);
-    }
-    if (again) q = alpha > 0.f ? laq_codes_exact(a4, alpha, qmax) : 0u;
+    const uint32_t q = normal ? laq_codes(a4, alpha, r_alpha, qmax) : (alpha > 0.f ? laq_codes_exact(a4, alpha, qmax) : 0u);
     if (!whole) qw += laq_dot(q, a4);
     b0 = __dp4a(rw.limb[i][0], q, b0);
     b1 = __dp4a(rw.limb[i][1], q, b1);
