@@ -245,7 +245,7 @@ __device__ __forceinline__ void laq_row(const float* w_row, int cols, int row, i
 // 2^23, two of them 8 bits apart below 2^31: codes of up to 4 bits).  Other rows, and more bits, take float64 sums.
 // Bound by instruction issue and latency: 5 instructions per weight and round and about 70 per warp for the sums, so a warp takes a
 // row of up to 1024 alone (no barrier) and three or four take wider ones.  A layer's four matrices, hidden 768, with the update: 145 us
-// with 8 weights a thread (3 warps for 768, 12 for 3072) and float32 sums of two 12-bit parts and a rest, now 107; the step of three
+// with 8 weights a thread (3 warps for 768, 12 for 3072) and float32 sums of two 12-bit parts and a rest, now 107 (75 in shared launches, below); the step of three
 // layers, 32 x 128 tokens, 1347 -> 1263 us (rows of 768 on three, two, one warp 1324, 1285, 1263).
 template <int V> struct LaqRow { float2 a[2 * V]; uint32_t limb[V][4], neg[V]; };   // |w|; bytes of four; ff where negative
 struct LaqShared { uint4 sums[2][LAQ_MAX_WARPS]; double d[32]; int i[64]; float f[32]; };
